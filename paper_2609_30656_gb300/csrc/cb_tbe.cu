@@ -16,14 +16,6 @@ using namespace cbtbe;
 
 namespace {
 
-#ifndef CB_FWD_CHUNK
-#define CB_FWD_CHUNK 512
-#endif
-#ifndef CB_BWD_CHUNK
-#define CB_BWD_CHUNK 512
-#endif
-constexpr int64_t kFwdChunk = CB_FWD_CHUNK;  // lookups per forward chunk
-constexpr int64_t kBwdChunk = CB_BWD_CHUNK;  // sorted positions per reduce chunk
 constexpr uint64_t kLookbackTimeoutNs = 1000000000ull;  // 1 s bounded wait
 constexpr int kNumTimers = 7;
 const char* const kComponentNames[kNumTimers] = {"fwd.prep",   "fwd.gather", "fwd.fixup",
@@ -182,8 +174,7 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
     };
     const int64_t T = h->T;
     const int64_t nc = std::max<size_t>(h->fwd_classes.size(), h->bwd_classes.size());
-    const int64_t chunk = std::min(kFwdChunk, kBwdChunk);
-    const int64_t max_chunks = n / chunk + T + 1;
+    const int64_t max_chunks = chunk_count_limit(n, h->num_sms, T);
     Workspace ws;
     ws.max_chunks = max_chunks;
     ws.table_pos = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
@@ -283,7 +274,8 @@ Problem make_problem(const cb_tbe* h, int32_t B, const void* indices, int64_t n,
     return P;
 }
 
-Plan make_plan(const cb_tbe* h, const Workspace& w, bool bwd, int64_t chunk_len) {
+Plan make_plan(const cb_tbe* h, const Workspace& w, bool bwd, int64_t n) {
+    const int64_t chunk_len = chunk_len_for(n, h->num_sms);
     Plan Q;
     Q.chunk_len = static_cast<int32_t>(chunk_len);
     // Chunk boundaries move to the end of the bag / run they cut unless it is
@@ -370,8 +362,8 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     if (st != CB_OK) return st;
     Workspace w;
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
-    Plan Q = make_plan(h, w, true, kBwdChunk);
-    const int64_t bound = n / kBwdChunk + h->T + 1;
+    Plan Q = make_plan(h, w, true, n);
+    const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
     const bool packed = per_sample_weights != nullptr || h->mode == CB_POOL_MEAN;
 
     // (1) keys and payloads
@@ -737,8 +729,8 @@ cb_status cb_tbe_forward(cb_tbe* h, int32_t batch, const void* indices, int64_t 
     if (st != CB_OK) return st;
     Workspace w;
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
-    Plan Q = make_plan(h, w, false, kFwdChunk);
-    const int64_t bound = n / kFwdChunk + h->T + 1;
+    Plan Q = make_plan(h, w, false, n);
+    const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
     launch_plan(P, Q, 0, nullptr, nullptr, h->num_sms, true, stream);
     h->launches += 2;
     record(h, h->ev_fwd[1], stream);
@@ -778,8 +770,8 @@ cb_status cb_tbe_weight_grad(cb_tbe* h, int32_t batch, const void* indices, int6
     if (st != CB_OK) return st;
     Workspace w;
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
-    Plan Q = make_plan(h, w, false, kFwdChunk);
-    const int64_t bound = n / kFwdChunk + h->T + 1;
+    Plan Q = make_plan(h, w, false, n);
+    const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
     launch_plan(P, Q, 0, nullptr, nullptr, h->num_sms, true, stream);
     h->launches += 2;
     for (size_t c = 0; c < h->fwd_classes.size(); ++c) {

@@ -24,7 +24,6 @@ using namespace cbtbe;
 namespace {
 
 constexpr size_t kScratchBytes = size_t(16) << 20;  // 16 MiB per device
-constexpr int64_t kChunk = 512;                      // lookups per chunk, as in the handle path
 constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -130,14 +129,15 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         class_start.push_back(static_cast<int32_t>(class_tables.size()));
     }
 
-    // Layout of the static scratch for this call; refuse calls that do not fit.
+    // Layout of the static scratch for this call; refuse calls that do not fit
+    // with the longest chunks. Shorter ones, as the handle's forward takes for
+    // fewer lookups, are used where their plan fits too.
     const int64_t T = num_tables, nc = static_cast<int64_t>(classes.size());
-    const int64_t max_chunks = num_indices / kChunk + T + 1;
     // Each chunk takes a descriptor, an owner word and two carry rows; refuse a
     // call whose chunks alone exceed the array before any product below can
     // wrap around (num_indices near 2^63).
     const size_t per_chunk = sizeof(Chunk) + sizeof(int64_t) + 2 * sizeof(float) * static_cast<size_t>(dmax);
-    if (max_chunks > static_cast<int64_t>(kScratchBytes / per_chunk)) return CB_ERR_CAPACITY;
+    if (num_indices / kMaxChunk + T + 1 > static_cast<int64_t>(kScratchBytes / per_chunk)) return CB_ERR_CAPACITY;
     size_t off = 0;
     const size_t o_err = off; off += up256(sizeof(int));
     const size_t o_zero = off; off += up256(2048);
@@ -147,18 +147,27 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
     const size_t o_pos = off; off += up256(sizeof(int64_t) * (T + 1));
     const size_t o_ord = off; off += up256(sizeof(int64_t) * (T + 1));
     const size_t o_cb = off; off += up256(sizeof(int64_t) * (nc + 1));
-    const size_t o_ch = off; off += up256(sizeof(Chunk) * max_chunks);
-    const size_t o_hd = off; off += up256(sizeof(float) * max_chunks * dmax);
-    const size_t o_tl = off; off += up256(sizeof(float) * max_chunks * dmax);
-    const size_t o_to = off; off += up256(sizeof(int64_t) * max_chunks);
     const size_t o_nx = off; off += up256(sizeof(uint32_t) * (nc + 1));  // chunk counters
-    if (off > kScratchBytes) return CB_ERR_CAPACITY;
+    const size_t o_ch = off;
+    auto scratch_end = [&](int64_t chunks) {
+        return o_ch + up256(sizeof(Chunk) * chunks) + 2 * up256(sizeof(float) * chunks * dmax) +
+               up256(sizeof(int64_t) * chunks);
+    };
+    if (scratch_end(chunk_count_bound(num_indices, kMaxChunk, T)) > kScratchBytes) return CB_ERR_CAPACITY;
 
     int device = -1;
-    if (cudaGetDevice(&device) != cudaSuccess) {
+    int num_sms = 1;
+    if (cudaGetDevice(&device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
         cudaGetLastError();
         return CB_ERR_CUDA;
     }
+    int64_t chunk_len = chunk_len_for(num_indices, num_sms);
+    if (scratch_end(chunk_count_bound(num_indices, chunk_len, T)) > kScratchBytes) chunk_len = kMaxChunk;
+    const int64_t max_chunks = chunk_count_bound(num_indices, chunk_len, T);
+    const size_t o_hd = o_ch + up256(sizeof(Chunk) * max_chunks);
+    const size_t o_tl = o_hd + up256(sizeof(float) * max_chunks * dmax);
+    const size_t o_to = o_tl + up256(sizeof(float) * max_chunks * dmax);
     unsigned char* base = nullptr;
     cb_status st = scratch_address(device, &base);
     if (st != CB_OK) return st;
@@ -194,8 +203,6 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
     P.mean = mode == CB_POOL_MEAN;
     P.dmax = dmax;
     P.out_dtype = CB_F32;
-    int num_sms = 1;
-    cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device);
     launch_validate_offsets(P, num_sms, stream);
     if (num_indices == 0) {
         if (cudaMemsetAsync(out, 0, sizeof(float) * batch * doff, stream) != cudaSuccess) {
@@ -204,8 +211,8 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         }
     } else {
         Plan Q;
-        Q.chunk_len = static_cast<int32_t>(kChunk);
-        Q.snap_cap = static_cast<int32_t>(4 * kChunk);  // as the handle's forward
+        Q.chunk_len = static_cast<int32_t>(chunk_len);
+        Q.snap_cap = static_cast<int32_t>(4 * chunk_len);  // as the handle's forward
         Q.num_classes = static_cast<int32_t>(nc);
         Q.class_tables = reinterpret_cast<const int32_t*>(base + o_ct);
         Q.class_table_start = reinterpret_cast<const int32_t*>(base + o_cs);

@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(1024) bwd_finalize_kernel(Problem P, BwdOut O)
 // ---------------------------------------------------------------- (6) fix-up
 
 // Runs split over chunks (hot rows longer than the snap cap): each warp scans
-// 32 chunks at a time for tail pieces and combines each such run in fp64. Runs
+// `span` chunks at a time for tail pieces and combines each such run in fp64. Runs
 // spread over more than kHeavyPieces chunks go to a list that bwd_heavy_kernel
 // combines with a whole block each.
 constexpr int64_t kHeavyPieces = 32;
@@ -388,12 +388,12 @@ __device__ __forceinline__ void store_grad4(float* dst, int x0, const double (&a
 
 __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_constant__ Problem P,
                                                                  const __grid_constant__ Plan Q,
-                                                                 const __grid_constant__ BwdOut O) {
+                                                                 const __grid_constant__ BwdOut O, int span) {
     if (*O.cap_fail) return;
     const int lane = threadIdx.x & 31;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    for (int64_t base = warp_id_global() * 32; base < total; base += warps_in_grid() * 32) {
-        const int64_t mine = base + lane < total ? Q.tail_owner[base + lane] : -1;
+    for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
+        const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
         for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
             const int b = __ffs(mask) - 1;
             const int64_t j = base + b;
@@ -464,12 +464,12 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_heavy_kernel(const __grid_co
 // the tail slot of the chunk where the run begins. One warp per such run.
 __global__ void __launch_bounds__(kWarpThreads) bwd_apply_split_kernel(const __grid_constant__ Problem P,
                                                                        const __grid_constant__ Plan Q,
-                                                                       const __grid_constant__ BwdOut O) {
+                                                                       const __grid_constant__ BwdOut O, int span) {
     if (*O.cap_fail) return;
     const int lane = threadIdx.x & 31;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    for (int64_t base = warp_id_global() * 32; base < total; base += warps_in_grid() * 32) {
-        const int64_t mine = base + lane < total ? Q.tail_owner[base + lane] : -1;
+    for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
+        const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
         for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
             const int b = __ffs(mask) - 1;
             const int64_t j = base + b;
@@ -535,18 +535,16 @@ void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const v
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
     cudaMemsetAsync(O.heavy_count, 0, sizeof(uint32_t), s);
-    const int64_t need = (chunk_bound + kWarpThreads - 1) / kWarpThreads;  // 32 chunks per warp
-    const int grid = static_cast<int>(max64(1, min64(need, static_cast<int64_t>(num_sms) * 8)));
-    bwd_fixup_kernel<<<grid, kWarpThreads, 0, s>>>(P, Q, O);
+    const int span = fixup_span(chunk_bound, num_sms);
+    bwd_fixup_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, O, span);
     const int hgrid = static_cast<int>(max64(1, min64(O.max_heavy, static_cast<int64_t>(num_sms) * 4)));
     bwd_heavy_kernel<<<hgrid, kWarpThreads, 0, s>>>(P, Q, O);
 }
 
 void launch_bwd_apply_split(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                             int num_sms, cudaStream_t s) {
-    const int64_t need = (chunk_bound + kWarpThreads - 1) / kWarpThreads;  // 32 chunks per warp
-    const int grid = static_cast<int>(max64(1, min64(need, static_cast<int64_t>(num_sms) * 8)));
-    bwd_apply_split_kernel<<<grid, kWarpThreads, 0, s>>>(P, Q, O);
+    const int span = fixup_span(chunk_bound, num_sms);
+    bwd_apply_split_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, O, span);
 }
 
 }  // namespace cbtbe

@@ -7,14 +7,14 @@ namespace cbtbe {
 
 // A heavy bag split over chunks: its tail piece (chunk where it starts) plus the
 // head pieces of the following chunks, added in fp64, then scaled. Each warp
-// scans 32 chunks at a time for tails (rare once boundaries snap to bag ends).
+// scans `span` chunks at a time for tails (rare once boundaries snap to bag ends).
 __global__ void __launch_bounds__(kWarpThreads) fwd_fixup_kernel(const __grid_constant__ Problem P,
                                                                  const __grid_constant__ Plan Q,
-                                                                 void* out) {
+                                                                 void* out, int span) {
     const int lane = threadIdx.x & 31;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    for (int64_t base = warp_id_global() * 32; base < total; base += warps_in_grid() * 32) {
-        const int64_t mine = base + lane < total ? Q.tail_owner[base + lane] : -1;
+    for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
+        const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
         for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
             const int b = __ffs(mask) - 1;
             const int64_t j = base + b;
@@ -52,9 +52,8 @@ void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int 
 
 void launch_fwd_fixup(const Problem& P, const Plan& Q, void* out, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
-    const int64_t need = (chunk_bound + kWarpThreads - 1) / kWarpThreads;  // 32 chunks per warp
-    const int grid = static_cast<int>(max64(1, min64(need, static_cast<int64_t>(num_sms) * 8)));
-    fwd_fixup_kernel<<<grid, kWarpThreads, 0, s>>>(P, Q, out);
+    const int span = fixup_span(chunk_bound, num_sms);
+    fwd_fixup_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, out, span);
 }
 
 }  // namespace cbtbe

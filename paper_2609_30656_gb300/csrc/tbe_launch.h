@@ -39,6 +39,50 @@ struct SortPass {
     uint64_t timeout_ns;
 };
 
+// Lookups per chunk. A walker's warp takes a chunk at a time, so a call needs
+// several chunks for each walker warp that the GPU holds (24 to 40 per SM): with
+// 512 lookups per chunk a call of up to a few million lookups left most SMs
+// without work, and one warp's chain of loads was the call's time. So
+// n / (num_sms * kChunksPerSm) lookups, rounded up to whole 32-lookup batches,
+// at least one batch and at most kMaxChunk. Measured whole calls, 512 against
+// this rule: forward of 512 lookups (1 table) 74 -> 23 us, of 1.6 M lookups (20
+// tables, odd dims) 277 -> 151 us; forward + backward of 106 K one-hot lookups
+// (26 tables) 682 -> 415 us; forward + fused Adagrad on 1.3 M lookups (16
+// tables) 1377 -> 572 us (698 at 64 chunks per SM, 945 at 32); from 10 M lookups
+// on the chunks are 512 long, where the sweep of 256, 512 and 1024 had its best.
+#ifndef CB_CHUNKS_PER_SM
+#define CB_CHUNKS_PER_SM 128
+#endif
+constexpr int64_t kChunksPerSm = CB_CHUNKS_PER_SM;
+constexpr int64_t kMaxChunk = 512;
+constexpr int64_t kMinChunk = 32;
+inline int64_t chunk_len_for(int64_t n, int num_sms) {
+    const int64_t per = n / (num_sms * kChunksPerSm) + 1;
+    const int64_t len = (per + 31) / 32 * 32;
+    return len < kMinChunk ? kMinChunk : (len > kMaxChunk ? kMaxChunk : len);
+}
+// Chunks of a call of n lookups over T tables: a whole number per table.
+inline int64_t chunk_count_bound(int64_t n, int64_t chunk_len, int64_t T) { return n / chunk_len + T + 1; }
+// An upper bound on the chunks of every call of up to n lookups (the count is
+// not monotone in n where the chunk length grows).
+inline int64_t chunk_count_limit(int64_t n, int num_sms, int64_t T) {
+    const int64_t most = num_sms * kChunksPerSm;
+    const int64_t small = n / kMinChunk < most ? n / kMinChunk : most;
+    return (small > n / kMaxChunk ? small : n / kMaxChunk) + T + 1;
+}
+// Chunks that one warp of a fix-up kernel scans at a time: 32 when there are
+// plenty, fewer so that the split segments of a small call spread over the GPU.
+inline int fixup_span(int64_t chunk_bound, int num_sms) {
+    const int64_t warps = static_cast<int64_t>(num_sms) * 64;
+    const int64_t span = (chunk_bound + warps - 1) / warps;
+    return static_cast<int>(span < 1 ? 1 : (span > 32 ? 32 : span));
+}
+inline int fixup_grid(int64_t chunk_bound, int span, int num_sms) {
+    const int64_t need = (chunk_bound + 8 * span - 1) / (8 * span);  // 8 warps per block
+    const int64_t cap = static_cast<int64_t>(num_sms) * 8;
+    return static_cast<int>(need < 1 ? 1 : (need < cap ? need : cap));
+}
+
 // Payload bag of a lookup whose index is out of range: outside every table's
 // bags, so the reduce reads the zero row for it.
 constexpr uint32_t kDeadBag = 0xffffffffu;
