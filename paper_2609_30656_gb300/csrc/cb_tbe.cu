@@ -48,27 +48,11 @@ class Ranges {
 struct KernelClass {
     int dtype;  // storage dtype (forward) or CB_F32 (backward)
     int vpl;    // 16-byte vectors per lane: 1, 2 or 4
-    int gc;     // rows per warp step fixed at compile time (0: run time)
+    int gc;     // rows per warp step
     std::vector<int32_t> tables;
 };
 
 int elem_bytes(int dt) { return dt == CB_F32 ? 4 : 2; }
-
-int vpl_for(int row_vecs) { return row_vecs <= 32 ? 1 : (row_vecs <= 64 ? 2 : 4); }
-
-// Lanes per row and rows per warp step for a row of `vecs` 16-byte vectors.
-void lane_split(int vecs, int32_t* lanes, int32_t* groups) {
-    if (vecs >= 32) {
-        *lanes = 32;
-        *groups = 1;
-    } else if ((vecs & (vecs - 1)) == 0) {
-        *lanes = vecs;
-        *groups = 32 / vecs;
-    } else {
-        *lanes = vecs;  // not a power of two: one row per warp step
-        *groups = 1;
-    }
-}
 
 size_t align_up(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
@@ -135,6 +119,7 @@ struct cb_tbe {
     int passes = 1;
     std::vector<TableDev> tables;
     std::vector<KernelClass> fwd_classes, bwd_classes;
+    bool fwd_one_dtype = true;  // every table has one storage type
     // persistent device memory: tables, class lists, error word, a never-written word
     void* persist = nullptr;
     TableDev* d_tables = nullptr;
@@ -577,9 +562,7 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
         td.doff = static_cast<int32_t>(doff);
         td.dtype = d.dtype;
         td.row_vecs = static_cast<int32_t>(row_bytes / 16);
-        lane_split(td.row_vecs, &td.lanes, &td.groups);
         td.grad_vecs = d.dim * out_eb / 16;  // grad_out row, in the output's type
-        lane_split(td.grad_vecs, &td.grad_lanes, &td.grad_groups);
         row_base += d.rows;
         doff += d.dim;
         h->dmax = std::max(h->dmax, d.dim);
@@ -601,24 +584,22 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     h->key_bits = bits;
     h->passes = (bits + 7) / 8;
 
-    // Kernel classes: forward by (storage dtype, vectors per lane), backward by
-    // vectors per lane of the grad_out row (fp32, or the mixed-precision type).
+    // Kernel classes: tables whose rows (forward: storage type) or grad_out rows
+    // (backward: fp32, or the mixed-precision type) have one layout over a warp.
     for (int32_t t = 0; t < num_tables; ++t) {
-        TableDev& td = h->tables[t];
-        const int fv = vpl_for(td.row_vecs), bv = vpl_for(td.grad_vecs);
-        const int fg = compile_time_groups(fv, td.lanes, td.groups);
-        const int bg = compile_time_groups(bv, td.grad_lanes, td.grad_groups);
-        auto put = [&](std::vector<KernelClass>& cls, int dt, int v, int gc) {
-            for (size_t c = 0; c < cls.size(); ++c)
-                if (cls[c].dtype == dt && cls[c].vpl == v && cls[c].gc == gc) {
-                    cls[c].tables.push_back(t);
-                    return static_cast<int>(c);
+        const TableDev& td = h->tables[t];
+        auto put = [&](std::vector<KernelClass>& cls, int dt, int vecs) {
+            const int v = row_vectors_per_lane(vecs), gc = rows_per_step(vecs);
+            for (KernelClass& c : cls)
+                if (c.dtype == dt && c.vpl == v && c.gc == gc) {
+                    c.tables.push_back(t);
+                    return;
                 }
             cls.push_back({dt, v, gc, {t}});
-            return static_cast<int>(cls.size() - 1);
         };
-        td.fwd_class = put(h->fwd_classes, td.dtype, fv, fg);
-        td.bwd_class = put(h->bwd_classes, h->out_dtype, bv, bg);
+        put(h->fwd_classes, td.dtype, td.row_vecs);
+        h->fwd_one_dtype = h->fwd_one_dtype && td.dtype == h->tables[0].dtype;
+        put(h->bwd_classes, h->out_dtype, td.grad_vecs);
     }
 
     if (cudaGetDevice(&h->device) != cudaSuccess ||
@@ -735,10 +716,15 @@ cb_status cb_tbe_forward(cb_tbe* h, int32_t batch, const void* indices, int64_t 
     h->launches += 2;
     record(h, h->ev_fwd[1], stream);
     nv.phase("fwd.gather");
-    for (size_t c = 0; c < h->fwd_classes.size(); ++c) {
-        launch_fwd_gather(P, Q, out, static_cast<int>(c), h->fwd_classes[c].dtype,
-                          h->fwd_classes[c].vpl, h->fwd_classes[c].gc, bound, h->num_sms, stream);
+    if (h->fwd_one_dtype && h->fwd_classes.size() > 1) {
+        launch_fwd_gather(P, Q, out, -1, h->fwd_classes[0].dtype, 0, 0, bound, h->num_sms, stream);
         h->launches += 1;
+    } else {
+        for (size_t c = 0; c < h->fwd_classes.size(); ++c) {
+            launch_fwd_gather(P, Q, out, static_cast<int>(c), h->fwd_classes[c].dtype,
+                              h->fwd_classes[c].vpl, h->fwd_classes[c].gc, bound, h->num_sms, stream);
+            h->launches += 1;
+        }
     }
     record(h, h->ev_fwd[2], stream);
     nv.phase("fwd.fixup");
@@ -775,7 +761,7 @@ cb_status cb_tbe_weight_grad(cb_tbe* h, int32_t batch, const void* indices, int6
     launch_plan(P, Q, 0, nullptr, nullptr, h->num_sms, true, stream);
     h->launches += 2;
     for (size_t c = 0; c < h->fwd_classes.size(); ++c) {
-        // The compiled row layouts cover one vector per lane; wider rows loop.
+        // One vector per lane; wider rows loop.
         const int gc = h->fwd_classes[c].vpl == 1 ? h->fwd_classes[c].gc : 0;
         launch_weight_grad(P, Q, grad_out, grad_weights, static_cast<int>(c), h->fwd_classes[c].dtype, gc,
                            bound, h->num_sms, stream);

@@ -50,19 +50,6 @@ cb_status scratch_address(int device, unsigned char** out) {
 
 size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
-void split(int vecs, int32_t* lanes, int32_t* groups) {
-    if (vecs >= 32) {
-        *lanes = 32;
-        *groups = 1;
-    } else if ((vecs & (vecs - 1)) == 0) {
-        *lanes = vecs;
-        *groups = 32 / vecs;
-    } else {
-        *lanes = vecs;
-        *groups = 1;
-    }
-}
-
 }  // namespace
 
 extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t num_tables,
@@ -103,11 +90,8 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         x.doff = static_cast<int32_t>(doff);
         x.dtype = d.dtype;
         x.row_vecs = static_cast<int32_t>(row_bytes / 16);
-        split(x.row_vecs, &x.lanes, &x.groups);
         x.grad_vecs = d.dim / 4;
-        split(x.grad_vecs, &x.grad_lanes, &x.grad_groups);
-        const int vpl = x.row_vecs <= 32 ? 1 : (x.row_vecs <= 64 ? 2 : 4);
-        const int gc = compile_time_groups(vpl, x.lanes, x.groups);
+        const int vpl = row_vectors_per_lane(x.row_vecs), gc = rows_per_step(x.row_vecs);
         int c = -1;
         for (size_t k = 0; k < classes.size(); ++k)
             if (classes[k].dtype == d.dtype && classes[k].vpl == vpl && classes[k].gc == gc)
@@ -117,7 +101,6 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
             c = static_cast<int>(classes.size() - 1);
         }
         classes[c].t.push_back(t);
-        x.fwd_class = c;
         row_base += d.rows;
         doff += d.dim;
         dmax = d.dim > dmax ? d.dim : dmax;
@@ -226,7 +209,11 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         Q.tail_owner = reinterpret_cast<int64_t*>(base + o_to);
         Q.chunk_next = reinterpret_cast<uint32_t*>(base + o_nx);  // zeroed by the plan
         launch_plan(P, Q, 0, nullptr, nullptr, num_sms, true, stream);
-        for (size_t c = 0; c < classes.size(); ++c)
+        bool one_dtype = true;
+        for (const Cls& c : classes) one_dtype = one_dtype && c.dtype == classes[0].dtype;
+        if (one_dtype && classes.size() > 1)
+            launch_fwd_gather(P, Q, out, -1, classes[0].dtype, 0, 0, max_chunks, num_sms, stream);
+        else for (size_t c = 0; c < classes.size(); ++c)
             launch_fwd_gather(P, Q, out, static_cast<int>(c), classes[c].dtype, classes[c].vpl,
                               classes[c].gc, max_chunks, num_sms, stream);
         launch_fwd_fixup(P, Q, out, max_chunks, num_sms, stream);

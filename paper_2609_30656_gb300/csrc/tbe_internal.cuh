@@ -68,9 +68,6 @@ constexpr int kWarpThreads = 256;  // block size of the warp-per-chunk kernels
 #ifndef CB_REDUCE_FAST_BATCH
 #define CB_REDUCE_FAST_BATCH 1
 #endif
-#ifndef CB_ROW_WALKER
-#define CB_ROW_WALKER 1  // 0: every layout takes the general walker (walk_chunk)
-#endif
 constexpr int64_t kNoSeg = INT64_MAX;
 
 // Per-table facts the kernels need, built once at create time.
@@ -87,14 +84,7 @@ struct TableDev {
     int32_t doff;       // column offset of this table in the [B, sum dims] output
     int32_t dtype;      // cb_dtype
     int32_t row_vecs;   // 16-byte vectors per stored row
-    int32_t lanes;      // lanes per stored row in the gather (V)
-    int32_t groups;     // stored rows per warp step (G, V * G <= 32)
-    int32_t grad_vecs;  // 16-byte vectors per fp32 gradient row (dim / 4)
-    int32_t grad_lanes;
-    int32_t grad_groups;
-    int32_t fwd_class;
-    int32_t bwd_class;
-    int32_t pad;
+    int32_t grad_vecs;  // 16-byte vectors per grad_out row, in the output's type
 };
 
 // A run of at most chunk_len item positions of one table.
@@ -156,6 +146,20 @@ __device__ __forceinline__ int64_t warp_id_global() {
 }
 __device__ __forceinline__ int64_t warps_in_grid() {
     return (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+}
+
+// Blocks of `threads` that one SM holds, and the grid of a persistent kernel
+// whose warps take `chunk_bound` chunks.
+template <class KernelT>
+inline int resident_blocks(KernelT kernel, int threads) {
+    int per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    return per_sm;
+}
+inline int warp_grid(int64_t chunk_bound, int64_t cap) {
+    const int64_t need = (chunk_bound + (kWarpThreads / 32) - 1) / (kWarpThreads / 32);
+    return static_cast<int>(max64(1, min64(need, cap)));
 }
 
 // The walkers' chunk order: a warp takes the next chunk of its class from a
@@ -341,21 +345,45 @@ __device__ __forceinline__ void accumulate(float (&a)[Storage<DT>::kElems], cons
 
 // ---------------------------------------------------------------- the walker
 //
-// Pol (policy) supplies:
-//   kDtype, kElems, kVpl (16-byte vectors per lane), kUnroll (rows in flight per
-//   lane), kWeighted
-//   int64_t seg_begin(s), seg_end(s)    positions of segment s (s < seg_hi)
-//   Raw fetch(q), static Raw none()      raw payload of item q (loads only)
-//   void decode(Raw, uint32_t& a, float& w)  row number within `base`
-//                                            (kInvalid = skip) and coefficient
-//   const uint4* base; uint32_t stride       row a starts at base + a * stride
-//   void emit(seg, len, started, ends, tot, lane-in-group v, is_group0)
-//                                            len = segment length when complete
+// A warp walks one chunk of item positions in batches of 32. A row is spread
+// over V = 32 / G lanes, 16 bytes per lane and vector, VPL vectors per lane
+// (G = 1 for more than one), so a warp step gathers G rows; G is the largest
+// power of two with rows that fit V lanes. Lanes past a row that is not a power
+// of two of vectors load one of the row's own vectors again (the same cache
+// lines, no branch) and never store what they sum. Before a batch's rows are
+// loaded, the warp finds every segment ending inside the batch from a window of
+// 32 segment ends (one per lane): the positions of those ends become a 32-bit
+// mask, and their segment numbers go to a per-warp list in shared memory, in
+// order. Adding a row then costs a shuffle, one multiply-add for its address,
+// the loads and the adds, and the mask is tested once per group of loads; a
+// segment end costs one list read and the store of the sum. Empty segments
+// (empty bags) are written out during the scan.
+//
 // Positions inside the walker are relative to the chunk start and clamped to
 // [kRelLo, kRelHi], which keeps every comparison with [0, len] exact in 32 bits.
 // The segment range of the chunk is [first, seg_hi); segments that start at or
 // after the chunk end belong to the next chunk, except after the last chunk of a
 // table (trailing empty bags), which `last` allows.
+//
+// Pol (policy) supplies:
+//   kDtype, kElems, kVpl (16-byte vectors per lane), kUnroll (row steps in
+//   flight), kWeighted, kTwoLevel
+//   kEmptySegments     segments may be empty
+//   kUnrollGroups      unroll a batch's load groups
+//   kFastBatch         separate unrolled path for batches with no segment end
+//   kPrefetch          load groups ahead whose rows are prefetched into L1 (0: none)
+//   int64_t seg_begin(s), seg_end(s)    positions of segment s (s < seg_hi)
+//   Raw fetch(q), static Raw none()      raw payload of item q (loads only)
+//   void decode(Raw, uint32_t& a, float& w)  row number within `base`
+//                                            (kInvalid = skip) and coefficient
+//   const uint4* base; uint32_t stride       row a starts at base + a * stride
+//   void put(seg, len, started, ends, tot, v, is_group0)   a segment's sum, or
+//                                            its piece in this chunk
+//   void seg_meta(seg)                       metadata of a segment that began in
+//                                            this chunk (once per segment; lanes
+//                                            may call it for different segments
+//                                            at the same time)
+//   void put_empty(seg, v, is_group0)        the output of an empty segment
 
 constexpr uint32_t kInvalid = 0xffffffffu;
 constexpr int32_t kRelLo = -1;
@@ -366,8 +394,6 @@ struct ChunkCtx {
     int32_t len;       // items in the chunk
     int32_t first;     // first segment
     int32_t seg_hi;    // segments of this table end before seg_hi
-    int32_t lanes;     // V
-    int32_t groups;    // G
     int32_t row_vecs;  // vectors per row
     bool last;         // owns trailing segments that start at the chunk end
 };
@@ -377,47 +403,49 @@ __device__ __forceinline__ int32_t rel_pos(int64_t x, int64_t k0) {
     return r < kRelLo ? kRelLo : (r > kRelHi ? kRelHi : static_cast<int32_t>(r));
 }
 
-// GC > 0: the row layout is known at compile time (G = GC rows per warp step,
-// V = 32 / GC lanes per row); GC == 0: taken from the chunk at run time (rows
-// whose vector count is not a power of two).
-template <class Pol, int GC>
-__device__ __forceinline__ void walk_chunk(Pol& pol, const ChunkCtx& c, const uint4* zero_row,
-                                           int lane) {
+// Number of a row's layout: 0..5 for 32, 16, .., 1 rows per step (1, 2, 4, .., 32
+// lanes per row), 6 and 7 for 2 and 4 vectors per lane.
+__device__ __forceinline__ int row_layout(int row_vecs) { return 32 - __clz(row_vecs - 1); }
+
+struct EndSlot {
+    int32_t seg;
+    int32_t len;  // segment length; -1 when it began in an earlier chunk, 0 for the
+                  // piece of one that runs past the chunk end
+};
+
+// A row's cache lines requested into L1 ahead of its load, without a register.
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
+template <class Pol, int G>
+__device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uint4* zero_row,
+                                          int lane, EndSlot* slots) {
     constexpr int E = Pol::kElems;
     constexpr int VPL = Pol::kVpl;
-    constexpr int U = Pol::kUnroll;
+    static_assert(G >= 1 && G <= 32 && (G & (G - 1)) == 0, "rows per warp step");
+    static_assert(VPL == 1 || G == 1, "several vectors per lane: one row per step");
+    constexpr int V = 32 / G;
+    constexpr int kSteps = 32 / G;                                      // row steps per batch
+    constexpr int UG = Pol::kUnroll < kSteps ? Pol::kUnroll : kSteps;  // row steps per load group
+    constexpr int kGroupItems = UG * G;
+    constexpr uint32_t kGroupMask = kGroupItems == 32 ? kFull : (1u << (kGroupItems & 31)) - 1u;
+    constexpr uint32_t kStepMask = G == 32 ? kFull : (1u << (G & 31)) - 1u;
     constexpr bool W = Pol::kWeighted;
-    constexpr bool kExact = GC > 0 && VPL == 1;  // each lane owns one vector of one row
-    const int V = GC > 0 ? 32 / GC : c.lanes;
-    const int G = GC > 0 ? GC : c.groups;
+    constexpr bool kTwoLevel = Pol::kTwoLevel;
+    constexpr int kGroupUnroll = Pol::kUnrollGroups ? 32 / kGroupItems : 1;
     const int g = lane / V;
     const int v = lane - g * V;
-    const int ustop = min(U, 32 / G);  // row groups per step
-    const int step = ustop * G;        // items per step (<= 32, divides 32)
     const int32_t len = c.len;
-    // Lanes past the row (non power-of-two rows) and vectors past it read zeros.
-    const uint4* vzero[VPL];
-    bool vlive[VPL];
+    const char* lane_base = reinterpret_cast<const char*>(pol.base + (v < c.row_vecs ? v : 0));
+    const uint32_t row_bytes = pol.stride * 16u;
+    const uint4* zrow = zero_row + v;
+    const uint32_t below = (1u << lane) - 1u;
+    // Vector v + 32k of the row, relative to the lane's first (0 past the row).
+    int voff[VPL];
 #pragma unroll
-    for (int k = 0; k < VPL; ++k) {
-        vlive[k] = kExact || (g < G && v + 32 * k < c.row_vecs);
-        vzero[k] = zero_row + (v + 32 * k) % 128;
-    }
+    for (int k = 0; k < VPL; ++k) voff[k] = k > 0 && v + 32 * k < c.row_vecs ? 32 * k : 0;
 
-    // Segment-end window: lane i holds the (relative) end of segment win + i.
-    int32_t win = c.first;
-    int32_t my_end = (win + lane < c.seg_hi) ? rel_pos(pol.seg_end(win + lane), c.k0) : kRelHi;
-    int32_t seg = c.first;
-    int32_t s_cur = kRelHi, e_cur = kRelHi;
-    if (seg < c.seg_hi) {
-        s_cur = rel_pos(pol.seg_begin(seg), c.k0);
-        e_cur = __shfl_sync(kFull, my_end, 0);
-    }
-
-    // fp32 rows (tables or gradients) sum in two levels (see the fold below);
-    // half-precision rows, whose tolerance is far looser, use one level, which
-    // frees registers for occupancy.
-    constexpr bool kTwoLevel = Pol::kTwoLevel;
     float ain[VPL][E], aout[VPL][kTwoLevel ? E : 1];
 #pragma unroll
     for (int k = 0; k < VPL; ++k) {
@@ -426,113 +454,16 @@ __device__ __forceinline__ void walk_chunk(Pol& pol, const ChunkCtx& c, const ui
 #pragma unroll
         for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[k][x] = 0.f;
     }
-
-    auto flush = [&]() {
-        float tot[VPL][E];
+    auto add = [&](const uint4 (&x)[VPL], float w) {
 #pragma unroll
-        for (int k = 0; k < VPL; ++k)
-#pragma unroll
-            for (int x = 0; x < E; ++x) tot[k][x] = kTwoLevel ? aout[k][x] + ain[k][x] : ain[k][x];
-        for (int off = V; off < V * G; off <<= 1) {
-#pragma unroll
-            for (int k = 0; k < VPL; ++k)
-#pragma unroll
-                for (int x = 0; x < E; ++x) tot[k][x] += __shfl_xor_sync(kFull, tot[k][x], off);
-        }
-        pol.emit(seg, e_cur - s_cur, s_cur >= 0, e_cur <= len, tot, v, g == 0);
-#pragma unroll
-        for (int k = 0; k < VPL; ++k) {
-#pragma unroll
-            for (int x = 0; x < E; ++x) ain[k][x] = 0.f;
-#pragma unroll
-            for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[k][x] = 0.f;
-        }
+        for (int k = 0; k < VPL; ++k) accumulate<Pol::kDtype, W>(ain[k], x[k], w);
     };
-    auto advance = [&]() {
-        ++seg;
-        s_cur = e_cur;
-        if (seg >= c.seg_hi) {
-            s_cur = e_cur = kRelHi;
-            return;
-        }
-        if (seg - win >= 32) {
-            win = seg;
-            my_end = (win + lane < c.seg_hi) ? rel_pos(pol.seg_end(win + lane), c.k0) : kRelHi;
-        }
-        e_cur = __shfl_sync(kFull, my_end, seg - win);
-    };
-
-    typename Pol::Raw nxt = Pol::none();
-    if (lane < len) nxt = pol.fetch(c.k0 + lane);
-
-    for (int32_t base = 0; base < len; base += 32) {
-        const int nb = min(32, len - base);
-        const typename Pol::Raw cur = nxt;
-        // Prefetch the next batch's raw payload while this batch's rows are in
-        // flight; it is only decoded when its batch comes up.
-        nxt = Pol::none();
-        if (base + 32 + lane < len) nxt = pol.fetch(c.k0 + base + 32 + lane);
-        uint32_t my_a = kInvalid;  // lanes >= nb hold kInvalid
-        float my_w = 0.f;
-        if (lane < nb) pol.decode(cur, my_a, my_w);
-
-        for (int i0 = 0; i0 < nb; i0 += step) {
-            // Issue every row load of the step first; an invalid or padding item
-            // reads the zero row, so it adds nothing and needs no bookkeeping.
-            uint4 buf[U][VPL];
-            float wt[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = i0 + u * G + g;
-                const uint32_t a = __shfl_sync(kFull, my_a, i & 31);
-                wt[u] = W ? __shfl_sync(kFull, my_w, i & 31) : 1.f;
-                const bool ok = u < ustop && a != kInvalid;
-                const uint4* rp = pol.base + static_cast<size_t>(a) * pol.stride;
-#pragma unroll
-                for (int k = 0; k < VPL; ++k)
-                    buf[u][k] = __ldg((ok && vlive[k]) ? rp + v + 32 * k : vzero[k]);
-            }
-            // Then add them in position order, emitting segments as they end.
-            if (i0 + step <= nb && e_cur > base + i0 + step - 1) {
-                // Common case: a full step inside the current segment.
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-#pragma unroll
-                    for (int k = 0; k < VPL; ++k) accumulate<Pol::kDtype, W>(ain[k], buf[u][k], wt[u]);
-                continue;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int ifirst = i0 + u * G;
-                if (ifirst >= nb) break;
-                const int32_t qlast = base + min(ifirst + G, nb) - 1;  // last item of this row group
-                if (e_cur > qlast) {
-#pragma unroll
-                    for (int k = 0; k < VPL; ++k) accumulate<Pol::kDtype, W>(ain[k], buf[u][k], wt[u]);
-                } else {
-                    // One or more segments end inside this row group.
-                    const int32_t q = base + ifirst + g;
-                    bool added = false;
-                    do {
-                        if (!added && q < e_cur) {
-#pragma unroll
-                            for (int k = 0; k < VPL; ++k)
-                                accumulate<Pol::kDtype, W>(ain[k], buf[u][k], wt[u]);
-                            added = true;
-                        }
-                        flush();
-                        advance();
-                    } while (e_cur <= qlast);
-                    if (!added) {
-#pragma unroll
-                        for (int k = 0; k < VPL; ++k) accumulate<Pol::kDtype, W>(ain[k], buf[u][k], wt[u]);
-                    }
-                }
-            }
-        }
-        // Two-level summation: at most 32 / G terms per lane enter `ain` before
-        // it is folded into `aout`, which bounds the fp32 rounding error.
-        if (kTwoLevel) {
+    // Two-level summation: at most 32 / G terms per lane enter `ain` before it is
+    // folded into `aout`, which bounds the fp32 rounding error (fp32 rows, tables
+    // or gradients; half-precision rows, whose tolerance is far looser, use one
+    // level, which frees registers for occupancy).
+    auto fold = [&]() {
+        if constexpr (kTwoLevel) {
 #pragma unroll
             for (int k = 0; k < VPL; ++k)
 #pragma unroll
@@ -541,128 +472,13 @@ __device__ __forceinline__ void walk_chunk(Pol& pol, const ChunkCtx& c, const ui
                     ain[k][x] = 0.f;
                 }
         }
-    }
-
-    // Segments still open at the chunk end: finish those that end here, emit the
-    // piece of the one that continues, and (last chunk only) the trailing empties.
-    while (seg < c.seg_hi) {
-        if (!c.last && s_cur >= len) break;
-        const bool done = e_cur <= len;
-        flush();
-        if (!done) break;
-        advance();
-    }
-}
-
-// ---------------------------------------------------------------- the row walker
-//
-// walk_rows has walk_chunk's contract for the common layout, one 16-byte vector
-// per lane and G = 32 / V rows per warp step fixed at compile time, and is built
-// around batches of 32 item positions. Before a batch's rows are loaded, the
-// warp finds every segment ending inside the batch from a window of 32 segment
-// ends (one per lane): the positions of those ends become a 32-bit mask, and
-// their segment numbers go to a per-warp list in shared memory, in order. Adding
-// a row then costs a shuffle, one multiply-add for its address, the load and
-// the adds, and the mask is tested once per group of loads; a segment end costs
-// one list read and the store of the sum. Empty segments (empty bags) are
-// written out during the scan. Pol additionally supplies:
-//   static constexpr bool kEmptySegments    segments may be empty
-//   static constexpr bool kUnrollGroups     unroll a batch's load groups
-//   static constexpr bool kFastBatch        separate unrolled path for batches
-//                                            with no segment end
-//   static constexpr int kPrefetch          load groups ahead whose rows are
-//                                            prefetched into L1 (0: none)
-//   void put(seg, len, started, ends, tot, v, is_group0)   emit without the
-//                                            per-segment metadata
-//   void seg_meta(seg)                       metadata of a segment that began in
-//                                            this chunk (once per segment; lanes
-//                                            may call it for different segments
-//                                            at the same time)
-//   void put_empty(seg, v, is_group0)        the output of an empty segment
-
-struct EndSlot {
-    int32_t seg;
-    int32_t len;  // segment length, or -1 when it began in an earlier chunk
-};
-
-// Loads of rows staged in shared memory (D > 0): each group of UG row steps is
-// copied with cp.async into a per-warp ring of D + 1 groups of slots (16 bytes
-// per lane and step), D groups ahead of the one being added, so that D * UG
-// steps of rows are in flight per warp without holding registers. A slot is
-// refilled one group after it was read, when its values have been added. The
-// decoded payloads of the next batch are kept for the prefetch across the
-// batch boundary. D = 0: the rows are loaded into registers one group at a
-// time.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(smem))),
-                 "l"(gmem)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(smem))),
-                 "l"(gmem)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(smem))),
-                 "l"(gmem)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// A row's cache lines requested into L1 ahead of its load, without a register.
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-// KS > 0 (with D = 0): the items' raw payloads (indices and weights, or
-// sorted payloads) are staged with cp.async KS batches ahead into a per-warp
-// ring of KS + 1 batch slots (Pol::kStageBytes per lane), instead of being
-// loaded into registers one batch ahead.
-template <class Pol, int G, int D = 0, int KS = 0>
-__device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uint4* zero_row,
-                                          int lane, EndSlot* slots, uint4* ring = nullptr,
-                                          char* stage = nullptr) {
-    static_assert(G == 1 || G == 2 || G == 4 || G == 8, "rows per warp step");
-    static_assert(Pol::kVpl == 1, "one vector per lane");
-    constexpr int E = Pol::kElems;
-    constexpr int V = 32 / G;
-    constexpr int kSteps = 32 / G;                                      // row steps per batch
-    constexpr int UG = Pol::kUnroll < kSteps ? Pol::kUnroll : kSteps;  // row steps per load group
-    constexpr int kGroupItems = UG * G;
-    constexpr uint32_t kGroupMask = kGroupItems == 32 ? kFull : (1u << kGroupItems) - 1u;
-    constexpr uint32_t kStepMask = (1u << G) - 1u;
-    constexpr bool W = Pol::kWeighted;
-    constexpr bool kTwoLevel = Pol::kTwoLevel;
-    constexpr int kGroupUnroll = Pol::kUnrollGroups ? 32 / kGroupItems : 1;
-    const int g = lane / V;
-    const int v = lane - g * V;
-    const int32_t len = c.len;
-    const char* lane_base = reinterpret_cast<const char*>(pol.base + v);
-    const uint32_t row_bytes = pol.stride * 16u;
-    const uint4* zrow = zero_row + v;
-    const uint32_t below = (1u << lane) - 1u;
-
-    float ain[E], aout[kTwoLevel ? E : 1];
-#pragma unroll
-    for (int x = 0; x < E; ++x) ain[x] = 0.f;
-#pragma unroll
-    for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[x] = 0.f;
+    };
 
     // Window: lane j holds the relative end of segment seg + j.
     int32_t seg = c.first;
     int32_t s_cur = seg < c.seg_hi ? rel_pos(pol.seg_begin(seg), c.k0) : kRelHi;
     int32_t my_end = seg + lane < c.seg_hi ? rel_pos(pol.seg_end(seg + lane), c.k0) : kRelHi;
     uint32_t mask = 0;
-    int ce_async = 0;  // next entry of the segment-end list (staged loads)
 
     // Segments ending at or before `bend` (the batch starts at `base`) leave the
     // window: non-empty ones are listed and marked in `mask`, empty ones owned
@@ -709,18 +525,23 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
     auto flush = [&](const EndSlot s, bool ends) {
         // Kept inside this chunk's segment range whatever the list holds.
         const int32_t sseg = min(max(s.seg, c.first), c.seg_hi - 1);
-        float tot[1][E];
+        float tot[VPL][E];
 #pragma unroll
-        for (int x = 0; x < E; ++x) tot[0][x] = kTwoLevel ? aout[x] + ain[x] : ain[x];
+        for (int k = 0; k < VPL; ++k)
+#pragma unroll
+            for (int x = 0; x < E; ++x) tot[k][x] = kTwoLevel ? aout[k][x] + ain[k][x] : ain[k][x];
 #pragma unroll
         for (int off = V; off < 32; off <<= 1)
 #pragma unroll
             for (int x = 0; x < E; ++x) tot[0][x] += __shfl_xor_sync(kFull, tot[0][x], off);
         pol.put(sseg, s.len, s.len >= 0, ends, tot, v, g == 0);
 #pragma unroll
-        for (int x = 0; x < E; ++x) ain[x] = 0.f;
+        for (int k = 0; k < VPL; ++k) {
 #pragma unroll
-        for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[x] = 0.f;
+            for (int x = 0; x < E; ++x) ain[k][x] = 0.f;
+#pragma unroll
+            for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[k][x] = 0.f;
+        }
     };
 
     // One batch's rows: CLEAN = 32 valid items (no padding, no skipped item).
@@ -730,7 +551,7 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
 #pragma unroll(kGroupUnroll)
         for (int i0 = 0; i0 < 32; i0 += kGroupItems) {
             if (!CLEAN && i0 >= nb) break;
-            uint4 buf[UG];
+            uint4 buf[UG][VPL];
             float wt[UG];
 #pragma unroll
             for (int u = 0; u < UG; ++u) {
@@ -738,7 +559,8 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
                 const uint32_t a = __shfl_sync(kFull, my_a, src);
                 wt[u] = W ? __shfl_sync(kFull, my_w, src) : 1.f;
                 const uint4* p = reinterpret_cast<const uint4*>(lane_base + static_cast<uint64_t>(a) * row_bytes);
-                buf[u] = __ldg(CLEAN || a != kInvalid ? p : zrow);
+#pragma unroll
+                for (int k = 0; k < VPL; ++k) buf[u][k] = __ldg(CLEAN || a != kInvalid ? p + voff[k] : zrow);
             }
             // The rows of the group kPrefetch groups ahead in this batch start
             // moving into L1 while this group's loads are waited for.
@@ -748,21 +570,24 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
 #pragma unroll
                     for (int u = 0; u < UG; ++u) {
                         const uint32_t a = __shfl_sync(kFull, my_a, pf + u * G + g);
-                        if (a != kInvalid) prefetch_l1(lane_base + static_cast<uint64_t>(a) * row_bytes);
+#pragma unroll
+                        for (int k = 0; k < VPL; ++k)
+                            if (a != kInvalid)
+                                prefetch_l1(lane_base + static_cast<uint64_t>(a) * row_bytes + 16 * voff[k]);
                     }
                 }
             }
             const uint32_t m = (mask >> i0) & kGroupMask;
             if (m == 0) {
 #pragma unroll
-                for (int u = 0; u < UG; ++u) accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
+                for (int u = 0; u < UG; ++u) add(buf[u], wt[u]);
                 continue;
             }
 #pragma unroll
             for (int u = 0; u < UG; ++u) {
                 uint32_t mu = (m >> (u * G)) & kStepMask;
                 if (mu == 0) {
-                    accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
+                    add(buf[u], wt[u]);
                     continue;
                 }
                 // Segments end after item i0 + u*G + p for each set bit p; this
@@ -771,149 +596,26 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
                 do {
                     const int p = __ffs(mu) - 1;
                     if (!added && g <= p) {
-                        accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
+                        add(buf[u], wt[u]);
                         added = true;
                     }
                     flush(slots[ce++], true);
                     mu &= mu - 1;
                 } while (mu);
-                if (!added) accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
+                if (!added) add(buf[u], wt[u]);
             }
         }
     };
 
-    if constexpr (D > 0) {
-        constexpr int kGroups = 32 / kGroupItems;  // load groups per batch
-        // groups in flight: at most a batch's, so the prefetch reaches at most
-        // one batch ahead
-        constexpr int DD = D < kGroups ? D : kGroups;
-        constexpr int kRing = DD + 1;              // groups of slots in the ring
-        // The rows of load group q (0 .. kGroups-1) of a batch whose decoded
-        // row numbers are `aa` and first position `bbase` go to ring group `rg`.
-        auto issue = [&](int rg, uint32_t aa, int q, int32_t bbase) {
-#pragma unroll
-            for (int u = 0; u < UG; ++u) {
-                const int src = q * kGroupItems + u * G + g;
-                const uint32_t a = __shfl_sync(kFull, aa, src);
-                const char* p = (a != kInvalid && bbase + src < len)
-                                    ? lane_base + static_cast<uint64_t>(a) * row_bytes
-                                    : reinterpret_cast<const char*>(zrow);
-                cp_async16(ring + (rg * UG + u) * 32 + lane, p);
-            }
-            cp_async_commit();
-        };
-        // Decoded payloads of this batch and the next; raw payloads two ahead.
-        uint32_t a0 = kInvalid, a1 = kInvalid;
-        float w0 = 0.f, w1 = 0.f;
-        typename Pol::Raw raw = Pol::none();
-        if (lane < len) raw = pol.fetch(c.k0 + lane);
-        if (lane < len) pol.decode(raw, a0, w0);
-        raw = Pol::none();
-        if (32 + lane < len) raw = pol.fetch(c.k0 + 32 + lane);
-#pragma unroll
-        for (int q = 0; q < DD; ++q) issue(q, a0, q, 0);
-        int rd = 0;  // ring group read next
-        for (int32_t base = 0; base < len; base += 32) {
-            const int nb = min(32, len - base);
-            a1 = kInvalid;
-            w1 = 0.f;
-            if (base + 32 + lane < len) pol.decode(raw, a1, w1);
-            raw = Pol::none();
-            if (base + 64 + lane < len) raw = pol.fetch(c.k0 + base + 64 + lane);
-            scan(base, base + nb);
-            for (int q = 0; q < kGroups; ++q) {
-                if (base + q * kGroupItems >= len) {
-                    // past the chunk: the groups still in flight carry zeros
-                    continue;
-                }
-                cp_async_wait<DD - 1>();
-                uint4 buf[UG];
-                float wt[UG];
-#pragma unroll
-                for (int u = 0; u < UG; ++u) {
-                    buf[u] = ring[(rd * UG + u) * 32 + lane];
-                    wt[u] = W ? __shfl_sync(kFull, w0, q * kGroupItems + u * G + g) : 1.f;
-                }
-                // refill the ring group read one group ago with group q + DD
-                const int wr = rd == 0 ? kRing - 1 : rd - 1;
-                if (q + DD < kGroups) issue(wr, a0, q + DD, base);
-                else issue(wr, a1, q + DD - kGroups, base + 32);
-                rd = rd + 1 == kRing ? 0 : rd + 1;
-                const uint32_t m = (mask >> (q * kGroupItems)) & kGroupMask;
-                if (m == 0) {
-#pragma unroll
-                    for (int u = 0; u < UG; ++u) accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
-                    continue;
-                }
-#pragma unroll
-                for (int u = 0; u < UG; ++u) {
-                    uint32_t mu = (m >> (u * G)) & kStepMask;
-                    if (mu == 0) {
-                        accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
-                        continue;
-                    }
-                    bool added = false;
-                    do {
-                        const int p = __ffs(mu) - 1;
-                        if (!added && g <= p) {
-                            accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
-                            added = true;
-                        }
-                        flush(slots[ce_async++], true);
-                        mu &= mu - 1;
-                    } while (mu);
-                    if (!added) accumulate<Pol::kDtype, W>(ain, buf[u], wt[u]);
-                }
-            }
-            ce_async = 0;
-            if (kTwoLevel) {
-#pragma unroll
-                for (int x = 0; x < E; ++x) {
-                    aout[x] += ain[x];
-                    ain[x] = 0.f;
-                }
-            }
-            a0 = a1;
-            w0 = w1;
-        }
-        cp_async_wait_all();
-        __syncwarp();
-        scan(len, len);
-        if (seg < c.seg_hi && s_cur < len) {
-            if (s_cur >= 0 && lane == 0) pol.seg_meta(seg);
-            flush(EndSlot{seg, s_cur >= 0 ? 0 : -1}, false);
-        }
-        return;
-    }
-
     typename Pol::Raw nxt = Pol::none();
-    constexpr int kStage = KS > 0 ? KS : 1;
-    auto stage_slot = [&](int k) { return stage + (k * 32 + lane) * Pol::kStageBytes; };
-    int srd = 0;  // staging slot of the batch read next
-    if constexpr (KS > 0) {
-#pragma unroll
-        for (int k = 0; k < kStage; ++k) {
-            if (k * 32 + lane < len) pol.stage(stage_slot(k), c.k0 + k * 32 + lane);
-            cp_async_commit();
-        }
-    } else {
-        if (lane < len) nxt = pol.fetch(c.k0 + lane);
-    }
+    if (lane < len) nxt = pol.fetch(c.k0 + lane);
     for (int32_t base = 0; base < len; base += 32) {
         const int nb = min(32, len - base);
-        typename Pol::Raw cur = nxt;
-        if constexpr (KS > 0) {
-            cp_async_wait<kStage - 1>();
-            cur = lane < nb ? pol.staged(stage_slot(srd)) : Pol::none();
-            // refill the slot read one batch ago with the batch KS ahead
-            const int swr = srd == 0 ? kStage : srd - 1;
-            if (base + kStage * 32 + lane < len) pol.stage(stage_slot(swr), c.k0 + base + kStage * 32 + lane);
-            cp_async_commit();
-            srd = srd == kStage ? 0 : srd + 1;
-        } else {
-            nxt = Pol::none();
-            if (base + 32 + lane < len) nxt = pol.fetch(c.k0 + base + 32 + lane);
-        }
+        // The next batch's raw payload is loaded while this batch's rows are in
+        // flight; it is only decoded when its batch comes up.
+        const typename Pol::Raw cur = nxt;
+        nxt = Pol::none();
+        if (base + 32 + lane < len) nxt = pol.fetch(c.k0 + base + 32 + lane);
         uint32_t my_a = kInvalid;
         float my_w = 0.f;
         if (lane < nb) pol.decode(cur, my_a, my_w);
@@ -929,9 +631,11 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
                     const int src = i0 + u * G + g;
                     const uint32_t a = __shfl_sync(kFull, my_a, src);
                     const float w = W ? __shfl_sync(kFull, my_w, src) : 1.f;
-                    const uint4 x = __ldg(reinterpret_cast<const uint4*>(
-                        lane_base + static_cast<uint64_t>(a) * row_bytes));
-                    accumulate<Pol::kDtype, W>(ain, x, w);
+                    const uint4* p = reinterpret_cast<const uint4*>(lane_base + static_cast<uint64_t>(a) * row_bytes);
+                    uint4 x[VPL];
+#pragma unroll
+                    for (int k = 0; k < VPL; ++k) x[k] = __ldg(p + voff[k]);
+                    add(x, w);
                 }
             }
         } else if (clean) {
@@ -939,19 +643,7 @@ __device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uin
         } else {
             rows(std::false_type{}, my_a, my_w, nb);
         }
-        // Two-level summation: at most 32 / G terms per lane enter `ain` before
-        // it is folded into `aout`, which bounds the fp32 rounding error.
-        if (kTwoLevel) {
-#pragma unroll
-            for (int x = 0; x < E; ++x) {
-                aout[x] += ain[x];
-                ain[x] = 0.f;
-            }
-        }
-    }
-    if constexpr (KS > 0) {
-        cp_async_wait_all();
-        __syncwarp();
+        fold();
     }
     // Empty segments at the chunk end (last chunk of a table), and chunks with
     // no items; then the piece of the segment that runs past the chunk end.

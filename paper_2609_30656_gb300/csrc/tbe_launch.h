@@ -83,6 +83,15 @@ inline int fixup_grid(int64_t chunk_bound, int span, int num_sms) {
     return static_cast<int>(need < 1 ? 1 : (need < cap ? need : cap));
 }
 
+// The walkers' layout of a row of `vecs` 16-byte vectors: vectors per lane, and
+// rows per warp step (the most whose lanes, a power of two per row, fit a warp).
+inline int row_vectors_per_lane(int vecs) { return vecs <= 32 ? 1 : (vecs <= 64 ? 2 : 4); }
+inline int rows_per_step(int vecs) {
+    int lanes = 1;
+    while (lanes < vecs && lanes < 32) lanes *= 2;
+    return 32 / lanes;
+}
+
 // Payload bag of a lookup whose index is out of range: outside every table's
 // bags, so the reduce reads the zero row for it.
 constexpr uint32_t kDeadBag = 0xffffffffu;
@@ -176,13 +185,6 @@ void launch_bwd_reduce_f16(const Problem& P, const Plan& Q, const BwdOut& O, con
 void launch_bwd_reduce_bf16(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out, int cls,
                             int vpl, int gc, bool packed, bool apply, int64_t chunk_bound, int num_sms,
                             cudaStream_t s);
-// Rows per warp step fixed at compile time for a row of `vecs` 16-byte vectors
-// spread as (lanes, groups), or 0 when the layout is only known at run time.
-inline int compile_time_groups(int vpl, int lanes, int groups) {
-    if (vpl > 1) return 1;
-    if (lanes * groups == 32 && (groups == 1 || groups == 2 || groups == 4 || groups == 8)) return groups;
-    return 0;
-}
 void launch_weight_grad(const Problem& P, const Plan& Q, const void* grad_out, float* grad_w, int cls,
                         int dtype, int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,

@@ -29,16 +29,7 @@ namespace cbtbe {
 
 template <class KernelT>
 inline int occupancy_grid(KernelT kernel, int threads, int num_sms) {
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    return per_sm * num_sms;
-}
-
-inline int warp_grid(int64_t chunk_bound, int cap) {
-    const int64_t need = (chunk_bound + (kWarpThreads / 32) - 1) / (kWarpThreads / 32);
-    return static_cast<int>(max64(1, min64(need, cap)));
+    return resident_blocks(kernel, threads) * num_sms;
 }
 
 // ---------------------------------------------------------------- optimizer step
@@ -196,11 +187,6 @@ struct BwdPolicy {
     };
     __device__ __forceinline__ static Raw none() { return {0xffffffffu}; }
     __device__ __forceinline__ Raw fetch(int64_t q) const { return {load_stream(O.vals_sorted + q)}; }
-    static constexpr int kStageBytes = 4;
-    __device__ __forceinline__ void stage(char* dst, int64_t q) const { cp_async4(dst, O.vals_sorted + q); }
-    __device__ __forceinline__ Raw staged(const char* src) const {
-        return {*reinterpret_cast<const uint32_t*>(src)};
-    }
     // Sorted item: the bag whose grad_out row it gathers, and w_i * s_b.
     __device__ __forceinline__ void decode(const Raw& x, uint32_t& a, float& w) const {
         int64_t bag;
@@ -229,11 +215,6 @@ struct BwdPolicy {
         O.grad_offsets[seg - out_shift] = float_lo + static_cast<int64_t>(seg - seg_lo) * dim;
     }
     __device__ __forceinline__ void put_empty(int32_t, int, bool) const {}
-    __device__ __forceinline__ void emit(int32_t seg, int32_t L, bool started, bool ends,
-                                         float (&tot)[VPL][kElems], int v, bool group0) const {
-        if (started && (threadIdx.x & 31) == 0) seg_meta(seg);
-        put(seg, L, started, ends, tot, v, group0);
-    }
     // Lane v of a row group holds vectors v + 32k of the grad_out row: columns
     // [(v + 32k) * kElems, + kElems), written as fp32 gradients.
     __device__ __forceinline__ void put(int32_t seg, int32_t, bool started, bool ends,
@@ -289,8 +270,9 @@ struct BwdPolicy {
 #endif
 template <int GO, int VPL, bool PACKED, int GC, bool APPLY>
 constexpr int reduce_min_blocks() {
-    if (APPLY) return CB_REDUCE_APPLY_MIN_BLOCKS;
-    return GO != CB_F32 && VPL == 1 && GC > 0 && GC != 4 && !PACKED ? CB_REDUCE_HALF_MIN_BLOCKS
+    if (APPLY && VPL == 1) return CB_REDUCE_APPLY_MIN_BLOCKS;
+    if (VPL == 4) return 2;  // 16 columns per lane, in two levels
+    return GO != CB_F32 && VPL == 1 && GC != 4 && !PACKED ? CB_REDUCE_HALF_MIN_BLOCKS
                                                                     : CB_REDUCE_MIN_BLOCKS;
 }
 
@@ -326,23 +308,11 @@ __global__ void __launch_bounds__(kWarpThreads, reduce_min_blocks<GO, VPL, PACKE
         // The run of out-of-range lookups (the table's spare key, last) is
         // walked but never output: its items read the zero row.
         c.seg_hi = static_cast<int32_t>(O.live_end[t]);
-        c.lanes = td.grad_lanes;
-        c.groups = td.grad_groups;
         c.row_vecs = td.grad_vecs;
         c.last = false;
         if (lane == 0) Q.tail_owner[j] = -1;
-        if constexpr (GC > 0 && VPL == 1 && CB_ROW_WALKER) {
-            __shared__ EndSlot slots[kWarpThreads / 32][32];
-#if defined(CB_REDUCE_STAGE) && CB_REDUCE_STAGE > 0
-            __shared__ __align__(16) char stage[kWarpThreads / 32][(CB_REDUCE_STAGE + 1) * 32 * 4];
-            walk_rows<BwdPolicy<GO, VPL, PACKED, APPLY>, GC, 0, CB_REDUCE_STAGE>(
-                pol, c, P.zero_row, lane, slots[threadIdx.x >> 5], nullptr, stage[threadIdx.x >> 5]);
-#else
-            walk_rows<BwdPolicy<GO, VPL, PACKED, APPLY>, GC>(pol, c, P.zero_row, lane, slots[threadIdx.x >> 5]);
-#endif
-        } else {
-            walk_chunk<BwdPolicy<GO, VPL, PACKED, APPLY>, GC>(pol, c, P.zero_row, lane);
-        }
+        __shared__ EndSlot slots[kWarpThreads / 32][32];
+        walk_rows<BwdPolicy<GO, VPL, PACKED, APPLY>, GC>(pol, c, P.zero_row, lane, slots[threadIdx.x >> 5]);
         j = __shfl_sync(kFull, nxt, 0);
     }
 }
@@ -365,9 +335,9 @@ void launch_bwd_reduce_t(const Problem& P, const Plan& Q, const BwdOut& O, const
         return;                                                                          \
     }
     CB_CASE(1, 1, false) CB_CASE(1, 2, false) CB_CASE(1, 4, false) CB_CASE(1, 8, false)
-    CB_CASE(1, 0, false) CB_CASE(2, 1, false) CB_CASE(4, 1, false)
+    CB_CASE(1, 16, false) CB_CASE(1, 32, false) CB_CASE(2, 1, false) CB_CASE(4, 1, false)
     CB_CASE(1, 1, true) CB_CASE(1, 2, true) CB_CASE(1, 4, true) CB_CASE(1, 8, true)
-    CB_CASE(1, 0, true) CB_CASE(2, 1, true) CB_CASE(4, 1, true)
+    CB_CASE(1, 16, true) CB_CASE(1, 32, true) CB_CASE(2, 1, true) CB_CASE(4, 1, true)
 #undef CB_CASE
 }
 

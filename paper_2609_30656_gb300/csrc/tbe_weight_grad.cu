@@ -56,7 +56,7 @@ __device__ __forceinline__ float dot_row(const uint4& x, const char* g, int go_d
     return acc;
 }
 
-// GC > 0: rows of exactly V = 32 / GC vectors (one per lane), GC lookups per
+// GC > 0: rows of up to V = 32 / GC vectors (one per lane), GC lookups per
 // warp step. GC == 0: any row size, one lookup per step, each lane taking
 // vectors lane, lane + 32, ... of the row.
 template <int DT, int GC>
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kWarpThreads) weight_grad_kernel(const __grid_
                     const uint4* rp = rows + static_cast<int64_t>(a) * nvec;
                     const char* gp = go_base + go * eb;
                     if (GC > 0) {
-                        dot[u] = dot_row<DT>(__ldg(rp + v), gp + v * E * eb, P.out_dtype);
+                        if (v < nvec) dot[u] = dot_row<DT>(__ldg(rp + v), gp + v * E * eb, P.out_dtype);
                     } else {
                         for (int vec = v; vec < nvec; vec += 32)
                             dot[u] += dot_row<DT>(__ldg(rp + vec), gp + vec * E * eb, P.out_dtype);
@@ -157,6 +157,8 @@ void launch_dtype(const Problem& P, const Plan& Q, const void* go, float* gw, in
         case 2: launch_one<DT, 2>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
         case 4: launch_one<DT, 4>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
         case 8: launch_one<DT, 8>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
+        case 16: launch_one<DT, 16>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
+        case 32: launch_one<DT, 32>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
         default: launch_one<DT, 0>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
     }
 }
