@@ -61,6 +61,7 @@ struct Workspace {
     int64_t* table_pos = nullptr;
     int64_t* ord_chunk_base = nullptr;
     int64_t* class_chunk_base = nullptr;
+    int64_t* table_chunk = nullptr;
     Chunk* chunks = nullptr;
     float* carry_head = nullptr;
     float* carry_tail = nullptr;
@@ -71,6 +72,7 @@ struct Workspace {
     int64_t* sp_table_pos = nullptr;
     int64_t* sp_ord = nullptr;
     int64_t* sp_class_base = nullptr;
+    int64_t* sp_table_chunk = nullptr;
     Chunk* sp_tiles = nullptr;
     int64_t sp_max_tiles = 0;
     // backward
@@ -84,15 +86,10 @@ struct Workspace {
     uint32_t* tile_digits = nullptr;
     uint32_t* seg_sums = nullptr;
     int segments = 1;
-    int64_t* tile_heads = nullptr;
-    int64_t* tile_base = nullptr;
-    uint32_t* uniq = nullptr;
-    uint32_t* seg_start = nullptr;
-    int64_t* table_first = nullptr;
-    int64_t* live_end = nullptr;
+    uint32_t* heads = nullptr;
+    int64_t* run_count = nullptr;
     int64_t* out_first = nullptr;
     int64_t* float_base = nullptr;
-    int64_t* num_unique = nullptr;
     int64_t* out_sizes = nullptr;  // [2] U and F of a fused step (no caller buffers)
     int* cap_fail = nullptr;
     int4* heavy = nullptr;
@@ -131,6 +128,7 @@ struct cb_tbe {
     int32_t* d_all_start = nullptr;   // {0, T}
     int* d_error = nullptr;
     uint32_t* d_never_set = nullptr;
+    uint32_t* d_tables_done = nullptr;
     uint4* d_zero_row = nullptr;  // 2 KB of zeros
     // grown on demand
     void* ws = nullptr;
@@ -165,6 +163,7 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
     ws.table_pos = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.ord_chunk_base = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.class_chunk_base = static_cast<int64_t*>(take(sizeof(int64_t) * (nc + 1)));
+    ws.table_chunk = static_cast<int64_t*>(take(sizeof(int64_t) * T));
     ws.chunks = static_cast<Chunk*>(take(sizeof(Chunk) * max_chunks));
     ws.carry_head = static_cast<float*>(take(sizeof(float) * max_chunks * h->dmax));
     ws.carry_tail = static_cast<float*>(take(sizeof(float) * max_chunks * h->dmax));
@@ -179,6 +178,7 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
     ws.sp_table_pos = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.sp_ord = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.sp_class_base = static_cast<int64_t*>(take(sizeof(int64_t) * 2));
+    ws.sp_table_chunk = static_cast<int64_t*>(take(sizeof(int64_t) * T));
     ws.sp_tiles = static_cast<Chunk*>(take(sizeof(Chunk) * ws.sp_max_tiles));
     ws.sort_tiles = ws.sp_max_tiles;
     if (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) {
@@ -196,16 +196,10 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
         ws.tile_digits = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * ws.sort_tiles));
         ws.seg_sums = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * T * ws.segments));
     }
-    const int64_t rt = rle_num_tiles(n);
-    ws.tile_heads = static_cast<int64_t*>(take(sizeof(int64_t) * rt));
-    ws.tile_base = static_cast<int64_t*>(take(sizeof(int64_t) * rt));
-    ws.uniq = static_cast<uint32_t*>(take(sizeof(uint32_t) * n));
-    ws.seg_start = static_cast<uint32_t*>(take(sizeof(uint32_t) * (n + 1)));
-    ws.table_first = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
-    ws.live_end = static_cast<int64_t*>(take(sizeof(int64_t) * T));
+    ws.heads = static_cast<uint32_t*>(take(sizeof(uint32_t) * max_chunks));
+    ws.run_count = static_cast<int64_t*>(take(sizeof(int64_t) * T));
     ws.out_first = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.float_base = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
-    ws.num_unique = static_cast<int64_t*>(take(sizeof(int64_t)));
     ws.out_sizes = static_cast<int64_t*>(take(sizeof(int64_t) * 2));
     ws.cap_fail = static_cast<int*>(take(sizeof(int)));
     ws.max_heavy = max_chunks / 32 + 1;  // a heavy run owns more than 32 chunks
@@ -263,15 +257,16 @@ Plan make_plan(const cb_tbe* h, const Workspace& w, bool bwd, int64_t n) {
     const int64_t chunk_len = chunk_len_for(n, h->num_sms);
     Plan Q;
     Q.chunk_len = static_cast<int32_t>(chunk_len);
-    // Chunk boundaries move to the end of the bag / run they cut unless it is
-    // longer than this, so only heavy bags and hot rows are split.
-    Q.snap_cap = static_cast<int32_t>(bwd ? chunk_len : 4 * chunk_len);
+    // Chunk boundaries move to the end of the bag they cut unless it is longer
+    // than this, so only heavy bags are split.
+    Q.snap_cap = static_cast<int32_t>(4 * chunk_len);
     Q.num_classes = static_cast<int32_t>(bwd ? h->bwd_classes.size() : h->fwd_classes.size());
     Q.class_tables = bwd ? h->d_bwd_class_tables : h->d_fwd_class_tables;
     Q.class_table_start = bwd ? h->d_bwd_class_start : h->d_fwd_class_start;
     Q.table_pos = w.table_pos;
     Q.ord_chunk_base = w.ord_chunk_base;
     Q.class_chunk_base = w.class_chunk_base;
+    Q.table_chunk = w.table_chunk;
     Q.chunks = w.chunks;
     Q.max_chunks = w.max_chunks;
     Q.carry_head = w.carry_head;
@@ -352,7 +347,7 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     const bool packed = per_sample_weights != nullptr || h->mode == CB_POOL_MEAN;
 
     // (1) keys and payloads
-    launch_plan(P, Q, 0, nullptr, nullptr, h->num_sms, true, stream);
+    launch_plan(P, Q, false, h->num_sms, stream);
     h->launches += 2;
     const bool lookback = (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) != 0;
     if (lookback && cudaMemsetAsync(w.hist, 0, w.status_bytes, stream) != cudaSuccess) return CB_ERR_CUDA;
@@ -375,12 +370,13 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     SQ.table_pos = w.sp_table_pos;
     SQ.ord_chunk_base = w.sp_ord;
     SQ.class_chunk_base = w.sp_class_base;
+    SQ.table_chunk = w.sp_table_chunk;
     SQ.chunks = w.sp_tiles;
     SQ.max_chunks = w.sp_max_tiles;
     SQ.carry_head = SQ.carry_tail = nullptr;
     SQ.tail_owner = nullptr;
     SQ.chunk_next = nullptr;
-    launch_plan(P, SQ, 2, nullptr, nullptr, h->num_sms, true, stream);
+    launch_plan(P, SQ, true, h->num_sms, stream);
     h->launches += 2;
     if (lookback) {
         launch_sort_hist(w.keys[0], w.sp_tiles, w.sp_class_base + 1, w.sp_max_tiles, h->d_tables,
@@ -428,19 +424,16 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     h->last_sorted = w.vals[cur];
     h->last_sorted_n = n;
 
-    // (3) runs of equal ids, (4) per-table ranges and capacity check
-    launch_rle(w.keys[cur], n, w.tile_heads, w.tile_base, w.num_unique, w.uniq, w.seg_start, stream);
-    h->launches += 3;
+    // (3) runs of equal keys, (4) per-table ranges and capacity check
     BwdOut O;
-    O.seg_start = w.seg_start;
+    O.keys_sorted = w.keys[cur];
     O.vals_sorted = w.vals[cur];
     O.packed = packed ? w.packed : nullptr;
-    O.uniq = w.uniq;
-    O.num_unique_ws = w.num_unique;
-    O.table_first = w.table_first;
-    O.live_end = w.live_end;
+    O.heads = w.heads;
+    O.run_count = w.run_count;
     O.out_first = w.out_first;
     O.float_base = w.float_base;
+    O.tables_done = h->d_tables_done;
     O.cap_fail = w.cap_fail;
     O.heavy = w.heavy;
     O.heavy_count = w.heavy_count;
@@ -472,20 +465,17 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
         O.state = nullptr;
     }
     const bool reduce = a || g->grads;  // a sizing call stops after the run counts
-    launch_bwd_finalize(P, O, stream);
-    h->launches += 1;
-    if (reduce) launch_plan(P, Q, 1, w.seg_start, w.num_unique, h->num_sms, false, stream);
-    if (reduce) h->launches += 1;
+    launch_bwd_runs(P, Q, O, bound, stream);
+    h->launches += 2;
     record(h, h->ev_bwd[3], stream);
     nv.phase("bwd.reduce");
 
     // (5) segmented reduce, (6) fix-up of runs split across chunks
     if (reduce) {
-        for (size_t c = 0; c < h->bwd_classes.size(); ++c) {
-            launch_bwd_reduce(P, Q, O, grad_out, static_cast<int>(c), h->bwd_classes[c].vpl, h->bwd_classes[c].gc,
-                              packed, a != nullptr, bound, h->num_sms, stream);
-            h->launches += 1;
-        }
+        const KernelClass& k = h->bwd_classes[0];
+        launch_bwd_reduce(P, Q, O, grad_out, h->bwd_classes.size() > 1 ? -1 : 0, k.vpl, k.gc, packed, a != nullptr,
+                          bound, h->num_sms, stream);
+        h->launches += 1;
         launch_bwd_fixup(P, Q, O, bound, h->num_sms, stream);
         h->launches += 2;
         if (a) {
@@ -628,7 +618,7 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     for (int32_t t = 0; t < num_tables; ++t) all[t] = t;
     const size_t o_all = off; off += align_up(sizeof(int32_t) * num_tables);
     const size_t o_alls = off; off += align_up(sizeof(int32_t) * 2);
-    const size_t o_err = off; off += align_up(sizeof(int) + sizeof(uint32_t));
+    const size_t o_err = off; off += align_up(sizeof(int) + 2 * sizeof(uint32_t));
     const size_t o_zero = off; off += align_up(2048);
     if (cudaMalloc(&h->persist, off) != cudaSuccess) {
         cudaGetLastError();
@@ -645,6 +635,7 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     h->d_all_start = reinterpret_cast<int32_t*>(p + o_alls);
     h->d_error = reinterpret_cast<int*>(p + o_err);
     h->d_never_set = reinterpret_cast<uint32_t*>(p + o_err + sizeof(int));
+    h->d_tables_done = h->d_never_set + 1;
     h->d_zero_row = reinterpret_cast<uint4*>(p + o_zero);
     bool ok = cudaMemcpy(h->d_tables, h->tables.data(), sizeof(TableDev) * num_tables,
                          cudaMemcpyHostToDevice) == cudaSuccess;
@@ -660,7 +651,7 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
                           cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemcpy(h->d_all_start, all_start.data(), sizeof(int32_t) * 2,
                           cudaMemcpyHostToDevice) == cudaSuccess;
-    ok = ok && cudaMemset(h->d_error, 0, sizeof(int) + sizeof(uint32_t)) == cudaSuccess;
+    ok = ok && cudaMemset(h->d_error, 0, sizeof(int) + 2 * sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMemset(h->d_zero_row, 0, 2048) == cudaSuccess;
     if (ok && (flags & CB_TIMING)) {
         for (auto& e : h->ev_fwd) ok = ok && cudaEventCreate(&e) == cudaSuccess;
@@ -712,7 +703,7 @@ cb_status cb_tbe_forward(cb_tbe* h, int32_t batch, const void* indices, int64_t 
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
     Plan Q = make_plan(h, w, false, n);
     const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
-    launch_plan(P, Q, 0, nullptr, nullptr, h->num_sms, true, stream);
+    launch_plan(P, Q, false, h->num_sms, stream);
     h->launches += 2;
     record(h, h->ev_fwd[1], stream);
     nv.phase("fwd.gather");
@@ -758,7 +749,7 @@ cb_status cb_tbe_weight_grad(cb_tbe* h, int32_t batch, const void* indices, int6
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
     Plan Q = make_plan(h, w, false, n);
     const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
-    launch_plan(P, Q, 0, nullptr, nullptr, h->num_sms, true, stream);
+    launch_plan(P, Q, false, h->num_sms, stream);
     h->launches += 2;
     for (size_t c = 0; c < h->fwd_classes.size(); ++c) {
         // One vector per lane; wider rows loop.

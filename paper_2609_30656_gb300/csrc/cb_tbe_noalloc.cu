@@ -130,6 +130,7 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
     const size_t o_pos = off; off += up256(sizeof(int64_t) * (T + 1));
     const size_t o_ord = off; off += up256(sizeof(int64_t) * (T + 1));
     const size_t o_cb = off; off += up256(sizeof(int64_t) * (nc + 1));
+    const size_t o_tc = off; off += up256(sizeof(int64_t) * T);
     const size_t o_nx = off; off += up256(sizeof(uint32_t) * (nc + 1));  // chunk counters
     const size_t o_ch = off;
     auto scratch_end = [&](int64_t chunks) {
@@ -202,13 +203,14 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         Q.table_pos = reinterpret_cast<int64_t*>(base + o_pos);
         Q.ord_chunk_base = reinterpret_cast<int64_t*>(base + o_ord);
         Q.class_chunk_base = reinterpret_cast<int64_t*>(base + o_cb);
+        Q.table_chunk = reinterpret_cast<int64_t*>(base + o_tc);
         Q.chunks = reinterpret_cast<Chunk*>(base + o_ch);
         Q.max_chunks = max_chunks;
         Q.carry_head = reinterpret_cast<float*>(base + o_hd);
         Q.carry_tail = reinterpret_cast<float*>(base + o_tl);
         Q.tail_owner = reinterpret_cast<int64_t*>(base + o_to);
         Q.chunk_next = reinterpret_cast<uint32_t*>(base + o_nx);  // zeroed by the plan
-        launch_plan(P, Q, 0, nullptr, nullptr, num_sms, true, stream);
+        launch_plan(P, Q, false, num_sms, stream);
         bool one_dtype = true;
         for (const Cls& c : classes) one_dtype = one_dtype && c.dtype == classes[0].dtype;
         if (one_dtype && classes.size() > 1)

@@ -5,11 +5,10 @@
 // Steps: (1) key generation: one warp per chunk of lookups walks the bags and
 // writes key_i = key_base_t + indices[i] with a payload (the bag id, or the
 // lookup position plus a packed (bag, w_i * s_b) pair when a coefficient is
-// needed); (2) radix sort of each table's range;
-// (3) run-length pass over the sorted ids; (4) per-table unique ranges and
+// needed); (2) radix sort of each table's range; (3) runs of equal sorted keys,
+// counted per chunk of sorted positions, and (4) per-table output ranges and
 // packed gradient offsets; (5) segmented reduce of the gathered grad_out
-// slices, one warp per chunk of sorted positions; (6) fp64 fix-up of runs that
-// straddle chunks.
+// slices, one warp per chunk; (6) fp64 fix-up of runs that straddle chunks.
 #include <cuda_bf16.h>
 
 #include "tbe_internal.cuh"
@@ -17,10 +16,6 @@
 #include "tbe_reduce.cuh"
 
 namespace cbtbe {
-
-constexpr int kRleThreads = 256;
-constexpr int kRleItems = 16;
-constexpr int kRleTile = kRleThreads * kRleItems;
 
 // ---------------------------------------------------------------- (1) keys
 
@@ -183,202 +178,166 @@ __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q,
 
 // ---------------------------------------------------------------- (3) runs
 
-// Head flags of the kRleItems sorted keys starting at `base` (thread-blocked):
-// bit i is set when key[base + i] starts a run. Full groups load as four
-// 16-byte vectors; the key before the group comes from the previous lane.
-__device__ __forceinline__ uint32_t head_flags(const uint32_t* keys, int64_t n, int64_t base) {
-    uint32_t k[kRleItems];
-    if (base + kRleItems <= n) {
-        const uint4* v = reinterpret_cast<const uint4*>(keys + base);
-#pragma unroll
-        for (int i = 0; i < kRleItems / 4; ++i) {
-            const uint4 x = __ldg(v + i);
-            k[4 * i] = x.x;
-            k[4 * i + 1] = x.y;
-            k[4 * i + 2] = x.z;
-            k[4 * i + 3] = x.w;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < kRleItems; ++i) k[i] = base + i < n ? __ldg(keys + base + i) : 0u;
-    }
+// A table's sorted positions are cut into cells of chunk_len positions (the last
+// one shorter), numbered as its chunks. Per cell: how many runs begin in it (low
+// half) and where the first does (high half; kNoHead: none). One warp per cell,
+// all of its keys loaded before any is compared. The keys are read once more by
+// the reduce; nothing else about the runs is stored.
+constexpr uint32_t kNoHead = 0xffffu;
+
+__global__ void __launch_bounds__(kWarpThreads) bwd_heads_kernel(const __grid_constant__ Problem P,
+                                                                 const __grid_constant__ Plan Q,
+                                                                 const __grid_constant__ BwdOut O) {
+    constexpr int kBatches = kMaxChunk / 32;
     const int lane = threadIdx.x & 31;
-    uint32_t prev = __shfl_up_sync(kFull, k[kRleItems - 1], 1);
-    if (lane == 0 && base > 0 && base <= n) prev = __ldg(keys + base - 1);
-    uint32_t flags = 0;
+    const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
+    const int64_t j = warp_id_global();
+    if (j >= total) return;
+    const int t = Q.chunks[j].table;
+    const int64_t p0 = Q.table_pos[t], p1 = max64(p0, Q.table_pos[t + 1]);
+    const int64_t x0 = min64(p0 + (j - Q.table_chunk[t]) * Q.chunk_len, p1);
+    const int32_t len = static_cast<int32_t>(min64(Q.chunk_len, p1 - x0));
+    const uint32_t* keys = O.keys_sorted + x0;
+    uint32_t k[kBatches];
 #pragma unroll
-    for (int i = 0; i < kRleItems; ++i) {
-        const uint32_t before = i == 0 ? prev : k[i - 1];
-        const bool head = base + i < n && (base + i == 0 || k[i] != before);
-        flags |= head ? (1u << i) : 0u;
+    for (int i = 0; i < kBatches; ++i) k[i] = 32 * i + lane < len ? __ldg(keys + 32 * i + lane) : 0u;
+    uint32_t before = x0 > p0 ? __ldg(keys - 1) : ~k[0];  // (lane 0) a table's first key starts a run
+    uint32_t count = 0, first = kNoHead;
+#pragma unroll
+    for (int i = 0; i < kBatches; ++i) {
+        if (32 * i >= len) break;  // warp-uniform
+        uint32_t prev = __shfl_up_sync(kFull, k[i], 1);
+        if (lane == 0) prev = before;
+        const uint32_t b = __ballot_sync(kFull, 32 * i + lane < len && k[i] != prev);
+        count += __popc(b);
+        if (first == kNoHead && b) first = 32 * i + __ffs(b) - 1;
+        before = __shfl_sync(kFull, k[i], 31);
     }
-    return flags;
-}
-
-__global__ void __launch_bounds__(kRleThreads) rle_count_kernel(const uint32_t* keys, int64_t n,
-                                                                 int64_t* tile_heads) {
-    __shared__ int64_t sh[33];
-    const int64_t base = static_cast<int64_t>(blockIdx.x) * kRleTile + threadIdx.x * kRleItems;
-    const int64_t c = __popc(head_flags(keys, n, base));
-    int64_t total;
-    block_excl_scan(c, sh, &total);
-    if (threadIdx.x == 0) tile_heads[blockIdx.x] = total;
-}
-
-// One block over the tile counts in rounds of 1024 x 8: thread i takes 8
-// consecutive counts of the round (a warp reads 2 KB contiguous), one block
-// scan per round, the round's total carried into the next: 45 us on cfg5.
-// (With each thread owning 1/1024 of the counts every warp load touched 32
-// lines: 55 us; with 16 counts per thread, at 64 registers: 57 us.)
-__global__ void __launch_bounds__(1024) rle_scan_kernel(const int64_t* tile_heads, int64_t tiles,
-                                                        int64_t* tile_base, int64_t* num_unique) {
-    constexpr int kPer = 8;
-    __shared__ int64_t sh[33];
-    int64_t carry = 0;
-    for (int64_t c0 = 0; c0 < tiles; c0 += static_cast<int64_t>(blockDim.x) * kPer) {
-        const int64_t i0 = c0 + static_cast<int64_t>(threadIdx.x) * kPer;
-        int64_t v[kPer];
-        int64_t sum = 0;
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            v[u] = i0 + u < tiles ? tile_heads[i0 + u] : 0;
-            sum += v[u];
-        }
-        int64_t total;
-        int64_t run = carry + block_excl_scan(sum, sh, &total);
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            if (i0 + u < tiles) tile_base[i0 + u] = run;
-            run += v[u];
-        }
-        carry += total;
-    }
-    if (threadIdx.x == 0) *num_unique = carry;
-}
-
-#ifndef CB_RLE_FNS
-#define CB_RLE_FNS 1  // find a lane's n-th head with __fns (0: clear the earlier heads one by one)
-#endif
-
-// Each warp writes its run heads (unique key, start position) 32 at a time,
-// coalesced: lane l writes the warp's head x = x0 + l, found by a search over
-// the lanes' head prefixes (the owning lane) and then among that lane's 16 head
-// flags. With few repeats nearly every position is a head, and per-thread
-// stores would land 16 apart across the warp.
-__global__ void __launch_bounds__(kRleThreads) rle_write_kernel(const uint32_t* keys, int64_t n,
-                                                                const int64_t* tile_base,
-                                                                const int64_t* num_unique,
-                                                                uint32_t* uniq, uint32_t* seg_start) {
-    __shared__ int64_t sh[33];
-    const int lane = threadIdx.x & 31;
-    const int64_t base = static_cast<int64_t>(blockIdx.x) * kRleTile + threadIdx.x * kRleItems;
-    const uint32_t flags = head_flags(keys, n, base);
-    int64_t total;
-    const int64_t k = block_excl_scan(__popc(flags), sh, &total);
-    const int64_t wk = __shfl_sync(kFull, k, 0);                  // the warp's first head in the tile
-    const int32_t mine = static_cast<int32_t>(k - wk);            // this lane's first head in the warp
-    const int32_t wtot = __shfl_sync(kFull, mine + __popc(flags), 31);
-    uint32_t* uo = uniq + tile_base[blockIdx.x] + wk;
-    uint32_t* so = seg_start + tile_base[blockIdx.x] + wk;
-    const int64_t wbase = base - static_cast<int64_t>(lane) * kRleItems;  // lane 0's first position
-    for (int32_t x0 = 0; x0 < wtot; x0 += 32) {
-        const int32_t x = x0 + lane;
-        int j = 0;  // the last lane whose first head is at or before x: it holds head x
-#pragma unroll
-        for (int b = 16; b >= 1; b >>= 1)
-            if (__shfl_sync(kFull, mine, j + b) <= x) j += b;
-        uint32_t f = __shfl_sync(kFull, flags, j);
-        const int32_t mj = __shfl_sync(kFull, mine, j);
-        if (x < wtot) {
-            // head x is the lane's (x - mj + 1)-th head: that set bit of its flags
-            int bit;
-            if (CB_RLE_FNS) {
-                bit = static_cast<int>(__fns(f, 0, x - mj + 1));
-            } else {
-                for (int32_t r = x - mj; r > 0; --r) f &= f - 1;  // drop the lane's earlier heads
-                bit = __ffs(f) - 1;
-            }
-            const int64_t pos = wbase + static_cast<int64_t>(j) * kRleItems + bit;
-            uo[x] = __ldg(keys + pos);
-            so[x] = static_cast<uint32_t>(pos);
-        }
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) seg_start[*num_unique] = static_cast<uint32_t>(n);
+    if (lane == 0) O.heads[j] = count | (first << 16);
 }
 
 // ---------------------------------------------------------------- (4) ranges
 
-__global__ void __launch_bounds__(1024) bwd_finalize_kernel(Problem P, BwdOut O) {
+// One block per table scans its cells' counts into the reduce's chunks: a cell in
+// which a run begins becomes the chunk from that run on (the positions before it
+// join the chunk before), a cell without one stays a chunk inside a run, a piece
+// for the fix-up. So only runs that cover whole cells are split, and a piece
+// holds nothing but its run. The last block to finish lays out the output: first
+// row and first float of every table, the totals, and the capacity check.
+__global__ void __launch_bounds__(1024) bwd_runs_kernel(const __grid_constant__ Problem P,
+                                                        const __grid_constant__ Plan Q,
+                                                        const __grid_constant__ BwdOut O) {
+    constexpr int kPer = 4;
     __shared__ int64_t sh[33];
-    __shared__ int64_t run_rows, run_floats;
-    const int64_t U = *O.num_unique_ws;
-    // First run of each table: the first run key at or above key_base_t.
-    for (int t = threadIdx.x; t <= P.T; t += blockDim.x) {
-        const int64_t kb = t < P.T ? P.tables[t].key_base
-                                   : P.tables[P.T - 1].key_base + P.tables[P.T - 1].rows + 1;
-        int64_t a = 0, b = U;
-        while (a < b) {
-            const int64_t m = (a + b) >> 1;
-            if (static_cast<int64_t>(O.uniq[m]) < kb) a = m + 1; else b = m;
+    __shared__ bool sh_last;
+    const int t = blockIdx.x, tid = threadIdx.x;
+    if (t == 0)  // the walkers' chunk counters
+        for (int c = tid; c <= Q.num_classes; c += blockDim.x) Q.chunk_next[c] = 0;
+    const int64_t p0 = Q.table_pos[t], p1 = max64(p0, Q.table_pos[t + 1]);
+    const int64_t C = Q.chunk_len;
+    const int64_t c0 = Q.table_chunk[t];
+    const int64_t cells = min64(max64(1, (p1 - p0 + C - 1) / C), Q.max_chunks - c0);
+    int64_t carry = 0;
+    for (int64_t i0 = 0; i0 < cells; i0 += static_cast<int64_t>(blockDim.x) * kPer) {
+        const int64_t i = i0 + static_cast<int64_t>(tid) * kPer;
+        uint32_t h[kPer + 1];
+        int64_t sum = 0;
+#pragma unroll
+        for (int u = 0; u <= kPer; ++u) h[u] = i + u < cells && p1 > p0 ? O.heads[c0 + i + u] : kNoHead << 16;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) sum += h[u] & 0xffffu;
+        int64_t total;
+        int64_t run = carry + block_excl_scan(sum, sh, &total);
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            if (i + u < cells) {
+                const uint32_t f = h[u] >> 16, fn = h[u + 1] >> 16;
+                const int64_t x0 = min64(p0 + (i + u) * C, p1);
+                const int64_t k0 = f == kNoHead ? x0 : x0 + f;
+                int64_t k1 = p1;
+                if (i + u + 1 < cells) k1 = min64(p0 + (i + u + 1) * C, p1) + (fn == kNoHead ? 0 : fn);
+                Chunk ch;
+                ch.k0 = k0;
+                ch.first = run;
+                ch.table = t;
+                ch.len = static_cast<uint32_t>(max64(0, k1 - k0)) | (f == kNoHead && p1 > p0 ? 0x80000000u : 0u);
+                Q.chunks[c0 + i + u] = ch;
+            }
+            run += h[u] & 0xffffu;
         }
-        O.table_first[t] = a;
+        carry += total;
     }
-    if (threadIdx.x == 0) run_rows = run_floats = 0;
+    if (tid == 0) {
+        // A table's last run may hold its out-of-range lookups (the spare key):
+        // it is not output.
+        const TableDev& td = P.tables[t];
+        const bool dead = p1 > p0 && static_cast<int64_t>(O.keys_sorted[p1 - 1]) == td.key_base + td.rows;
+        O.run_count[t] = carry - (dead ? 1 : 0);
+        __threadfence();
+        sh_last = atomicAdd(O.tables_done, 1u) == static_cast<uint32_t>(P.T) - 1;
+    }
     __syncthreads();
-    // A table's last run may hold its out-of-range lookups (the spare key):
-    // it is not output. Output rows and floats are scanned over the rest.
+    if (!sh_last) return;
+    __threadfence();
+    int64_t rows = 0, floats = 0;
     for (int t0 = 0; t0 < P.T; t0 += blockDim.x) {
-        const int t = t0 + threadIdx.x;
-        int64_t live = 0, dim = 0;
-        if (t < P.T) {
-            const TableDev& td = P.tables[t];
-            const int64_t a = O.table_first[t], b = O.table_first[t + 1];
-            const bool dead = b > a && static_cast<int64_t>(O.uniq[b - 1]) == td.key_base + td.rows;
-            O.live_end[t] = dead ? b - 1 : b;
-            live = (dead ? b - 1 : b) - a;
-            dim = td.dim;
-        }
+        const int u = t0 + tid;
+        const int64_t live = u < P.T ? __ldcg(O.run_count + u) : 0;
+        const int64_t dim = u < P.T ? P.tables[u].dim : 0;
         int64_t rows_total, floats_total;
         const int64_t ex_rows = block_excl_scan(live, sh, &rows_total);
         const int64_t ex_floats = block_excl_scan(live * dim, sh, &floats_total);
-        if (t < P.T) {
-            O.out_first[t] = run_rows + ex_rows;
-            O.float_base[t] = run_floats + ex_floats;
+        if (u < P.T) {
+            O.out_first[u] = rows + ex_rows;
+            O.float_base[u] = floats + ex_floats;
+            if (O.table_offsets) O.table_offsets[u] = rows + ex_rows;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            run_rows += rows_total;
-            run_floats += floats_total;
-        }
-        __syncthreads();
+        rows += rows_total;
+        floats += floats_total;
     }
-    const int64_t Uo = run_rows, F = run_floats;
-    if (O.table_offsets)
-        for (int t = threadIdx.x; t <= P.T; t += blockDim.x) O.table_offsets[t] = t < P.T ? O.out_first[t] : Uo;
-    if (threadIdx.x == 0) {
-        O.out_first[P.T] = Uo;
-        O.float_base[P.T] = F;
-        *O.num_unique = Uo;
-        *O.num_floats = F;
+    if (tid == 0) {
+        O.out_first[P.T] = rows;
+        O.float_base[P.T] = floats;
+        if (O.table_offsets) O.table_offsets[P.T] = rows;
+        *O.num_unique = rows;
+        *O.num_floats = floats;
         int fail = 0;
         // After a timed-out sort pass the sorted order is not trustworthy.
         if (*reinterpret_cast<volatile int*>(P.error) == CB_ERR_TIMEOUT) fail = 1;
-        if (O.grads && (Uo > O.cap_rows || F > O.cap_floats)) {
+        if (O.grads && (rows > O.cap_rows || floats > O.cap_floats)) {
             set_error(P.error, CB_ERR_CAPACITY);
             fail = 1;
         }
         *O.cap_fail = fail;
-        if (O.grads && !fail) O.grad_offsets[Uo] = F;
+        if (O.grads && !fail) O.grad_offsets[rows] = floats;
+        *O.tables_done = 0;
     }
 }
 
 // ---------------------------------------------------------------- (6) fix-up
 
-// Runs split over chunks (hot rows longer than the snap cap): each warp scans
+// Runs split over chunks (hot rows that cover whole cells): each warp scans
 // `span` chunks at a time for tail pieces and combines each such run in fp64. Runs
 // spread over more than kHeavyPieces chunks go to a list that bwd_heavy_kernel
 // combines with a whole block each.
 constexpr int64_t kHeavyPieces = 32;
+
+// The chunks after chunk j that hold the rest of its open run: the pieces that
+// follow it (a piece holds one run only).
+__device__ __forceinline__ int64_t run_pieces(const Plan& Q, int64_t j, int t, int64_t total, int lane) {
+    int64_t m = 0;
+    for (;;) {
+        const int64_t i = j + 1 + m + lane;
+        bool more = false;
+        if (i < total) {
+            const Chunk& ch = Q.chunks[i];
+            more = (ch.len >> 31) != 0 && ch.table == t;
+        }
+        const uint32_t b = __ballot_sync(kFull, more);
+        if (b != kFull) return m + __ffs(~b) - 1;
+        m += 32;
+    }
+}
 
 __device__ __forceinline__ void store_grad4(float* dst, int x0, const double (&acc)[4]) {
     *reinterpret_cast<float4*>(dst + x0) =
@@ -398,8 +357,8 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_co
             const int b = __ffs(mask) - 1;
             const int64_t j = base + b;
             const int64_t seg = __shfl_sync(kFull, mine, b);
-            const int64_t e = O.seg_start[seg + 1];
-            const int64_t m = pieces_after(Q, j, e, total);
+            const int t = Q.chunks[j].table;
+            const int64_t m = run_pieces(Q, j, t, total, lane);
             if (m > kHeavyPieces) {
                 if (lane == 0) {
                     const uint32_t slot = atomicAdd(O.heavy_count, 1u);
@@ -409,11 +368,10 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_co
                 }
                 continue;
             }
-            const int t = Q.chunks[j].table;
             const TableDev& td = P.tables[t];
             // A fused step takes the combined row from the chunk's tail slot.
             float* dst = O.apply ? Q.carry_tail + j * P.dmax
-                                 : O.grads + O.float_base[t] + (seg - O.table_first[t]) * td.dim;
+                                 : O.grads + O.float_base[t] + seg * td.dim;
             combine_pieces(Q, j, m, td.dim, P.dmax, lane,
                            [&](int x0, double (&acc)[4]) { store_grad4(dst, x0, acc); });
         }
@@ -446,7 +404,7 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_heavy_kernel(const __grid_co
         __syncthreads();
         if (w == 0) {
             float* dst = O.apply ? Q.carry_tail + j * P.dmax
-                                 : O.grads + O.float_base[t] + (seg - O.table_first[t]) * td.dim;
+                                 : O.grads + O.float_base[t] + seg * td.dim;
             const float* tail = Q.carry_tail + j * P.dmax;
             for (int x0 = lane * 4; x0 < td.dim; x0 += 128) {
                 const float4 a = *reinterpret_cast<const float4*>(tail + x0);
@@ -473,10 +431,11 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_apply_split_kernel(const __g
         for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
             const int b = __ffs(mask) - 1;
             const int64_t j = base + b;
-            const int64_t seg = __shfl_sync(kFull, mine, b);
-            const int t = Q.chunks[j].table;
+            const Chunk ch = Q.chunks[j];
+            const int t = ch.table;
             const TableDev& td = P.tables[t];
-            const int64_t row = static_cast<int64_t>(O.uniq[seg]) - td.key_base;
+            // the chunk's last position belongs to the run
+            const int64_t row = static_cast<int64_t>(O.keys_sorted[ch.k0 + (ch.len & 0x7fffffffu) - 1]) - td.key_base;
             const float* g = Q.carry_tail + j * P.dmax;
             float sq = 0.f;
             for (int x0 = lane * 4; x0 < td.dim; x0 += 128) {
@@ -503,19 +462,10 @@ void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed
     }
 }
 
-int64_t rle_num_tiles(int64_t n) { return (n + kRleTile - 1) / kRleTile; }
-
-void launch_rle(const uint32_t* keys, int64_t n, int64_t* tile_heads, int64_t* tile_base,
-                int64_t* num_unique, uint32_t* uniq, uint32_t* seg_start, cudaStream_t s) {
-    const int64_t tiles = rle_num_tiles(n);
-    rle_count_kernel<<<static_cast<unsigned>(tiles), kRleThreads, 0, s>>>(keys, n, tile_heads);
-    rle_scan_kernel<<<1, 1024, 0, s>>>(tile_heads, tiles, tile_base, num_unique);
-    rle_write_kernel<<<static_cast<unsigned>(tiles), kRleThreads, 0, s>>>(keys, n, tile_base,
-                                                                         num_unique, uniq, seg_start);
-}
-
-void launch_bwd_finalize(const Problem& P, const BwdOut& O, cudaStream_t s) {
-    bwd_finalize_kernel<<<1, 1024, 0, s>>>(P, O);
+void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound, cudaStream_t s) {
+    const int64_t blocks = (chunk_bound + kWarpThreads / 32 - 1) / (kWarpThreads / 32);
+    bwd_heads_kernel<<<static_cast<unsigned>(max64(blocks, 1)), kWarpThreads, 0, s>>>(P, Q, O);
+    bwd_runs_kernel<<<static_cast<unsigned>(P.T), 1024, 0, s>>>(P, Q, O);
 }
 
 void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out, int cls,

@@ -33,40 +33,19 @@ constexpr int kWarpThreads = 256;  // block size of the warp-per-chunk kernels
 #ifndef CB_WALK_ROWS
 #define CB_WALK_ROWS 4  // 16-byte rows in flight per lane in the walker (with one vector per lane)
 #endif
-// Load groups ahead whose rows are prefetched into L1 (0: none), per kernel
-// (measured on cfg5 / cfg5u): the Zipf gather slows down by 2.4x with one
-// group ahead (its hot rows already live in L1), the reduce gains ~1 %.
-#ifndef CB_WALK_PREFETCH
-#define CB_WALK_PREFETCH 0
-#endif
-#ifndef CB_REDUCE_PREFETCH
-#define CB_REDUCE_PREFETCH 1
-#endif
+// The backward reduce's own targets, and those of its form with the optimizer
+// step fused (measured beside reduce_min_blocks).
 #ifndef CB_REDUCE_MIN_BLOCKS
-#define CB_REDUCE_MIN_BLOCKS 3  // the backward reduce's own targets (from the same sweep)
+#define CB_REDUCE_MIN_BLOCKS 3
 #endif
 #ifndef CB_REDUCE_ROWS
 #define CB_REDUCE_ROWS 8
 #endif
-// Row-walker code shape, per kernel (measured on cfg5): the forward keeps one
-// copy of the segment-end code per batch (unrolling it over the load groups
-// overflowed the instruction cache and doubled the gather time) and, since
-// warps take chunks from a counter, no separate unrolled path for batches with
-// no segment end either (gather 4.74 -> 4.49 ms without it); the fp32 backward
-// reduce also keeps one copy of its run-end code per batch but unrolls the
-// batches with no run end (reduce 5.40 -> 5.19 ms on cfg5; 18.45 -> 18.59 ms on
-// uniform indices, where nearly every batch has run ends).
-#ifndef CB_WALK_UNROLL_GROUPS
-#define CB_WALK_UNROLL_GROUPS 0
+#ifndef CB_REDUCE_APPLY_MIN_BLOCKS
+#define CB_REDUCE_APPLY_MIN_BLOCKS 4
 #endif
-#ifndef CB_WALK_FAST_BATCH
-#define CB_WALK_FAST_BATCH 0
-#endif
-#ifndef CB_REDUCE_UNROLL_GROUPS
-#define CB_REDUCE_UNROLL_GROUPS 0
-#endif
-#ifndef CB_REDUCE_FAST_BATCH
-#define CB_REDUCE_FAST_BATCH 1
+#ifndef CB_REDUCE_APPLY_ROWS
+#define CB_REDUCE_APPLY_ROWS 4
 #endif
 constexpr int64_t kNoSeg = INT64_MAX;
 
@@ -90,9 +69,11 @@ struct TableDev {
 // A run of at most chunk_len item positions of one table.
 struct Chunk {
     int64_t k0;     // first item position
-    int64_t first;  // first segment touching k0 (bag id, or unique-row index)
+    int64_t first;  // forward: first bag touching k0; backward: first run of the table
+                    // that begins at or after k0
     int32_t table;
-    uint32_t len;   // bit 31: last chunk of its table; bits 0..30: item count
+    uint32_t len;   // bits 0..30: item count; bit 31: last chunk of its table (forward),
+                    // or k0 lies inside a run begun earlier (backward)
 };
 
 struct Problem {
@@ -121,6 +102,7 @@ struct Plan {
     int64_t* table_pos;                // [T + 1] first item position of each table
     int64_t* ord_chunk_base;           // [T + 1] first chunk of class_tables[i]
     int64_t* class_chunk_base;         // [num_classes + 1]
+    int64_t* table_chunk;              // [T] first chunk of each table
     Chunk* chunks;                     // [max_chunks]
     int64_t max_chunks;
     float* carry_head;                 // [max_chunks, dmax] piece of a segment begun earlier
@@ -343,60 +325,22 @@ __device__ __forceinline__ void accumulate(float (&a)[Storage<DT>::kElems], cons
     }
 }
 
-// ---------------------------------------------------------------- the walker
+// ---------------------------------------------------------------- the walkers
 //
-// A warp walks one chunk of item positions in batches of 32. A row is spread
-// over V = 32 / G lanes, 16 bytes per lane and vector, VPL vectors per lane
-// (G = 1 for more than one), so a warp step gathers G rows; G is the largest
-// power of two with rows that fit V lanes. Lanes past a row that is not a power
-// of two of vectors load one of the row's own vectors again (the same cache
-// lines, no branch) and never store what they sum. Before a batch's rows are
-// loaded, the warp finds every segment ending inside the batch from a window of
-// 32 segment ends (one per lane): the positions of those ends become a 32-bit
-// mask, and their segment numbers go to a per-warp list in shared memory, in
-// order. Adding a row then costs a shuffle, one multiply-add for its address,
-// the loads and the adds, and the mask is tested once per group of loads; a
-// segment end costs one list read and the store of the sum. Empty segments
-// (empty bags) are written out during the scan.
-//
-// Positions inside the walker are relative to the chunk start and clamped to
-// [kRelLo, kRelHi], which keeps every comparison with [0, len] exact in 32 bits.
-// The segment range of the chunk is [first, seg_hi); segments that start at or
-// after the chunk end belong to the next chunk, except after the last chunk of a
-// table (trailing empty bags), which `last` allows.
-//
-// Pol (policy) supplies:
-//   kDtype, kElems, kVpl (16-byte vectors per lane), kUnroll (row steps in
-//   flight), kWeighted, kTwoLevel
-//   kEmptySegments     segments may be empty
-//   kUnrollGroups      unroll a batch's load groups
-//   kFastBatch         separate unrolled path for batches with no segment end
-//   kPrefetch          load groups ahead whose rows are prefetched into L1 (0: none)
-//   int64_t seg_begin(s), seg_end(s)    positions of segment s (s < seg_hi)
-//   Raw fetch(q), static Raw none()      raw payload of item q (loads only)
-//   void decode(Raw, uint32_t& a, float& w)  row number within `base`
-//                                            (kInvalid = skip) and coefficient
-//   const uint4* base; uint32_t stride       row a starts at base + a * stride
-//   void put(seg, len, started, ends, tot, v, is_group0)   a segment's sum, or
-//                                            its piece in this chunk
-//   void seg_meta(seg)                       metadata of a segment that began in
-//                                            this chunk (once per segment; lanes
-//                                            may call it for different segments
-//                                            at the same time)
-//   void put_empty(seg, v, is_group0)        the output of an empty segment
+// A warp walks one chunk of item positions in batches of 32 (forward: Gather in
+// tbe_forward.cuh; backward: Reduce in tbe_reduce.cuh). A row is spread over
+// V = 32 / G lanes, 16 bytes per lane and vector, VPL vectors per lane (G = 1 for
+// more than one), so a warp step gathers G rows; V is the smallest power of two
+// that holds the row. Lanes past a row that is not a power of two of vectors load
+// one of the row's own vectors again (the same cache lines, no branch) and never
+// store what they sum. Several steps' rows are loaded together, then added
+// segment by segment.
 
+// Forward positions are relative to the chunk start and clamped to
+// [kRelLo, kRelHi], which keeps every comparison with [0, len] exact in 32 bits.
 constexpr uint32_t kInvalid = 0xffffffffu;
 constexpr int32_t kRelLo = -1;
 constexpr int32_t kRelHi = 1 << 30;
-
-struct ChunkCtx {
-    int64_t k0;        // absolute position of the chunk's first item
-    int32_t len;       // items in the chunk
-    int32_t first;     // first segment
-    int32_t seg_hi;    // segments of this table end before seg_hi
-    int32_t row_vecs;  // vectors per row
-    bool last;         // owns trailing segments that start at the chunk end
-};
 
 __device__ __forceinline__ int32_t rel_pos(int64_t x, int64_t k0) {
     const int64_t r = x - k0;
@@ -413,245 +357,9 @@ struct EndSlot {
                   // piece of one that runs past the chunk end
 };
 
-// A row's cache lines requested into L1 ahead of its load, without a register.
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-template <class Pol, int G>
-__device__ __forceinline__ void walk_rows(Pol& pol, const ChunkCtx& c, const uint4* zero_row,
-                                          int lane, EndSlot* slots) {
-    constexpr int E = Pol::kElems;
-    constexpr int VPL = Pol::kVpl;
-    static_assert(G >= 1 && G <= 32 && (G & (G - 1)) == 0, "rows per warp step");
-    static_assert(VPL == 1 || G == 1, "several vectors per lane: one row per step");
-    constexpr int V = 32 / G;
-    constexpr int kSteps = 32 / G;                                      // row steps per batch
-    constexpr int UG = Pol::kUnroll < kSteps ? Pol::kUnroll : kSteps;  // row steps per load group
-    constexpr int kGroupItems = UG * G;
-    constexpr uint32_t kGroupMask = kGroupItems == 32 ? kFull : (1u << (kGroupItems & 31)) - 1u;
-    constexpr uint32_t kStepMask = G == 32 ? kFull : (1u << (G & 31)) - 1u;
-    constexpr bool W = Pol::kWeighted;
-    constexpr bool kTwoLevel = Pol::kTwoLevel;
-    constexpr int kGroupUnroll = Pol::kUnrollGroups ? 32 / kGroupItems : 1;
-    const int g = lane / V;
-    const int v = lane - g * V;
-    const int32_t len = c.len;
-    const char* lane_base = reinterpret_cast<const char*>(pol.base + (v < c.row_vecs ? v : 0));
-    const uint32_t row_bytes = pol.stride * 16u;
-    const uint4* zrow = zero_row + v;
-    const uint32_t below = (1u << lane) - 1u;
-    // Vector v + 32k of the row, relative to the lane's first (0 past the row).
-    int voff[VPL];
-#pragma unroll
-    for (int k = 0; k < VPL; ++k) voff[k] = k > 0 && v + 32 * k < c.row_vecs ? 32 * k : 0;
-
-    float ain[VPL][E], aout[VPL][kTwoLevel ? E : 1];
-#pragma unroll
-    for (int k = 0; k < VPL; ++k) {
-#pragma unroll
-        for (int x = 0; x < E; ++x) ain[k][x] = 0.f;
-#pragma unroll
-        for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[k][x] = 0.f;
-    }
-    auto add = [&](const uint4 (&x)[VPL], float w) {
-#pragma unroll
-        for (int k = 0; k < VPL; ++k) accumulate<Pol::kDtype, W>(ain[k], x[k], w);
-    };
-    // Two-level summation: at most 32 / G terms per lane enter `ain` before it is
-    // folded into `aout`, which bounds the fp32 rounding error (fp32 rows, tables
-    // or gradients; half-precision rows, whose tolerance is far looser, use one
-    // level, which frees registers for occupancy).
-    auto fold = [&]() {
-        if constexpr (kTwoLevel) {
-#pragma unroll
-            for (int k = 0; k < VPL; ++k)
-#pragma unroll
-                for (int x = 0; x < E; ++x) {
-                    aout[k][x] += ain[k][x];
-                    ain[k][x] = 0.f;
-                }
-        }
-    };
-
-    // Window: lane j holds the relative end of segment seg + j.
-    int32_t seg = c.first;
-    int32_t s_cur = seg < c.seg_hi ? rel_pos(pol.seg_begin(seg), c.k0) : kRelHi;
-    int32_t my_end = seg + lane < c.seg_hi ? rel_pos(pol.seg_end(seg + lane), c.k0) : kRelHi;
-    uint32_t mask = 0;
-
-    // Segments ending at or before `bend` (the batch starts at `base`) leave the
-    // window: non-empty ones are listed and marked in `mask`, empty ones owned
-    // by this chunk are written out. Ends are non-decreasing, so the finished
-    // segments are a prefix of the window.
-    auto scan = [&](int32_t base, int32_t bend) {
-        __syncwarp();  // every lane is done reading the previous batch's list
-        mask = 0;
-        int nend = 0;
-        for (;;) {
-            int32_t my_beg = __shfl_up_sync(kFull, my_end, 1);
-            if (lane == 0) my_beg = s_cur;
-            const bool nonempty = my_end > my_beg;
-            const bool done = my_end <= bend && (nonempty || my_end < len || c.last);
-            const uint32_t dm = __ballot_sync(kFull, done);
-            const uint32_t ne = __ballot_sync(kFull, done && nonempty);
-            if (done && nonempty) {
-                // (index masked: malformed offsets, which are reported, can
-                // break the prefix property but never reach past the list)
-                slots[(nend + __popc(ne & below)) & 31] = EndSlot{seg + lane, my_beg >= 0 ? my_end - my_beg : -1};
-                if (my_beg >= 0) pol.seg_meta(seg + lane);
-            }
-            if constexpr (Pol::kEmptySegments) {
-                for (uint32_t em = dm & ~ne; em; em &= em - 1) pol.put_empty(seg + __ffs(em) - 1, v, g == 0);
-            }
-            mask |= __reduce_or_sync(kFull, (done && nonempty) ? 1u << ((my_end - base - 1) & 31) : 0u);
-            nend += __popc(ne);
-            const int nd = __popc(dm);
-            if (nd == 0) break;
-            const int32_t last_end = __shfl_sync(kFull, my_end, nd - 1);
-            const int32_t moved = __shfl_down_sync(kFull, my_end, nd & 31);
-            s_cur = last_end;
-            seg += nd;
-            my_end = lane + nd < 32 ? moved
-                                    : (seg + lane < c.seg_hi ? rel_pos(pol.seg_end(seg + lane), c.k0) : kRelHi);
-            // A full window that finished before `bend` leaves more to find; at
-            // the chunk end, so may one that finished exactly there (empty
-            // segments at the end of the table's last chunk).
-            if (nd < 32 || (last_end >= bend && !(Pol::kEmptySegments && bend == len))) break;
-        }
-        __syncwarp();
-    };
-
-    auto flush = [&](const EndSlot s, bool ends) {
-        // Kept inside this chunk's segment range whatever the list holds.
-        const int32_t sseg = min(max(s.seg, c.first), c.seg_hi - 1);
-        float tot[VPL][E];
-#pragma unroll
-        for (int k = 0; k < VPL; ++k)
-#pragma unroll
-            for (int x = 0; x < E; ++x) tot[k][x] = kTwoLevel ? aout[k][x] + ain[k][x] : ain[k][x];
-#pragma unroll
-        for (int off = V; off < 32; off <<= 1)
-#pragma unroll
-            for (int x = 0; x < E; ++x) tot[0][x] += __shfl_xor_sync(kFull, tot[0][x], off);
-        pol.put(sseg, s.len, s.len >= 0, ends, tot, v, g == 0);
-#pragma unroll
-        for (int k = 0; k < VPL; ++k) {
-#pragma unroll
-            for (int x = 0; x < E; ++x) ain[k][x] = 0.f;
-#pragma unroll
-            for (int x = 0; x < (kTwoLevel ? E : 1); ++x) aout[k][x] = 0.f;
-        }
-    };
-
-    // One batch's rows: CLEAN = 32 valid items (no padding, no skipped item).
-    auto rows = [&](auto clean_tag, uint32_t my_a, float my_w, int nb) {
-        constexpr bool CLEAN = decltype(clean_tag)::value;
-        int ce = 0;
-#pragma unroll(kGroupUnroll)
-        for (int i0 = 0; i0 < 32; i0 += kGroupItems) {
-            if (!CLEAN && i0 >= nb) break;
-            uint4 buf[UG][VPL];
-            float wt[UG];
-#pragma unroll
-            for (int u = 0; u < UG; ++u) {
-                const int src = i0 + u * G + g;
-                const uint32_t a = __shfl_sync(kFull, my_a, src);
-                wt[u] = W ? __shfl_sync(kFull, my_w, src) : 1.f;
-                const uint4* p = reinterpret_cast<const uint4*>(lane_base + static_cast<uint64_t>(a) * row_bytes);
-#pragma unroll
-                for (int k = 0; k < VPL; ++k) buf[u][k] = __ldg(CLEAN || a != kInvalid ? p + voff[k] : zrow);
-            }
-            // The rows of the group kPrefetch groups ahead in this batch start
-            // moving into L1 while this group's loads are waited for.
-            if constexpr (Pol::kPrefetch > 0) {
-                const int pf = i0 + Pol::kPrefetch * kGroupItems;
-                if (pf < 32) {
-#pragma unroll
-                    for (int u = 0; u < UG; ++u) {
-                        const uint32_t a = __shfl_sync(kFull, my_a, pf + u * G + g);
-#pragma unroll
-                        for (int k = 0; k < VPL; ++k)
-                            if (a != kInvalid)
-                                prefetch_l1(lane_base + static_cast<uint64_t>(a) * row_bytes + 16 * voff[k]);
-                    }
-                }
-            }
-            const uint32_t m = (mask >> i0) & kGroupMask;
-            if (m == 0) {
-#pragma unroll
-                for (int u = 0; u < UG; ++u) add(buf[u], wt[u]);
-                continue;
-            }
-#pragma unroll
-            for (int u = 0; u < UG; ++u) {
-                uint32_t mu = (m >> (u * G)) & kStepMask;
-                if (mu == 0) {
-                    add(buf[u], wt[u]);
-                    continue;
-                }
-                // Segments end after item i0 + u*G + p for each set bit p; this
-                // group's item (p index g) belongs to the first of them with g <= p.
-                bool added = false;
-                do {
-                    const int p = __ffs(mu) - 1;
-                    if (!added && g <= p) {
-                        add(buf[u], wt[u]);
-                        added = true;
-                    }
-                    flush(slots[ce++], true);
-                    mu &= mu - 1;
-                } while (mu);
-                if (!added) add(buf[u], wt[u]);
-            }
-        }
-    };
-
-    typename Pol::Raw nxt = Pol::none();
-    if (lane < len) nxt = pol.fetch(c.k0 + lane);
-    for (int32_t base = 0; base < len; base += 32) {
-        const int nb = min(32, len - base);
-        // The next batch's raw payload is loaded while this batch's rows are in
-        // flight; it is only decoded when its batch comes up.
-        const typename Pol::Raw cur = nxt;
-        nxt = Pol::none();
-        if (base + 32 + lane < len) nxt = pol.fetch(c.k0 + base + 32 + lane);
-        uint32_t my_a = kInvalid;
-        float my_w = 0.f;
-        if (lane < nb) pol.decode(cur, my_a, my_w);
-        scan(base, base + nb);
-        const bool clean = __all_sync(kFull, my_a != kInvalid);
-        if (Pol::kFastBatch && clean && mask == 0) {
-            // The whole batch adds into the open segment: every load group
-            // unrolled, so loads of later groups overlap the adds of earlier ones.
-#pragma unroll
-            for (int i0 = 0; i0 < 32; i0 += kGroupItems) {
-#pragma unroll
-                for (int u = 0; u < UG; ++u) {
-                    const int src = i0 + u * G + g;
-                    const uint32_t a = __shfl_sync(kFull, my_a, src);
-                    const float w = W ? __shfl_sync(kFull, my_w, src) : 1.f;
-                    const uint4* p = reinterpret_cast<const uint4*>(lane_base + static_cast<uint64_t>(a) * row_bytes);
-                    uint4 x[VPL];
-#pragma unroll
-                    for (int k = 0; k < VPL; ++k) x[k] = __ldg(p + voff[k]);
-                    add(x, w);
-                }
-            }
-        } else if (clean) {
-            rows(std::true_type{}, my_a, my_w, nb);
-        } else {
-            rows(std::false_type{}, my_a, my_w, nb);
-        }
-        fold();
-    }
-    // Empty segments at the chunk end (last chunk of a table), and chunks with
-    // no items; then the piece of the segment that runs past the chunk end.
-    scan(len, len);
-    if (seg < c.seg_hi && s_cur < len) {
-        if (s_cur >= 0 && lane == 0) pol.seg_meta(seg);
-        flush(EndSlot{seg, s_cur >= 0 ? 0 : -1}, false);
-    }
+// A cache line requested into L2 ahead of its load, without a register.
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // ---------------------------------------------------------------- fix-up

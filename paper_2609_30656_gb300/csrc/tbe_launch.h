@@ -105,17 +105,15 @@ struct KeyGen {
 
 struct BwdOut {
     // workspace
-    const uint32_t* seg_start;   // [U + 1]
+    const uint32_t* keys_sorted; // [n] key_base_t + r
     const uint32_t* vals_sorted; // [n]
     const uint2* packed;         // [n] or null
-    const uint32_t* uniq;        // [U] sorted keys of the runs (key_base_t + r)
-    int64_t* num_unique_ws;      // U, runs of out-of-range lookups included
-    int64_t* table_first;        // [T + 1] first run of each table
-    int64_t* live_end;           // [T] one past table t's last run of real rows
-                                 // (table_first[t + 1], less the out-of-range run)
+    uint32_t* heads;             // [max_chunks] runs begun per chunk cell, and the first's offset
+    int64_t* run_count;          // [T] runs of real rows per table
     int64_t* out_first;          // [T + 1] first output row of each table (runs of
                                  // out-of-range lookups are not output)
     int64_t* float_base;         // [T + 1]
+    uint32_t* tables_done;       // zero between calls
     int* cap_fail;
     int4* heavy;                 // [max_heavy] runs left for the block-wide combine
     uint32_t* heavy_count;       // zeroed before the fix-up
@@ -142,8 +140,8 @@ constexpr int kApplyAdagrad = 2;
 void launch_validate_offsets(const Problem& P, int num_sms, cudaStream_t s);
 // The optimizer step of O.apply from the row-sparse gradient in O's caller buffers.
 void launch_apply_sparse(const Problem& P, const BwdOut& O, int num_sms, cudaStream_t s);
-void launch_plan(const Problem& P, const Plan& Q, int mode, const uint32_t* seg_start,
-                 const int64_t* num_unique, int num_sms, bool tables_too, cudaStream_t s);
+// The chunk plan over the lookups, or (tiles) table-aligned tiles for the sort.
+void launch_plan(const Problem& P, const Plan& Q, bool tiles, int num_sms, cudaStream_t s);
 
 void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int dtype, int vpl,
                        int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
@@ -165,10 +163,9 @@ int radix_pass_launches();  // kernels launch_radix_pass enqueues
 
 void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed, int64_t chunk_bound,
                    int num_sms, cudaStream_t s);
-int64_t rle_num_tiles(int64_t n);
-void launch_rle(const uint32_t* keys, int64_t n, int64_t* tile_heads, int64_t* tile_base,
-                int64_t* num_unique, uint32_t* uniq, uint32_t* seg_start, cudaStream_t s);
-void launch_bwd_finalize(const Problem& P, const BwdOut& O, cudaStream_t s);
+// Runs of equal sorted keys: counts per chunk cell, the reduce's chunks (cut at
+// run ends), and the sizes and first output rows of every table.
+void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound, cudaStream_t s);
 // The segmented reduce (apply: with the optimizer step fused), dispatched on
 // the grad_out type P.out_dtype; one translation unit per type.
 void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out, int cls,

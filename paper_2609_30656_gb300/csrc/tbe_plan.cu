@@ -50,7 +50,10 @@ __global__ void __launch_bounds__(1024) plan_tables_kernel(Problem P, Plan Q) {
             }
             int64_t total;
             const int64_t ex = block_excl_scan(cnt, sh, &total);
-            if (i < b) Q.ord_chunk_base[i] = running + ex;
+            if (i < b) {
+                Q.ord_chunk_base[i] = running + ex;
+                Q.table_chunk[Q.class_tables[i]] = running + ex;
+            }
             __syncthreads();
             if (tid == 0) running += total;
             __syncthreads();
@@ -63,9 +66,8 @@ __global__ void __launch_bounds__(1024) plan_tables_kernel(Problem P, Plan Q) {
     }
 }
 
-// Segment bounds around a position: the first bag of table t starting at or
-// after x (lower bound over the table's offsets), or the run of sorted ids
-// containing x.
+// The first bag of table t starting at or after x (lower bound over the table's
+// offsets).
 __device__ __forceinline__ int64_t bag_lower_bound(const Problem& P, int t, int64_t x) {
     const int64_t blo = static_cast<int64_t>(t) * P.B, bhi = blo + P.B;
     int64_t a = blo, b = bhi + 1;
@@ -76,35 +78,22 @@ __device__ __forceinline__ int64_t bag_lower_bound(const Problem& P, int t, int6
     return a;  // in [blo, bhi + 1]
 }
 
-__device__ __forceinline__ int64_t run_containing(const uint32_t* seg_start, int64_t U, int64_t x) {
-    int64_t a = 0, b = U + 1;
-    while (a < b) {
-        const int64_t m = (a + b) >> 1;
-        if (static_cast<int64_t>(seg_start[m]) <= x) a = m + 1; else b = m;
-    }
-    return max64(a - 1, 0);
-}
-
-// A chunk boundary at x moves to the end of the segment it falls in, unless
-// that segment is longer than the cap: short bags and runs are then never
-// split, and only heavy ones leave pieces for the fix-up. Monotone in x, so
-// consecutive chunks stay contiguous (a chunk may come out empty). One search
-// gives both the moved boundary and the first segment of a chunk starting
-// there:
-//   mode 0: the bag touching the chunk start (the bag starting exactly there if
-//           any, the first of equal starts; else the one containing it);
-//   mode 1: the run of sorted ids containing the chunk start;
-//   mode 2: tiles only (radix sort), no moving, first left at 0.
+// A chunk boundary at x moves to the end of the bag it falls in, unless that bag
+// is longer than the cap: short bags are then never split, and only heavy ones
+// leave pieces for the fix-up. Monotone in x, so consecutive chunks stay
+// contiguous (a chunk may come out empty). One search gives both the moved
+// boundary and the first bag touching it (the one starting exactly there if any,
+// the first of equal starts; else the one containing it). Sort tiles (`tiles`)
+// are not moved, and have no first bag.
 struct Boundary {
     int64_t k;      // position
     int64_t first;  // first segment of a chunk starting at k
 };
 
-__device__ __forceinline__ Boundary boundary(const Problem& P, const Plan& Q, int mode, int t,
-                                             const uint32_t* seg_start, int64_t U, int64_t x, int64_t p0,
-                                             int64_t p1) {
+__device__ __forceinline__ Boundary boundary(const Problem& P, const Plan& Q, bool tiles, int t, int64_t x,
+                                             int64_t p0, int64_t p1) {
     const bool may_move = Q.snap_cap > 0 && x > p0 && x < p1;
-    if (mode == 0) {
+    if (!tiles) {
         const int64_t blo = static_cast<int64_t>(t) * P.B, bhi = blo + P.B;
         const int64_t a = bag_lower_bound(P, t, x);  // first bag starting at or after x
         const int64_t e = a <= bhi ? load_index(P.offsets, a, P.is32) : -1;
@@ -118,25 +107,15 @@ __device__ __forceinline__ Boundary boundary(const Problem& P, const Plan& Q, in
         const int64_t first = (a <= bhi && e == k) ? a : a - 1;
         return {k, min64(max64(first, blo), bhi)};
     }
-    if (mode == 1) {
-        const int64_t u = run_containing(seg_start, U, x);
-        const int64_t s0 = seg_start[u], e = seg_start[u + 1];
-        // Runs are never empty (seg_start increases), so the run containing e is u + 1.
-        if (may_move && s0 != x && e - s0 <= Q.snap_cap && e <= p1) return {e, u + 1};
-        return {x, u};
-    }
     return {x, 0};
 }
 
 // 8 blocks of 256 threads per SM (32 registers): the grid (8 per SM) runs in
 // one wave of latency-bound searches.
-__global__ void __launch_bounds__(256, 8) plan_chunks_kernel(Problem P, Plan Q, int mode,
-                                                             const uint32_t* seg_start,
-                                                             const int64_t* num_unique) {
+__global__ void __launch_bounds__(256, 8) plan_chunks_kernel(Problem P, Plan Q, bool tiles) {
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t C = Q.chunk_len;
-    const int64_t U = mode == 1 ? *num_unique : 0;
     if (blockIdx.x == 0 && Q.chunk_next)  // the walkers' chunk counters (none for sort tiles)
         for (int c = threadIdx.x; c <= Q.num_classes; c += blockDim.x) Q.chunk_next[c] = 0;
     for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < total;
@@ -155,8 +134,8 @@ __global__ void __launch_bounds__(256, 8) plan_chunks_kernel(Problem P, Plan Q, 
         const bool last = local >= nch - 1;
         const int64_t x0 = min64(p0 + local * C, p1);
         const int64_t x1 = last ? p1 : min64(p0 + (local + 1) * C, p1);
-        const Boundary b0 = boundary(P, Q, mode, t, seg_start, U, x0, p0, p1);
-        const int64_t k1 = last ? x1 : boundary(P, Q, mode, t, seg_start, U, x1, p0, p1).k;
+        const Boundary b0 = boundary(P, Q, tiles, t, x0, p0, p1);
+        const int64_t k1 = last ? x1 : boundary(P, Q, tiles, t, x1, p0, p1).k;
         Chunk ch;
         ch.k0 = b0.k;
         ch.first = b0.first;
@@ -172,12 +151,11 @@ void launch_validate_offsets(const Problem& P, int num_sms, cudaStream_t s) {
     validate_offsets_kernel<<<max(blocks, 1), 256, 0, s>>>(P);
 }
 
-void launch_plan(const Problem& P, const Plan& Q, int mode, const uint32_t* seg_start,
-                 const int64_t* num_unique, int num_sms, bool tables_too, cudaStream_t s) {
-    if (tables_too) plan_tables_kernel<<<1, 1024, 0, s>>>(P, Q);
+void launch_plan(const Problem& P, const Plan& Q, bool tiles, int num_sms, cudaStream_t s) {
+    plan_tables_kernel<<<1, 1024, 0, s>>>(P, Q);
     const int blocks = static_cast<int>(
         min64((Q.max_chunks + 255) / 256, static_cast<int64_t>(num_sms) * 8));
-    plan_chunks_kernel<<<max(blocks, 1), 256, 0, s>>>(P, Q, mode, seg_start, num_unique);
+    plan_chunks_kernel<<<max(blocks, 1), 256, 0, s>>>(P, Q, tiles);
 }
 
 }  // namespace cbtbe

@@ -10,21 +10,6 @@
 #include "tbe_internal.cuh"
 #include "tbe_launch.h"
 
-// The reduce with the optimizer step fused carries more state (the table row
-// and its update), so it spilled at 3 blocks with 8 rows; measured on cfg5
-// (fused SGD / Adagrad ms): 8 rows at 3 blocks 14.46 / 17.24, 4 at 4 13.25 /
-// 15.47, 4 at 5 13.00 / 15.05, 2 at 5 12.93 / 14.83, 2 at 6 13.22 / 14.88,
-// 1 at 5 13.73 / 15.67.
-#ifndef CB_REDUCE_APPLY_ROWS
-#define CB_REDUCE_APPLY_ROWS 2  // rows in flight per lane with the optimizer step fused
-#endif
-#ifndef CB_REDUCE_HALF_ROWS
-#define CB_REDUCE_HALF_ROWS 4  // rows in flight per lane for fp16 / bf16 grad_out
-#endif
-#ifndef CB_REDUCE_HALF_FAST_BATCH
-#define CB_REDUCE_HALF_FAST_BATCH 1  // fp16 / bf16 grad_out: unrolled path for batches with no run end
-#endif
-
 namespace cbtbe {
 
 template <class KernelT>
@@ -130,10 +115,9 @@ struct GradRow {
 };
 
 template <int N>
-__device__ __noinline__ void apply_row(const Problem& P, const BwdOut& O, int t, int32_t seg,
+__device__ __noinline__ void apply_row(const Problem& P, const BwdOut& O, int t, uint32_t row,
                                        const GradRow<N> g, bool group0) {
     const TableDev& td = P.tables[t];
-    const int64_t row = static_cast<int64_t>(__ldg(O.uniq + seg)) - td.key_base;
     float sq = 0.f;
 #pragma unroll
     for (int k = 0; k < N; ++k)
@@ -148,136 +132,329 @@ __device__ __noinline__ void apply_row(const Problem& P, const BwdOut& O, int t,
 
 // ---------------------------------------------------------------- (5) reduce
 
+// One chunk of a table's sorted positions, walked by one warp in batches of 32.
+// A run ends where the next sorted key differs: one ballot over the keys of a
+// batch gives the mask of its ends, and runs are output in order, so the row a
+// run goes to follows from the chunk's first run by counting. (Taking the ends
+// from a list of run starts took a window scan per batch, a list in shared
+// memory, and two more passes over the keys to write the run keys and starts: on
+// the three batches below 1102 / 1294 / 3162 us, and 65 / 65 / 120 us more for the
+// runs.)
+// The end of a run is a few instructions, repeated in every step of a load
+// group: add, store, advance the output row. Runs cut by the chunk's edges leave
+// their piece in the carry rows. Out-of-range lookups sort to the table's end
+// under its spare key; the walk stops there.
 // APPLY: the optimizer step is fused where a run's sum ends (compiled as its
 // own kernels, so the gradient-writing reduce carries none of its code).
-template <int GO, int VPL, bool PACKED, bool APPLY>
-struct BwdPolicy {
-    static constexpr int kDtype = GO;  // grad_out storage: fp32, or fp16 / bf16 (mixed precision)
-    static constexpr int kElems = Storage<GO>::kElems;
-    static constexpr bool kTwoLevel = true;  // gradients keep the fp32 bound for every grad_out type
-    static constexpr int kVpl = VPL;
-    // Half grad_out rows (8 values per lane, usually 2 rows per warp step) take
-    // the forward's code shape: fewer rows in flight, one copy of the run-end
-    // code per batch.
-    static constexpr int kRows = APPLY ? CB_REDUCE_APPLY_ROWS : (GO == CB_F32 ? CB_REDUCE_ROWS : CB_REDUCE_HALF_ROWS);
-    static constexpr int kUnroll = kRows / VPL > 0 ? kRows / VPL : 1;
-    static constexpr bool kWeighted = PACKED;
-    static constexpr bool kUnrollGroups = GO == CB_F32 ? CB_REDUCE_UNROLL_GROUPS : false;
-    static constexpr bool kFastBatch = GO == CB_F32 ? CB_REDUCE_FAST_BATCH : CB_REDUCE_HALF_FAST_BATCH;
-    static constexpr int kPrefetch = CB_REDUCE_PREFETCH;
+template <int GO, int VPL, bool PACKED, bool APPLY, int G>
+struct Reduce {
+    static constexpr int E = Storage<GO>::kElems;  // grad_out storage: fp32, or fp16 / bf16 (mixed precision)
+    static constexpr int V = 32 / G;
+    static constexpr int kWide = (APPLY ? CB_REDUCE_APPLY_ROWS : CB_REDUCE_ROWS) / VPL;
+    static constexpr int UG = kWide < V ? kWide : V;  // row steps per load group
+    static constexpr int kItems = UG * G;
+    static constexpr uint32_t kItemMask = kItems == 32 ? kFull : (1u << (kItems & 31)) - 1u;
+    static constexpr uint32_t kStepMask = G == 32 ? kFull : (1u << (G & 31)) - 1u;
+    static constexpr bool kFastBatch = VPL == 1 && !APPLY;
+    static_assert(VPL == 1 || G == 1, "several vectors per lane: one row per step");
 
     const Problem& P;  // kernel parameters: read in place, not held in registers
     const Plan& Q;
     const BwdOut& O;
-    const uint4* base;  // grad_out + Doff_t, one row per bag of this table
-    int64_t float_lo;   // first float of this table in grads
-    uint32_t stride;    // 16-byte vectors per grad_out row
-    int32_t chunk;
-    int32_t bag_lo;
-    int32_t seg_lo;     // first run of this table
-    int32_t out_shift;  // run index - output row (runs of out-of-range lookups of
-                        // earlier tables are not output)
-    int32_t dim;
-    int32_t table;
+    int32_t j;  // the chunk
+    int32_t t;
+    int lane, g, v;
+    int32_t row_vecs, dim;
+    bool at_head;   // the open run began in an earlier chunk
+    float* dst;     // this lane's columns of the open run's output row
+    float* next;    // and of the run after it
+    float ain[VPL][E], aout[VPL][E];
 
-    __device__ __forceinline__ int64_t seg_begin(int32_t s) const { return __ldg(O.seg_start + s); }
-    __device__ __forceinline__ int64_t seg_end(int32_t s) const { return __ldg(O.seg_start + s + 1); }
-    struct Raw {
-        uint32_t v;
-    };
-    __device__ __forceinline__ static Raw none() { return {0xffffffffu}; }
-    __device__ __forceinline__ Raw fetch(int64_t q) const { return {load_stream(O.vals_sorted + q)}; }
-    // Sorted item: the bag whose grad_out row it gathers, and w_i * s_b.
-    __device__ __forceinline__ void decode(const Raw& x, uint32_t& a, float& w) const {
-        int64_t bag;
-        if (PACKED) {
-            if (x.v >= P.n) {  // only after an aborted sort pass: skip the item
-                a = kInvalid;
-                w = 0.f;
-                return;
-            }
-            const uint2 pk = __ldg(O.packed + x.v);
-            bag = pk.x;
-            w = __uint_as_float(pk.y);
-        } else {
-            bag = x.v;
-            w = 1.f;
-        }
-        const int64_t b = bag - bag_lo;
-        a = (b >= 0 && b < P.B) ? static_cast<uint32_t>(b) : kInvalid;
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int k = 0; k < VPL; ++k)
+#pragma unroll
+            for (int x = 0; x < E; ++x) ain[k][x] = aout[k][x] = 0.f;
     }
-    static constexpr bool kEmptySegments = false;
-    // Row id (row_base_t + r = key - t) and float offset of a run that begins
-    // in this chunk, at its output row.
-    __device__ __forceinline__ void seg_meta(int32_t seg) const {
-        if (APPLY) return;  // a fused step writes no gradient buffers
-        O.unique_ids[seg - out_shift] = static_cast<int64_t>(__ldg(O.uniq + seg)) - table;
-        O.grad_offsets[seg - out_shift] = float_lo + static_cast<int64_t>(seg - seg_lo) * dim;
+    __device__ __forceinline__ void add(const uint4 (&x)[VPL], float w) {
+#pragma unroll
+        for (int k = 0; k < VPL; ++k) accumulate<GO, PACKED>(ain[k], x[k], w);
     }
-    __device__ __forceinline__ void put_empty(int32_t, int, bool) const {}
-    // Lane v of a row group holds vectors v + 32k of the grad_out row: columns
-    // [(v + 32k) * kElems, + kElems), written as fp32 gradients.
-    __device__ __forceinline__ void put(int32_t seg, int32_t, bool started, bool ends,
-                                        float (&tot)[VPL][kElems], int v, bool group0) const {
-        const int64_t fo = float_lo + static_cast<int64_t>(seg - seg_lo) * dim;
-        if (started && !ends && (threadIdx.x & 31) == 0) Q.tail_owner[chunk] = seg;
+    __device__ __forceinline__ void store(float* at, const float (&t4)[VPL][E]) const {
+#pragma unroll
+        for (int k = 0; k < VPL; ++k)
+            if (v + 32 * k < row_vecs)
+#pragma unroll
+                for (int x = 0; x < E; x += 4)
+                    store_stream(reinterpret_cast<float4*>(at + 32 * k * E + x),
+                                 make_float4(t4[k][x], t4[k][x + 1], t4[k][x + 2], t4[k][x + 3]));
+    }
+    __device__ __forceinline__ float* carry(float* rows) const {
+        return rows + static_cast<int64_t>(j) * P.dmax + v * E;
+    }
+    // The sums of the open run over the lane groups, and a clean start.
+    __device__ __forceinline__ void total(float (&tot)[VPL][E]) {
+#pragma unroll
+        for (int k = 0; k < VPL; ++k)
+#pragma unroll
+            for (int x = 0; x < E; ++x) tot[k][x] = aout[k][x] + ain[k][x];
+#pragma unroll
+        for (int off = V; off < 32; off <<= 1)
+#pragma unroll
+            for (int x = 0; x < E; ++x) tot[0][x] += __shfl_xor_sync(kFull, tot[0][x], off);
+        zero();
+    }
+    // The end of a run (its key: `key`).
+    __device__ __forceinline__ void flush(uint32_t key) {
+        float tot[VPL][E];
+        total(tot);
         if constexpr (APPLY) {
-            if (started && ends) {
-                GradRow<VPL * kElems / 4> r;
+            if (!at_head) {
+                GradRow<VPL * E / 4> r;
 #pragma unroll
                 for (int k = 0; k < VPL; ++k)
 #pragma unroll
-                    for (int x = 0; x < kElems / 4; ++x) {
-                        const int col = (v + 32 * k) * kElems + 4 * x;
-                        r.v[k * (kElems / 4) + x] = make_float4(tot[k][4 * x], tot[k][4 * x + 1],
-                                                                tot[k][4 * x + 2], tot[k][4 * x + 3]);
-                        r.col[k * (kElems / 4) + x] = col < dim ? col : -1;
+                    for (int x = 0; x < E / 4; ++x) {
+                        const int col = (v + 32 * k) * E + 4 * x;
+                        r.v[k * (E / 4) + x] = make_float4(tot[k][4 * x], tot[k][4 * x + 1], tot[k][4 * x + 2],
+                                                           tot[k][4 * x + 3]);
+                        r.col[k * (E / 4) + x] = col < dim ? col : -1;
                     }
-                apply_row<VPL * kElems / 4>(P, O, table, seg, r, group0);
+                apply_row<VPL * E / 4>(P, O, t, key - static_cast<uint32_t>(P.tables[t].key_base), r, g == 0);
                 return;
             }
+            if (g == 0) store(dst, tot);
+            at_head = false;
+        } else {
+            if (g == 0) store(dst, tot);
+            at_head = false;
+            dst = next;
+            next += dim;
         }
-        if (!group0) return;
-        float* dst;
-        if (started && ends) dst = O.grads + fo;
-        else dst = (started ? Q.carry_tail : Q.carry_head) + static_cast<int64_t>(chunk) * P.dmax;
+    }
+
+    struct Item {
+        uint32_t key, after, val;
+    };
+    struct Walk {
+        const uint32_t* keys;
+        const uint32_t* vals;
+        int32_t len, table_end;  // items of the chunk; end of the table, relative to the chunk
+    };
+    __device__ __forceinline__ Item fetch(const Walk& w, int32_t q) const {
+        Item x{0u, 0u, 0u};
+        if (q < w.len) {
+            x.key = __ldg(w.keys + q);
+            x.after = q + 1 < w.table_end ? __ldg(w.keys + q + 1) : ~x.key;
+            x.val = load_stream(w.vals + q);
+        }
+        return x;
+    }
+    // (bag, bits of w_i * s_b) of a sorted item.
+    __device__ __forceinline__ uint2 coefficient(const Item& x) const {
+        if constexpr (PACKED) return __ldg(O.packed + min(x.val, static_cast<uint32_t>(P.n - 1)));
+        return make_uint2(x.val, 0u);
+    }
+
+    // grad_out rows of this table's bags start at `rows`, `stride` bytes apart.
+    __device__ __forceinline__ void walk(const Walk& w, const char* rows, uint32_t stride, bool piece, int64_t out_row,
+                                         int64_t out_float) {
+        const TableDev& td = P.tables[t];
+        const uint32_t dead = static_cast<uint32_t>(td.key_base + td.rows);
+        const uint32_t bag_lo = static_cast<uint32_t>(t) * static_cast<uint32_t>(P.B);
+        rows += (v < row_vecs ? v : 0) * 16;
+        int voff[VPL];  // lanes past the row load one of its vectors again and never store what they sum
 #pragma unroll
-        for (int k = 0; k < VPL; ++k) {
-            const int vec = v + 32 * k;
-            if (vec * kElems < dim) {
-                float4* d4 = reinterpret_cast<float4*>(dst + vec * kElems);
-#pragma unroll
-                for (int x = 0; x < kElems / 4; ++x)
-                    store_stream(d4 + x, make_float4(tot[k][4 * x], tot[k][4 * x + 1], tot[k][4 * x + 2],
-                                                     tot[k][4 * x + 3]));
+        for (int k = 0; k < VPL; ++k) voff[k] = k > 0 && v + 32 * k < row_vecs ? 512 * k : 0;
+        zero();
+        at_head = piece;
+        if constexpr (APPLY) {
+            dst = carry(Q.carry_head);
+        } else {
+            next = O.grads + out_float + v * E;
+            dst = piece ? carry(Q.carry_head) : next;
+            if (piece) out_row -= 1, out_float -= dim;  // the first end is that of the run before
+            else next += dim;
+        }
+        bool open = piece;  // the run of the next item began before it
+        Item nxt = fetch(w, lane), far{};
+        uint2 npk = coefficient(nxt);
+        if (PACKED) far = fetch(w, 32 + lane);
+        for (int32_t base = 0; base < w.len; base += 32) {
+            // The next batch's items are loaded while this batch's rows are in
+            // flight (with coefficients, which depend on them: one batch further).
+            const Item cur = nxt;
+            const uint2 pk = npk;
+            if (PACKED) {
+                nxt = far;
+                far = fetch(w, base + 64 + lane);
+            } else {
+                nxt = fetch(w, base + 32 + lane);
             }
+            npk = coefficient(nxt);
+            const bool have = base + lane < w.len && cur.key != dead;
+            const int nb = __popc(__ballot_sync(kFull, have));  // dead lookups are the last
+            if (nb == 0) break;
+            const bool end = have && cur.key != cur.after;
+            const uint32_t mask = __ballot_sync(kFull, end);
+            if constexpr (!APPLY) {
+                // Row id (row_base_t + r = key - t) and float offset of a run.
+                if (end) {
+                    const int r = __popc(mask & ((1u << lane) - 1u));
+                    O.unique_ids[out_row + r] = static_cast<int64_t>(cur.key) - t;
+                    O.grad_offsets[out_row + r] = out_float + static_cast<int64_t>(r) * dim;
+                }
+                out_row += __popc(mask);
+                out_float += static_cast<int64_t>(__popc(mask)) * dim;
+            } else if (end) {
+                // The table rows that this batch steps start moving into L2.
+                const char* row = static_cast<const char*>(td.data) +
+                                  static_cast<uint64_t>(cur.key - static_cast<uint32_t>(td.key_base)) * td.row_vecs * 16u;
+                for (int x = 0; x < td.row_vecs * 16; x += 128) prefetch_l2(row + x);
+                if (O.apply == kApplyAdagrad) prefetch_l2(O.state[t] + (cur.key - static_cast<uint32_t>(td.key_base)));
+            }
+            // Row of the bag within the table's (kept inside it whatever the payload).
+            const uint32_t my_a = have ? min(pk.x - bag_lo, static_cast<uint32_t>(P.B - 1)) : 0u;
+            // runs of one lookup, begun in this chunk
+            const uint32_t singles = mask & ((mask << 1) | (open ? 0u : 1u));
+            if (kFastBatch && mask == 0 && nb == 32) {
+                // The whole batch adds into the open run: every load group
+                // unrolled, so loads of later groups overlap the adds of earlier ones.
+#pragma unroll
+                for (int i = 0; i < 32; i += G) {
+                    const uint32_t a = __shfl_sync(kFull, my_a, i + g);
+                    const float c = PACKED ? __uint_as_float(__shfl_sync(kFull, pk.y, i + g)) : 1.f;
+                    const char* p = rows + static_cast<uint64_t>(a) * stride;
+                    uint4 x[VPL];
+#pragma unroll
+                    for (int k = 0; k < VPL; ++k) x[k] = __ldg(reinterpret_cast<const uint4*>(p + voff[k]));
+                    add(x, c);
+                }
+            } else
+#pragma unroll 1
+            for (int i0 = 0; i0 < nb; i0 += kItems) {
+                uint4 buf[UG][VPL];
+                float wt[UG];
+#pragma unroll
+                for (int u = 0; u < UG; ++u) {
+                    const int src = i0 + u * G + g;
+                    const uint32_t a = __shfl_sync(kFull, my_a, src);
+                    wt[u] = PACKED ? __uint_as_float(__shfl_sync(kFull, pk.y, src)) : 1.f;
+                    const char* p = rows + static_cast<uint64_t>(a) * stride;
+#pragma unroll
+                    for (int k = 0; k < VPL; ++k) buf[u][k] = __ldg(reinterpret_cast<const uint4*>(p + voff[k]));
+                }
+                const uint32_t m = (mask >> i0) & kItemMask;
+                if (m == 0 && i0 + kItems <= nb) {
+#pragma unroll
+                    for (int u = 0; u < UG; ++u) add(buf[u], wt[u]);
+                    continue;
+                }
+#pragma unroll
+                for (int u = 0; u < UG; ++u) {
+                    const int left = nb - (i0 + u * G);  // items from this step on
+                    if (left <= 0) break;
+                    uint32_t mu = (m >> (u * G)) & kStepMask;
+                    if (mu == 0) {
+                        if (G == 1 || g < left) add(buf[u], wt[u]);
+                        continue;
+                    }
+                    if constexpr (!APPLY) {
+                        if (((singles >> (i0 + u * G)) & kStepMask) == kStepMask) {
+                            // Every lane group's item is a whole run: each stores its own.
+                            float one[VPL][E] = {};
+#pragma unroll
+                            for (int k = 0; k < VPL; ++k) accumulate<GO, PACKED>(one[k], buf[u][k], wt[u]);
+                            store(dst + g * dim, one);
+                            dst += G * dim;
+                            next += G * dim;
+                            continue;
+                        }
+                    }
+                    if constexpr (G == 1) {
+                        add(buf[u], wt[u]);
+                        flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u) : 0u);
+                    } else {
+                        // Runs end after item i0 + u*G + p for each set bit p; this lane
+                        // group's item (p index g) belongs to the first of them with g <= p.
+                        bool added = g >= left;
+                        do {
+                            const int p = __ffs(mu) - 1;
+                            if (!added && g <= p) {
+                                add(buf[u], wt[u]);
+                                added = true;
+                            }
+                            flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u * G + p) : 0u);
+                            mu &= mu - 1;
+                        } while (mu);
+                        if (!added) add(buf[u], wt[u]);
+                    }
+                }
+            }
+            open = !((mask >> (nb - 1)) & 1u);
+            // Two-level summation: at most 32 / G terms per lane enter `ain`
+            // before it is folded into `aout`, which bounds the rounding error.
+#pragma unroll
+            for (int k = 0; k < VPL; ++k)
+#pragma unroll
+                for (int x = 0; x < E; ++x) {
+                    aout[k][x] += ain[k][x];
+                    ain[k][x] = 0.f;
+                }
+        }
+        if (open) {
+            // The run goes on in the next chunk: this chunk's piece of it.
+            float tot[VPL][E];
+            total(tot);
+            if (!at_head && lane == 0) {
+                // its number in the table, for the fix-up
+                Q.tail_owner[j] = APPLY ? 0 : out_row - O.out_first[t];
+            }
+            if (g == 0) store(carry(at_head ? Q.carry_head : Q.carry_tail), tot);
         }
     }
 };
 
-// Resident blocks per SM the reduce is compiled for: half-precision grad_out
-// slices with one vector per lane, no coefficient and no optimizer step fit 5
-// blocks' registers (48) without spilling, and more resident warps raise the
-// rate of the L2-served gathers; the optimizer-step form runs 5 blocks with
-// 2 rows in flight (CB_REDUCE_APPLY_ROWS); fp32 slices (8 rows in flight per
-// lane, whose uniform-index gathers come from DRAM and want the bytes in
-// flight) and the other forms keep CB_REDUCE_MIN_BLOCKS.
-#ifndef CB_REDUCE_HALF_MIN_BLOCKS
-#define CB_REDUCE_HALF_MIN_BLOCKS 5
-#endif
-#ifndef CB_REDUCE_APPLY_MIN_BLOCKS
-#define CB_REDUCE_APPLY_MIN_BLOCKS 5  // the reduce with the optimizer step fused
-#endif
-template <int GO, int VPL, bool PACKED, int GC, bool APPLY>
+// Resident blocks per SM the reduce is compiled for: 3 with 8 rows in flight per
+// lane, so that slices that come from DRAM or a distant L2 have the bytes in
+// flight; 4 with 4 rows when the optimizer step is fused, which carries the table
+// row too; 2 for four vectors per lane (16 columns in two levels). Measured, reduce
+// of 41 M lookups on skewed indices (fp32 grad_out) / 12 M uniform (bf16) / 26 M
+// weighted uniform (fp32), us: 8 rows at 3 blocks 1140 / 952 / 2675; 4 at 4 1133 /
+// 1167 (4 at 5) / 2925; 12 at 2 1331 / - / 2613; 16 at 2 - / 1017 / -. Fused Adagrad
+// step of 1.3 M lookups: 4 rows at 4 blocks 256, 2 at 5 262, 4 at 3 277.
+template <int VPL, bool APPLY>
 constexpr int reduce_min_blocks() {
-    if (APPLY && VPL == 1) return CB_REDUCE_APPLY_MIN_BLOCKS;
-    if (VPL == 4) return 2;  // 16 columns per lane, in two levels
-    return GO != CB_F32 && VPL == 1 && GC != 4 && !PACKED ? CB_REDUCE_HALF_MIN_BLOCKS
-                                                                    : CB_REDUCE_MIN_BLOCKS;
+    return VPL == 4 ? 2 : (APPLY && VPL == 1 ? CB_REDUCE_APPLY_MIN_BLOCKS : CB_REDUCE_MIN_BLOCKS);
 }
 
 template <int GO, int VPL, bool PACKED, int GC, bool APPLY>
-__global__ void __launch_bounds__(kWarpThreads, reduce_min_blocks<GO, VPL, PACKED, GC, APPLY>())
+__device__ __forceinline__ void reduce_chunk(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out,
+                                             int64_t j, const Chunk& ch, const TableDev& td, int lane) {
+    constexpr int eb = GO == CB_F32 ? 4 : 2;
+    const int t = ch.table;
+    Reduce<GO, VPL, PACKED, APPLY, GC> r{P, Q, O};
+    r.j = static_cast<int32_t>(j);
+    r.t = t;
+    r.lane = lane;
+    r.g = lane / r.V;
+    r.v = lane - r.g * r.V;
+    r.row_vecs = td.grad_vecs;
+    r.dim = td.dim;
+    typename Reduce<GO, VPL, PACKED, APPLY, GC>::Walk w;
+    w.keys = O.keys_sorted + ch.k0;
+    w.vals = O.vals_sorted + ch.k0;
+    w.len = static_cast<int32_t>(ch.len & 0x7fffffffu);
+    w.table_end = static_cast<int32_t>(Q.table_pos[t + 1] - ch.k0);
+    if (lane == 0) Q.tail_owner[j] = -1;
+    if (w.len == 0) return;
+    // ch.first: the chunk's first run that begins in it (the one after the piece)
+    r.walk(w, static_cast<const char*>(grad_out) + static_cast<int64_t>(td.doff) * eb, P.sum_d * eb, (ch.len >> 31) != 0,
+           O.out_first[t] + ch.first, O.float_base[t] + ch.first * td.dim);
+}
+
+template <int GO, int VPL, bool PACKED, int GC, bool APPLY>
+__global__ void __launch_bounds__(kWarpThreads, reduce_min_blocks<VPL, APPLY>())
     bwd_reduce_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q,
                       const __grid_constant__ BwdOut O, const void* grad_out, int cls) {
     if (*O.cap_fail) return;
@@ -287,51 +464,56 @@ __global__ void __launch_bounds__(kWarpThreads, reduce_min_blocks<GO, VPL, PACKE
     for (int64_t j = first_chunk(Q, cls, cb, lane); j < ce;) {
         const int64_t nxt = fetch_next_chunk(Q, cls, cb, lane);
         const Chunk ch = Q.chunks[j];
-        const int t = ch.table;
-        const TableDev& td = P.tables[t];
-        BwdPolicy<GO, VPL, PACKED, APPLY> pol{P, Q, O};
-        constexpr int eb = GO == CB_F32 ? 4 : 2;
-        pol.base = reinterpret_cast<const uint4*>(static_cast<const char*>(grad_out) +
-                                                  static_cast<int64_t>(td.doff) * eb);
-        pol.float_lo = O.float_base[t];
-        pol.stride = static_cast<uint32_t>(P.sum_d * eb / 16);
-        pol.chunk = static_cast<int32_t>(j);
-        pol.bag_lo = t * P.B;
-        pol.seg_lo = static_cast<int32_t>(O.table_first[t]);
-        pol.out_shift = static_cast<int32_t>(O.table_first[t] - O.out_first[t]);
-        pol.dim = td.dim;
-        pol.table = t;
-        ChunkCtx c;
-        c.k0 = ch.k0;
-        c.len = static_cast<int32_t>(ch.len & 0x7fffffffu);
-        c.first = static_cast<int32_t>(max64(ch.first, O.table_first[t]));
-        // The run of out-of-range lookups (the table's spare key, last) is
-        // walked but never output: its items read the zero row.
-        c.seg_hi = static_cast<int32_t>(O.live_end[t]);
-        c.row_vecs = td.grad_vecs;
-        c.last = false;
-        if (lane == 0) Q.tail_owner[j] = -1;
-        __shared__ EndSlot slots[kWarpThreads / 32][32];
-        walk_rows<BwdPolicy<GO, VPL, PACKED, APPLY>, GC>(pol, c, P.zero_row, lane, slots[threadIdx.x >> 5]);
+        reduce_chunk<GO, VPL, PACKED, GC, APPLY>(P, Q, O, grad_out, j, ch, P.tables[ch.table], lane);
         j = __shfl_sync(kFull, nxt, 0);
     }
 }
 
-template <int GO, int VPL, bool PACKED, int GC, bool APPLY>
-static void launch_reduce_one(const Problem& P, const Plan& Q, const BwdOut& O, const void* go,
-                              int cls, int64_t chunk_bound, int num_sms, cudaStream_t s) {
-    static int cap = occupancy_grid(bwd_reduce_kernel<GO, VPL, PACKED, GC, APPLY>, kWarpThreads, num_sms);
-    bwd_reduce_kernel<GO, VPL, PACKED, GC, APPLY><<<warp_grid(chunk_bound, cap), kWarpThreads, 0, s>>>(
-        P, Q, O, go, cls);
+// Tables of several row layouts in one launch, as in the forward.
+template <int GO, bool PACKED, bool APPLY>
+__global__ void __launch_bounds__(kWarpThreads, CB_REDUCE_MIN_BLOCKS)
+    bwd_reduce_mixed_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q,
+                            const __grid_constant__ BwdOut O, const void* grad_out) {
+    if (*O.cap_fail) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t ce = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
+    for (int64_t j = first_chunk(Q, Q.num_classes, 0, lane); j < ce;) {
+        const int64_t nxt = fetch_next_chunk(Q, Q.num_classes, 0, lane);
+        const Chunk ch = Q.chunks[j];
+        const TableDev& td = P.tables[ch.table];
+        switch (row_layout(td.grad_vecs)) {
+            case 0: reduce_chunk<GO, 1, PACKED, 32, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            case 1: reduce_chunk<GO, 1, PACKED, 16, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            case 2: reduce_chunk<GO, 1, PACKED, 8, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            case 3: reduce_chunk<GO, 1, PACKED, 4, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            case 4: reduce_chunk<GO, 1, PACKED, 2, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            case 5: reduce_chunk<GO, 1, PACKED, 1, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            case 6: reduce_chunk<GO, 2, PACKED, 1, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+            default: reduce_chunk<GO, 4, PACKED, 1, APPLY>(P, Q, O, grad_out, j, ch, td, lane); break;
+        }
+        j = __shfl_sync(kFull, nxt, 0);
+    }
 }
 
+template <auto Kernel, class... Args>
+static void launch_reduce_grid(int64_t chunk_bound, int num_sms, cudaStream_t s, const Args&... args) {
+    static const int cap = resident_blocks(Kernel, kWarpThreads);
+    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(args...);
+}
+
+// cls < 0: all classes, in one launch.
 template <int GO, bool APPLY>
 void launch_bwd_reduce_t(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out,
                          int cls, int vpl, int gc, bool packed, int64_t chunk_bound, int num_sms,
                          cudaStream_t s) {
+    if (cls < 0) {
+        if (packed) launch_reduce_grid<bwd_reduce_mixed_kernel<GO, true, APPLY>>(chunk_bound, num_sms, s, P, Q, O, grad_out);
+        else launch_reduce_grid<bwd_reduce_mixed_kernel<GO, false, APPLY>>(chunk_bound, num_sms, s, P, Q, O, grad_out);
+        return;
+    }
 #define CB_CASE(V, G, PK)                                                                \
     if (vpl == V && gc == G && packed == PK) {                                            \
-        launch_reduce_one<GO, V, PK, G, APPLY>(P, Q, O, grad_out, cls, chunk_bound, num_sms, s); \
+        launch_reduce_grid<bwd_reduce_kernel<GO, V, PK, G, APPLY>>(chunk_bound, num_sms, s, P, Q, O, grad_out, cls); \
         return;                                                                          \
     }
     CB_CASE(1, 1, false) CB_CASE(1, 2, false) CB_CASE(1, 4, false) CB_CASE(1, 8, false)
