@@ -134,11 +134,18 @@ struct cb_tbe {
     void* ws = nullptr;
     size_t ws_bytes = 0;
     cudaStream_t last_stream = nullptr;
+    // A size query whose sorted runs the workspace still holds (n < 0: none):
+    // any call that writes the workspace ends it.
+    int64_t query_n = -1;
+    int32_t query_batch = 0;
+    bool query_packed = false;
     // Sorted payloads of the last backward that reached the sort (workspace).
     const uint32_t* last_sorted = nullptr;
     int64_t last_sorted_n = 0;
     cudaEvent_t ev_fwd[4] = {};
     cudaEvent_t ev_bwd[5] = {};
+    cudaEvent_t ev_finish = nullptr;  // start of a reduce that finishes a size query
+    bool bwd_finished = false;
     bool fwd_timed = false;
     bool bwd_timed = false;
     uint64_t launches = 0;
@@ -210,6 +217,7 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
 }
 
 cb_status ensure_workspace(cb_tbe* h, int64_t B, int64_t n) {
+    h->query_n = -1;
     const size_t need = layout(h, B, n, nullptr, nullptr);
     if (need <= h->ws_bytes) return CB_OK;
     if (h->ws) {
@@ -306,49 +314,14 @@ struct ApplyArgs {
     float* const* state;
 };
 
-// The backward: into the caller's sparse-gradient buffers (g), or, with an
-// optimizer step (a), into the tables themselves.
-cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t num_indices,
-                        const void* offsets, const float* per_sample_weights, const void* grad_out,
-                        cb_sparse_grad* g, const ApplyArgs* a, cudaStream_t stream) {
-    cb_status st = check_common(h, batch, indices, num_indices, offsets);
-    if (st != CB_OK) return st;
-    const int64_t n = num_indices;
-    if (n >= (int64_t(1) << 30)) return CB_ERR_INVALID_ARG;
-    if (n > 0 && batch > 0 && (!grad_out || (reinterpret_cast<uintptr_t>(grad_out) & 15u)))
-        return CB_ERR_INVALID_ARG;
-    if (!current_device_ok(h)) return CB_ERR_INVALID_ARG;
-    h->last_stream = stream;
-    h->bwd_timed = false;
-    h->last_sorted = nullptr;
-    Problem P = make_problem(h, batch, indices, n, offsets, per_sample_weights);
-    Ranges nv(a ? "cb_tbe_backward_apply" : "cb_tbe_backward");
-    nv.phase("bwd.keygen");
-    record(h, h->ev_bwd[0], stream);
-    if ((h->flags & CB_VALIDATE) && batch > 0) {
-        launch_validate_offsets(P, h->num_sms, stream);
-        h->launches += 1;
-    }
-    if ((n == 0 || batch == 0) && a) return finish_call(h, stream);  // no row is touched
-    if (n == 0 || batch == 0) {
-        bool ok = cudaMemsetAsync(g->table_offsets, 0, sizeof(int64_t) * (h->T + 1), stream) == cudaSuccess;
-        ok = ok && cudaMemsetAsync(g->num_unique, 0, sizeof(int64_t), stream) == cudaSuccess;
-        ok = ok && cudaMemsetAsync(g->num_floats, 0, sizeof(int64_t), stream) == cudaSuccess;
-        if (g->grads) ok = ok && cudaMemsetAsync(g->grad_offsets, 0, sizeof(int64_t), stream) == cudaSuccess;
-        if (!ok) return CB_ERR_CUDA;
-        return finish_call(h, stream);
-    }
-    st = ensure_workspace(h, batch, n);
-    if (st != CB_OK) return st;
-    Workspace w;
-    layout(h, batch, n, static_cast<char*>(h->ws), &w);
-    Plan Q = make_plan(h, w, true, n);
-    const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
-    const bool packed = per_sample_weights != nullptr || h->mode == CB_POOL_MEAN;
-
+// The backward's first two steps: keys and payloads of every lookup, and the radix
+// sort of each table's range. The sorted pairs end in buffers passes & 1.
+cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Plan& Q, int64_t bound, bool packed,
+                       Ranges& nv, cudaStream_t stream) {
     // (1) keys and payloads
     launch_plan(P, Q, false, h->num_sms, stream);
     h->launches += 2;
+    const int64_t n = P.n;
     const bool lookback = (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) != 0;
     if (lookback && cudaMemsetAsync(w.hist, 0, w.status_bytes, stream) != cudaSuccess) return CB_ERR_CUDA;
     KeyGen K;
@@ -423,6 +396,60 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     nv.phase("bwd.rle");
     h->last_sorted = w.vals[cur];
     h->last_sorted_n = n;
+    return CB_OK;
+}
+
+// The backward: into the caller's sparse-gradient buffers (g), or, with an
+// optimizer step (a), into the tables themselves. finish: from the sorted runs
+// that a size query of the same batch left in the workspace.
+cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t num_indices,
+                        const void* offsets, const float* per_sample_weights, const void* grad_out,
+                        cb_sparse_grad* g, const ApplyArgs* a, bool finish, cudaStream_t stream) {
+    cb_status st = check_common(h, batch, indices, num_indices, offsets);
+    if (st != CB_OK) return st;
+    const int64_t n = num_indices;
+    if (n >= (int64_t(1) << 30)) return CB_ERR_INVALID_ARG;
+    if (n > 0 && batch > 0 && (!grad_out || (reinterpret_cast<uintptr_t>(grad_out) & 15u)))
+        return CB_ERR_INVALID_ARG;
+    if (!current_device_ok(h)) return CB_ERR_INVALID_ARG;
+    const bool packed = per_sample_weights != nullptr || h->mode == CB_POOL_MEAN;
+    if (finish && n > 0 && batch > 0 &&
+        (h->query_n != n || h->query_batch != batch || h->query_packed != packed))
+        return CB_ERR_INVALID_ARG;
+    h->last_stream = stream;
+    h->bwd_timed = false;
+    if (!finish) h->last_sorted = nullptr;
+    Problem P = make_problem(h, batch, indices, n, offsets, per_sample_weights);
+    Ranges nv(a ? "cb_tbe_backward_apply" : "cb_tbe_backward");
+    nv.phase(finish ? "bwd.reduce" : "bwd.keygen");
+    record(h, finish ? h->ev_finish : h->ev_bwd[0], stream);
+    if ((h->flags & CB_VALIDATE) && batch > 0 && !finish) {
+        launch_validate_offsets(P, h->num_sms, stream);
+        h->launches += 1;
+    }
+    if ((n == 0 || batch == 0) && a) return finish_call(h, stream);  // no row is touched
+    if (n == 0 || batch == 0) {
+        bool ok = cudaMemsetAsync(g->table_offsets, 0, sizeof(int64_t) * (h->T + 1), stream) == cudaSuccess;
+        ok = ok && cudaMemsetAsync(g->num_unique, 0, sizeof(int64_t), stream) == cudaSuccess;
+        ok = ok && cudaMemsetAsync(g->num_floats, 0, sizeof(int64_t), stream) == cudaSuccess;
+        if (g->grads) ok = ok && cudaMemsetAsync(g->grad_offsets, 0, sizeof(int64_t), stream) == cudaSuccess;
+        if (!ok) return CB_ERR_CUDA;
+        return finish_call(h, stream);
+    }
+    if (!finish) {
+        st = ensure_workspace(h, batch, n);
+        if (st != CB_OK) return st;
+    }
+    h->query_n = -1;
+    Workspace w;
+    layout(h, batch, n, static_cast<char*>(h->ws), &w);
+    Plan Q = make_plan(h, w, true, n);
+    const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
+    if (!finish) {
+        st = sort_lookups(h, P, w, Q, bound, packed, nv, stream);
+        if (st != CB_OK) return st;
+    }
+    const int cur = h->passes & 1;  // the buffers that the last sort pass wrote
 
     // (3) runs of equal keys, (4) per-table ranges and capacity check
     BwdOut O;
@@ -465,10 +492,16 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
         O.state = nullptr;
     }
     const bool reduce = a || g->grads;  // a sizing call stops after the run counts
-    launch_bwd_runs(P, Q, O, bound, stream);
-    h->launches += 2;
-    record(h, h->ev_bwd[3], stream);
-    nv.phase("bwd.reduce");
+    if (finish) {
+        launch_bwd_outputs(P, O, stream);
+        h->launches += 1;
+    } else {
+        launch_bwd_runs(P, Q, O, bound, stream);
+        h->launches += 2;
+        record(h, h->ev_bwd[3], stream);
+        nv.phase("bwd.reduce");
+    }
+    h->bwd_finished = finish;
 
     // (5) segmented reduce, (6) fix-up of runs split across chunks
     if (reduce) {
@@ -485,7 +518,18 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     }
     record(h, h->ev_bwd[4], stream);
     h->bwd_timed = (h->flags & CB_TIMING) != 0;
+    if (!reduce) {
+        h->query_n = n;
+        h->query_batch = batch;
+        h->query_packed = packed;
+    }
     return finish_call(h, stream);
+}
+
+bool sparse_grad_ok(const cb_sparse_grad* g) {
+    if (!g || !g->table_offsets || !g->num_unique || !g->num_floats) return false;
+    return !g->grads || (g->unique_ids && g->grad_offsets && g->cap_rows >= 0 && g->cap_floats >= 0 &&
+                         (reinterpret_cast<uintptr_t>(g->grads) & 15u) == 0);
 }
 
 }  // namespace
@@ -656,6 +700,7 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     if (ok && (flags & CB_TIMING)) {
         for (auto& e : h->ev_fwd) ok = ok && cudaEventCreate(&e) == cudaSuccess;
         for (auto& e : h->ev_bwd) ok = ok && cudaEventCreate(&e) == cudaSuccess;
+        ok = ok && cudaEventCreate(&h->ev_finish) == cudaSuccess;
     }
     if (!ok) {
         cudaGetLastError();
@@ -765,11 +810,16 @@ cb_status cb_tbe_backward(cb_tbe* h, int32_t batch, const void* indices, int64_t
                           const void* offsets, const float* per_sample_weights,
                           const void* grad_out, cb_sparse_grad* g, cudaStream_t stream) {
     if (!h) return CB_ERR_INVALID_ARG;
-    if (!g || !g->table_offsets || !g->num_unique || !g->num_floats) return CB_ERR_INVALID_ARG;
-    if (g->grads && (!g->unique_ids || !g->grad_offsets || g->cap_rows < 0 || g->cap_floats < 0 ||
-                     (reinterpret_cast<uintptr_t>(g->grads) & 15u)))
-        return CB_ERR_INVALID_ARG;
-    return backward_impl(h, batch, indices, num_indices, offsets, per_sample_weights, grad_out, g, nullptr,
+    if (!sparse_grad_ok(g)) return CB_ERR_INVALID_ARG;
+    return backward_impl(h, batch, indices, num_indices, offsets, per_sample_weights, grad_out, g, nullptr, false,
+                         stream);
+}
+
+cb_status cb_tbe_backward_finish(cb_tbe* h, int32_t batch, const void* indices, int64_t num_indices,
+                                 const void* offsets, const float* per_sample_weights,
+                                 const void* grad_out, cb_sparse_grad* g, cudaStream_t stream) {
+    if (!h || !sparse_grad_ok(g) || !g->grads) return CB_ERR_INVALID_ARG;
+    return backward_impl(h, batch, indices, num_indices, offsets, per_sample_weights, grad_out, g, nullptr, true,
                          stream);
 }
 
@@ -783,7 +833,7 @@ cb_status cb_tbe_backward_apply(cb_tbe* h, int32_t batch, const void* indices, i
     a.lr = lr;
     a.eps = eps;
     a.state = state;
-    return backward_impl(h, batch, indices, num_indices, offsets, per_sample_weights, grad_out, nullptr, &a,
+    return backward_impl(h, batch, indices, num_indices, offsets, per_sample_weights, grad_out, nullptr, &a, false,
                          stream);
 }
 
@@ -839,7 +889,8 @@ cb_status cb_tbe_last_timings(cb_tbe* h, float* ms, int32_t n) {
     }
     if (h->bwd_timed) {
         if (cudaEventSynchronize(h->ev_bwd[4]) != cudaSuccess) return CB_ERR_CUDA;
-        for (int i = 0; i < 4; ++i) cudaEventElapsedTime(&v[3 + i], h->ev_bwd[i], h->ev_bwd[i + 1]);
+        for (int i = 0; i < 3; ++i) cudaEventElapsedTime(&v[3 + i], h->ev_bwd[i], h->ev_bwd[i + 1]);
+        cudaEventElapsedTime(&v[6], h->bwd_finished ? h->ev_finish : h->ev_bwd[3], h->ev_bwd[4]);
     }
     for (int i = 0; i < n && i < kNumTimers; ++i) ms[i] = v[i];
     return CB_OK;
@@ -867,6 +918,7 @@ void cb_tbe_destroy(cb_tbe* h) {
         if (e) cudaEventDestroy(e);
     for (auto& e : h->ev_bwd)
         if (e) cudaEventDestroy(e);
+    if (h->ev_finish) cudaEventDestroy(h->ev_finish);
     cudaGetLastError();
     delete h;
 }

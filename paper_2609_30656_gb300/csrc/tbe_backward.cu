@@ -218,12 +218,49 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_heads_kernel(const __grid_co
 
 // ---------------------------------------------------------------- (4) ranges
 
+// The output's layout from the tables' run counts (one block): first row and
+// first float of every table, the totals, and the capacity check.
+__device__ __forceinline__ void output_ranges(const Problem& P, const BwdOut& O, int64_t* sh) {
+    const int tid = threadIdx.x;
+    int64_t rows = 0, floats = 0;
+    for (int t0 = 0; t0 < P.T; t0 += blockDim.x) {
+        const int u = t0 + tid;
+        const int64_t live = u < P.T ? __ldcg(O.run_count + u) : 0;
+        const int64_t dim = u < P.T ? P.tables[u].dim : 0;
+        int64_t rows_total, floats_total;
+        const int64_t ex_rows = block_excl_scan(live, sh, &rows_total);
+        const int64_t ex_floats = block_excl_scan(live * dim, sh, &floats_total);
+        if (u < P.T) {
+            O.out_first[u] = rows + ex_rows;
+            O.float_base[u] = floats + ex_floats;
+            if (O.table_offsets) O.table_offsets[u] = rows + ex_rows;
+        }
+        rows += rows_total;
+        floats += floats_total;
+    }
+    if (tid == 0) {
+        O.out_first[P.T] = rows;
+        O.float_base[P.T] = floats;
+        if (O.table_offsets) O.table_offsets[P.T] = rows;
+        *O.num_unique = rows;
+        *O.num_floats = floats;
+        int fail = 0;
+        // After a timed-out sort pass the sorted order is not trustworthy.
+        if (*reinterpret_cast<volatile int*>(P.error) == CB_ERR_TIMEOUT) fail = 1;
+        if (O.grads && (rows > O.cap_rows || floats > O.cap_floats)) {
+            set_error(P.error, CB_ERR_CAPACITY);
+            fail = 1;
+        }
+        *O.cap_fail = fail;
+        if (O.grads && !fail) O.grad_offsets[rows] = floats;
+    }
+}
+
 // One block per table scans its cells' counts into the reduce's chunks: a cell in
 // which a run begins becomes the chunk from that run on (the positions before it
 // join the chunk before), a cell without one stays a chunk inside a run, a piece
 // for the fix-up. So only runs that cover whole cells are split, and a piece
-// holds nothing but its run. The last block to finish lays out the output: first
-// row and first float of every table, the totals, and the capacity check.
+// holds nothing but its run. The last block to finish lays out the output.
 __global__ void __launch_bounds__(1024) bwd_runs_kernel(const __grid_constant__ Problem P,
                                                         const __grid_constant__ Plan Q,
                                                         const __grid_constant__ BwdOut O) {
@@ -279,39 +316,15 @@ __global__ void __launch_bounds__(1024) bwd_runs_kernel(const __grid_constant__ 
     __syncthreads();
     if (!sh_last) return;
     __threadfence();
-    int64_t rows = 0, floats = 0;
-    for (int t0 = 0; t0 < P.T; t0 += blockDim.x) {
-        const int u = t0 + tid;
-        const int64_t live = u < P.T ? __ldcg(O.run_count + u) : 0;
-        const int64_t dim = u < P.T ? P.tables[u].dim : 0;
-        int64_t rows_total, floats_total;
-        const int64_t ex_rows = block_excl_scan(live, sh, &rows_total);
-        const int64_t ex_floats = block_excl_scan(live * dim, sh, &floats_total);
-        if (u < P.T) {
-            O.out_first[u] = rows + ex_rows;
-            O.float_base[u] = floats + ex_floats;
-            if (O.table_offsets) O.table_offsets[u] = rows + ex_rows;
-        }
-        rows += rows_total;
-        floats += floats_total;
-    }
-    if (tid == 0) {
-        O.out_first[P.T] = rows;
-        O.float_base[P.T] = floats;
-        if (O.table_offsets) O.table_offsets[P.T] = rows;
-        *O.num_unique = rows;
-        *O.num_floats = floats;
-        int fail = 0;
-        // After a timed-out sort pass the sorted order is not trustworthy.
-        if (*reinterpret_cast<volatile int*>(P.error) == CB_ERR_TIMEOUT) fail = 1;
-        if (O.grads && (rows > O.cap_rows || floats > O.cap_floats)) {
-            set_error(P.error, CB_ERR_CAPACITY);
-            fail = 1;
-        }
-        *O.cap_fail = fail;
-        if (O.grads && !fail) O.grad_offsets[rows] = floats;
-        *O.tables_done = 0;
-    }
+    output_ranges(P, O, sh);
+    if (tid == 0) *O.tables_done = 0;
+}
+
+// The ranges alone, for a call that finishes a size query.
+__global__ void __launch_bounds__(1024) bwd_outputs_kernel(const __grid_constant__ Problem P,
+                                                           const __grid_constant__ BwdOut O) {
+    __shared__ int64_t sh[33];
+    output_ranges(P, O, sh);
 }
 
 // ---------------------------------------------------------------- (6) fix-up
@@ -466,6 +479,10 @@ void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t c
     const int64_t blocks = (chunk_bound + kWarpThreads / 32 - 1) / (kWarpThreads / 32);
     bwd_heads_kernel<<<static_cast<unsigned>(max64(blocks, 1)), kWarpThreads, 0, s>>>(P, Q, O);
     bwd_runs_kernel<<<static_cast<unsigned>(P.T), 1024, 0, s>>>(P, Q, O);
+}
+
+void launch_bwd_outputs(const Problem& P, const BwdOut& O, cudaStream_t s) {
+    bwd_outputs_kernel<<<1, 1024, 0, s>>>(P, O);
 }
 
 void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out, int cls,

@@ -28,7 +28,7 @@ _POOL = {"sum": 0, "mean": 1}
 _IDX = {torch.int32: 0, torch.int64: 1}
 
 # Every entry point declared in include/cb_tbe.h.
-EXPORTS = ("cb_tbe_create", "cb_tbe_reserve", "cb_tbe_forward", "cb_tbe_backward",
+EXPORTS = ("cb_tbe_create", "cb_tbe_reserve", "cb_tbe_forward", "cb_tbe_backward", "cb_tbe_backward_finish",
            "cb_tbe_get_error", "cb_tbe_last_timings", "cb_tbe_component_name",
            "cb_tbe_launch_count", "cb_tbe_status_string", "cb_tbe_destroy",
            "cb_tbe_forward_noalloc", "cb_fm_forward", "cb_fm_backward", "cb_tbe_weight_grad",
@@ -72,6 +72,7 @@ def load_library() -> ctypes.CDLL:
     lib.cb_tbe_reserve.argtypes = [p, i32, i64]
     lib.cb_tbe_forward.argtypes = [p, i32, p, i64, p, p, p, p]
     lib.cb_tbe_backward.argtypes = [p, i32, p, i64, p, p, p, ctypes.POINTER(CbSparseGrad), p]
+    lib.cb_tbe_backward_finish.argtypes = lib.cb_tbe_backward.argtypes
     lib.cb_tbe_get_error.argtypes = [p]
     lib.cb_tbe_last_timings.argtypes = [p, ctypes.POINTER(ctypes.c_float), i32]
     lib.cb_tbe_component_name.argtypes = [i32]
@@ -94,7 +95,7 @@ def load_library() -> ctypes.CDLL:
     lib.cb_gather_ceiling_tma.argtypes = [p, i64, i32, p, i64, p, p, p]
     lib.cb_fm_forward.argtypes = [p, i32, i32, i32, i64, p, p]
     lib.cb_fm_backward.argtypes = [p, p, i32, i32, i32, i64, p, p]
-    for name in ("cb_tbe_create", "cb_tbe_reserve", "cb_tbe_forward", "cb_tbe_backward",
+    for name in ("cb_tbe_create", "cb_tbe_reserve", "cb_tbe_forward", "cb_tbe_backward", "cb_tbe_backward_finish",
                  "cb_tbe_get_error", "cb_tbe_last_timings", "cb_fm_forward", "cb_fm_backward",
                  "cb_tbe_weight_grad", "cb_tbe_backward_apply", "cb_kjt_replicate",
                  "cb_tbe_sorted_payloads", "cb_gather_ceiling", "cb_gather_ceiling_f16", "cb_gather_ceiling_tma"):
@@ -237,18 +238,23 @@ class TBE:
     def alloc_grad(self, cap_rows: int, cap_floats: int, size_only: bool = False) -> SparseGrad:
         dev = self.device
         T = len(self.dims)
+        sizes = torch.zeros(2, dtype=torch.int64, device=dev)
         return SparseGrad(
             unique_ids=torch.empty(max(cap_rows, 1), dtype=torch.int64, device=dev),
             table_offsets=torch.empty(T + 1, dtype=torch.int64, device=dev),
             grad_offsets=torch.empty(max(cap_rows, 0) + 1, dtype=torch.int64, device=dev),
             grads=None if size_only else torch.empty(max(cap_floats, 4), dtype=torch.float32,
                                                      device=dev),
-            num_unique_dev=torch.zeros(1, dtype=torch.int64, device=dev),
-            num_floats_dev=torch.zeros(1, dtype=torch.int64, device=dev))
+            num_unique_dev=sizes[:1], num_floats_dev=sizes[1:])
 
     def backward_into(self, g: SparseGrad, indices, offsets, grad_out,
                       per_sample_weights=None, cap_rows: int | None = None,
                       cap_floats: int | None = None) -> SparseGrad:
+        return self._backward_into(self._lib.cb_tbe_backward, g, indices, offsets, grad_out, per_sample_weights,
+                                   cap_rows, cap_floats)
+
+    def _backward_into(self, call, g: SparseGrad, indices, offsets, grad_out, per_sample_weights,
+                       cap_rows: int | None = None, cap_floats: int | None = None) -> SparseGrad:
         T = len(self.dims)
         batch = (offsets.numel() - 1) // T
         ind = self._dev(indices, self.index_dtype)
@@ -262,18 +268,23 @@ class TBE:
             0 if g.grads is None else (g.grads.numel() if cap_floats is None else cap_floats),
             g.num_unique_dev.data_ptr(), g.num_floats_dev.data_ptr())
         with torch.cuda.device(self.device):
-            _check(self._lib.cb_tbe_backward(self._h, batch, _ptr(ind), ind.numel(), _ptr(off),
-                                             _ptr(w), _ptr(go), ctypes.byref(cs), self._stream()),
-                   "cb_tbe_backward")
+            _check(call(self._h, batch, _ptr(ind), ind.numel(), _ptr(off), _ptr(w), _ptr(go),
+                        ctypes.byref(cs), self._stream()), "cb_tbe_backward")
         return g
 
     def backward(self, indices, offsets, grad_out, per_sample_weights=None) -> SparseGrad:
-        """Sizes the output with a counting call, then computes the gradient."""
-        probe = self.alloc_grad(0, 0, size_only=True)
-        self.backward_into(probe, indices, offsets, grad_out, per_sample_weights)
-        U, F = probe.num_unique, probe.num_floats
+        """Counts the gradient's rows and values, then computes it into buffers of that size."""
+        ind = self._dev(indices, self.index_dtype)
+        off = self._dev(offsets, self.index_dtype)
+        w = self._dev(per_sample_weights, torch.float32)
+        go = self._dev(grad_out, self.out_dtype)
+        T = len(self.dims)
+        sizes = torch.empty(T + 3, dtype=torch.int64, device=self.device)
+        probe = SparseGrad(sizes, sizes[2:], sizes, None, sizes[:1], sizes[1:2])
+        self.backward_into(probe, ind, off, go, w)
+        U, F = sizes[:2].tolist()
         g = self.alloc_grad(U, F)
-        return self.backward_into(g, indices, offsets, grad_out, per_sample_weights)
+        return self._backward_into(self._lib.cb_tbe_backward_finish, g, ind, off, go, w)
 
     def backward_apply(self, indices, offsets, grad_out, per_sample_weights=None,
                        optimizer: str = "sgd", lr: float = 0.01, eps: float = 1e-8,

@@ -1,0 +1,68 @@
+"""A size query finished from its own sorted runs (cb_tbe_backward_finish) gives the
+bits of a full backward, and is refused when the workspace holds no such query."""
+
+import ctypes
+
+import pytest
+import torch
+
+from tests.helpers import random_problem
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+def _finish(m, g, ind, off, go, w):
+    return m._backward_into(m._lib.cb_tbe_backward_finish, g, ind, off, go, w)
+
+
+@pytest.mark.parametrize("weighted,pooling", [(False, "sum"), (True, "sum"), (False, "mean")])
+@pytest.mark.parametrize("batch,max_len", [(1, 1), (40, 30), (300, 900)])
+def test_finish_gives_the_full_calls_bits(weighted, pooling, batch, max_len):
+    from paper_2609_30656_gb300.tbe import TBE
+    tables, ind, off, w = random_problem(5, dims=(8, 64, 256), rows=(3, 700, 90), batch=batch, max_len=max_len,
+                                         weighted=weighted, empty_frac=0.1)
+    ind, off = ind.to(DEV), off.to(DEV)
+    w = None if w is None else w.to(DEV)
+    go = torch.randn(batch, 328, device=DEV)
+    m = TBE([t.to(DEV) for t in tables], pooling=pooling, validate=True)
+    n = ind.numel()
+    full = m.alloc_grad(n, n * 256)
+    m.backward_into(full, ind, off, go, w)
+    got = m.backward(ind, off, go, w)
+    U, F = full.num_unique, full.num_floats
+    assert (got.num_unique, got.num_floats) == (U, F)
+    assert torch.equal(got.unique_ids[:U], full.unique_ids[:U])
+    assert torch.equal(got.grad_offsets[:U + 1], full.grad_offsets[:U + 1])
+    assert torch.equal(got.table_offsets, full.table_offsets)
+    assert torch.equal(got.grads[:F], full.grads[:F])
+
+
+def test_finish_needs_the_query_before_it():
+    from paper_2609_30656_gb300.tbe import CB_ERR_CAPACITY, TBE, CbTbeError
+    tables, ind, off, _ = random_problem(6, batch=30)
+    ind, off = ind.to(DEV), off.to(DEV)
+    go = torch.randn(30, sum(t.shape[1] for t in tables), device=DEV)
+    m = TBE([t.to(DEV) for t in tables])
+    n = ind.numel()
+    g = m.alloc_grad(n, n * 24)
+    probe = m.alloc_grad(0, 0, size_only=True)
+    with pytest.raises(CbTbeError):
+        _finish(m, g, ind, off, go, None)          # no query yet
+    m.backward_into(probe, ind, off, go)
+    with pytest.raises(CbTbeError):
+        _finish(m, g, ind[:-1], off, go, None)     # another batch
+    with pytest.raises(CbTbeError):
+        _finish(m, g, ind, off, go, torch.rand(n, device=DEV))  # another kind of payload
+    _finish(m, g, ind, off, go, None)
+    with pytest.raises(CbTbeError):
+        _finish(m, g, ind, off, go, None)          # finished already
+    m.backward_into(probe, ind, off, go)
+    m.forward(ind, off)
+    with pytest.raises(CbTbeError):
+        _finish(m, g, ind, off, go, None)          # the forward used the workspace
+    m.backward_into(probe, ind, off, go)
+    small = m.alloc_grad(1, 8)
+    _finish(m, small, ind, off, go, None)
+    assert m.get_error() == CB_ERR_CAPACITY
+    assert small.num_unique == probe.num_unique
