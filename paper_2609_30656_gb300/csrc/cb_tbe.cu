@@ -69,10 +69,8 @@ struct Workspace {
     uint32_t* chunk_next = nullptr;
     int64_t max_chunks = 0;
     // radix sort plan: table-aligned tiles
-    int64_t* sp_table_pos = nullptr;
-    int64_t* sp_ord = nullptr;
-    int64_t* sp_class_base = nullptr;
-    int64_t* sp_table_chunk = nullptr;
+    int64_t* sp_first = nullptr;
+    int64_t* sp_num = nullptr;
     Chunk* sp_tiles = nullptr;
     int64_t sp_max_tiles = 0;
     // backward
@@ -124,8 +122,6 @@ struct cb_tbe {
     int32_t* d_fwd_class_start = nullptr;
     int32_t* d_bwd_class_tables = nullptr;
     int32_t* d_bwd_class_start = nullptr;
-    int32_t* d_all_tables = nullptr;  // 0..T-1, one class: the radix sort plan
-    int32_t* d_all_start = nullptr;   // {0, T}
     int* d_error = nullptr;
     uint32_t* d_never_set = nullptr;
     uint32_t* d_tables_done = nullptr;
@@ -182,10 +178,8 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
     }
     ws.packed = static_cast<uint2*>(take(sizeof(uint2) * n));
     ws.sp_max_tiles = n / kSortTileKeys + T + 1;
-    ws.sp_table_pos = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
-    ws.sp_ord = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
-    ws.sp_class_base = static_cast<int64_t*>(take(sizeof(int64_t) * 2));
-    ws.sp_table_chunk = static_cast<int64_t*>(take(sizeof(int64_t) * T));
+    ws.sp_first = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
+    ws.sp_num = static_cast<int64_t*>(take(sizeof(int64_t)));
     ws.sp_tiles = static_cast<Chunk*>(take(sizeof(Chunk) * ws.sp_max_tiles));
     ws.sort_tiles = ws.sp_max_tiles;
     if (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) {
@@ -319,8 +313,14 @@ struct ApplyArgs {
 cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Plan& Q, int64_t bound, bool packed,
                        Ranges& nv, cudaStream_t stream) {
     // (1) keys and payloads
-    launch_plan(P, Q, false, h->num_sms, stream);
-    h->launches += 2;
+    TilePlan S0{};
+    S0.tile_len = kSortTileKeys;
+    S0.tiles = w.sp_tiles;
+    S0.max_tiles = w.sp_max_tiles;
+    S0.table_first_tile = w.sp_first;
+    S0.num_tiles = w.sp_num;
+    launch_plan(P, Q, &S0, bound, h->num_sms, stream);
+    h->launches += plan_launches(P);
     const int64_t n = P.n;
     const bool lookback = (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) != 0;
     if (lookback && cudaMemsetAsync(w.hist, 0, w.status_bytes, stream) != cudaSuccess) return CB_ERR_CUDA;
@@ -334,27 +334,10 @@ cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Pl
     nv.phase("bwd.sort");
 
     // (2) radix sort of each table's range, 8 bits of the row number per pass
-    Plan SQ;
-    SQ.chunk_len = static_cast<int32_t>(kSortTileKeys);
-    SQ.snap_cap = 0;
-    SQ.num_classes = 1;
-    SQ.class_tables = h->d_all_tables;
-    SQ.class_table_start = h->d_all_start;
-    SQ.table_pos = w.sp_table_pos;
-    SQ.ord_chunk_base = w.sp_ord;
-    SQ.class_chunk_base = w.sp_class_base;
-    SQ.table_chunk = w.sp_table_chunk;
-    SQ.chunks = w.sp_tiles;
-    SQ.max_chunks = w.sp_max_tiles;
-    SQ.carry_head = SQ.carry_tail = nullptr;
-    SQ.tail_owner = nullptr;
-    SQ.chunk_next = nullptr;
-    launch_plan(P, SQ, true, h->num_sms, stream);
-    h->launches += 2;
     if (lookback) {
-        launch_sort_hist(w.keys[0], w.sp_tiles, w.sp_class_base + 1, w.sp_max_tiles, h->d_tables,
+        launch_sort_hist(w.keys[0], w.sp_tiles, w.sp_num, w.sp_max_tiles, h->d_tables,
                          h->passes, w.hist, h->num_sms, stream);
-        launch_sort_bases(w.hist, w.sp_table_pos, h->T, h->passes, w.digit_base, stream);
+        launch_sort_bases(w.hist, w.table_pos, h->T, h->passes, w.digit_base, stream);
         h->launches += 2;
     }
     int cur = 0;
@@ -365,8 +348,8 @@ cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Pl
         S.keys_out = w.keys[cur ^ 1];
         S.vals_out = w.vals[cur ^ 1];
         S.tiles = w.sp_tiles;
-        S.num_tiles = w.sp_class_base + 1;
-        S.table_first_tile = w.sp_ord;
+        S.num_tiles = w.sp_num;
+        S.table_first_tile = w.sp_first;
         S.tables = h->d_tables;
         S.n = n;
         S.shift = 8 * p;
@@ -382,7 +365,7 @@ cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Pl
             launch_onesweep(S, w.sp_max_tiles, stream);
             h->launches += 1;
         } else {
-            S.table_pos = w.sp_table_pos;
+            S.table_pos = w.table_pos;
             S.tile_digits = w.tile_digits;
             S.seg_sums = w.seg_sums;
             S.T = h->T;
@@ -658,10 +641,6 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     const size_t o_fcs = off; off += align_up(sizeof(int32_t) * fcs.size());
     const size_t o_bct = off; off += align_up(sizeof(int32_t) * bct.size());
     const size_t o_bcs = off; off += align_up(sizeof(int32_t) * bcs.size());
-    std::vector<int32_t> all(num_tables), all_start{0, num_tables};
-    for (int32_t t = 0; t < num_tables; ++t) all[t] = t;
-    const size_t o_all = off; off += align_up(sizeof(int32_t) * num_tables);
-    const size_t o_alls = off; off += align_up(sizeof(int32_t) * 2);
     const size_t o_err = off; off += align_up(sizeof(int) + 2 * sizeof(uint32_t));
     const size_t o_zero = off; off += align_up(2048);
     if (cudaMalloc(&h->persist, off) != cudaSuccess) {
@@ -675,8 +654,6 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     h->d_fwd_class_start = reinterpret_cast<int32_t*>(p + o_fcs);
     h->d_bwd_class_tables = reinterpret_cast<int32_t*>(p + o_bct);
     h->d_bwd_class_start = reinterpret_cast<int32_t*>(p + o_bcs);
-    h->d_all_tables = reinterpret_cast<int32_t*>(p + o_all);
-    h->d_all_start = reinterpret_cast<int32_t*>(p + o_alls);
     h->d_error = reinterpret_cast<int*>(p + o_err);
     h->d_never_set = reinterpret_cast<uint32_t*>(p + o_err + sizeof(int));
     h->d_tables_done = h->d_never_set + 1;
@@ -690,10 +667,6 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     ok = ok && cudaMemcpy(h->d_bwd_class_tables, bct.data(), sizeof(int32_t) * bct.size(),
                           cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemcpy(h->d_bwd_class_start, bcs.data(), sizeof(int32_t) * bcs.size(),
-                          cudaMemcpyHostToDevice) == cudaSuccess;
-    ok = ok && cudaMemcpy(h->d_all_tables, all.data(), sizeof(int32_t) * num_tables,
-                          cudaMemcpyHostToDevice) == cudaSuccess;
-    ok = ok && cudaMemcpy(h->d_all_start, all_start.data(), sizeof(int32_t) * 2,
                           cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(h->d_error, 0, sizeof(int) + 2 * sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMemset(h->d_zero_row, 0, 2048) == cudaSuccess;
@@ -748,8 +721,8 @@ cb_status cb_tbe_forward(cb_tbe* h, int32_t batch, const void* indices, int64_t 
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
     Plan Q = make_plan(h, w, false, n);
     const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
-    launch_plan(P, Q, false, h->num_sms, stream);
-    h->launches += 2;
+    launch_plan(P, Q, nullptr, bound, h->num_sms, stream);
+    h->launches += plan_launches(P);
     record(h, h->ev_fwd[1], stream);
     nv.phase("fwd.gather");
     if (h->fwd_one_dtype && h->fwd_classes.size() > 1) {
@@ -794,8 +767,8 @@ cb_status cb_tbe_weight_grad(cb_tbe* h, int32_t batch, const void* indices, int6
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
     Plan Q = make_plan(h, w, false, n);
     const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
-    launch_plan(P, Q, false, h->num_sms, stream);
-    h->launches += 2;
+    launch_plan(P, Q, nullptr, bound, h->num_sms, stream);
+    h->launches += plan_launches(P);
     for (size_t c = 0; c < h->fwd_classes.size(); ++c) {
         // One vector per lane; wider rows loop.
         const int gc = h->fwd_classes[c].vpl == 1 ? h->fwd_classes[c].gc : 0;

@@ -140,8 +140,20 @@ constexpr int kApplyAdagrad = 2;
 void launch_validate_offsets(const Problem& P, int num_sms, cudaStream_t s);
 // The optimizer step of O.apply from the row-sparse gradient in O's caller buffers.
 void launch_apply_sparse(const Problem& P, const BwdOut& O, int num_sms, cudaStream_t s);
-// The chunk plan over the lookups, or (tiles) table-aligned tiles for the sort.
-void launch_plan(const Problem& P, const Plan& Q, bool tiles, int num_sms, cudaStream_t s);
+// Table-aligned tiles of the sort, and the words to clear before it.
+struct TilePlan {
+    int64_t tile_len;           // 0: no tiles
+    struct Chunk* tiles;        // [max_tiles]
+    int64_t max_tiles;
+    int64_t* table_first_tile;  // [T + 1]
+    int64_t* num_tiles;         // device scalar
+    uint32_t* zero;             // [zero_words]
+    int64_t zero_words;
+};
+// The chunk plan over the lookups and, with S, the sort's tiles.
+void launch_plan(const Problem& P, const Plan& Q, const TilePlan* S, int64_t chunk_bound, int num_sms,
+                 cudaStream_t s);
+int plan_launches(const Problem& P);  // kernels launch_plan enqueues
 
 void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int dtype, int vpl,
                        int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
