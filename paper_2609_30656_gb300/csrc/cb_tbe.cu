@@ -770,10 +770,8 @@ cb_status cb_tbe_weight_grad(cb_tbe* h, int32_t batch, const void* indices, int6
     launch_plan(P, Q, nullptr, bound, h->num_sms, stream);
     h->launches += plan_launches(P);
     for (size_t c = 0; c < h->fwd_classes.size(); ++c) {
-        // One vector per lane; wider rows loop.
-        const int gc = h->fwd_classes[c].vpl == 1 ? h->fwd_classes[c].gc : 0;
-        launch_weight_grad(P, Q, grad_out, grad_weights, static_cast<int>(c), h->fwd_classes[c].dtype, gc,
-                           bound, h->num_sms, stream);
+        launch_weight_grad(P, Q, grad_out, grad_weights, static_cast<int>(c), h->fwd_classes[c].dtype,
+                           h->fwd_classes[c].vpl, h->fwd_classes[c].gc, bound, h->num_sms, stream);
         h->launches += 1;
     }
     return finish_call(h, stream);

@@ -19,87 +19,6 @@ namespace cbtbe {
 
 // ---------------------------------------------------------------- (1) keys
 
-// The bag of each lookup, from a window of 32 bag ends held one per lane, in
-// positions relative to the chunk start: every position is below 2^30, so these
-// are exact in 32 bits (saturated, for malformed offsets, well inside the
-// sentinel kPastTable that marks ends past the table's last bag).
-constexpr int32_t kPastTable = INT32_MAX;
-
-__device__ __forceinline__ int32_t rel32(int64_t x, int64_t k0) {
-    const int64_t r = x - k0;
-    return static_cast<int32_t>(r < -(int64_t(1) << 30) ? -(int64_t(1) << 30)
-                                                        : (r > (int64_t(1) << 30) ? (int64_t(1) << 30) : r));
-}
-
-struct BagWindow32 {
-    int64_t win;        // first bag of the window
-    int32_t win_start;  // start of bag win
-    int32_t my_end;     // end of bag win + lane
-};
-
-__device__ __forceinline__ BagWindow32 bag_window32(const Problem& P, int64_t first, int64_t bag_hi,
-                                                    int64_t k0, int lane) {
-    BagWindow32 W;
-    W.win = first;
-    W.win_start = first < bag_hi ? rel32(load_index(P.offsets, first, P.is32), k0) : kPastTable;
-    W.my_end = first + lane < bag_hi ? rel32(load_index(P.offsets, first + lane + 1, P.is32), k0) : kPastTable;
-    return W;
-}
-
-// Every lane calls this with its relative position q; the window moves forward
-// 32 bags at a time until every valid lane has its bag (bag = -1 otherwise).
-__device__ __forceinline__ void find_bag32(const Problem& P, BagWindow32& W, int64_t bag_hi, int64_t k0,
-                                           int32_t q, bool valid, int lane, int64_t& bag, int32_t& s,
-                                           int32_t& e) {
-    bag = -1;
-    s = e = 0;
-    while (true) {
-        int cnt = 0;  // ends at or before q in the window
-#pragma unroll
-        for (int b = 16; b >= 1; b >>= 1)
-            if (__shfl_sync(kFull, W.my_end, cnt + b - 1) <= q) cnt += b;
-        if (__shfl_sync(kFull, W.my_end, 31) <= q) cnt = 32;
-        const int32_t e_sel = __shfl_sync(kFull, W.my_end, cnt < 32 ? cnt : 31);
-        const int32_t s_sel = __shfl_sync(kFull, W.my_end, cnt > 0 ? cnt - 1 : 0);
-        if (valid && bag < 0 && cnt < 32) {
-            bag = W.win + cnt;
-            e = e_sel;
-            s = cnt > 0 ? s_sel : W.win_start;
-        }
-        if (!__any_sync(kFull, valid && bag < 0)) break;
-        W.win_start = __shfl_sync(kFull, W.my_end, 31);
-        W.win += 32;
-        W.my_end = W.win + lane < bag_hi ? rel32(load_index(P.offsets, W.win + lane + 1, P.is32), k0) : kPastTable;
-    }
-}
-
-// The bags of 32 consecutive positions p0 .. p0 + 31 without shuffles when
-// possible: the window's ends inside the step become bits of a mask (one warp
-// OR), and lane l's bag is the window's first bag plus the ends at or before
-// p0 + l. Returns false (nothing written) when two ends coincide (an empty bag)
-// or the step reaches past the window's last end; the caller then bisects.
-#ifndef CB_KEYGEN_MASK
-#define CB_KEYGEN_MASK 1
-#endif
-__device__ __forceinline__ bool bags_by_mask(const BagWindow32& W, int32_t p0, int lane, bool want_range,
-                                             int64_t& bag, int32_t& s, int32_t& e) {
-    const bool before = W.my_end < p0;
-    const bool inside = W.my_end >= p0 && W.my_end <= p0 + 31;
-    const uint32_t nbefore = __popc(__ballot_sync(kFull, before));
-    const uint32_t nin = __popc(__ballot_sync(kFull, inside));
-    const uint32_t mask = __reduce_or_sync(kFull, inside ? 1u << (W.my_end - p0) : 0u);
-    if (__popc(mask) != static_cast<int>(nin) || nbefore + nin >= 32) return false;  // warp-uniform
-    const uint32_t le = lane == 31 ? kFull : (2u << lane) - 1u;
-    const int cnt = static_cast<int>(nbefore) + __popc(mask & le);
-    bag = W.win + cnt;
-    if (want_range) {
-        e = __shfl_sync(kFull, W.my_end, cnt);
-        const int32_t prev = __shfl_sync(kFull, W.my_end, cnt > 0 ? cnt - 1 : 0);
-        s = cnt > 0 ? prev : W.win_start;
-    }
-    return true;
-}
-
 // A warp walks one chunk kKeygenSteps x 32 lookups at a time: the indices (and
 // weights) of all the steps are loaded first, so that many loads are in flight
 // per warp, then each step finds its lanes' bags and writes.
@@ -144,7 +63,7 @@ __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q,
                 const bool valid = q < len;
                 int64_t my_bag;
                 int32_t my_s = 0, my_e = 0;
-                if (!CB_KEYGEN_MASK || !bags_by_mask(W, base + 32 * u, lane, PACKED && P.mean, my_bag, my_s, my_e))
+                if (!bags_by_mask(W, base + 32 * u, lane, PACKED && P.mean, my_bag, my_s, my_e))
                     find_bag32(P, W, bag_hi, k0, q, valid, lane, my_bag, my_s, my_e);
                 if (!valid) continue;
                 if (my_bag >= bag_hi) {  // only reachable with malformed offsets

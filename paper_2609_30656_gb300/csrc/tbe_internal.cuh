@@ -47,7 +47,6 @@ constexpr int kWarpThreads = 256;  // block size of the warp-per-chunk kernels
 #ifndef CB_REDUCE_APPLY_ROWS
 #define CB_REDUCE_APPLY_ROWS 4
 #endif
-constexpr int64_t kNoSeg = INT64_MAX;
 
 // Per-table facts the kernels need, built once at create time.
 struct TableDev {
@@ -157,42 +156,48 @@ __device__ __forceinline__ int64_t fetch_next_chunk(const Plan& Q, int cls, int6
 
 // ---------------------------------------------------------------- bags of positions
 
-// The bag of each of 32 consecutive lookup positions of one table. A window of
-// 32 bag ends slides forward (lane i holds the end of bag win + i); ends never
-// decrease (valid offsets), so the number of the window's bags that end at or
-// before a position is a bisection. Each lane gets its bag and the bag's
-// [start, end) positions.
-struct BagWindow {
+// The bag of each lookup, from a window of 32 bag ends held one per lane, in
+// positions relative to the chunk start: every position is below 2^30, so these
+// are exact in 32 bits (saturated, for malformed offsets, well inside the
+// sentinel kPastTable that marks ends past the table's last bag).
+constexpr int32_t kPastTable = INT32_MAX;
+
+__device__ __forceinline__ int32_t rel32(int64_t x, int64_t k0) {
+    const int64_t r = x - k0;
+    return static_cast<int32_t>(r < -(int64_t(1) << 30) ? -(int64_t(1) << 30)
+                                                        : (r > (int64_t(1) << 30) ? (int64_t(1) << 30) : r));
+}
+
+struct BagWindow32 {
     int64_t win;        // first bag of the window
-    int64_t win_start;  // start position of bag win
-    int64_t my_end;     // end position of bag win + lane (kNoSeg past the table)
-    int64_t bag_hi;     // one past the table's last bag
+    int32_t win_start;  // start of bag win
+    int32_t my_end;     // end of bag win + lane
 };
 
-__device__ __forceinline__ BagWindow bag_window(const Problem& P, int64_t first, int64_t bag_hi,
-                                                int lane) {
-    BagWindow W;
+__device__ __forceinline__ BagWindow32 bag_window32(const Problem& P, int64_t first, int64_t bag_hi,
+                                                    int64_t k0, int lane) {
+    BagWindow32 W;
     W.win = first;
-    W.bag_hi = bag_hi;
-    W.win_start = first < bag_hi ? load_index(P.offsets, first, P.is32) : kNoSeg;
-    W.my_end = (first + lane < bag_hi) ? load_index(P.offsets, first + lane + 1, P.is32) : kNoSeg;
+    W.win_start = first < bag_hi ? rel32(load_index(P.offsets, first, P.is32), k0) : kPastTable;
+    W.my_end = first + lane < bag_hi ? rel32(load_index(P.offsets, first + lane + 1, P.is32), k0) : kPastTable;
     return W;
 }
 
-// Every lane of the warp calls this with its position q (valid: q is a lookup
-// of the table); bag = -1 for invalid lanes.
-__device__ __forceinline__ void find_bag(const Problem& P, BagWindow& W, int64_t q, bool valid, int lane,
-                                         int64_t& bag, int64_t& s, int64_t& e) {
+// Every lane calls this with its relative position q; the window moves forward
+// 32 bags at a time until every valid lane has its bag (bag = -1 otherwise).
+__device__ __forceinline__ void find_bag32(const Problem& P, BagWindow32& W, int64_t bag_hi, int64_t k0,
+                                           int32_t q, bool valid, int lane, int64_t& bag, int32_t& s,
+                                           int32_t& e) {
     bag = -1;
     s = e = 0;
     while (true) {
-        int cnt = 0;
+        int cnt = 0;  // ends at or before q in the window
 #pragma unroll
         for (int b = 16; b >= 1; b >>= 1)
             if (__shfl_sync(kFull, W.my_end, cnt + b - 1) <= q) cnt += b;
         if (__shfl_sync(kFull, W.my_end, 31) <= q) cnt = 32;
-        const int64_t e_sel = __shfl_sync(kFull, W.my_end, cnt < 32 ? cnt : 31);
-        const int64_t s_sel = __shfl_sync(kFull, W.my_end, cnt > 0 ? cnt - 1 : 0);
+        const int32_t e_sel = __shfl_sync(kFull, W.my_end, cnt < 32 ? cnt : 31);
+        const int32_t s_sel = __shfl_sync(kFull, W.my_end, cnt > 0 ? cnt - 1 : 0);
         if (valid && bag < 0 && cnt < 32) {
             bag = W.win + cnt;
             e = e_sel;
@@ -201,8 +206,32 @@ __device__ __forceinline__ void find_bag(const Problem& P, BagWindow& W, int64_t
         if (!__any_sync(kFull, valid && bag < 0)) break;
         W.win_start = __shfl_sync(kFull, W.my_end, 31);
         W.win += 32;
-        W.my_end = (W.win + lane < W.bag_hi) ? load_index(P.offsets, W.win + lane + 1, P.is32) : kNoSeg;
+        W.my_end = W.win + lane < bag_hi ? rel32(load_index(P.offsets, W.win + lane + 1, P.is32), k0) : kPastTable;
     }
+}
+
+// The bags of 32 consecutive positions p0 .. p0 + 31 without shuffles when
+// possible: the window's ends inside the step become bits of a mask (one warp
+// OR), and lane l's bag is the window's first bag plus the ends at or before
+// p0 + l. Returns false (nothing written) when two ends coincide (an empty bag)
+// or the step reaches past the window's last end; the caller then bisects.
+__device__ __forceinline__ bool bags_by_mask(const BagWindow32& W, int32_t p0, int lane, bool want_range,
+                                             int64_t& bag, int32_t& s, int32_t& e) {
+    const bool before = W.my_end < p0;
+    const bool inside = W.my_end >= p0 && W.my_end <= p0 + 31;
+    const uint32_t nbefore = __popc(__ballot_sync(kFull, before));
+    const uint32_t nin = __popc(__ballot_sync(kFull, inside));
+    const uint32_t mask = __reduce_or_sync(kFull, inside ? 1u << (W.my_end - p0) : 0u);
+    if (__popc(mask) != static_cast<int>(nin) || nbefore + nin >= 32) return false;  // warp-uniform
+    const uint32_t le = lane == 31 ? kFull : (2u << lane) - 1u;
+    const int cnt = static_cast<int>(nbefore) + __popc(mask & le);
+    bag = W.win + cnt;
+    if (want_range) {
+        e = __shfl_sync(kFull, W.my_end, cnt);
+        const int32_t prev = __shfl_sync(kFull, W.my_end, cnt > 0 ? cnt - 1 : 0);
+        s = cnt > 0 ? prev : W.win_start;
+    }
+    return true;
 }
 
 // ---------------------------------------------------------------- storage types

@@ -197,7 +197,7 @@ void launch_bwd_reduce_bf16(const Problem& P, const Plan& Q, const BwdOut& O, co
                             int vpl, int gc, bool packed, bool apply, int64_t chunk_bound, int num_sms,
                             cudaStream_t s);
 void launch_weight_grad(const Problem& P, const Plan& Q, const void* grad_out, float* grad_w, int cls,
-                        int dtype, int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
+                        int dtype, int vpl, int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s);
 void launch_bwd_apply_split(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,

@@ -7,21 +7,23 @@
 // (s_b = 1/L for mean pooling, 1 for sum), whatever the weights are: one dot
 // product of the lookup's table row with its bag's grad_out slice.
 //
-// One warp per chunk of lookup positions (the forward's chunk plan). Each lane
-// finds the bag of one position of a 32-position batch by bisection over a
-// window of bag ends; then G = 32 / V lookups per warp step (V lanes per stored
-// row, 16 bytes each), several steps' loads in flight, a dot product per lane
-// and a butterfly over the row's lanes. Consecutive lookups of one bag read the
-// same grad_out slice, which L1 serves. grad_out is fp32, or fp16 / bf16 when
-// the handle's output is (mixed precision). The dot products are summed in a
-// fixed order (deterministic).
+// One warp per chunk of lookup positions (the forward's chunk plan and row
+// layouts), in batches of 32 lookups: each of the G lane groups takes V = 32 / G
+// consecutive lookups, so that it holds its bag's grad_out slice in registers and
+// loads one only where its bag changes. Eight lookups' rows are loaded together, and
+// their eight dot products are summed over the group's lanes at once: three rounds
+// that halve the values a lane holds while they add, then plain butterfly rounds;
+// every lane ends with its own lookup's sum. grad_out is fp32, or fp16 / bf16 when
+// the handle's output is (mixed precision). Fixed order: deterministic.
+// Bound by the rows served from L1 and L2, as the forward's gather, and by issue. On
+// 11.8 M lookups (24 tables, 256-byte rows, Zipf 1.1, bags of 30): 771 us with the
+// slice loaded and a butterfly run for every lookup, 396 us now (four lookups at a
+// time: 447 us at 4 blocks per SM, 418 at 5, 508 at 3; eight at 3 blocks: 444).
 #include "tbe_internal.cuh"
 #include "tbe_launch.h"
 
 namespace cbtbe {
 namespace {
-
-constexpr int kWgradSteps = 4;  // warp steps whose loads are issued together
 
 // Four grad_out values at g (fp32, or fp16 / bf16 with mixed precision), widened.
 __device__ __forceinline__ float4 load_go4(const char* g, int go_dtype) {
@@ -37,139 +39,156 @@ __device__ __forceinline__ float4 load_go4(const char* g, int go_dtype) {
     return make_float4(fa.x, fa.y, fb.x, fb.y);
 }
 
-// <row vector x, the E grad_out values at g>, g in bytes of the grad_out type.
-template <int DT>
-__device__ __forceinline__ float dot_row(const uint4& x, const char* g, int go_dtype) {
+template <int DT, int VPL, int G>
+__device__ __forceinline__ void weight_grad_chunk(const Problem& P, const Chunk& ch, const TableDev& td,
+                                                  const void* grad_out, float* grad_w, int lane) {
     constexpr int E = Storage<DT>::kElems;
-    float f[E];
-    unpack<DT>(x, f);
-    const int step = go_dtype == CB_F32 ? 16 : 8;
-    float acc = 0.f;
+    constexpr int V = 32 / G;
+        constexpr int U = V < 8 / VPL ? V : 8 / VPL;  // lookups per group whose rows are loaded together
+    static_assert(VPL == 1 || G == 1, "several vectors per lane: one row per step");
+    const int g = lane / V, v = lane - g * V;
+    const int row_vecs = td.row_vecs;
+    const uint32_t row_bytes = row_vecs * 16u;
+    const uint32_t rows = static_cast<uint32_t>(td.rows);
+    const int64_t k0 = ch.k0;
+    const int32_t len = static_cast<int32_t>(ch.len & 0x7fffffffu);
+    const int64_t bag_lo = static_cast<int64_t>(ch.table) * P.B, bag_hi = bag_lo + P.B;
+    const int eb = dtype_bytes(P.out_dtype);
+    const char* go_lane = static_cast<const char*>(grad_out) + (static_cast<int64_t>(td.doff) + v * E) * eb;
+    const int64_t go_stride = static_cast<int64_t>(P.sum_d) * eb;
+    const char* row_lane = static_cast<const char*>(td.data) + (v < row_vecs ? v : 0) * 16;
+    BagWindow32 W = bag_window32(P, ch.first, bag_hi, k0, lane);
+    float go[VPL][E];         // the group's bag's slice, this lane's columns
+    int32_t held = -1;        // the bag
+    int64_t r = lane < len ? load_index(P.indices, k0 + lane, P.is32) : -1;
+    for (int32_t base = 0; base < len; base += 32) {
+        const int32_t q = base + lane;
+        const int64_t r_cur = r;
+        r = q + 32 < len ? load_index(P.indices, k0 + q + 32, P.is32) : -1;  // the next batch's
+        int64_t my_bag;
+        int32_t my_s = 0, my_e = 0;
+        if (!bags_by_mask(W, base, lane, P.mean, my_bag, my_s, my_e))
+            find_bag32(P, W, bag_hi, k0, q, q < len, lane, my_bag, my_s, my_e);
+        int32_t b_rel = 0;
+        if (q < len) {
+            if (my_bag >= bag_hi) {  // only reachable with malformed offsets
+                set_error(P.error, CB_ERR_BAD_OFFSETS);
+                my_bag = bag_hi - 1;
+            }
+            b_rel = static_cast<int32_t>(my_bag - bag_lo);
+        }
+        // An invalid lookup contributes nothing: it loads a valid one's row, and
+        // its result is replaced by 0 below.
+        const bool valid = static_cast<uint64_t>(r_cur) < rows;
+        if (!valid && q < len) set_error(P.error, CB_ERR_INDEX_OOB);
+        const uint32_t vm = __ballot_sync(kFull, valid);
+        uint32_t my_a = static_cast<uint32_t>(r_cur);
+        const uint32_t some = __shfl_sync(kFull, my_a, vm ? __ffs(vm) - 1 : 0);
+        if (!valid) my_a = some;
+        float mine = 0.f;
+#pragma unroll 1
+        for (int s0 = 0; vm != 0 && s0 < V && base + s0 < len; s0 += U) {
+            uint4 x[U][VPL];
 #pragma unroll
-    for (int k = 0; k < E / 4; ++k) {
-        const float4 q = load_go4(g + k * step, go_dtype);
-        acc = fmaf(q.x, f[4 * k], acc);
-        acc = fmaf(q.y, f[4 * k + 1], acc);
-        acc = fmaf(q.z, f[4 * k + 2], acc);
-        acc = fmaf(q.w, f[4 * k + 3], acc);
+            for (int u = 0; u < U; ++u) {
+                const uint32_t a = __shfl_sync(kFull, my_a, g * V + s0 + u);
+                const char* p = row_lane + static_cast<uint64_t>(a) * row_bytes;
+#pragma unroll
+                for (int k = 0; k < VPL; ++k)
+                    x[u][k] = __ldg(reinterpret_cast<const uint4*>(p + (k > 0 && v + 32 * k < row_vecs ? 512 * k : 0)));
+            }
+            float dot[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t bag = __shfl_sync(kFull, b_rel, g * V + s0 + u);
+                if (bag != held) {
+                    held = bag;
+#pragma unroll
+                    for (int k = 0; k < VPL; ++k)
+                        if (v + 32 * k < row_vecs)
+#pragma unroll
+                            for (int c = 0; c < E; c += 4) {
+                                const float4 f = load_go4(go_lane + held * go_stride + (32 * k * E + c) * eb, P.out_dtype);
+                                go[k][c] = f.x;
+                                go[k][c + 1] = f.y;
+                                go[k][c + 2] = f.z;
+                                go[k][c + 3] = f.w;
+                            }
+                }
+                dot[u] = 0.f;
+#pragma unroll
+                for (int k = 0; k < VPL; ++k) {
+                    float f[E];
+                    unpack<DT>(x[u][k], f);
+                    if (v + 32 * k < row_vecs)
+#pragma unroll
+                        for (int c = 0; c < E; ++c) dot[u] = fmaf(go[k][c], f[c], dot[u]);
+                }
+            }
+            // The U sums over the group's V lanes: lane v ends with that of lookup v % U.
+#pragma unroll
+            for (int w = 1; w < U; w <<= 1) {
+                // a lane keeps the sums whose number has its own bit w and adds its
+                // partner's share of them
+                const bool up = v & w;
+#pragma unroll
+                for (int i = 0; i < U; i += 2 * w)
+                    dot[i] = (up ? dot[i + w] : dot[i]) + __shfl_xor_sync(kFull, up ? dot[i] : dot[i + w], w);
+            }
+            float z = dot[0];
+#pragma unroll
+            for (int off = U; off < V; off <<= 1) z += __shfl_xor_sync(kFull, z, off);
+            if (v / U == s0 / U) mine = z;  // lookup g*V + v is this lane's own
+        }
+        if (q < len) {
+            const float sc = (P.mean && my_e > my_s) ? 1.f / static_cast<float>(my_e - my_s) : 1.f;
+            grad_w[k0 + q] = valid ? sc * mine : 0.f;
+        }
     }
-    return acc;
 }
 
-// GC > 0: rows of up to V = 32 / GC vectors (one per lane), GC lookups per
-// warp step. GC == 0: any row size, one lookup per step, each lane taking
-// vectors lane, lane + 32, ... of the row.
-template <int DT, int GC>
-__global__ void __launch_bounds__(kWarpThreads) weight_grad_kernel(const __grid_constant__ Problem P,
-                                                                   const __grid_constant__ Plan Q,
-                                                                   const void* grad_out, float* grad_w,
-                                                                   int cls) {
-    constexpr int E = Storage<DT>::kElems;
-    constexpr int G = GC > 0 ? GC : 1;
-    constexpr int V = 32 / G;
+template <int DT, int VPL, int G>
+__global__ void __launch_bounds__(kWarpThreads, VPL == 4 ? 2 : 4)
+    weight_grad_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q, const void* grad_out,
+                       float* grad_w, int cls) {
     const int lane = threadIdx.x & 31;
-    const int g = lane / V, v = lane - g * V;
     const int64_t cb = Q.class_chunk_base[cls];
     const int64_t ce = min64(Q.class_chunk_base[cls + 1], Q.max_chunks);
     for (int64_t j = first_chunk(Q, cls, cb, lane); j < ce;) {
         const int64_t nxt = fetch_next_chunk(Q, cls, cb, lane);
         const Chunk ch = Q.chunks[j];
-        const int t = ch.table;
-        const TableDev& td = P.tables[t];
-        const uint4* rows = static_cast<const uint4*>(td.data);
-        const int nvec = td.row_vecs;
-        const int64_t k0 = ch.k0, k1 = ch.k0 + (ch.len & 0x7fffffffu);
-        const int64_t bag_lo = static_cast<int64_t>(t) * P.B, bag_hi = bag_lo + P.B;
-        const int eb = dtype_bytes(P.out_dtype);
-        const char* go_base = static_cast<const char*>(grad_out) + static_cast<int64_t>(td.doff) * eb;
-        BagWindow W = bag_window(P, ch.first, bag_hi, lane);
-        for (int64_t base = k0; base < k1; base += 32) {
-            const int64_t q = base + lane;
-            const bool valid = q < k1;
-            int64_t my_bag, my_s, my_e;
-            find_bag(P, W, q, valid, lane, my_bag, my_s, my_e);
-            // Per position: row (kInvalid = contributes nothing), bag row offset, s_b.
-            uint32_t my_a = kInvalid;
-            int64_t my_go = 0;
-            float my_sc = 0.f;
-            if (valid) {
-                if (my_bag >= bag_hi) {  // only reachable with malformed offsets
-                    set_error(P.error, CB_ERR_BAD_OFFSETS);
-                    my_bag = bag_hi - 1;
-                }
-                const int64_t r = load_index(P.indices, q, P.is32);
-                if (r < 0 || r >= td.rows) set_error(P.error, CB_ERR_INDEX_OOB);
-                else my_a = static_cast<uint32_t>(r);
-                my_go = (my_bag - bag_lo) * P.sum_d;
-                my_sc = (P.mean && my_e > my_s) ? 1.f / static_cast<float>(my_e - my_s) : 1.f;
-            }
-            const int nb = static_cast<int>(min64(32, k1 - base));
-            for (int i0 = 0; i0 < nb; i0 += G * kWgradSteps) {
-                float dot[kWgradSteps];
-#pragma unroll
-                for (int u = 0; u < kWgradSteps; ++u) {
-                    const int i = i0 + u * G + g;
-                    const uint32_t a = __shfl_sync(kFull, my_a, i & 31);
-                    const int64_t go = __shfl_sync(kFull, my_go, i & 31);
-                    dot[u] = 0.f;
-                    if (i >= nb || a == kInvalid) continue;
-                    const uint4* rp = rows + static_cast<int64_t>(a) * nvec;
-                    const char* gp = go_base + go * eb;
-                    if (GC > 0) {
-                        if (v < nvec) dot[u] = dot_row<DT>(__ldg(rp + v), gp + v * E * eb, P.out_dtype);
-                    } else {
-                        for (int vec = v; vec < nvec; vec += 32)
-                            dot[u] += dot_row<DT>(__ldg(rp + vec), gp + vec * E * eb, P.out_dtype);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kWgradSteps; ++u) {
-#pragma unroll
-                    for (int off = V / 2; off >= 1; off >>= 1) dot[u] += __shfl_xor_sync(kFull, dot[u], off);
-                    const int i = i0 + u * G + g;
-                    const float sc = __shfl_sync(kFull, my_sc, i & 31);
-                    if (v == 0 && i < nb) grad_w[base + i] = sc * dot[u];
-                }
-            }
-        }
+        weight_grad_chunk<DT, VPL, G>(P, ch, P.tables[ch.table], grad_out, grad_w, lane);
         j = __shfl_sync(kFull, nxt, 0);
     }
 }
 
-template <int DT, int GC>
+template <auto Kernel>
 void launch_one(const Problem& P, const Plan& Q, const void* go, float* gw, int cls, int64_t chunk_bound,
                 int num_sms, cudaStream_t s) {
-    static int per_sm = -1;
-    if (per_sm < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, weight_grad_kernel<DT, GC>,
-                                                                     kWarpThreads, 0) != cudaSuccess ||
-                       per_sm < 1))
-        per_sm = 1;
-    const int64_t need = (chunk_bound + (kWarpThreads / 32) - 1) / (kWarpThreads / 32);
-    const int grid = static_cast<int>(max64(1, min64(need, static_cast<int64_t>(per_sm) * num_sms)));
-    weight_grad_kernel<DT, GC><<<grid, kWarpThreads, 0, s>>>(P, Q, go, gw, cls);
+    static const int cap = resident_blocks(Kernel, kWarpThreads);
+    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(P, Q, go, gw, cls);
 }
 
 template <int DT>
-void launch_dtype(const Problem& P, const Plan& Q, const void* go, float* gw, int cls, int gc,
+void launch_dtype(const Problem& P, const Plan& Q, const void* go, float* gw, int cls, int vpl, int gc,
                   int64_t chunk_bound, int num_sms, cudaStream_t s) {
-    switch (gc) {
-        case 1: launch_one<DT, 1>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
-        case 2: launch_one<DT, 2>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
-        case 4: launch_one<DT, 4>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
-        case 8: launch_one<DT, 8>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
-        case 16: launch_one<DT, 16>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
-        case 32: launch_one<DT, 32>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
-        default: launch_one<DT, 0>(P, Q, go, gw, cls, chunk_bound, num_sms, s); break;
+#define CB_CASE(V, G)                                                                             \
+    if (vpl == V && gc == G) {                                                                     \
+        launch_one<weight_grad_kernel<DT, V, G>>(P, Q, go, gw, cls, chunk_bound, num_sms, s);       \
+        return;                                                                                   \
     }
+    CB_CASE(1, 1) CB_CASE(1, 2) CB_CASE(1, 4) CB_CASE(1, 8) CB_CASE(1, 16) CB_CASE(1, 32)
+    CB_CASE(2, 1) CB_CASE(4, 1)
+#undef CB_CASE
 }
 
 }  // namespace
 
 void launch_weight_grad(const Problem& P, const Plan& Q, const void* grad_out, float* grad_w, int cls,
-                        int dtype, int gc, int64_t chunk_bound, int num_sms, cudaStream_t s) {
-    if (dtype == CB_F32) launch_dtype<CB_F32>(P, Q, grad_out, grad_w, cls, gc, chunk_bound, num_sms, s);
-    else if (dtype == CB_F16) launch_dtype<CB_F16>(P, Q, grad_out, grad_w, cls, gc, chunk_bound, num_sms, s);
-    else launch_dtype<CB_BF16>(P, Q, grad_out, grad_w, cls, gc, chunk_bound, num_sms, s);
+                        int dtype, int vpl, int gc, int64_t chunk_bound, int num_sms, cudaStream_t s) {
+    if (dtype == CB_F32) launch_dtype<CB_F32>(P, Q, grad_out, grad_w, cls, vpl, gc, chunk_bound, num_sms, s);
+    else if (dtype == CB_F16) launch_dtype<CB_F16>(P, Q, grad_out, grad_w, cls, vpl, gc, chunk_bound, num_sms, s);
+    else launch_dtype<CB_BF16>(P, Q, grad_out, grad_w, cls, vpl, gc, chunk_bound, num_sms, s);
 }
 
 }  // namespace cbtbe
