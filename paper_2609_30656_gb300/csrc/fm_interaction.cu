@@ -12,13 +12,18 @@
 //
 //   grad_y[b, t*D + j] = g[b] * (sum_u v_buj - v_btj).
 //
-// The forward runs one warp per sample: the warp streams the sample's T*D
-// values with 16-byte loads and keeps per-column sums and sums of squares in
-// registers, reading every value once. The backward runs one block per sample
-// when the row fits the block's registers (up to 4096 16-byte vectors): the row
-// is loaded once, the column sums meet in shared memory, and the gradient row is
-// written from registers; other shapes take a warp per sample that reads the
-// row twice. Sums are taken in a fixed order, so results are deterministic.
+// A block takes S samples (one, unless a sample has fewer vectors than a block has
+// threads): R * nv threads per sample, thread (r, c) owning vector column c of
+// fields r, r + R, ..., loaded together and held in registers; the R partial
+// column sums meet in shared memory. So a sample is read once, with every load of
+// the block in flight, whatever T and D (D / 4 need not divide anything); only
+// samples of more than 16 fields per thread row are read in a loop, twice by the
+// gradient. Sums are taken in a fixed order, so results are deterministic.
+// Bound by HBM. Against a warp per sample (forward, and gradients whose vectors did
+// not divide 256), us from a flushed L2, forward + gradient: 16384 samples x 26
+// fields x 128: 54 + 76, now 48 + 70; 19881 x 23 x 96: 56 + 87, now 48 + 68;
+// 60000 x 10 x 8: 21 + 203, now 21 + 17; 65536 x 100 x 128: 507 + 986, now 472 + 959
+// (6.9 TB/s of compulsory bytes). One after the other, 16384 x 26 x 128: 118, now 107.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -28,6 +33,7 @@ namespace cbtbe {
 namespace {
 
 constexpr int kFmThreads = 256;
+constexpr int kFmFields = 16;  // fields per thread held in registers
 
 __device__ __forceinline__ void add4(float4& a, const float4& x) {
     a.x += x.x;
@@ -41,189 +47,124 @@ __device__ __forceinline__ void fma4(float4& a, const float4& x) {
     a.z = fmaf(x.z, x.z, a.z);
     a.w = fmaf(x.w, x.w, a.w);
 }
-__device__ __forceinline__ float4 shfl_xor4(const float4& a, int off) {
-    return make_float4(__shfl_xor_sync(0xffffffffu, a.x, off), __shfl_xor_sync(0xffffffffu, a.y, off),
-                       __shfl_xor_sync(0xffffffffu, a.z, off), __shfl_xor_sync(0xffffffffu, a.w, off));
+
+// The R partial sums of a column (part[c], part[c + nv], ...): up to kDirect of
+// them are added by whoever needs the total; more meet in a tree first, in which
+// `part` and `part2` (unless null) of thread (r, c) take those of (r + half, c).
+constexpr int kDirect = 16;
+__device__ __forceinline__ void tree_sum(float4* part, float4* part2, int r, int nv, int R) {
+    int half = 1;
+    while (half < R) half <<= 1;
+    for (half >>= 1; half >= 1; half >>= 1) {
+        if (r < half && r + half < R) {
+            add4(part[0], part[half * nv]);
+            if (part2) add4(part2[0], part2[half * nv]);
+        }
+        __syncthreads();
+    }
+}
+__device__ __forceinline__ float4 column_total(const float4* part, int nv, int R) {
+    float4 S = part[0];
+#pragma unroll 1
+    for (int q = 1; q < R; ++q) add4(S, part[q * nv]);
+    return S;
 }
 
-// Field layout over a warp, with nv = D / 4 vectors per field: G = 32 / nv
-// fields side by side per step when nv divides 32 (D <= 128, M = 1); otherwise
-// one field per step, lane l owning vector columns l + 32 m for m < M.
-template <int G, int M>
-struct FieldMap {
-    int g, c;  // field group of this lane, its first vector column
-    int nv;
-    __device__ FieldMap(int lane, int nv_) : nv(nv_) {
-        g = G > 1 ? lane / (32 / G) : 0;
-        c = G > 1 ? lane - g * (32 / G) : lane;
-    }
-    __device__ bool live(int m) const { return c + 32 * m < nv; }
-    __device__ int64_t at(int t, int m) const { return static_cast<int64_t>(t) * nv + c + 32 * m; }
+struct FmShape {
+    int B, T, nv;    // samples, fields, 16-byte vectors per field
+    int R, per, S;   // thread rows per sample, threads per sample (R * nv), samples per block
+    int64_t stride;  // floats from one sample to the next
 };
 
-// Column sums s (and sums of squares q) of one sample, combined over the G
-// field groups so every group holds the totals of its columns.
-template <int G, int M, bool SQUARES>
-__device__ __forceinline__ void column_sums(const float4* row, int T, const FieldMap<G, M>& f,
-                                            float4 (&s)[M], float4 (&q)[M]) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) s[m] = q[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-    int t = f.g;
-    for (; t + 3 * G < T; t += 4 * G) {
-        float4 x[4][M];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-                x[k][m] = f.live(m) ? __ldg(row + f.at(t + k * G, m)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int m = 0; m < M; ++m) {
-                add4(s[m], x[k][m]);
-                if (SQUARES) fma4(q[m], x[k][m]);
-            }
-    }
-    for (; t < T; t += G) {
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            const float4 x = f.live(m) ? __ldg(row + f.at(t, m)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            add4(s[m], x);
-            if (SQUARES) fma4(q[m], x);
-        }
-    }
-#pragma unroll
-    for (int off = 32 / G; off < 32; off <<= 1)
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            add4(s[m], shfl_xor4(s[m], off));
-            if (SQUARES) add4(q[m], shfl_xor4(q[m], off));
-        }
-}
-
-template <int G, int M>
-__global__ void __launch_bounds__(kFmThreads) fm_forward_kernel(const float* __restrict__ y, int B, int T,
-                                                                int nv, int64_t stride,
-                                                                float* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const FieldMap<G, M> f(lane, nv);
-    for (int64_t b = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; b < B;
-         b += nwarps) {
-        float4 s[M], q[M];
-        column_sums<G, M, true>(reinterpret_cast<const float4*>(y + b * stride), T, f, s, q);
-        float part = 0.f;
-        if (f.g == 0) {
-#pragma unroll
-            for (int m = 0; m < M; ++m)
-                if (f.live(m))
-                    part += (fmaf(s[m].x, s[m].x, -q[m].x) + fmaf(s[m].y, s[m].y, -q[m].y)) +
-                            (fmaf(s[m].z, s[m].z, -q[m].z) + fmaf(s[m].w, s[m].w, -q[m].w));
-        }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-        if (lane == 0) out[b] = 0.5f * part;
-    }
-}
-
-template <int G, int M>
-__global__ void __launch_bounds__(kFmThreads) fm_backward_kernel(const float* __restrict__ y,
-                                                                 const float* __restrict__ grad_fm, int B,
-                                                                 int T, int nv, int64_t stride,
-                                                                 float* __restrict__ grad_y) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const FieldMap<G, M> f(lane, nv);
-    for (int64_t b = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; b < B;
-         b += nwarps) {
-        const float4* row = reinterpret_cast<const float4*>(y + b * stride);
-        float4* dst = reinterpret_cast<float4*>(grad_y + b * stride);
-        float4 s[M], q[M];
-        column_sums<G, M, false>(row, T, f, s, q);
-        const float gb = __ldg(grad_fm + b);
-        for (int t = f.g; t < T; t += G) {
-#pragma unroll
-            for (int m = 0; m < M; ++m) {
-                if (!f.live(m)) continue;
-                const float4 x = row[f.at(t, m)];
-                dst[f.at(t, m)] = make_float4(gb * (s[m].x - x.x), gb * (s[m].y - x.y), gb * (s[m].z - x.z),
-                                              gb * (s[m].w - x.w));
-            }
-        }
-    }
-}
-
-// Backward with one block per sample when 256 threads tile the sample's row:
-// nv divides 256 (so thread i always owns vector column i % nv) and the row
-// has at most 256 * K vectors. The row stays in registers between the column
-// sums and the gradient, so it is read from memory once.
-constexpr int kRowThreads = 256;
-
-template <int K>
-__global__ void __launch_bounds__(kRowThreads) fm_backward_rows_kernel(const float* __restrict__ y,
-                                                                       const float* __restrict__ grad_fm,
-                                                                       int B, int T, int nv, int64_t stride,
-                                                                       float* __restrict__ grad_y) {
-    __shared__ float4 part[kRowThreads];
+// K > 0: up to K fields per thread, in registers. K = 0: any number, in a loop.
+// The gradient takes the samples from the last to the first: after a forward pass
+// the last ones are what L2 still holds.
+template <int K, bool BACKWARD>
+__global__ void __launch_bounds__(kFmThreads, K == 16 ? 2 : (K == 8 ? 4 : (K == 4 ? 6 : 8)))
+    fm_kernel(const float* __restrict__ y, const float* __restrict__ grad_fm, const FmShape f,
+              float* __restrict__ out) {
+    __shared__ float4 sum[kFmThreads], sq[BACKWARD ? 1 : kFmThreads];
     const int i = threadIdx.x;
-    const int c = i % nv, r = i / nv, R = kRowThreads / nv;
-    const int nvec = T * nv;  // vector k of the row is field k / nv, column k % nv
-    for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
-        const float4* row = reinterpret_cast<const float4*>(y + b * stride);
-        float4 x[K];
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int slot = i / f.per, w = i - slot * f.per, r = w / f.nv, c = w - r * f.nv;
+    const int64_t b0 = static_cast<int64_t>(blockIdx.x) * f.S + slot;
+    const bool live = slot < f.S && b0 < f.B;
+    const int64_t b = !live ? 0 : (BACKWARD ? f.B - 1 - b0 : b0);
+    const float4* row = reinterpret_cast<const float4*>(y + b * f.stride) + c;
+    constexpr int kHeld = K > 0 ? K : 1;
+    float4 x[kHeld];
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f), q = s;
+    if constexpr (K > 0) {
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-            const int k = i + kRowThreads * j;
-            x[j] = k < nvec ? __ldg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < K; ++k) {
+            const int t = r + k * f.R;
+            x[k] = live && t < f.T ? __ldg(row + static_cast<int64_t>(t) * f.nv) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int j = 0; j < K; ++j) add4(s, x[j]);
-        part[i] = s;
+        for (int k = 0; k < K; ++k) {
+            add4(s, x[k]);
+            if (!BACKWARD) fma4(q, x[k]);
+        }
+    } else if (live) {
+#pragma unroll 8
+        for (int t = r; t < f.T; t += f.R) {
+            const float4 z = __ldg(row + static_cast<int64_t>(t) * f.nv);
+            add4(s, z);
+            if (!BACKWARD) fma4(q, z);
+        }
+    }
+    sum[i] = s;
+    if (!BACKWARD) sq[i] = q;
+    __syncthreads();
+    const int left = f.R > kDirect ? 1 : f.R;
+    if (left == 1) tree_sum(sum + i, BACKWARD ? nullptr : sq + i, live ? r : f.R, f.nv, f.R);
+    if constexpr (!BACKWARD) {
+        // thread (0, c): its column's S^2 - Q; then a warp per sample adds the columns
+        __shared__ float cols[kFmThreads];
+        if (live && r == 0) {
+            const float4 S = column_total(sum + i, f.nv, left), Q = column_total(sq + i, f.nv, left);
+            cols[slot * f.nv + c] = (fmaf(S.x, S.x, -Q.x) + fmaf(S.y, S.y, -Q.y)) +
+                                    (fmaf(S.z, S.z, -Q.z) + fmaf(S.w, S.w, -Q.w));
+        }
         __syncthreads();
-        if (r == 0) {  // column c: the R partial sums in a fixed order
-            float4 S = part[c];
-            for (int q = 1; q < R; ++q) add4(S, part[q * nv + c]);
-            part[c] = S;
-        }
-        __syncthreads();
-        const float4 S = part[c];
-        const float gb = __ldg(grad_fm + b);
-        float4* dst = reinterpret_cast<float4*>(grad_y + b * stride);
+        const int lane = i & 31;
+        for (int k = i >> 5; k < f.S; k += blockDim.x >> 5) {
+            const int64_t bk = static_cast<int64_t>(blockIdx.x) * f.S + k;
+            if (bk >= f.B) break;
+            float part = 0.f;
+            for (int j = lane; j < f.nv; j += 32) part += cols[k * f.nv + j];
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-            const int k = i + kRowThreads * j;
-            if (k < nvec)
-                dst[k] = make_float4(gb * (S.x - x[j].x), gb * (S.y - x[j].y), gb * (S.z - x[j].z),
-                                     gb * (S.w - x[j].w));
+            for (int off = 16; off >= 1; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+            if (lane == 0) out[bk] = 0.5f * part;
         }
-        __syncthreads();  // `part` is reused by the next sample
+    } else if (live) {
+        const float4 S = column_total(sum + slot * f.per + c, f.nv, left);
+        const float g = __ldg(grad_fm + b);
+        float4* dst = reinterpret_cast<float4*>(out + b * f.stride) + c;
+        auto put = [&](int t, const float4& z) {
+            __stcs(dst + static_cast<int64_t>(t) * f.nv,
+                   make_float4(g * (S.x - z.x), g * (S.y - z.y), g * (S.z - z.z), g * (S.w - z.w)));
+        };
+        if constexpr (K > 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (r + k * f.R < f.T) put(r + k * f.R, x[k]);
+        } else {
+#pragma unroll 4
+            for (int t = r; t < f.T; t += f.R) put(t, row[static_cast<int64_t>(t) * f.nv]);
+        }
     }
 }
 
-int sm_count() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-        return 1;
-    return n;
-}
-
-// Warps per SM the grid asks for: enough 16-byte loads in flight to cover HBM
-// latency; samples beyond the grid are taken in a grid-stride loop.
-constexpr int kFmBlocksPerSm = 8;
-
-template <int G, int M>
-void launch_fm(bool backward, const float* y, const float* grad_fm, int B, int T, int nv,
-               int64_t stride, float* out, cudaStream_t s) {
-    const int64_t warps_per_block = kFmThreads / 32;
-    const int64_t need = (static_cast<int64_t>(B) + warps_per_block - 1) / warps_per_block;
-    const int grid = static_cast<int>(need < int64_t(sm_count()) * kFmBlocksPerSm ? need
-                                                                                   : int64_t(sm_count()) * kFmBlocksPerSm);
-    if (backward)
-        fm_backward_kernel<G, M><<<grid, kFmThreads, 0, s>>>(y, grad_fm, B, T, nv, stride, out);
-    else
-        fm_forward_kernel<G, M><<<grid, kFmThreads, 0, s>>>(y, B, T, nv, stride, out);
+template <bool BACKWARD>
+void launch_fm(const float* y, const float* grad_fm, const FmShape& f, float* out, cudaStream_t s) {
+    const unsigned grid = static_cast<unsigned>((f.B + f.S - 1) / f.S);
+    const int threads = (f.per * f.S + 31) / 32 * 32;
+    const int k = (f.T + f.R - 1) / f.R;
+    if (k <= 2) fm_kernel<2, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
+    else if (k <= 4) fm_kernel<4, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
+    else if (k <= 8) fm_kernel<8, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
+    else if (k <= kFmFields) fm_kernel<kFmFields, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
+    else fm_kernel<0, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
 }
 
 cb_status fm_call(bool backward, const float* y, const float* grad_fm, int32_t batch, int32_t num_fields,
@@ -236,40 +177,16 @@ cb_status fm_call(bool backward, const float* y, const float* grad_fm, int32_t b
         return CB_ERR_INVALID_ARG;
     if (batch == 0) return CB_OK;
     cudaGetLastError();  // an earlier, unrelated failure is not this call's
-    const int nv = dim / 4;
-    const int64_t nvec = static_cast<int64_t>(num_fields) * nv;
-    if (backward && kRowThreads % nv == 0 && nvec <= 16 * kRowThreads) {
-        const int k = nvec <= 4 * kRowThreads ? 4 : (nvec <= 8 * kRowThreads ? 8 : 16);
-        const int per_sm = k == 16 ? 2 : 4;
-        const int grid = static_cast<int>(batch < sm_count() * per_sm * 4 ? batch : sm_count() * per_sm * 4);
-        if (k == 4)
-            fm_backward_rows_kernel<4><<<grid, kRowThreads, 0, stream>>>(y, grad_fm, batch, num_fields, nv,
-                                                                        row_stride, out);
-        else if (k == 8)
-            fm_backward_rows_kernel<8><<<grid, kRowThreads, 0, stream>>>(y, grad_fm, batch, num_fields, nv,
-                                                                        row_stride, out);
-        else
-            fm_backward_rows_kernel<16><<<grid, kRowThreads, 0, stream>>>(y, grad_fm, batch, num_fields, nv,
-                                                                         row_stride, out);
-        return cudaGetLastError() == cudaSuccess ? CB_OK : CB_ERR_CUDA;
-    }
-    if (nv <= 32 && 32 % nv == 0) {
-        switch (32 / nv) {
-            case 1: launch_fm<1, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            case 2: launch_fm<2, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            case 4: launch_fm<4, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            case 8: launch_fm<8, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            case 16: launch_fm<16, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            default: launch_fm<32, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-        }
-    } else {
-        switch ((nv + 31) / 32) {
-            case 1: launch_fm<1, 1>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            case 2: launch_fm<1, 2>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            case 3: launch_fm<1, 3>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-            default: launch_fm<1, 4>(backward, y, grad_fm, batch, num_fields, nv, row_stride, out, stream); break;
-        }
-    }
+    FmShape f;
+    f.B = batch;
+    f.T = num_fields;
+    f.nv = dim / 4;
+    f.R = kFmThreads / f.nv < num_fields ? kFmThreads / f.nv : num_fields;
+    f.per = f.R * f.nv;
+    f.S = kFmThreads / f.per;
+    f.stride = row_stride;
+    if (backward) launch_fm<true>(y, grad_fm, f, out, stream);
+    else launch_fm<false>(y, grad_fm, f, out, stream);
     return cudaGetLastError() == cudaSuccess ? CB_OK : CB_ERR_CUDA;
 }
 
