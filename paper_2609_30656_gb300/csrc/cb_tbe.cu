@@ -82,8 +82,9 @@ struct Workspace {
     uint32_t* status = nullptr;
     uint32_t* tile_counters = nullptr;
     uint32_t* tile_digits = nullptr;
-    uint32_t* seg_sums = nullptr;
-    int segments = 1;
+    uint32_t* table_digits = nullptr;
+    int64_t digit_words = 0;  // zeroed before the sort, from zero_digits on
+    uint32_t* zero_digits = nullptr;
     uint32_t* heads = nullptr;
     int64_t* run_count = nullptr;
     int64_t* out_first = nullptr;
@@ -193,9 +194,17 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
         ws.tile_counters = base ? ws.status + static_cast<size_t>(h->passes) * ws.sort_tiles * 256 : nullptr;
         ws.status_bytes += sizeof(uint32_t) * hist_words + sizeof(uint32_t) * 4;  // cleared from `hist` on
     } else {
-        ws.segments = radix_segments(ws.sp_max_tiles, static_cast<int>(T));
-        ws.tile_digits = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * ws.sort_tiles));
-        ws.seg_sums = static_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * T * ws.segments));
+        // Few tiles: every pass's counts, zeroed at the start. Many: one pass's
+        // counts, and every pass's counts per table, zeroed at the start. Calls of
+        // few tiles fit into what a call of many takes.
+        const int64_t tile_words = 256 * ws.sort_tiles, table_words = 256 * T * h->passes;
+        const int64_t few_tiles = std::min(ws.sort_tiles, kFewSortTiles);
+        ws.tile_digits = static_cast<uint32_t*>(
+            take(sizeof(uint32_t) * std::max(tile_words + table_words, 256 * few_tiles * h->passes)));
+        const bool few = ws.sort_tiles <= kFewSortTiles;
+        ws.table_digits = base && !few ? ws.tile_digits + tile_words : nullptr;
+        ws.zero_digits = few ? ws.tile_digits : ws.table_digits;
+        ws.digit_words = few ? tile_words * h->passes : table_words;
     }
     ws.heads = static_cast<uint32_t*>(take(sizeof(uint32_t) * max_chunks));
     ws.run_count = static_cast<int64_t*>(take(sizeof(int64_t) * T));
@@ -319,15 +328,22 @@ cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Pl
     S0.max_tiles = w.sp_max_tiles;
     S0.table_first_tile = w.sp_first;
     S0.num_tiles = w.sp_num;
+    const bool lookback = (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) != 0;
+    const bool few = !lookback && w.sp_max_tiles <= kFewSortTiles;
+    if (!lookback) {
+        S0.zero = w.zero_digits;
+        S0.zero_words = w.digit_words;
+    }
     launch_plan(P, Q, &S0, bound, h->num_sms, stream);
     h->launches += plan_launches(P);
     const int64_t n = P.n;
-    const bool lookback = (h->flags & (CB_SORT_LOOKBACK | CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)) != 0;
     if (lookback && cudaMemsetAsync(w.hist, 0, w.status_bytes, stream) != cudaSuccess) return CB_ERR_CUDA;
     KeyGen K;
     K.keys = w.keys[0];
     K.vals = w.vals[0];
     K.packed = packed ? w.packed : nullptr;
+    K.tile_digits = few ? w.tile_digits : nullptr;
+    K.table_first_tile = w.sp_first;
     launch_keygen(P, Q, K, packed, bound, h->num_sms, stream);
     h->launches += 1;
     record(h, h->ev_bwd[1], stream);
@@ -366,12 +382,13 @@ cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Pl
             h->launches += 1;
         } else {
             S.table_pos = w.table_pos;
-            S.tile_digits = w.tile_digits;
-            S.seg_sums = w.seg_sums;
+            const int64_t words = 256 * w.sort_tiles;
+            S.tile_digits = few ? w.tile_digits + p * words : w.tile_digits;
+            S.next_digits = few && p + 1 < h->passes ? S.tile_digits + words : nullptr;
+            S.table_digits = few ? nullptr : w.table_digits + static_cast<int64_t>(p) * 256 * h->T;
             S.T = h->T;
-            S.segments = w.segments;
             launch_radix_pass(S, w.sp_max_tiles, stream);
-            h->launches += radix_pass_launches();
+            h->launches += radix_pass_launches(w.sp_max_tiles);
         }
         cur ^= 1;
     }

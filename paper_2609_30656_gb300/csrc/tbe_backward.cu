@@ -30,7 +30,8 @@ constexpr int kKeygenSteps = CB_KEYGEN_STEPS;
 // Compiled with no minimum of resident blocks: 48 registers, 5 blocks of 256
 // threads per SM. (A minimum of 1 let it take 72 registers, 3 blocks: cfg5
 // 0.63 -> 0.75 ms; a minimum of 6, 40 registers: cfg5u 0.63 -> 0.71 ms.)
-template <bool PACKED>
+// COUNT: the first sort pass's digits are counted on the way (few tiles).
+template <bool PACKED, bool COUNT>
 __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q, KeyGen K) {
     const int lane = threadIdx.x & 31;
     const int64_t total = min(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
@@ -46,6 +47,9 @@ __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q,
         const int64_t bag_lo = static_cast<int64_t>(t) * P.B, bag_hi = bag_lo + P.B;
         uint32_t* keys = K.keys + k0;
         uint32_t* vals = K.vals + k0;
+        // the chunk's first position within its table, and the table's counts
+        const int64_t in_table = k0 - Q.table_pos[t];
+        uint32_t* digits = COUNT ? K.tile_digits + K.table_first_tile[t] * 256 : nullptr;
         BagWindow32 W = bag_window32(P, ch.first, bag_hi, k0, lane);
         for (int32_t base = 0; base < len; base += 32 * kKeygenSteps) {
             int64_t idx[kKeygenSteps];
@@ -81,6 +85,7 @@ __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q,
                     bag = kDeadBag;
                 }
                 keys[q] = static_cast<uint32_t>(key_base + r);
+                if (COUNT) atomicAdd(digits + (in_table + q) / kSortTileKeys * 256 + (r & 255), 1u);
                 if (PACKED) {
                     float c = wt[u];
                     if (P.mean && my_e > my_s) c = c / static_cast<float>(my_e - my_s);
@@ -383,15 +388,19 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_apply_split_kernel(const __g
 
 // ---------------------------------------------------------------- launchers
 
+template <auto Kernel>
+static void launch_keygen_one(const Problem& P, const Plan& Q, const KeyGen& K, int64_t chunk_bound, int num_sms,
+                              cudaStream_t s) {
+    static const int cap = resident_blocks(Kernel, kWarpThreads);
+    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(P, Q, K);
+}
+
 void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed, int64_t chunk_bound,
                    int num_sms, cudaStream_t s) {
-    if (packed) {
-        static int cap = occupancy_grid(keygen_kernel<true>, kWarpThreads, num_sms);
-        keygen_kernel<true><<<warp_grid(chunk_bound, cap), kWarpThreads, 0, s>>>(P, Q, K);
-    } else {
-        static int cap = occupancy_grid(keygen_kernel<false>, kWarpThreads, num_sms);
-        keygen_kernel<false><<<warp_grid(chunk_bound, cap), kWarpThreads, 0, s>>>(P, Q, K);
-    }
+    if (packed && K.tile_digits) launch_keygen_one<keygen_kernel<true, true>>(P, Q, K, chunk_bound, num_sms, s);
+    else if (packed) launch_keygen_one<keygen_kernel<true, false>>(P, Q, K, chunk_bound, num_sms, s);
+    else if (K.tile_digits) launch_keygen_one<keygen_kernel<false, true>>(P, Q, K, chunk_bound, num_sms, s);
+    else launch_keygen_one<keygen_kernel<false, false>>(P, Q, K, chunk_bound, num_sms, s);
 }
 
 void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound, cudaStream_t s) {

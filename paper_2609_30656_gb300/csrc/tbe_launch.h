@@ -24,10 +24,10 @@ struct SortPass {
     int shift;                   // digit = ((key - key_base_t) >> shift) & 255
     // reduce-then-scan
     const int64_t* table_pos;    // [T + 1] first position of each table
-    uint32_t* tile_digits;       // [tiles][256]: digit counts, then first output slots
-    uint32_t* seg_sums;          // [T][segments][256]
+    uint32_t* tile_digits;       // [tiles][256]: digit counts (many tiles: then first output slots)
+    uint32_t* next_digits;       // few tiles: the next pass's counts, zeroed (null: last pass)
+    uint32_t* table_digits;      // many tiles: [T][256] digit counts per table, zeroed
     int T;
-    int segments;                // parts of each table's tiles in the slot scan
     // single sweep with look-back
     const uint32_t* digit_base;  // [T][stride]: this pass's 256 first output slots per table
     int base_stride;             // passes * 256
@@ -101,6 +101,8 @@ struct KeyGen {
     uint32_t* vals;    // [n] bag id (kDeadBag when out of range), or lookup position
                        // when `packed` is used
     uint2* packed;     // [n] (bag id or kDeadBag, bits of w_i * s_b) by lookup position, or null
+    uint32_t* tile_digits;         // counts of the first sort pass, zeroed (null: counted later)
+    const int64_t* table_first_tile;
 };
 
 struct BwdOut {
@@ -167,11 +169,16 @@ void launch_sort_hist(const uint32_t* keys, const struct Chunk* tiles, const int
 void launch_sort_bases(const uint32_t* hist, const int64_t* table_pos, int T, int passes,
                        uint32_t* base, cudaStream_t s);
 void launch_onesweep(const SortPass& S, int64_t tile_bound, cudaStream_t s);
-// Parts per table of the slot scan for a tile bound (about 16 tiles each).
-int radix_segments(int64_t tile_bound, int T);
-// One reduce-then-scan pass: tile counts, segment sums, slots, scatter.
+// Up to this many tiles, a pass is one kernel: every scatter tile sums the counts
+// of its table's tiles itself, and counts the next pass's digits as it writes.
+// (A pass's three kernels become one, 6 fewer in a backward of three passes: sort of
+// 330 K lookups in 8 tables 58 -> 40 us, of 106 K in 26 tables 52 -> 35 us, of 1.3 M
+// in 16 tables 76 -> 74 us. A tile reads its table's counts, so the reads grow with
+// the square of a table's tiles: 512 tiles of one table read 268 MB from L2.)
+constexpr int64_t kFewSortTiles = 512;
+// One reduce-then-scan pass: tile counts and slots, unless few tiles; scatter.
 void launch_radix_pass(const SortPass& S, int64_t tile_bound, cudaStream_t s);
-int radix_pass_launches();  // kernels launch_radix_pass enqueues
+int radix_pass_launches(int64_t tile_bound);  // kernels launch_radix_pass enqueues
 
 void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed, int64_t chunk_bound,
                    int num_sms, cudaStream_t s);

@@ -9,9 +9,11 @@
 // (warp match + per-warp counters, stable by position), lays them out by digit
 // in shared memory and writes each digit's run to that digit's slots of the
 // output. The first output slot of each (tile, digit) is found one of two ways:
-//   reduce-then-scan (default): one kernel counts every tile's digits, two
-//     more scan the counts per table (segment sums, then offsets), and the
-//     scatter reads its slots; no block waits on another.
+//   reduce-then-scan (default): one kernel counts every tile's digits, one
+//     scans the counts per table, and the scatter reads its slots; no block
+//     waits on another. With few tiles the scatter sums the counts itself, and
+//     the counts come from the kernel that wrote the keys (key generation, or
+//     the pass before).
 //   single sweep (CB_SORT_LOOKBACK): one streaming kernel counts every pass's
 //     digit histogram per table; each pass then reads and writes every pair
 //     once, a block publishing its per-digit counts and finding those of the
@@ -115,11 +117,7 @@ __device__ __forceinline__ void rank_tile(const uint32_t (&key)[kSortTile / NT],
 // The tile laid out by digit in shared memory (slot = the warp's start of the
 // digit, which holds the digit's tile-local start plus the counts of earlier
 // warps, + the rank): every slot first (the counters are read-only here), then
-// the stores. With CB_SORT_KV_PAIRS each (key, payload) pair goes to shared
-// memory as one 8-byte word.
-#ifndef CB_SORT_KV_PAIRS
-#define CB_SORT_KV_PAIRS 0
-#endif
+// the stores.
 template <int NT>
 __device__ __forceinline__ void scatter_tile(const uint32_t (&key)[kSortTile / NT], const uint32_t (&val)[kSortTile / NT],
                                              uint32_t (&rank2)[kSortTile / NT / 2], int tile_count, uint32_t key_base,
@@ -140,12 +138,8 @@ __device__ __forceinline__ void scatter_tile(const uint32_t (&key)[kSortTile / N
         const int local = wid * (32 * NI) + j * 32 + lane;
         if (local < tile_count) {
             const uint32_t pos = (j & 1) ? (rank2[j >> 1] >> 16) : (rank2[j >> 1] & 0xffffu);
-            if (CB_SORT_KV_PAIRS) {
-                reinterpret_cast<uint2*>(sh_keys)[pos] = make_uint2(key[j], val[j]);
-            } else {
-                sh_keys[pos] = key[j];
-                sh_vals[pos] = val[j];
-            }
+            sh_keys[pos] = key[j];
+            sh_vals[pos] = val[j];
         }
     }
 }
@@ -153,10 +147,12 @@ __device__ __forceinline__ void scatter_tile(const uint32_t (&key)[kSortTile / N
 // Consecutive shared slots of one digit go to consecutive global slots
 // (destination = sh_goff[digit] + slot). Half a tile at a time: its shared
 // reads, its destinations, its stores.
-template <int NT>
+// NEXT: the digits of the next pass are counted for the tile that each pair lands
+// in (tile first + (destination - p0) / kSortTile, at most last).
+template <int NT, bool NEXT = false>
 __device__ __forceinline__ void write_tile(const SortPass& S, int tile_count, uint32_t key_base,
                                            const int32_t* sh_goff, const uint32_t* sh_keys,
-                                           const uint32_t* sh_vals) {
+                                           const uint32_t* sh_vals, int32_t p0 = 0, int32_t first = 0, int32_t last = 0) {
     const int tid = threadIdx.x;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -166,14 +162,8 @@ __device__ __forceinline__ void write_tile(const SortPass& S, int tile_count, ui
 #pragma unroll
         for (int j = 0; j < kHalf; ++j) {
             const int i = tid + (h * kHalf + j) * NT;
-            if (CB_SORT_KV_PAIRS) {
-                const uint2 kv = i < tile_count ? reinterpret_cast<const uint2*>(sh_keys)[i] : make_uint2(0u, 0u);
-                key[j] = kv.x;
-                val[j] = kv.y;
-            } else {
-                key[j] = i < tile_count ? sh_keys[i] : 0u;
-                val[j] = i < tile_count ? sh_vals[i] : 0u;
-            }
+            key[j] = i < tile_count ? sh_keys[i] : 0u;
+            val[j] = i < tile_count ? sh_vals[i] : 0u;
         }
 #pragma unroll
         for (int j = 0; j < kHalf; ++j)
@@ -184,6 +174,11 @@ __device__ __forceinline__ void write_tile(const SortPass& S, int tile_count, ui
             if (i < tile_count && dst[j] >= 0 && dst[j] < S.n) {
                 S.keys_out[dst[j]] = key[j];
                 S.vals_out[dst[j]] = val[j];
+                if (NEXT) {
+                    const int32_t tile = min(first + max(dst[j] - p0, 0) / kSortTile, last);
+                    atomicAdd(S.next_digits + static_cast<int64_t>(tile) * kRadix +
+                                  sort_digit(key[j], key_base, S.shift + 8), 1u);
+                }
             }
         }
     }
@@ -336,98 +331,34 @@ __global__ void __launch_bounds__(kSortThreads, CB_COUNT_MIN_BLOCKS) radix_count
     for (int j = 0; j < kSortItems; ++j)
         if (tid + j * kSortThreads < count) atomicAdd(&sh[sort_digit(k[j], rb, S.shift)], 1u);
     __syncthreads();
-    S.tile_digits[tile * kRadix + tid] = sh[tid];
+    const uint32_t c = sh[tid];
+    S.tile_digits[tile * kRadix + tid] = c;
+    if (c) atomicAdd(S.table_digits + static_cast<int64_t>(tc.table) * kRadix + tid, c);
 }
 
-// Table t's tiles [f, e) cut into S.segments equal parts; part s is [a, b).
-__device__ __forceinline__ void segment_range(const SortPass& S, int t, int s, int64_t* a, int64_t* b) {
-    const int64_t f = S.table_first_tile[t], e = S.table_first_tile[t + 1];
-    const int64_t per = (e - f + S.segments - 1) / S.segments;
-    *a = min64(f + s * per, e);
-    *b = min64(*a + per, e);
-}
-
-// (b) Per (table, segment) block, thread d: the segment's count of digit d.
-__global__ void __launch_bounds__(kRadix) radix_segsum_kernel(const SortPass S) {
-    const int t = blockIdx.x / S.segments, sg = blockIdx.x % S.segments, d = threadIdx.x;
-    int64_t a, b;
-    segment_range(S, t, sg, &a, &b);
-    const uint32_t* c = S.tile_digits + d;
-    uint32_t sum = 0;
-    int64_t k = a;
-    for (; k + 8 <= b; k += 8) {
-        uint32_t v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = c[(k + u) * kRadix];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) sum += v[u];
-    }
-    for (; k < b; ++k) sum += c[k * kRadix];
-    S.seg_sums[(static_cast<int64_t>(t) * S.segments + sg) * kRadix + d] = sum;
-}
-
-// (c) Per (table, segment) block, thread d: the first output slot of digit d in
-// each of the segment's tiles, replacing its count. The slots of digit d in
-// table t start at the table's first position plus the table's counts of the
-// smaller digits; within the digit, tiles (and segments) keep their order.
-__global__ void __launch_bounds__(kRadix) radix_offsets_kernel(const SortPass S) {
-    __shared__ int64_t sh_scan[33];
-    const int t = blockIdx.x / S.segments, sg = blockIdx.x % S.segments, d = threadIdx.x;
-    const uint32_t* ss = S.seg_sums + static_cast<int64_t>(t) * S.segments * kRadix + d;
-    uint32_t total = 0, before = 0;
-    for (int q = 0; q < S.segments; ++q) {
-        const uint32_t v = ss[q * kRadix];
-        before += q < sg ? v : 0u;
-        total += v;
-    }
-    int64_t all;
-    const int64_t digit_start = block_excl_scan(total, sh_scan, &all);
-    // positions are below 2^30: 32 bits hold every slot
-    uint32_t run = static_cast<uint32_t>(S.table_pos[t] + digit_start) + before;
-    int64_t a, b;
-    segment_range(S, t, sg, &a, &b);
-    uint32_t* c = S.tile_digits + d;
-    int64_t k = a;
-    for (; k + 8 <= b; k += 8) {
-        uint32_t v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = c[(k + u) * kRadix];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            c[(k + u) * kRadix] = run;
-            run += v[u];
-        }
-    }
-    for (; k < b; ++k) {
-        const uint32_t v = c[k * kRadix];
-        c[k * kRadix] = run;
-        run += v;
-    }
-}
-
-// (b + c) in one kernel (CB_SORT_TABLE_SCAN): one block of 1024 threads per
-// table; thread (part, d) owns digit d over a quarter of the table's tiles.
-// It sums the part's counts (16 loads in flight), the block turns the four
-// parts' sums into each (part, digit)'s first slot (table start + the table's
-// counts of smaller digits + the earlier parts' counts of the digit), and the
-// thread replaces every count of its part by the tile's first slot. No block
-// waits on another; the per-(table, segment) blocks of (b) and (c) were
-// latency-bound on short loops.
-#ifndef CB_SORT_TABLE_SCAN
-#define CB_SORT_TABLE_SCAN 1
-#endif
-constexpr int kScanParts = 4;
+// (b) The first output slot of every (tile, digit), replacing its count: the
+// table's first position, plus the table's counts of smaller digits, plus the
+// counts of the digit in the table's earlier tiles. A block takes kScanDigits digits
+// of a table (8 blocks per table) and a thread one digit over 1/16 of the table's
+// tiles, up to kScanLoads loads in flight (6 tables of 500 tiles: sort 402 -> 373 us
+// against one block per table and four threads per digit, 24 us a pass; 64 tables of
+// 100 tiles, 643 us that way: 656 with 32 parts).
+constexpr int kScanDigits = 32;
+constexpr int kScanParts = 16;
 constexpr int kScanLoads = 16;
 
-__global__ void __launch_bounds__(kRadix * kScanParts) radix_table_scan_kernel(const SortPass S) {
-    __shared__ uint32_t sh_part[kScanParts][kRadix];
+__global__ void __launch_bounds__(kScanDigits * kScanParts) radix_slots_kernel(const SortPass S) {
+    __shared__ uint32_t sh_part[kScanParts][kScanDigits];
     __shared__ uint32_t sh_start[kRadix];
     __shared__ int64_t sh_scan[33];
-    const int t = blockIdx.x;
-    const int d = threadIdx.x & (kRadix - 1), part = threadIdx.x / kRadix;
+    const int groups = kRadix / kScanDigits;
+    const int t = blockIdx.x / groups, tid = threadIdx.x;
+    const int lane = tid & (kScanDigits - 1), part = tid / kScanDigits;
+    const int d = (blockIdx.x % groups) * kScanDigits + lane;
     const int64_t f = S.table_first_tile[t], e = S.table_first_tile[t + 1];
     const int64_t per = (e - f + kScanParts - 1) / kScanParts;
     const int64_t a = min64(f + part * per, e), b = min64(a + per, e);
+    const uint32_t mine = tid < kRadix ? S.table_digits[static_cast<int64_t>(t) * kRadix + tid] : 0u;
     uint32_t* c = S.tile_digits + d;
     uint32_t sum = 0;
     int64_t k = a;
@@ -439,22 +370,14 @@ __global__ void __launch_bounds__(kRadix * kScanParts) radix_table_scan_kernel(c
         for (int u = 0; u < kScanLoads; ++u) sum += v[u];
     }
     for (; k < b; ++k) sum += c[k * kRadix];
-    sh_part[part][d] = sum;
-    __syncthreads();
-    uint32_t total = 0, before = 0;
-#pragma unroll
-    for (int q = 0; q < kScanParts; ++q) {
-        const uint32_t x = sh_part[q][d];
-        before += q < part ? x : 0u;
-        total += x;
-    }
-    // digit starts: the scan over the first part's threads (0..255, one per digit)
+    sh_part[part][lane] = sum;
     int64_t all;
-    const int64_t ex = block_excl_scan(part == 0 ? total : 0u, sh_scan, &all);
+    const int64_t ex = block_excl_scan(mine, sh_scan, &all);
     // positions are below 2^30: 32 bits hold every slot
-    if (part == 0) sh_start[d] = static_cast<uint32_t>(S.table_pos[t] + ex);
+    if (tid < kRadix) sh_start[tid] = static_cast<uint32_t>(S.table_pos[t] + ex);
     __syncthreads();
-    uint32_t run = sh_start[d] + before;
+    uint32_t run = sh_start[d];
+    for (int q = 0; q < part; ++q) run += sh_part[q][lane];
     for (k = a; k + kScanLoads <= b; k += kScanLoads) {
         uint32_t v[kScanLoads];
 #pragma unroll
@@ -472,8 +395,9 @@ __global__ void __launch_bounds__(kRadix * kScanParts) radix_table_scan_kernel(c
     }
 }
 
-// (d) The scatter of tile blockIdx.x: the ranking of the single-sweep kernel,
-// with the first output slot of every digit read from (c). NT threads per tile
+// (c) The scatter of tile blockIdx.x: the ranking of the single-sweep kernel,
+// with the first output slot of every digit read from (b), or (FEW) summed here
+// from the counts of the table's tiles. NT threads per tile
 // (NT / 32 warps ranking kSortTile / NT keys per thread); threads 0..255 own one
 // digit each in the prefix step.
 #ifndef CB_SCATTER_THREADS
@@ -482,7 +406,7 @@ __global__ void __launch_bounds__(kRadix * kScanParts) radix_table_scan_kernel(c
 constexpr int kScatterThreads = CB_SCATTER_THREADS;
 static_assert(kScatterThreads >= kRadix && kSortTile % kScatterThreads == 0, "scatter block shape");
 
-template <int NT>
+template <int NT, bool FEW>
 __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1024 / NT) radix_scatter_kernel(const SortPass S) {
     constexpr int NI = kSortTile / NT;
     constexpr int NW = NT / 32;
@@ -498,9 +422,16 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1024 / NT) radix_scatter_k
     if (tile >= *S.num_tiles) return;  // the grid is an upper bound on the tiles
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     for (int i = tid; i < NW * (kRadix + 1); i += NT) (&sh_warp[0][0])[i] = 0;
-    // digit tid's first output slot
-    const uint32_t slot = tid < kRadix ? S.tile_digits[tile * kRadix + tid] : 0u;
     const Chunk tc = S.tiles[tile];
+    // digit tid's first output slot; FEW: the counts it follows from
+    uint32_t slot = 0, digit_total = 0;
+    int64_t first_tile = 0, last_tile = 0;
+    if constexpr (FEW) {
+        first_tile = S.table_first_tile[tc.table];
+        last_tile = S.table_first_tile[tc.table + 1] - 1;
+    } else {
+        slot = tid < kRadix ? S.tile_digits[tile * kRadix + tid] : 0u;
+    }
     const int64_t tile_base = tc.k0;
     const int tile_count = static_cast<int>(min64(tc.len & 0x7fffffffu, S.n - tile_base));
     const uint32_t key_base = static_cast<uint32_t>(S.tables[tc.table].key_base);
@@ -511,6 +442,23 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1024 / NT) radix_scatter_k
         const bool valid = local < tile_count;
         key[j] = valid ? __ldg(S.keys_in + tile_base + local) : 0u;
         val[j] = valid ? __ldg(S.vals_in + tile_base + local) : 0u;
+    }
+    if constexpr (FEW) {
+        if (tid < kRadix) {
+            const uint32_t* c = S.tile_digits + tid;
+            for (int64_t k0 = first_tile; k0 <= last_tile; k0 += 8) {
+                uint32_t v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = k0 + u <= last_tile ? __ldg(c + (k0 + u) * kRadix) : 0u;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    digit_total += v[u];
+                    slot += k0 + u < tile ? v[u] : 0u;
+                }
+            }
+        }
+        int64_t all;
+        slot += static_cast<uint32_t>(S.table_pos[tc.table] + block_excl_scan(digit_total, sh_scan, &all));
     }
     __syncthreads();
     uint32_t rank2[NI / 2];
@@ -536,7 +484,12 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1024 / NT) radix_scatter_k
     __syncthreads();
     scatter_tile<NT>(key, val, rank2, tile_count, key_base, S.shift, sh_warp, sh_keys, sh_vals);
     __syncthreads();
-    write_tile<NT>(S, tile_count, key_base, sh_goff, sh_keys, sh_vals);
+    if (FEW && S.next_digits)
+        write_tile<NT, true>(S, tile_count, key_base, sh_goff, sh_keys, sh_vals,
+                             static_cast<int32_t>(S.table_pos[tc.table]), static_cast<int32_t>(first_tile),
+                             static_cast<int32_t>(last_tile));
+    else
+        write_tile<NT>(S, tile_count, key_base, sh_goff, sh_keys, sh_vals);
 }
 
 // ---------------------------------------------------------------- single sweep
@@ -617,31 +570,28 @@ void launch_sort_bases(const uint32_t* hist, const int64_t* table_pos, int T, in
 
 constexpr int kSortDynSmem = 2 * kSortTile * sizeof(uint32_t);  // 32 KB
 
-int radix_segments(int64_t tile_bound, int T) {
-    const int64_t per_table = tile_bound / max64(T, 1) + 1;
-    return static_cast<int>(min64(max64((per_table + 15) / 16, 1), 1024));
+template <bool FEW>
+void launch_scatter(const SortPass& S, unsigned grid, cudaStream_t s) {
+    // static + dynamic shared memory may pass the 48 KB default
+    static const bool configured = cudaFuncSetAttribute(radix_scatter_kernel<kScatterThreads, FEW>,
+                                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                        kSortDynSmem) == cudaSuccess;
+    (void)configured;
+    radix_scatter_kernel<kScatterThreads, FEW><<<grid, kScatterThreads, kSortDynSmem, s>>>(S);
 }
 
 void launch_radix_pass(const SortPass& S, int64_t tile_bound, cudaStream_t s) {
     const unsigned grid = static_cast<unsigned>(max64(tile_bound, 1));
-    const unsigned parts = static_cast<unsigned>(S.T) * static_cast<unsigned>(S.segments);
+    if (tile_bound <= kFewSortTiles) {
+        launch_scatter<true>(S, grid, s);
+        return;
+    }
     radix_count_kernel<<<grid, kSortThreads, 0, s>>>(S);
-    if (CB_SORT_TABLE_SCAN) {
-        radix_table_scan_kernel<<<static_cast<unsigned>(S.T), kRadix * kScanParts, 0, s>>>(S);
-    } else {
-        radix_segsum_kernel<<<parts, kRadix, 0, s>>>(S);
-        radix_offsets_kernel<<<parts, kRadix, 0, s>>>(S);
-    }
-    static bool configured = false;
-    if (!configured) {  // static + dynamic shared memory may pass the 48 KB default
-        cudaFuncSetAttribute(radix_scatter_kernel<kScatterThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSortDynSmem);
-        configured = true;
-    }
-    radix_scatter_kernel<kScatterThreads><<<grid, kScatterThreads, kSortDynSmem, s>>>(S);
+    radix_slots_kernel<<<static_cast<unsigned>(S.T) * (kRadix / kScanDigits), kScanDigits * kScanParts, 0, s>>>(S);
+    launch_scatter<false>(S, grid, s);
 }
 
-int radix_pass_launches() { return CB_SORT_TABLE_SCAN ? 3 : 4; }
+int radix_pass_launches(int64_t tile_bound) { return tile_bound <= kFewSortTiles ? 1 : 3; }
 
 void launch_onesweep(const SortPass& S, int64_t tile_bound, cudaStream_t s) {
     static bool configured = false;
