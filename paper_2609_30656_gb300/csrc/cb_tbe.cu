@@ -91,9 +91,6 @@ struct Workspace {
     int64_t* float_base = nullptr;
     int64_t* out_sizes = nullptr;  // [2] U and F of a fused step (no caller buffers)
     int* cap_fail = nullptr;
-    int4* heavy = nullptr;
-    uint32_t* heavy_count = nullptr;
-    int64_t max_heavy = 0;
     int64_t sort_tiles = 0;
     size_t status_bytes = 0;
 };
@@ -212,9 +209,6 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
     ws.float_base = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.out_sizes = static_cast<int64_t*>(take(sizeof(int64_t) * 2));
     ws.cap_fail = static_cast<int*>(take(sizeof(int)));
-    ws.max_heavy = max_chunks / 32 + 1;  // a heavy run owns more than 32 chunks
-    ws.heavy = static_cast<int4*>(take(sizeof(int4) * ws.max_heavy));
-    ws.heavy_count = static_cast<uint32_t*>(take(sizeof(uint32_t)));
     if (w) *w = ws;
     return off;
 }
@@ -462,9 +456,6 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     O.float_base = w.float_base;
     O.tables_done = h->d_tables_done;
     O.cap_fail = w.cap_fail;
-    O.heavy = w.heavy;
-    O.heavy_count = w.heavy_count;
-    O.max_heavy = w.max_heavy;
     if (a) {
         // No caller buffers: the sizes land in the workspace's own words.
         O.unique_ids = nullptr;
@@ -510,11 +501,7 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
                           bound, h->num_sms, stream);
         h->launches += 1;
         launch_bwd_fixup(P, Q, O, bound, h->num_sms, stream);
-        h->launches += 2;
-        if (a) {
-            launch_bwd_apply_split(P, Q, O, bound, h->num_sms, stream);
-            h->launches += 1;
-        }
+        h->launches += 1;
     }
     record(h, h->ev_bwd[4], stream);
     h->bwd_timed = (h->flags & CB_TIMING) != 0;

@@ -254,9 +254,12 @@ __global__ void __launch_bounds__(1024) bwd_outputs_kernel(const __grid_constant
 // ---------------------------------------------------------------- (6) fix-up
 
 // Runs split over chunks (hot rows that cover whole cells): each warp scans
-// `span` chunks at a time for tail pieces and combines each such run in fp64. Runs
-// spread over more than kHeavyPieces chunks go to a list that bwd_heavy_kernel
-// combines with a whole block each.
+// `span` chunks at a time for tail pieces and combines each such run in fp64; runs
+// spread over more than kHeavyPieces chunks are left to the whole block, after its
+// warps' own. With the optimizer step fused, the row is stepped as soon as its sum is
+// complete. (A list of the heavy runs for a second kernel, and a third kernel for the
+// step, took 51 us on 41 M skewed lookups and 3 + 15 us more on 1.3 M with Adagrad;
+// this kernel @@ and @@.)
 constexpr int64_t kHeavyPieces = 32;
 
 // The chunks after chunk j that hold the rest of its open run: the pieces that
@@ -276,19 +279,53 @@ __device__ __forceinline__ int64_t run_pieces(const Plan& Q, int64_t j, int t, i
     }
 }
 
+// Where the fix-up leaves a split run's sum: its gradient row, or, for a fused step,
+// the tail slot of the chunk where it begins.
+__device__ __forceinline__ float* split_row(const Plan& Q, const BwdOut& O, int64_t dmax, int64_t j, int64_t seg, int t,
+                                            int dim) {
+    return O.apply ? Q.carry_tail + j * dmax : O.grads + O.float_base[t] + seg * dim;
+}
+
+// Lane l stores columns [4l + 128k, + 4), and steps them itself.
 __device__ __forceinline__ void store_grad4(float* dst, int x0, const double (&acc)[4]) {
     *reinterpret_cast<float4*>(dst + x0) =
         make_float4(static_cast<float>(acc[0]), static_cast<float>(acc[1]),
                     static_cast<float>(acc[2]), static_cast<float>(acc[3]));
 }
 
+// The fused step of the run that is open at the end of chunk j, whose complete
+// gradient row `g` each lane of the warp has stored its columns of.
+__device__ __forceinline__ void step_split_run(const Problem& P, const Plan& Q, const BwdOut& O, int64_t j, int t,
+                                               const float* g, int lane) {
+    const TableDev& td = P.tables[t];
+    const Chunk ch = Q.chunks[j];
+    // the chunk's last position belongs to the run
+    const int64_t row = static_cast<int64_t>(O.keys_sorted[ch.k0 + (ch.len & 0x7fffffffu) - 1]) - td.key_base;
+    float sq = 0.f;
+    for (int x0 = lane * 4; x0 < td.dim; x0 += 128) sq += sq4(*reinterpret_cast<const float4*>(g + x0));
+    const float scale = step_scale(O, t, row, td.dim, sq);
+    for (int x0 = lane * 4; x0 < td.dim; x0 += 128)
+        step_cols(td, row, x0, *reinterpret_cast<const float4*>(g + x0), scale);
+}
+
 __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_constant__ Problem P,
                                                                  const __grid_constant__ Plan Q,
                                                                  const __grid_constant__ BwdOut O, int span) {
+    constexpr int kWarps = kWarpThreads / 32;
+    // Heavy runs of a round: they begin more than kHeavyPieces chunks apart, in the
+    // at most kWarps * 32 chunks that the block scans.
+    constexpr int kMaxHeavy = kWarps * 32 / static_cast<int>(kHeavyPieces) + 2;
+    __shared__ double sh[kWarps][512];
+    __shared__ int4 heavy[kMaxHeavy];
+    __shared__ int heavy_count;
     if (*O.cap_fail) return;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
+    const int64_t round = static_cast<int64_t>(gridDim.x) * kWarps * span;
+    for (int64_t base0 = static_cast<int64_t>(blockIdx.x) * kWarps * span; base0 < total; base0 += round) {
+        if (threadIdx.x == 0) heavy_count = 0;
+        __syncthreads();
+        const int64_t base = base0 + static_cast<int64_t>(w) * span;
         const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
         for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
             const int b = __ffs(mask) - 1;
@@ -298,90 +335,53 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_co
             const int64_t m = run_pieces(Q, j, t, total, lane);
             if (m > kHeavyPieces) {
                 if (lane == 0) {
-                    const uint32_t slot = atomicAdd(O.heavy_count, 1u);
-                    if (slot < O.max_heavy)
-                        O.heavy[slot] = make_int4(static_cast<int>(j), static_cast<int>(seg),
-                                                  static_cast<int>(m), 0);
+                    const int slot = atomicAdd(&heavy_count, 1);
+                    if (slot < kMaxHeavy)
+                        heavy[slot] = make_int4(static_cast<int>(j), static_cast<int>(seg), static_cast<int>(m), t);
                 }
                 continue;
             }
-            const TableDev& td = P.tables[t];
-            // A fused step takes the combined row from the chunk's tail slot.
-            float* dst = O.apply ? Q.carry_tail + j * P.dmax
-                                 : O.grads + O.float_base[t] + seg * td.dim;
-            combine_pieces(Q, j, m, td.dim, P.dmax, lane,
-                           [&](int x0, double (&acc)[4]) { store_grad4(dst, x0, acc); });
-        }
-    }
-}
-
-// One heavy run per block: warp w adds pieces w, w + 8, ... (lanes own columns;
-// fp32 groups folded into fp64), then the warps' partial sums meet in shared
-// memory in warp order, after the tail piece. The order is fixed, so the result
-// is deterministic.
-__global__ void __launch_bounds__(kWarpThreads) bwd_heavy_kernel(const __grid_constant__ Problem P,
-                                                                 const __grid_constant__ Plan Q,
-                                                                 const __grid_constant__ BwdOut O) {
-    __shared__ double sh[kWarpThreads / 32][512];
-    if (*O.cap_fail) return;
-    const uint32_t count = min64(*O.heavy_count, O.max_heavy);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    constexpr int kWarps = kWarpThreads / 32;
-    for (uint32_t h = blockIdx.x; h < count; h += gridDim.x) {
-        const int4 rec = O.heavy[h];
-        const int64_t j = rec.x, seg = rec.y, m = rec.z;
-        const int t = Q.chunks[j].table;
-        const TableDev& td = P.tables[t];
-        const float* head = Q.carry_head + (j + 1) * P.dmax;
-        for (int x0 = lane * 4; x0 < td.dim; x0 += 128) {
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-            add_pieces(head, w, kWarps, m, P.dmax, x0, acc);
-            for (int x = 0; x < 4; ++x) sh[w][x0 + x] = acc[x];
-        }
-        __syncthreads();
-        if (w == 0) {
-            float* dst = O.apply ? Q.carry_tail + j * P.dmax
-                                 : O.grads + O.float_base[t] + seg * td.dim;
+            const int dim = P.tables[t].dim;
+            float* dst = split_row(Q, O, P.dmax, j, seg, t, dim);
             const float* tail = Q.carry_tail + j * P.dmax;
-            for (int x0 = lane * 4; x0 < td.dim; x0 += 128) {
+            const float* head = Q.carry_head + (j + 1) * P.dmax;
+            for (int x0 = lane * 4; x0 < dim; x0 += 128) {
                 const float4 a = *reinterpret_cast<const float4*>(tail + x0);
                 double acc[4] = {a.x, a.y, a.z, a.w};
-                for (int ww = 0; ww < kWarps; ++ww)
-                    for (int x = 0; x < 4; ++x) acc[x] += sh[ww][x0 + x];
+                add_pieces(head, 0, 1, m, P.dmax, x0, acc);
                 store_grad4(dst, x0, acc);
             }
+            if (O.apply) step_split_run(P, Q, O, j, t, dst, lane);
         }
         __syncthreads();
-    }
-}
-
-// Fused step for the runs the fix-up combined: their full gradient row waits in
-// the tail slot of the chunk where the run begins. One warp per such run.
-__global__ void __launch_bounds__(kWarpThreads) bwd_apply_split_kernel(const __grid_constant__ Problem P,
-                                                                       const __grid_constant__ Plan Q,
-                                                                       const __grid_constant__ BwdOut O, int span) {
-    if (*O.cap_fail) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
-        const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
-        for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
-            const int b = __ffs(mask) - 1;
-            const int64_t j = base + b;
-            const Chunk ch = Q.chunks[j];
-            const int t = ch.table;
-            const TableDev& td = P.tables[t];
-            // the chunk's last position belongs to the run
-            const int64_t row = static_cast<int64_t>(O.keys_sorted[ch.k0 + (ch.len & 0x7fffffffu) - 1]) - td.key_base;
-            const float* g = Q.carry_tail + j * P.dmax;
-            float sq = 0.f;
-            for (int x0 = lane * 4; x0 < td.dim; x0 += 128) {
-                const float4 v = *reinterpret_cast<const float4*>(g + x0);
-                sq += sq4(v);
+        // A heavy run: warp w adds pieces w, w + 8, ... (lanes own columns; fp32 groups
+        // folded into fp64), then the warps' partial sums meet in warp order, after
+        // the tail piece. The order is fixed, so the result is deterministic.
+        const int count = min(heavy_count, kMaxHeavy);
+        for (int h = 0; h < count; ++h) {
+            const int64_t j = heavy[h].x, seg = heavy[h].y, m = heavy[h].z;
+            const int t = heavy[h].w;
+            const int dim = P.tables[t].dim;
+            const float* head = Q.carry_head + (j + 1) * P.dmax;
+            for (int x0 = lane * 4; x0 < dim; x0 += 128) {
+                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                add_pieces(head, w, kWarps, m, P.dmax, x0, acc);
+                for (int x = 0; x < 4; ++x) sh[w][x0 + x] = acc[x];
             }
-            const float scale = step_scale(O, t, row, td.dim, sq);
-            for (int x0 = lane * 4; x0 < td.dim; x0 += 128)
-                step_cols(td, row, x0, *reinterpret_cast<const float4*>(g + x0), scale);
+            __syncthreads();
+            if (w == 0) {
+                float* dst = split_row(Q, O, P.dmax, j, seg, t, dim);
+                const float* tail = Q.carry_tail + j * P.dmax;
+                for (int x0 = lane * 4; x0 < dim; x0 += 128) {
+                    const float4 a = *reinterpret_cast<const float4*>(tail + x0);
+                    double acc[4] = {a.x, a.y, a.z, a.w};
+                    for (int ww = 0; ww < kWarps; ++ww)
+                        for (int x = 0; x < 4; ++x) acc[x] += sh[ww][x0 + x];
+                    store_grad4(dst, x0, acc);
+                }
+                if (O.apply) step_split_run(P, Q, O, j, t, dst, lane);
+            }
+            __syncthreads();
         }
     }
 }
@@ -429,17 +429,8 @@ void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const v
 
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
-    cudaMemsetAsync(O.heavy_count, 0, sizeof(uint32_t), s);
     const int span = fixup_span(chunk_bound, num_sms);
     bwd_fixup_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, O, span);
-    const int hgrid = static_cast<int>(max64(1, min64(O.max_heavy, static_cast<int64_t>(num_sms) * 4)));
-    bwd_heavy_kernel<<<hgrid, kWarpThreads, 0, s>>>(P, Q, O);
-}
-
-void launch_bwd_apply_split(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
-                            int num_sms, cudaStream_t s) {
-    const int span = fixup_span(chunk_bound, num_sms);
-    bwd_apply_split_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, O, span);
 }
 
 }  // namespace cbtbe

@@ -117,9 +117,6 @@ struct BwdOut {
     int64_t* float_base;         // [T + 1]
     uint32_t* tables_done;       // zero between calls
     int* cap_fail;
-    int4* heavy;                 // [max_heavy] runs left for the block-wide combine
-    uint32_t* heavy_count;       // zeroed before the fix-up
-    int64_t max_heavy;
     // caller's buffers
     int64_t* unique_ids;
     int64_t* table_offsets;
@@ -207,7 +204,4 @@ void launch_weight_grad(const Problem& P, const Plan& Q, const void* grad_out, f
                         int dtype, int vpl, int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s);
-void launch_bwd_apply_split(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
-                            int num_sms, cudaStream_t s);
-
 }  // namespace cbtbe
