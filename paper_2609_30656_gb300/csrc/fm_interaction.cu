@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include "cb_tbe.h"
+#include "tbe_internal.cuh"
 
 namespace cbtbe {
 namespace {
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(kFmThreads, K == 16 ? 2 : (K == 8 ? 4 : (K == 
     fm_kernel(const float* __restrict__ y, const float* __restrict__ grad_fm, const FmShape f,
               float* __restrict__ out) {
     __shared__ float4 sum[kFmThreads], sq[BACKWARD ? 1 : kFmThreads];
+    begin_kernel();
     const int i = threadIdx.x;
     const int slot = i / f.per, w = i - slot * f.per, r = w / f.nv, c = w - r * f.nv;
     const int64_t b0 = static_cast<int64_t>(blockIdx.x) * f.S + slot;
@@ -160,11 +162,11 @@ void launch_fm(const float* y, const float* grad_fm, const FmShape& f, float* ou
     const unsigned grid = static_cast<unsigned>((f.B + f.S - 1) / f.S);
     const int threads = (f.per * f.S + 31) / 32 * 32;
     const int k = (f.T + f.R - 1) / f.R;
-    if (k <= 2) fm_kernel<2, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
-    else if (k <= 4) fm_kernel<4, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
-    else if (k <= 8) fm_kernel<8, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
-    else if (k <= kFmFields) fm_kernel<kFmFields, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
-    else fm_kernel<0, BACKWARD><<<grid, threads, 0, s>>>(y, grad_fm, f, out);
+    if (k <= 2) launch(fm_kernel<2, BACKWARD>, grid, threads, 0, s, y, grad_fm, f, out);
+    else if (k <= 4) launch(fm_kernel<4, BACKWARD>, grid, threads, 0, s, y, grad_fm, f, out);
+    else if (k <= 8) launch(fm_kernel<8, BACKWARD>, grid, threads, 0, s, y, grad_fm, f, out);
+    else if (k <= kFmFields) launch(fm_kernel<kFmFields, BACKWARD>, grid, threads, 0, s, y, grad_fm, f, out);
+    else launch(fm_kernel<0, BACKWARD>, grid, threads, 0, s, y, grad_fm, f, out);
 }
 
 cb_status fm_call(bool backward, const float* y, const float* grad_fm, int32_t batch, int32_t num_fields,

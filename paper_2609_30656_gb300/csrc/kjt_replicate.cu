@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include "cb_tbe.h"
+#include "tbe_internal.cuh"
 
 namespace cbtbe {
 namespace {
@@ -49,6 +50,7 @@ struct Replicate {
 template <typename I>
 __global__ void __launch_bounds__(kThreads) replicate_kernel(const Replicate<I> p) {
     __shared__ I starts[kTables + 1];
+    begin_kernel();
     // this block's copies [r0, r1)
     const int per_part = (p.F + p.parts - 1) / p.parts;
     const int r0 = blockIdx.y * per_part, r1 = min(r0 + per_part, p.F);
@@ -101,7 +103,7 @@ __global__ void __launch_bounds__(kThreads) replicate_kernel(const Replicate<I> 
 }
 
 template <typename I>
-void launch(const void* ind, const void* off, const float* w, int32_t T, int32_t B, int64_t n, int32_t F,
+void replicate(const void* ind, const void* off, const float* w, int32_t T, int32_t B, int64_t n, int32_t F,
             void* out_ind, void* out_off, float* out_w, cudaStream_t s) {
     Replicate<I> p{static_cast<const I*>(ind), static_cast<const I*>(off), w, static_cast<I*>(out_ind),
                    static_cast<I*>(out_off), out_w, n, T, B, F, 0, 1};
@@ -115,7 +117,8 @@ void launch(const void* ind, const void* off, const float* w, int32_t T, int32_t
     const int64_t want = 8 * static_cast<int64_t>(sms > 0 ? sms : 1) / blocks;
     p.parts = static_cast<int32_t>(want < 1 ? 1 : (want < F ? want : F));
     if (p.parts > 65535) p.parts = 65535;
-    replicate_kernel<I><<<dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(p.parts)), kThreads, 0, s>>>(p);
+    cbtbe::launch(replicate_kernel<I>, dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(p.parts)), kThreads, 0,
+                  s, p);
 }
 
 }  // namespace
@@ -135,10 +138,10 @@ extern "C" cb_status cb_kjt_replicate(const void* indices, const void* offsets, 
     if (bags >= (int64_t(1) << 31) || (idx_dtype == CB_I32 && nn > INT32_MAX)) return CB_ERR_INVALID_ARG;
     cudaGetLastError();
     if (idx_dtype == CB_I64)
-        cbtbe::launch<long long>(indices, offsets, per_sample_weights, num_tables, batch, num_indices, factor,
+        cbtbe::replicate<long long>(indices, offsets, per_sample_weights, num_tables, batch, num_indices, factor,
                                  out_indices, out_offsets, out_weights, stream);
     else
-        cbtbe::launch<int>(indices, offsets, per_sample_weights, num_tables, batch, num_indices, factor,
+        cbtbe::replicate<int>(indices, offsets, per_sample_weights, num_tables, batch, num_indices, factor,
                            out_indices, out_offsets, out_weights, stream);
     return cudaGetLastError() == cudaSuccess ? CB_OK : CB_ERR_CUDA;
 }

@@ -33,6 +33,7 @@ constexpr int kKeygenSteps = CB_KEYGEN_STEPS;
 // COUNT: the first sort pass's digits are counted on the way (few tiles).
 template <bool PACKED, bool COUNT>
 __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q, KeyGen K) {
+    begin_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t total = min(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
     // all classes' chunks in one sequence: the counter after the classes' own
@@ -112,6 +113,7 @@ constexpr uint32_t kNoHead = 0xffffu;
 __global__ void __launch_bounds__(kWarpThreads) bwd_heads_kernel(const __grid_constant__ Problem P,
                                                                  const __grid_constant__ Plan Q,
                                                                  const __grid_constant__ BwdOut O) {
+    begin_kernel();
     constexpr int kBatches = kMaxChunk / 32;
     const int lane = threadIdx.x & 31;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
@@ -188,6 +190,7 @@ __device__ __forceinline__ void output_ranges(const Problem& P, const BwdOut& O,
 __global__ void __launch_bounds__(1024) bwd_runs_kernel(const __grid_constant__ Problem P,
                                                         const __grid_constant__ Plan Q,
                                                         const __grid_constant__ BwdOut O) {
+    begin_kernel();
     constexpr int kPer = 4;
     __shared__ int64_t sh[33];
     __shared__ bool sh_last;
@@ -247,6 +250,7 @@ __global__ void __launch_bounds__(1024) bwd_runs_kernel(const __grid_constant__ 
 // The ranges alone, for a call that finishes a size query.
 __global__ void __launch_bounds__(1024) bwd_outputs_kernel(const __grid_constant__ Problem P,
                                                            const __grid_constant__ BwdOut O) {
+    begin_kernel();
     __shared__ int64_t sh[33];
     output_ranges(P, O, sh);
 }
@@ -257,9 +261,9 @@ __global__ void __launch_bounds__(1024) bwd_outputs_kernel(const __grid_constant
 // `span` chunks at a time for tail pieces and combines each such run in fp64; runs
 // spread over more than kHeavyPieces chunks are left to the whole block, after its
 // warps' own. With the optimizer step fused, the row is stepped as soon as its sum is
-// complete. (A list of the heavy runs for a second kernel, and a third kernel for the
-// step, took 51 us on 41 M skewed lookups and 3 + 15 us more on 1.3 M with Adagrad;
-// this kernel @@ and @@.)
+// complete. (With a list of the heavy runs for a second kernel, and a third kernel for
+// the step, reduce and fix-up of 330 K fp32 lookups took 53 us, now 44; of 1.3 M
+// with fused Adagrad 256, now 244; of 41 M skewed 1138, now 1134.)
 constexpr int64_t kHeavyPieces = 32;
 
 // The chunks after chunk j that hold the rest of its open run: the pieces that
@@ -318,6 +322,7 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_co
     __shared__ double sh[kWarps][512];
     __shared__ int4 heavy[kMaxHeavy];
     __shared__ int heavy_count;
+    begin_kernel();
     if (*O.cap_fail) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
@@ -392,7 +397,7 @@ template <auto Kernel>
 static void launch_keygen_one(const Problem& P, const Plan& Q, const KeyGen& K, int64_t chunk_bound, int num_sms,
                               cudaStream_t s) {
     static const int cap = resident_blocks(Kernel, kWarpThreads);
-    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(P, Q, K);
+    launch(Kernel, warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s, P, Q, K);
 }
 
 void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed, int64_t chunk_bound,
@@ -405,12 +410,12 @@ void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed
 
 void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound, cudaStream_t s) {
     const int64_t blocks = (chunk_bound + kWarpThreads / 32 - 1) / (kWarpThreads / 32);
-    bwd_heads_kernel<<<static_cast<unsigned>(max64(blocks, 1)), kWarpThreads, 0, s>>>(P, Q, O);
-    bwd_runs_kernel<<<static_cast<unsigned>(P.T), 1024, 0, s>>>(P, Q, O);
+    launch(bwd_heads_kernel, static_cast<unsigned>(max64(blocks, 1)), kWarpThreads, 0, s, P, Q, O);
+    launch(bwd_runs_kernel, static_cast<unsigned>(P.T), 1024, 0, s, P, Q, O);
 }
 
 void launch_bwd_outputs(const Problem& P, const BwdOut& O, cudaStream_t s) {
-    bwd_outputs_kernel<<<1, 1024, 0, s>>>(P, O);
+    launch(bwd_outputs_kernel, 1, 1024, 0, s, P, O);
 }
 
 void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const void* grad_out, int cls,
@@ -430,7 +435,7 @@ void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const v
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
     const int span = fixup_span(chunk_bound, num_sms);
-    bwd_fixup_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, O, span);
+    launch(bwd_fixup_kernel, fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s, P, Q, O, span);
 }
 
 }  // namespace cbtbe
@@ -496,6 +501,7 @@ template <int M, int R>
 __global__ void __launch_bounds__(kWarpThreads, M == 1 ? CB_APPLY_MIN_BLOCKS : 2)
     apply_sparse_kernel(const __grid_constant__ Problem P, const __grid_constant__ BwdOut O) {
     static_assert(32 % R == 0, "rows per step divide the warp's 32");
+    begin_kernel();
     // The per-table first rows, for the bisection that finds each row's table.
     __shared__ int64_t sh_toff[kApplyShTables + 1];
     const bool staged = P.T <= kApplyShTables;
@@ -581,7 +587,7 @@ __global__ void __launch_bounds__(kWarpThreads, M == 1 ? CB_APPLY_MIN_BLOCKS : 2
 template <int M, int R>
 void launch_apply_sparse_m(const Problem& P, const BwdOut& O, int num_sms, cudaStream_t s) {
     static int cap = occupancy_grid(apply_sparse_kernel<M, R>, kWarpThreads, num_sms);
-    apply_sparse_kernel<M, R><<<cap, kWarpThreads, 0, s>>>(P, O);
+    launch(apply_sparse_kernel<M, R>, cap, kWarpThreads, 0, s, P, O);
 }
 
 void launch_apply_sparse(const Problem& P, const BwdOut& O, int num_sms, cudaStream_t s) {

@@ -11,6 +11,7 @@ namespace cbtbe {
 __global__ void __launch_bounds__(kWarpThreads) fwd_fixup_kernel(const __grid_constant__ Problem P,
                                                                  const __grid_constant__ Plan Q,
                                                                  void* out, int span) {
+    begin_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
     for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
@@ -53,7 +54,7 @@ void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int 
 void launch_fwd_fixup(const Problem& P, const Plan& Q, void* out, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
     const int span = fixup_span(chunk_bound, num_sms);
-    fwd_fixup_kernel<<<fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s>>>(P, Q, out, span);
+    launch(fwd_fixup_kernel, fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s, P, Q, out, span);
 }
 
 }  // namespace cbtbe

@@ -355,6 +355,7 @@ __global__ void __launch_bounds__(kWarpThreads, gather_min_blocks<VPL, WEIGHTED,
     fwd_gather_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q, void* out,
                       int cls) {
     __shared__ EndSlot slots[kWarpThreads / 32][32];
+    begin_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t cb = Q.class_chunk_base[cls];
     const int64_t ce = min64(Q.class_chunk_base[cls + 1], Q.max_chunks);
@@ -374,6 +375,7 @@ template <int DT, bool WEIGHTED>
 __global__ void __launch_bounds__(kWarpThreads, CB_WALK_MIN_BLOCKS_MIXED)
     fwd_gather_mixed_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q, void* out) {
     __shared__ EndSlot slots[kWarpThreads / 32][32];
+    begin_kernel();
     const int lane = threadIdx.x & 31;
     EndSlot* mine = slots[threadIdx.x >> 5];
     const int64_t ce = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(kWarpThreads, CB_WALK_MIN_BLOCKS_MIXED)
 template <auto Kernel, class... Args>
 static void launch_gather(int64_t chunk_bound, int num_sms, cudaStream_t s, const Args&... args) {
     static const int cap = resident_blocks(Kernel, kWarpThreads);
-    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(args...);
+    launch(Kernel, warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s, args...);
 }
 
 // Row layouts compiled for: one vector per lane with 1 to 32 rows per step, or

@@ -12,6 +12,7 @@
 namespace cbtbe {
 
 __global__ void validate_offsets_kernel(Problem P) {
+    begin_kernel();
     const int64_t nb = static_cast<int64_t>(P.T) * P.B;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k <= nb;
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(1024) plan_tables_kernel(const __grid_constant
                                                            const __grid_constant__ Plan Q,
                                                            const __grid_constant__ TilePlan S) {
     __shared__ int64_t sh[33];
+    begin_kernel();
     plan_tables(P, Q, S.tile_len, Q.table_pos, Q.ord_chunk_base, S.table_first_tile, sh);
 }
 
@@ -158,6 +160,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
                                                       const __grid_constant__ TilePlan S) {
     __shared__ int64_t sh_pos[kPlanTables + 1], sh_ord[kPlanTables + 1], sh_tile[kPlanTables + 1];
     __shared__ int64_t sh[33];
+    begin_kernel();
     const bool own = P.T <= kPlanTables;
     const int64_t* pos = own ? sh_pos : Q.table_pos;
     const int64_t* ord = own ? sh_ord : Q.ord_chunk_base;
@@ -227,17 +230,18 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
 void launch_validate_offsets(const Problem& P, int num_sms, cudaStream_t s) {
     const int64_t nb = static_cast<int64_t>(P.T) * P.B + 1;
     const int blocks = static_cast<int>(min64((nb + 255) / 256, int64_t(num_sms) * 8));
-    validate_offsets_kernel<<<max(blocks, 1), 256, 0, s>>>(P);
+    launch(validate_offsets_kernel, max(blocks, 1), 256, 0, s, P);
 }
 
 void launch_plan(const Problem& P, const Plan& Q, const TilePlan* S, int64_t chunk_bound, int num_sms, cudaStream_t s) {
     const TilePlan none{};
-    if (P.T > kPlanTables) plan_tables_kernel<<<1, 1024, 0, s>>>(P, Q, S ? *S : none);
+    if (P.T > kPlanTables) launch(plan_tables_kernel, 1, 1024, 0, s, P, Q, S ? *S : none);
     const int64_t cap = static_cast<int64_t>(num_sms) * 6;
     if (chunk_bound <= cap * 32)
-        plan_kernel<8><<<static_cast<unsigned>((chunk_bound + 31) / 32), 256, 0, s>>>(P, Q, S ? *S : none);
+        launch(plan_kernel<8>, static_cast<unsigned>((chunk_bound + 31) / 32), 256, 0, s, P, Q, S ? *S : none);
     else
-        plan_kernel<1><<<static_cast<unsigned>(min64((chunk_bound + 255) / 256, cap)), 256, 0, s>>>(P, Q, S ? *S : none);
+        launch(plan_kernel<1>, static_cast<unsigned>(min64((chunk_bound + 255) / 256, cap)), 256, 0, s, P, Q,
+               S ? *S : none);
 }
 int plan_launches(const Problem& P) { return P.T > kPlanTables ? 2 : 1; }
 

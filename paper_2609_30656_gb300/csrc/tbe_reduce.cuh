@@ -457,6 +457,7 @@ template <int GO, int VPL, bool PACKED, int GC, bool APPLY>
 __global__ void __launch_bounds__(kWarpThreads, reduce_min_blocks<VPL, APPLY>())
     bwd_reduce_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q,
                       const __grid_constant__ BwdOut O, const void* grad_out, int cls) {
+    begin_kernel();
     if (*O.cap_fail) return;
     const int lane = threadIdx.x & 31;
     const int64_t cb = Q.class_chunk_base[cls];
@@ -474,6 +475,7 @@ template <int GO, bool PACKED, bool APPLY>
 __global__ void __launch_bounds__(kWarpThreads, CB_REDUCE_MIN_BLOCKS)
     bwd_reduce_mixed_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q,
                             const __grid_constant__ BwdOut O, const void* grad_out) {
+    begin_kernel();
     if (*O.cap_fail) return;
     const int lane = threadIdx.x & 31;
     const int64_t ce = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
@@ -498,7 +500,7 @@ __global__ void __launch_bounds__(kWarpThreads, CB_REDUCE_MIN_BLOCKS)
 template <auto Kernel, class... Args>
 static void launch_reduce_grid(int64_t chunk_bound, int num_sms, cudaStream_t s, const Args&... args) {
     static const int cap = resident_blocks(Kernel, kWarpThreads);
-    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(args...);
+    launch(Kernel, warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s, args...);
 }
 
 // cls < 0: all classes, in one launch.

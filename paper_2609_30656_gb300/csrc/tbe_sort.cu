@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) onesweep_kernel(SortPass S) {
     __shared__ int64_t sh_scan[33];
     __shared__ uint32_t sh_tile;
     __shared__ int sh_abort;
+    begin_kernel();
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) {
@@ -313,6 +314,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) onesweep_kernel(SortPass S) {
 #endif
 __global__ void __launch_bounds__(kSortThreads, CB_COUNT_MIN_BLOCKS) radix_count_kernel(const SortPass S) {
     __shared__ uint32_t sh[kRadix];
+    begin_kernel();
     const int64_t tile = blockIdx.x;
     if (tile >= *S.num_tiles) return;  // the grid is an upper bound on the tiles
     const int tid = threadIdx.x;
@@ -351,6 +353,7 @@ __global__ void __launch_bounds__(kScanDigits * kScanParts) radix_slots_kernel(c
     __shared__ uint32_t sh_part[kScanParts][kScanDigits];
     __shared__ uint32_t sh_start[kRadix];
     __shared__ int64_t sh_scan[33];
+    begin_kernel();
     const int groups = kRadix / kScanDigits;
     const int t = blockIdx.x / groups, tid = threadIdx.x;
     const int lane = tid & (kScanDigits - 1), part = tid / kScanDigits;
@@ -418,6 +421,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1024 / NT) radix_scatter_k
     __shared__ int32_t sh_goff[kRadix];                    // global destination - local index
     __shared__ int64_t sh_scan[33];
 
+    begin_kernel();
     const int64_t tile = blockIdx.x;
     if (tile >= *S.num_tiles) return;  // the grid is an upper bound on the tiles
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -501,6 +505,7 @@ __global__ void __launch_bounds__(256) sort_hist_kernel(const uint32_t* keys, co
                                                         const TableDev* tables, int passes,
                                                         uint32_t* hist) {
     __shared__ uint32_t sh[4 * kRadix];
+    begin_kernel();
     const int64_t nt = *num_tiles;
     const int64_t per = (nt + gridDim.x - 1) / gridDim.x;
     const int64_t lo = static_cast<int64_t>(blockIdx.x) * per, hi = min64(lo + per, nt);
@@ -547,6 +552,7 @@ __global__ void __launch_bounds__(256) sort_hist_kernel(const uint32_t* keys, co
 __global__ void sort_base_kernel(const uint32_t* hist, const int64_t* table_pos, int passes,
                                  uint32_t* base) {
     __shared__ int64_t sh[33];
+    begin_kernel();
     const int t = blockIdx.x, d = threadIdx.x;
     for (int p = 0; p < passes; ++p) {
         const int64_t i = (static_cast<int64_t>(t) * passes + p) * kRadix + d;
@@ -560,12 +566,12 @@ void launch_sort_hist(const uint32_t* keys, const Chunk* tiles, const int64_t* n
                       int64_t tile_bound, const TableDev* tables, int passes, uint32_t* hist,
                       int num_sms, cudaStream_t s) {
     const int grid = static_cast<int>(max64(1, min64(tile_bound, static_cast<int64_t>(num_sms) * 4)));
-    sort_hist_kernel<<<grid, 256, 0, s>>>(keys, tiles, num_tiles, tables, passes, hist);
+    launch(sort_hist_kernel, grid, 256, 0, s, keys, tiles, num_tiles, tables, passes, hist);
 }
 
 void launch_sort_bases(const uint32_t* hist, const int64_t* table_pos, int T, int passes,
                        uint32_t* base, cudaStream_t s) {
-    sort_base_kernel<<<T, kRadix, 0, s>>>(hist, table_pos, passes, base);
+    launch(sort_base_kernel, T, kRadix, 0, s, hist, table_pos, passes, base);
 }
 
 constexpr int kSortDynSmem = 2 * kSortTile * sizeof(uint32_t);  // 32 KB
@@ -577,7 +583,7 @@ void launch_scatter(const SortPass& S, unsigned grid, cudaStream_t s) {
                                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                         kSortDynSmem) == cudaSuccess;
     (void)configured;
-    radix_scatter_kernel<kScatterThreads, FEW><<<grid, kScatterThreads, kSortDynSmem, s>>>(S);
+    launch(radix_scatter_kernel<kScatterThreads, FEW>, grid, kScatterThreads, kSortDynSmem, s, S);
 }
 
 void launch_radix_pass(const SortPass& S, int64_t tile_bound, cudaStream_t s) {
@@ -586,8 +592,8 @@ void launch_radix_pass(const SortPass& S, int64_t tile_bound, cudaStream_t s) {
         launch_scatter<true>(S, grid, s);
         return;
     }
-    radix_count_kernel<<<grid, kSortThreads, 0, s>>>(S);
-    radix_slots_kernel<<<static_cast<unsigned>(S.T) * (kRadix / kScanDigits), kScanDigits * kScanParts, 0, s>>>(S);
+    launch(radix_count_kernel, grid, kSortThreads, 0, s, S);
+    launch(radix_slots_kernel, static_cast<unsigned>(S.T) * (kRadix / kScanDigits), kScanDigits * kScanParts, 0, s, S);
     launch_scatter<false>(S, grid, s);
 }
 
@@ -599,7 +605,7 @@ void launch_onesweep(const SortPass& S, int64_t tile_bound, cudaStream_t s) {
         cudaFuncSetAttribute(onesweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortDynSmem);
         configured = true;
     }
-    onesweep_kernel<<<static_cast<unsigned>(max64(tile_bound, 1)), kSortThreads, kSortDynSmem, s>>>(S);
+    launch(onesweep_kernel, static_cast<unsigned>(max64(tile_bound, 1)), kSortThreads, kSortDynSmem, s, S);
 }
 
 }  // namespace cbtbe

@@ -151,6 +151,7 @@ template <int DT, int VPL, int G>
 __global__ void __launch_bounds__(kWarpThreads, VPL == 4 ? 2 : 4)
     weight_grad_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q, const void* grad_out,
                        float* grad_w, int cls) {
+    begin_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t cb = Q.class_chunk_base[cls];
     const int64_t ce = min64(Q.class_chunk_base[cls + 1], Q.max_chunks);
@@ -166,7 +167,7 @@ template <auto Kernel>
 void launch_one(const Problem& P, const Plan& Q, const void* go, float* gw, int cls, int64_t chunk_bound,
                 int num_sms, cudaStream_t s) {
     static const int cap = resident_blocks(Kernel, kWarpThreads);
-    Kernel<<<warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s>>>(P, Q, go, gw, cls);
+    launch(Kernel, warp_grid(chunk_bound, static_cast<int64_t>(cap) * num_sms), kWarpThreads, 0, s, P, Q, go, gw, cls);
 }
 
 template <int DT>
