@@ -98,10 +98,10 @@ struct Gather {
     // finished bags are a prefix of the window. At the chunk end, the bag that
     // runs past it is listed too, as a piece (`runs_on`).
     __device__ __forceinline__ uint32_t scan(int32_t base, int32_t bend) {
+        runs_on = false;
         __syncwarp();  // every lane is done reading the previous batch's list
         uint32_t mask = 0;
         int nend = 0;
-        runs_on = false;
         for (;;) {
             int32_t my_beg = __shfl_up_sync(kFull, my_end, 1);
             if (lane == 0) my_beg = s_cur;

@@ -411,9 +411,9 @@ struct EndSlot {
                   // piece of one that runs past the chunk end
 };
 
-// A cache line requested into L2 ahead of its load, without a register.
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+// A cache line requested into L1 ahead of its load, without a register.
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
 // ---------------------------------------------------------------- fix-up

@@ -169,8 +169,8 @@ void launch_onesweep(const SortPass& S, int64_t tile_bound, cudaStream_t s);
 // Up to this many tiles, a pass is one kernel: every scatter tile sums the counts
 // of its table's tiles itself, and counts the next pass's digits as it writes.
 // (A pass's three kernels become one, 6 fewer in a backward of three passes: sort of
-// 330 K lookups in 8 tables 58 -> 40 us, of 106 K in 26 tables 52 -> 35 us, of 1.3 M
-// in 16 tables 76 -> 74 us. A tile reads its table's counts, so the reads grow with
+// 330 K lookups in 8 tables 58 -> 31 us, of 106 K in 26 tables 52 -> 27 us, of 1.3 M
+// in 16 tables 76 -> 56 us. A tile reads its table's counts, so the reads grow with
 // the square of a table's tiles: 512 tiles of one table read 268 MB from L2.)
 constexpr int64_t kFewSortTiles = 512;
 // One reduce-then-scan pass: tile counts and slots, unless few tiles; scatter.

@@ -105,9 +105,10 @@ __device__ __forceinline__ float step_scale(const BwdOut& O, int t, int64_t row,
 
 // The fused step on one complete run's row, as the walker holds it: lane v of
 // each row group owns vectors v + 32k; every group holds the same totals and
-// group 0 writes. Out of line: the walker ends runs in many places, and a copy
-// of the step in each of them overflowed the instruction cache (measured on
-// cfg5: fused SGD step 36.8 ms inline, 21 ms out of line).
+// group 0 writes. `m0`: the row's previous Adagrad state (in lane 0). The row's
+// loads are issued before the scale is summed. Out of line: the walker ends runs
+// in many places, and a copy of the step in each of them overflowed the
+// instruction cache.
 template <int N>
 struct GradRow {
     float4 v[N];   // four gradient columns each
@@ -116,18 +117,27 @@ struct GradRow {
 
 template <int N>
 __device__ __noinline__ void apply_row(const Problem& P, const BwdOut& O, int t, uint32_t row,
-                                       const GradRow<N> g, bool group0) {
+                                       const GradRow<N> g, float m0, bool group0) {
     const TableDev& td = P.tables[t];
-    float sq = 0.f;
+    char* p = row_ptr(td, row);
+    const int dtype = td.dtype;
+    uint4 x[N];
 #pragma unroll
     for (int k = 0; k < N; ++k)
-        if (group0 && g.col[k] >= 0)
-            sq += sq4(g.v[k]);
-    const float scale = step_scale(O, t, row, td.dim, sq);
+        if (group0 && g.col[k] >= 0) x[k] = load_cols(p, dtype, g.col[k]);
+    float scale = O.lr;
+    if (O.apply == kApplyAdagrad) {
+        float sq = 0.f;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (group0 && g.col[k] >= 0)
+                sq += sq4(g.v[k]);
+        scale = adagrad_scale(O, O.state[t] + row, td.dim, sq, m0);
+    }
     if (!group0) return;
 #pragma unroll
     for (int k = 0; k < N; ++k)
-        if (g.col[k] >= 0) step_cols(td, row, g.col[k], g.v[k], scale);
+        if (g.col[k] >= 0) store_step(p, dtype, g.col[k], x[k], g.v[k], scale);
 }
 
 // ---------------------------------------------------------------- (5) reduce
@@ -150,7 +160,8 @@ template <int GO, int VPL, bool PACKED, bool APPLY, int G>
 struct Reduce {
     static constexpr int E = Storage<GO>::kElems;  // grad_out storage: fp32, or fp16 / bf16 (mixed precision)
     static constexpr int V = 32 / G;
-    static constexpr int kWide = (APPLY ? CB_REDUCE_APPLY_ROWS : CB_REDUCE_ROWS) / VPL;
+    static constexpr int kRows = APPLY ? CB_REDUCE_APPLY_ROWS : CB_REDUCE_ROWS;
+    static constexpr int kWide = kRows > VPL ? kRows / VPL : 1;
     static constexpr int UG = kWide < V ? kWide : V;  // row steps per load group
     static constexpr int kItems = UG * G;
     static constexpr uint32_t kItemMask = kItems == 32 ? kFull : (1u << (kItems & 31)) - 1u;
@@ -204,8 +215,8 @@ struct Reduce {
             for (int x = 0; x < E; ++x) tot[0][x] += __shfl_xor_sync(kFull, tot[0][x], off);
         zero();
     }
-    // The end of a run (its key: `key`).
-    __device__ __forceinline__ void flush(uint32_t key) {
+    // The end of a run (fused step: its key, and its row's previous state).
+    __device__ __forceinline__ void flush(uint32_t key, float m0) {
         float tot[VPL][E];
         total(tot);
         if constexpr (APPLY) {
@@ -220,7 +231,7 @@ struct Reduce {
                                                            tot[k][4 * x + 3]);
                         r.col[k * (E / 4) + x] = col < dim ? col : -1;
                     }
-                apply_row<VPL * E / 4>(P, O, t, key - static_cast<uint32_t>(P.tables[t].key_base), r, g == 0);
+                apply_row<VPL * E / 4>(P, O, t, key - static_cast<uint32_t>(P.tables[t].key_base), r, m0, g == 0);
                 return;
             }
             if (g == 0) store(dst, tot);
@@ -297,6 +308,7 @@ struct Reduce {
             if (nb == 0) break;
             const bool end = have && cur.key != cur.after;
             const uint32_t mask = __ballot_sync(kFull, end);
+            float state = 0.f;
             if constexpr (!APPLY) {
                 // Row id (row_base_t + r = key - t) and float offset of a run.
                 if (end) {
@@ -307,11 +319,12 @@ struct Reduce {
                 out_row += __popc(mask);
                 out_float += static_cast<int64_t>(__popc(mask)) * dim;
             } else if (end) {
-                // The table rows that this batch steps start moving into L2.
-                const char* row = static_cast<const char*>(td.data) +
-                                  static_cast<uint64_t>(cur.key - static_cast<uint32_t>(td.key_base)) * td.row_vecs * 16u;
-                for (int x = 0; x < td.row_vecs * 16; x += 128) prefetch_l2(row + x);
-                if (O.apply == kApplyAdagrad) prefetch_l2(O.state[t] + (cur.key - static_cast<uint32_t>(td.key_base)));
+                // The table rows that this batch steps start moving into L1, and
+                // their states into the lanes that hold the runs' ends.
+                const uint32_t r = cur.key - static_cast<uint32_t>(td.key_base);
+                const char* row = static_cast<const char*>(td.data) + static_cast<uint64_t>(r) * td.row_vecs * 16u;
+                for (int x = 0; x < td.row_vecs * 16; x += 128) prefetch_l1(row + x);
+                if (O.apply == kApplyAdagrad) state = O.state[t][r];
             }
             // Row of the bag within the table's (kept inside it whatever the payload).
             const uint32_t my_a = have ? min(pk.x - bag_lo, static_cast<uint32_t>(P.B - 1)) : 0u;
@@ -373,7 +386,8 @@ struct Reduce {
                     }
                     if constexpr (G == 1) {
                         add(buf[u], wt[u]);
-                        flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u) : 0u);
+                        flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u) : 0u,
+                              APPLY ? __shfl_sync(kFull, state, i0 + u) : 0.f);
                     } else {
                         // Runs end after item i0 + u*G + p for each set bit p; this lane
                         // group's item (p index g) belongs to the first of them with g <= p.
@@ -384,7 +398,8 @@ struct Reduce {
                                 add(buf[u], wt[u]);
                                 added = true;
                             }
-                            flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u * G + p) : 0u);
+                            flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u * G + p) : 0u,
+                                  APPLY ? __shfl_sync(kFull, state, i0 + u * G + p) : 0.f);
                             mu &= mu - 1;
                         } while (mu);
                         if (!added) add(buf[u], wt[u]);
@@ -422,7 +437,8 @@ struct Reduce {
 // of 41 M lookups on skewed indices (fp32 grad_out) / 12 M uniform (bf16) / 26 M
 // weighted uniform (fp32), us: 8 rows at 3 blocks 1140 / 952 / 2675; 4 at 4 1133 /
 // 1167 (4 at 5) / 2925; 12 at 2 1331 / - / 2613; 16 at 2 - / 1017 / -. Fused Adagrad
-// step of 1.3 M lookups: 4 rows at 4 blocks 256, 2 at 5 262, 4 at 3 277.
+// step of 1.3 M lookups: 4 rows at 4 blocks 206, 4 at 3 213, 2 at 4 210, 2 at 5 220
+// (244 with a row's state and stored values loaded only where its run ends).
 template <int VPL, bool APPLY>
 constexpr int reduce_min_blocks() {
     return VPL == 4 ? 2 : (APPLY && VPL == 1 ? CB_REDUCE_APPLY_MIN_BLOCKS : CB_REDUCE_MIN_BLOCKS);

@@ -171,14 +171,24 @@ __device__ __forceinline__ void write_tile(const SortPass& S, int tile_count, ui
 #pragma unroll
         for (int j = 0; j < kHalf; ++j) {
             const int i = tid + (h * kHalf + j) * NT;
-            if (i < tile_count && dst[j] >= 0 && dst[j] < S.n) {
+            const bool in = i < tile_count && dst[j] >= 0 && dst[j] < S.n;
+            if (in) {
                 S.keys_out[dst[j]] = key[j];
                 S.vals_out[dst[j]] = val[j];
-                if (NEXT) {
-                    const int32_t tile = min(first + max(dst[j] - p0, 0) / kSortTile, last);
-                    atomicAdd(S.next_digits + static_cast<int64_t>(tile) * kRadix +
-                                  sort_digit(key[j], key_base, S.shift + 8), 1u);
-                }
+            }
+            if (NEXT) {
+                // The lanes that count where the first counting lane does are added by
+                // it together: a hot row's pairs are neighbours here, and would queue
+                // up at one counter.
+                const int32_t tile = min(first + max(dst[j] - p0, 0) / kSortTile, last);
+                const uint32_t at = static_cast<uint32_t>(tile) * kRadix + sort_digit(key[j], key_base, S.shift + 8);
+                const uint32_t active = __ballot_sync(kFull, in);
+                const int lead = active ? __ffs(active) - 1 : 0;
+                const uint32_t lead_at = __shfl_sync(kFull, at, lead);
+                const uint32_t same = __ballot_sync(kFull, in && at == lead_at);
+                const int lane = tid & 31;
+                if (in && (lane == lead || !((same >> lane) & 1u)))
+                    atomicAdd(S.next_digits + at, lane == lead ? static_cast<uint32_t>(__popc(same)) : 1u);
             }
         }
     }
