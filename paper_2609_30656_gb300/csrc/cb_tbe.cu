@@ -725,12 +725,15 @@ cb_status cb_tbe_forward(cb_tbe* h, int32_t batch, const void* indices, int64_t 
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
     Plan Q = make_plan(h, w, false, n);
     const int64_t bound = chunk_count_bound(n, Q.chunk_len, h->T);
-    launch_plan(P, Q, nullptr, bound, h->num_sms, stream);
-    h->launches += plan_launches(P);
+    const bool planned = h->fwd_one_dtype && fwd_plans_itself(bound, h->T, h->num_sms);
+    if (!planned) {
+        launch_plan(P, Q, nullptr, bound, h->num_sms, stream);
+        h->launches += plan_launches(P);
+    }
     record(h, h->ev_fwd[1], stream);
     nv.phase("fwd.gather");
-    if (h->fwd_one_dtype && h->fwd_classes.size() > 1) {
-        launch_fwd_gather(P, Q, out, -1, h->fwd_classes[0].dtype, 0, 0, bound, h->num_sms, stream);
+    if (planned || (h->fwd_one_dtype && h->fwd_classes.size() > 1)) {
+        launch_fwd_gather(P, Q, out, planned ? kPlanned : kAllClasses, h->fwd_classes[0].dtype, 0, 0, bound, h->num_sms, stream);
         h->launches += 1;
     } else {
         for (size_t c = 0; c < h->fwd_classes.size(); ++c) {

@@ -210,11 +210,12 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         Q.carry_tail = reinterpret_cast<float*>(base + o_tl);
         Q.tail_owner = reinterpret_cast<int64_t*>(base + o_to);
         Q.chunk_next = reinterpret_cast<uint32_t*>(base + o_nx);  // zeroed by the plan
-        launch_plan(P, Q, nullptr, max_chunks, num_sms, stream);
         bool one_dtype = true;
         for (const Cls& c : classes) one_dtype = one_dtype && c.dtype == classes[0].dtype;
-        if (one_dtype && classes.size() > 1)
-            launch_fwd_gather(P, Q, out, -1, classes[0].dtype, 0, 0, max_chunks, num_sms, stream);
+        const bool planned = one_dtype && fwd_plans_itself(max_chunks, T, num_sms);
+        if (!planned) launch_plan(P, Q, nullptr, max_chunks, num_sms, stream);
+        if (planned || (one_dtype && classes.size() > 1))
+            launch_fwd_gather(P, Q, out, planned ? kPlanned : kAllClasses, classes[0].dtype, 0, 0, max_chunks, num_sms, stream);
         else for (size_t c = 0; c < classes.size(); ++c)
             launch_fwd_gather(P, Q, out, static_cast<int>(c), classes[c].dtype, classes[c].vpl,
                               classes[c].gc, max_chunks, num_sms, stream);

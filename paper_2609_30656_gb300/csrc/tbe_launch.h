@@ -154,6 +154,15 @@ void launch_plan(const Problem& P, const Plan& Q, const TilePlan* S, int64_t chu
                  cudaStream_t s);
 int plan_launches(const Problem& P);  // kernels launch_plan enqueues
 
+constexpr int kAllClasses = -1, kPlanned = -2;  // `cls` of launch_fwd_gather
+// Whether a forward of one storage type runs without a plan kernel.
+#ifndef CB_PLANNED_BLOCKS
+#define CB_PLANNED_BLOCKS 2
+#endif
+constexpr int kPlannedBlocks = CB_PLANNED_BLOCKS;  // resident blocks per SM of the kernel that does
+inline bool fwd_plans_itself(int64_t chunk_bound, int64_t T, int num_sms) {
+    return T <= 1024 && chunk_bound <= static_cast<int64_t>(num_sms) * 8 * kPlannedBlocks;
+}
 void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int dtype, int vpl,
                        int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);
 void launch_fwd_fixup(const Problem& P, const Plan& Q, void* out, int64_t chunk_bound,
