@@ -80,17 +80,20 @@ __device__ __forceinline__ float sq4(float4 g) {
     return fmaf(g.w, g.w, fmaf(g.z, g.z, fmaf(g.y, g.y, __fmul_rn(g.x, g.x))));
 }
 
-// The Adagrad scale from the summed squares and the row's previous state `m0`
-// (meaningful in lane 0); lane 0 stores the new state.
-__device__ __forceinline__ float adagrad_scale(const BwdOut& O, float* st, int dim, float sq, float m0) {
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) sq += __shfl_xor_sync(kFull, sq, off);
+// The Adagrad scale of a row spread over V lanes (a warp's lane groups may hold
+// different rows) from each lane's share `sq` of the summed squares and the row's
+// previous state `m0` (meaningful in the group's first lane, which stores the new
+// state if `active`).
+__device__ __forceinline__ float adagrad_scale(const BwdOut& O, float* st, int dim, float sq, float m0, int V,
+                                               bool active) {
+    const int lane = threadIdx.x & 31;
+    for (int off = V / 2; off >= 1; off >>= 1) sq += __shfl_xor_sync(kFull, sq, off);
     float m = 0.f;
-    if ((threadIdx.x & 31) == 0) {
+    if ((lane & (V - 1)) == 0 && active) {
         m = m0 + sq / static_cast<float>(dim);
         *st = m;
     }
-    m = __shfl_sync(kFull, m, 0);
+    m = __shfl_sync(kFull, m, lane & ~(V - 1));
     return O.lr / (sqrtf(m) + O.eps);
 }
 
@@ -100,41 +103,41 @@ __device__ __forceinline__ float adagrad_scale(const BwdOut& O, float* st, int d
 __device__ __forceinline__ float step_scale(const BwdOut& O, int t, int64_t row, int dim, float sq) {
     if (O.apply != kApplyAdagrad) return O.lr;
     float* st = O.state[t] + row;
-    return adagrad_scale(O, st, dim, sq, (threadIdx.x & 31) == 0 ? *st : 0.f);
+    return adagrad_scale(O, st, dim, sq, (threadIdx.x & 31) == 0 ? *st : 0.f, 32, true);
 }
 
-// The fused step on one complete run's row, as the walker holds it: lane v of
-// each row group owns vectors v + 32k; every group holds the same totals and
-// group 0 writes. `m0`: the row's previous Adagrad state (in lane 0). The row's
-// loads are issued before the scale is summed. Out of line: the walker ends runs
-// in many places, and a copy of the step in each of them overflowed the
-// instruction cache.
+// The fused step on complete runs' rows, as the walker holds them: a lane group of
+// V lanes holds one row, lane v of it vectors v + 32k. Either every group holds the
+// same totals and one of them is `active`, or each holds a run of its own. `m0`:
+// the row's previous Adagrad state (in the group's first lane). The row's loads are
+// issued before the scale is summed. Out of line: the walker ends runs in many
+// places, and a copy of the step in each of them overflowed the instruction cache.
 template <int N>
 struct GradRow {
     float4 v[N];   // four gradient columns each
     int col[N];    // first column of each, or -1 past the row
 };
 
-template <int N>
+template <int N, int V>
 __device__ __noinline__ void apply_row(const Problem& P, const BwdOut& O, int t, uint32_t row,
-                                       const GradRow<N> g, float m0, bool group0) {
+                                       const GradRow<N> g, float m0, bool active) {
     const TableDev& td = P.tables[t];
     char* p = row_ptr(td, row);
     const int dtype = td.dtype;
     uint4 x[N];
 #pragma unroll
     for (int k = 0; k < N; ++k)
-        if (group0 && g.col[k] >= 0) x[k] = load_cols(p, dtype, g.col[k]);
+        if (active && g.col[k] >= 0) x[k] = load_cols(p, dtype, g.col[k]);
     float scale = O.lr;
     if (O.apply == kApplyAdagrad) {
         float sq = 0.f;
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            if (group0 && g.col[k] >= 0)
+            if (g.col[k] >= 0)
                 sq += sq4(g.v[k]);
-        scale = adagrad_scale(O, O.state[t] + row, td.dim, sq, m0);
+        scale = adagrad_scale(O, O.state[t] + row, td.dim, sq, m0, V, active);
     }
-    if (!group0) return;
+    if (!active) return;
 #pragma unroll
     for (int k = 0; k < N; ++k)
         if (g.col[k] >= 0) store_step(p, dtype, g.col[k], x[k], g.v[k], scale);
@@ -215,23 +218,27 @@ struct Reduce {
             for (int x = 0; x < E; ++x) tot[0][x] += __shfl_xor_sync(kFull, tot[0][x], off);
         zero();
     }
+    // The fused step of the run that this lane's group holds.
+    __device__ __forceinline__ void step(uint32_t key, const float (&tot)[VPL][E], float m0, bool active) const {
+        GradRow<VPL * E / 4> r;
+#pragma unroll
+        for (int k = 0; k < VPL; ++k)
+#pragma unroll
+            for (int x = 0; x < E / 4; ++x) {
+                const int col = (v + 32 * k) * E + 4 * x;
+                r.v[k * (E / 4) + x] = make_float4(tot[k][4 * x], tot[k][4 * x + 1], tot[k][4 * x + 2],
+                                                   tot[k][4 * x + 3]);
+                r.col[k * (E / 4) + x] = col < dim ? col : -1;
+            }
+        apply_row<VPL * E / 4, V>(P, O, t, key - static_cast<uint32_t>(P.tables[t].key_base), r, m0, active);
+    }
     // The end of a run (fused step: its key, and its row's previous state).
     __device__ __forceinline__ void flush(uint32_t key, float m0) {
         float tot[VPL][E];
         total(tot);
         if constexpr (APPLY) {
             if (!at_head) {
-                GradRow<VPL * E / 4> r;
-#pragma unroll
-                for (int k = 0; k < VPL; ++k)
-#pragma unroll
-                    for (int x = 0; x < E / 4; ++x) {
-                        const int col = (v + 32 * k) * E + 4 * x;
-                        r.v[k * (E / 4) + x] = make_float4(tot[k][4 * x], tot[k][4 * x + 1], tot[k][4 * x + 2],
-                                                           tot[k][4 * x + 3]);
-                        r.col[k * (E / 4) + x] = col < dim ? col : -1;
-                    }
-                apply_row<VPL * E / 4>(P, O, t, key - static_cast<uint32_t>(P.tables[t].key_base), r, m0, g == 0);
+                step(key, tot, m0, g == 0);
                 return;
             }
             if (g == 0) store(dst, tot);
@@ -372,17 +379,20 @@ struct Reduce {
                         if (G == 1 || g < left) add(buf[u], wt[u]);
                         continue;
                     }
-                    if constexpr (!APPLY) {
-                        if (((singles >> (i0 + u * G)) & kStepMask) == kStepMask) {
-                            // Every lane group's item is a whole run: each stores its own.
-                            float one[VPL][E] = {};
+                    if (((singles >> (i0 + u * G)) & kStepMask) == kStepMask) {
+                        // Every lane group's item is a whole run: each stores (or steps) its own.
+                        float one[VPL][E] = {};
 #pragma unroll
-                            for (int k = 0; k < VPL; ++k) accumulate<GO, PACKED>(one[k], buf[u][k], wt[u]);
+                        for (int k = 0; k < VPL; ++k) accumulate<GO, PACKED>(one[k], buf[u][k], wt[u]);
+                        if constexpr (APPLY) {
+                            step(__shfl_sync(kFull, cur.key, i0 + u * G + g), one,
+                                 __shfl_sync(kFull, state, i0 + u * G + g), true);
+                        } else {
                             store(dst + g * dim, one);
                             dst += G * dim;
                             next += G * dim;
-                            continue;
                         }
+                        continue;
                     }
                     if constexpr (G == 1) {
                         add(buf[u], wt[u]);
@@ -438,7 +448,8 @@ struct Reduce {
 // weighted uniform (fp32), us: 8 rows at 3 blocks 1140 / 952 / 2675; 4 at 4 1133 /
 // 1167 (4 at 5) / 2925; 12 at 2 1331 / - / 2613; 16 at 2 - / 1017 / -. Fused Adagrad
 // step of 1.3 M lookups: 4 rows at 4 blocks 206, 4 at 3 213, 2 at 4 210, 2 at 5 220
-// (244 with a row's state and stored values loaded only where its run ends).
+// (244 with a row's state and stored values loaded only where its run ends; 178, as
+// now, with the runs of one lookup stepped by a lane group each).
 template <int VPL, bool APPLY>
 constexpr int reduce_min_blocks() {
     return VPL == 4 ? 2 : (APPLY && VPL == 1 ? CB_REDUCE_APPLY_MIN_BLOCKS : CB_REDUCE_MIN_BLOCKS);
@@ -486,9 +497,13 @@ __global__ void __launch_bounds__(kWarpThreads, reduce_min_blocks<VPL, APPLY>())
     }
 }
 
-// Tables of several row layouts in one launch, as in the forward.
+// Tables of several row layouts in one launch, as in the forward. 2 blocks per SM:
+// at 3 the compiler spills 100 to 160 bytes (26 M weighted lookups, dims 64/128/256:
+// 2672 us at 3, 2581 at 2; fused Adagrad of 490 K: 162 and 129; fp32 gradients of
+// 330 K: 47 and 48).
+constexpr int kMixedReduceBlocks = 2;
 template <int GO, bool PACKED, bool APPLY>
-__global__ void __launch_bounds__(kWarpThreads, CB_REDUCE_MIN_BLOCKS)
+__global__ void __launch_bounds__(kWarpThreads, kMixedReduceBlocks)
     bwd_reduce_mixed_kernel(const __grid_constant__ Problem P, const __grid_constant__ Plan Q,
                             const __grid_constant__ BwdOut O, const void* grad_out) {
     begin_kernel();
