@@ -171,7 +171,7 @@ typedef struct {
  *   G[row_base_t + r] = sum over lookups i of table t with indices[i] == r of
  *                       w_i * s_b(i) * grad_out[b(i), Doff_t : Doff_t + D_t]
  * computed by an on-device stable radix sort of (row id, lookup) pairs, a
- * run-length pass and a segmented reduction. Arguments as in cb_tbe_forward;
+ * pass over the runs and a segmented reduction. Arguments as in cb_tbe_forward;
  * grad_out is device [B, sum of dims] of the output type (fp32 unless mixed
  * precision), 16-byte aligned; gradients are fp32. When U > cap_rows
  * or F > cap_floats nothing is written to unique_ids / grad_offsets / grads,

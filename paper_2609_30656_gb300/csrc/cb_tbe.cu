@@ -86,6 +86,7 @@ struct Workspace {
     int64_t digit_words = 0;  // zeroed before the sort, from zero_digits on
     uint32_t* zero_digits = nullptr;
     uint32_t* heads = nullptr;
+    uint32_t* head_bits = nullptr;
     int64_t* run_count = nullptr;
     int64_t* out_first = nullptr;
     int64_t* float_base = nullptr;
@@ -204,6 +205,8 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
         ws.digit_words = few ? tile_words * h->passes : table_words;
     }
     ws.heads = static_cast<uint32_t*>(take(sizeof(uint32_t) * max_chunks));
+    // (the reduce loads up to two words past a cell's)
+    ws.head_bits = static_cast<uint32_t*>(take(sizeof(uint32_t) * (max_chunks + 1) * (kMaxChunk / 32)));
     ws.run_count = static_cast<int64_t*>(take(sizeof(int64_t) * T));
     ws.out_first = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
     ws.float_base = static_cast<int64_t*>(take(sizeof(int64_t) * (T + 1)));
@@ -451,6 +454,7 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     O.vals_sorted = w.vals[cur];
     O.packed = packed ? w.packed : nullptr;
     O.heads = w.heads;
+    O.head_bits = w.head_bits;
     O.run_count = w.run_count;
     O.out_first = w.out_first;
     O.float_base = w.float_base;

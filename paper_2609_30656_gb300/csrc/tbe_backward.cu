@@ -105,9 +105,9 @@ __global__ void __launch_bounds__(kWarpThreads) keygen_kernel(Problem P, Plan Q,
 
 // A table's sorted positions are cut into cells of chunk_len positions (the last
 // one shorter), numbered as its chunks. Per cell: how many runs begin in it (low
-// half) and where the first does (high half; kNoHead: none). One warp per cell,
-// all of its keys loaded before any is compared. The keys are read once more by
-// the reduce; nothing else about the runs is stored.
+// half) and where the first does (high half; kNoHead: none), and a flag per
+// position for the reduce. One warp per cell, all of its keys loaded before any is
+// compared.
 constexpr uint32_t kNoHead = 0xffffu;
 
 __global__ void __launch_bounds__(kWarpThreads) bwd_heads_kernel(const __grid_constant__ Problem P,
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_heads_kernel(const __grid_co
 #pragma unroll
     for (int i = 0; i < kBatches; ++i) k[i] = 32 * i + lane < len ? __ldg(keys + 32 * i + lane) : 0u;
     uint32_t before = x0 > p0 ? __ldg(keys - 1) : ~k[0];  // (lane 0) a table's first key starts a run
-    uint32_t count = 0, first = kNoHead;
+    uint32_t count = 0, first = kNoHead, flags = 0;
 #pragma unroll
     for (int i = 0; i < kBatches; ++i) {
         if (32 * i >= len) break;  // warp-uniform
@@ -137,8 +137,10 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_heads_kernel(const __grid_co
         const uint32_t b = __ballot_sync(kFull, 32 * i + lane < len && k[i] != prev);
         count += __popc(b);
         if (first == kNoHead && b) first = 32 * i + __ffs(b) - 1;
+        if (lane == i) flags = b;
         before = __shfl_sync(kFull, k[i], 31);
     }
+    if (lane < (len + 31) / 32) O.head_bits[j * (Q.chunk_len / 32) + lane] = flags;
     if (lane == 0) O.heads[j] = count | (first << 16);
 }
 

@@ -1,5 +1,5 @@
-// tbe_internal.cuh -- device-side structures and the segmented gather-reduce
-// walker shared by the forward gather-pool and the backward segmented reduce.
+// tbe_internal.cuh -- device-side structures and steps shared by the forward
+// gather-pool and the backward segmented reduce.
 //
 // Both hot loops have the same shape: a run of items in position order, grouped
 // into consecutive segments (forward: the bags of a table, delimited by the
@@ -8,8 +8,8 @@
 // coefficient-weighted sum of its rows. The pooled bag of the paper's sparse_arch
 // (Sec. IV.A.2) and its de-duplicated adjoint are both this shape.
 //
-// Work is cut into fixed-size chunks of item positions, so every warp does the
-// same amount of gathering whatever the bag-length distribution (heavy tails,
+// Work is cut into chunks of item positions of one size per call, so every warp
+// does the same amount of gathering whatever the bag-length distribution (heavy tails,
 // empty bags, one-hot bags). A segment that straddles chunk boundaries is summed
 // piecewise; its pieces are combined afterwards in chunk order, in fp64, by a
 // fix-up pass, so results are deterministic.
@@ -42,7 +42,7 @@ constexpr int kWarpThreads = 256;  // block size of the warp-per-chunk kernels
 #define CB_REDUCE_ROWS 8
 #endif
 #ifndef CB_REDUCE_APPLY_MIN_BLOCKS
-#define CB_REDUCE_APPLY_MIN_BLOCKS 4
+#define CB_REDUCE_APPLY_MIN_BLOCKS 3
 #endif
 #ifndef CB_REDUCE_APPLY_ROWS
 #define CB_REDUCE_APPLY_ROWS 4

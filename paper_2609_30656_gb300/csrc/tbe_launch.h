@@ -111,6 +111,7 @@ struct BwdOut {
     const uint32_t* vals_sorted; // [n]
     const uint2* packed;         // [n] or null
     uint32_t* heads;             // [max_chunks] runs begun per chunk cell, and the first's offset
+    uint32_t* head_bits;         // [max_chunks][chunk_len / 32] a flag per position: a run begins
     int64_t* run_count;          // [T] runs of real rows per table
     int64_t* out_first;          // [T + 1] first output row of each table (runs of
                                  // out-of-range lookups are not output)

@@ -2,7 +2,8 @@
 // ids; per run the coefficient-weighted sum of the gathered grad_out slices,
 // the de-duplicated adjoint of the pooled bag of Sec. IV.A.2), and the
 // optimizer step that can be fused where a run's sum ends. Included by
-// tbe_backward.cu (gradient output) and tbe_backward_apply.cu (fused step).
+// tbe_reduce_{f32,f16,bf16}.cu and tbe_backward_apply.cu (instantiations) and by
+// tbe_backward.cu (the step of split runs and of the second pass).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -146,17 +147,19 @@ __device__ __noinline__ void apply_row(const Problem& P, const BwdOut& O, int t,
 // ---------------------------------------------------------------- (5) reduce
 
 // One chunk of a table's sorted positions, walked by one warp in batches of 32.
-// A run ends where the next sorted key differs: one ballot over the keys of a
-// batch gives the mask of its ends, and runs are output in order, so the row a
-// run goes to follows from the chunk's first run by counting. (Taking the ends
+// The kernel that counted the run heads left a flag per position: 32 of them are
+// the mask of a batch's run ends, and runs are output in order, so the row a run
+// goes to follows from the chunk's first run by counting; only the keys at run
+// ends are read. (Taking the ends
 // from a list of run starts took a window scan per batch, a list in shared
 // memory, and two more passes over the keys to write the run keys and starts: on
 // the three batches below 1102 / 1294 / 3162 us, and 65 / 65 / 120 us more for the
-// runs.)
+// runs; comparing the keys here, read twice, 1133 / 946 / 2585; with the flags 1116 /
+// 946 / 2543.)
 // The end of a run is a few instructions, repeated in every step of a load
 // group: add, store, advance the output row. Runs cut by the chunk's edges leave
 // their piece in the carry rows. Out-of-range lookups sort to the table's end
-// under its spare key; the walk stops there.
+// under its spare key: their run is summed (of some row of the table) and dropped.
 // APPLY: the optimizer step is fused where a run's sum ends (compiled as its
 // own kernels, so the gradient-writing reduce carries none of its code).
 template <int GO, int VPL, bool PACKED, bool APPLY, int G>
@@ -169,7 +172,7 @@ struct Reduce {
     static constexpr int kItems = UG * G;
     static constexpr uint32_t kItemMask = kItems == 32 ? kFull : (1u << (kItems & 31)) - 1u;
     static constexpr uint32_t kStepMask = G == 32 ? kFull : (1u << (G & 31)) - 1u;
-    static constexpr bool kFastBatch = VPL == 1 && !APPLY;
+    static constexpr bool kFastBatch = VPL == 1;
     static_assert(VPL == 1 || G == 1, "several vectors per lane: one row per step");
 
     const Problem& P;  // kernel parameters: read in place, not held in registers
@@ -251,27 +254,20 @@ struct Reduce {
         }
     }
 
-    struct Item {
-        uint32_t key, after, val;
-    };
     struct Walk {
         const uint32_t* keys;
         const uint32_t* vals;
+        const uint32_t* bits;    // head flags from the chunk's cell on
+        int32_t shift;           // of the chunk's first position within them
         int32_t len, table_end;  // items of the chunk; end of the table, relative to the chunk
     };
-    __device__ __forceinline__ Item fetch(const Walk& w, int32_t q) const {
-        Item x{0u, 0u, 0u};
-        if (q < w.len) {
-            x.key = __ldg(w.keys + q);
-            x.after = q + 1 < w.table_end ? __ldg(w.keys + q + 1) : ~x.key;
-            x.val = load_stream(w.vals + q);
-        }
-        return x;
+    __device__ __forceinline__ uint32_t fetch(const Walk& w, int32_t q) const {
+        return q < w.len ? load_stream(w.vals + q) : 0u;
     }
     // (bag, bits of w_i * s_b) of a sorted item.
-    __device__ __forceinline__ uint2 coefficient(const Item& x) const {
-        if constexpr (PACKED) return __ldg(O.packed + min(x.val, static_cast<uint32_t>(P.n - 1)));
-        return make_uint2(x.val, 0u);
+    __device__ __forceinline__ uint2 coefficient(uint32_t val) const {
+        if constexpr (PACKED) return __ldg(O.packed + min(val, static_cast<uint32_t>(P.n - 1)));
+        return make_uint2(val, 0u);
     }
 
     // grad_out rows of this table's bags start at `rows`, `stride` bytes apart.
@@ -295,13 +291,18 @@ struct Reduce {
             else next += dim;
         }
         bool open = piece;  // the run of the next item began before it
-        Item nxt = fetch(w, lane), far{};
+        uint32_t nxt = fetch(w, lane), far = 0u;
         uint2 npk = coefficient(nxt);
         if (PACKED) far = fetch(w, 32 + lane);
+        // Item q ends its run where the flag of position q + 1 is set: a batch's mask
+        // is 32 flags from bit shift + 1 + base on, across two words.
+        const uint32_t* word = w.bits + ((w.shift + 1) >> 5);
+        const int skew = (w.shift + 1) & 31;
+        uint32_t lo = __ldg(word), hi = __ldg(word + 1);
+        bool dead_run = false;  // the open run is the one of out-of-range lookups
         for (int32_t base = 0; base < w.len; base += 32) {
             // The next batch's items are loaded while this batch's rows are in
             // flight (with coefficients, which depend on them: one batch further).
-            const Item cur = nxt;
             const uint2 pk = npk;
             if (PACKED) {
                 nxt = far;
@@ -310,17 +311,26 @@ struct Reduce {
                 nxt = fetch(w, base + 32 + lane);
             }
             npk = coefficient(nxt);
-            const bool have = base + lane < w.len && cur.key != dead;
-            const int nb = __popc(__ballot_sync(kFull, have));  // dead lookups are the last
-            if (nb == 0) break;
-            const bool end = have && cur.key != cur.after;
-            const uint32_t mask = __ballot_sync(kFull, end);
+            const int nb = min(32, w.len - base);
+            uint32_t mask = __funnelshift_r(lo, hi, skew) & (nb == 32 ? kFull : (1u << nb) - 1u);
+            lo = hi;
+            hi = __ldg(word + (base >> 5) + 2);
+            if (base + nb == w.table_end) {
+                // The table's last run ends here. It is not output if it holds the
+                // out-of-range lookups.
+                dead_run = __ldg(w.keys + w.table_end - 1) == dead;
+                const uint32_t last = 1u << (nb - 1);
+                mask = dead_run ? mask & ~last : mask | last;
+            }
+            const bool have = lane < nb;
+            const bool end = (mask >> lane) & 1u;
+            const uint32_t key = end ? __ldg(w.keys + base + lane) : 0u;
             float state = 0.f;
             if constexpr (!APPLY) {
                 // Row id (row_base_t + r = key - t) and float offset of a run.
                 if (end) {
                     const int r = __popc(mask & ((1u << lane) - 1u));
-                    O.unique_ids[out_row + r] = static_cast<int64_t>(cur.key) - t;
+                    O.unique_ids[out_row + r] = static_cast<int64_t>(key) - t;
                     O.grad_offsets[out_row + r] = out_float + static_cast<int64_t>(r) * dim;
                 }
                 out_row += __popc(mask);
@@ -328,7 +338,7 @@ struct Reduce {
             } else if (end) {
                 // The table rows that this batch steps start moving into L1, and
                 // their states into the lanes that hold the runs' ends.
-                const uint32_t r = cur.key - static_cast<uint32_t>(td.key_base);
+                const uint32_t r = key - static_cast<uint32_t>(td.key_base);
                 const char* row = static_cast<const char*>(td.data) + static_cast<uint64_t>(r) * td.row_vecs * 16u;
                 for (int x = 0; x < td.row_vecs * 16; x += 128) prefetch_l1(row + x);
                 if (O.apply == kApplyAdagrad) state = O.state[t][r];
@@ -385,7 +395,7 @@ struct Reduce {
 #pragma unroll
                         for (int k = 0; k < VPL; ++k) accumulate<GO, PACKED>(one[k], buf[u][k], wt[u]);
                         if constexpr (APPLY) {
-                            step(__shfl_sync(kFull, cur.key, i0 + u * G + g), one,
+                            step(__shfl_sync(kFull, key, i0 + u * G + g), one,
                                  __shfl_sync(kFull, state, i0 + u * G + g), true);
                         } else {
                             store(dst + g * dim, one);
@@ -396,7 +406,7 @@ struct Reduce {
                     }
                     if constexpr (G == 1) {
                         add(buf[u], wt[u]);
-                        flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u) : 0u,
+                        flush(APPLY ? __shfl_sync(kFull, key, i0 + u) : 0u,
                               APPLY ? __shfl_sync(kFull, state, i0 + u) : 0.f);
                     } else {
                         // Runs end after item i0 + u*G + p for each set bit p; this lane
@@ -408,7 +418,7 @@ struct Reduce {
                                 add(buf[u], wt[u]);
                                 added = true;
                             }
-                            flush(APPLY ? __shfl_sync(kFull, cur.key, i0 + u * G + p) : 0u,
+                            flush(APPLY ? __shfl_sync(kFull, key, i0 + u * G + p) : 0u,
                                   APPLY ? __shfl_sync(kFull, state, i0 + u * G + p) : 0.f);
                             mu &= mu - 1;
                         } while (mu);
@@ -427,7 +437,7 @@ struct Reduce {
                     ain[k][x] = 0.f;
                 }
         }
-        if (open) {
+        if (open && !dead_run && __ldg(w.keys + w.len - 1) != dead) {
             // The run goes on in the next chunk: this chunk's piece of it.
             float tot[VPL][E];
             total(tot);
@@ -442,14 +452,15 @@ struct Reduce {
 
 // Resident blocks per SM the reduce is compiled for: 3 with 8 rows in flight per
 // lane, so that slices that come from DRAM or a distant L2 have the bytes in
-// flight; 4 with 4 rows when the optimizer step is fused, which carries the table
+// flight; 3 with 4 rows when the optimizer step is fused, which carries the table
 // row too; 2 for four vectors per lane (16 columns in two levels). Measured, reduce
 // of 41 M lookups on skewed indices (fp32 grad_out) / 12 M uniform (bf16) / 26 M
 // weighted uniform (fp32), us: 8 rows at 3 blocks 1140 / 952 / 2675; 4 at 4 1133 /
 // 1167 (4 at 5) / 2925; 12 at 2 1331 / - / 2613; 16 at 2 - / 1017 / -. Fused Adagrad
-// step of 1.3 M lookups: 4 rows at 4 blocks 206, 4 at 3 213, 2 at 4 210, 2 at 5 220
-// (244 with a row's state and stored values loaded only where its run ends; 178, as
-// now, with the runs of one lookup stepped by a lane group each).
+// step of 1.3 M lookups (Adagrad) / 41 M (SGD): 4 rows at 3 blocks 174 / 1928, 4 at 4
+// 180 / 2051; without the batches with no run end unrolled - / 2154; without the runs
+// of one lookup stepped by a lane group each 223 / 2140; with a row's state and
+// stored values loaded only where its run ends 244 / -.
 template <int VPL, bool APPLY>
 constexpr int reduce_min_blocks() {
     return VPL == 4 ? 2 : (APPLY && VPL == 1 ? CB_REDUCE_APPLY_MIN_BLOCKS : CB_REDUCE_MIN_BLOCKS);
@@ -471,6 +482,9 @@ __device__ __forceinline__ void reduce_chunk(const Problem& P, const Plan& Q, co
     typename Reduce<GO, VPL, PACKED, APPLY, GC>::Walk w;
     w.keys = O.keys_sorted + ch.k0;
     w.vals = O.vals_sorted + ch.k0;
+    // the chunk's cell: positions [x0, x0 + chunk_len) of the table
+    w.bits = O.head_bits + j * (Q.chunk_len / 32);
+    w.shift = static_cast<int32_t>(ch.k0 - Q.table_pos[t] - (j - Q.table_chunk[t]) * Q.chunk_len);
     w.len = static_cast<int32_t>(ch.len & 0x7fffffffu);
     w.table_end = static_cast<int32_t>(Q.table_pos[t + 1] - ch.k0);
     if (lane == 0) Q.tail_owner[j] = -1;

@@ -30,9 +30,9 @@ def _problem(vectors, dtype, seed, batch=150):
     for _ in dims:
         x = torch.ones(batch, dtype=torch.int64)
         x[40:90] = torch.randint(0, 6, (50,), generator=g)
-        x[90:140] = torch.randint(0, 60, (50,), generator=g)
-        x[95] = 700
-        x[140:] = 0  # trailing empty bags
+        x[90:-10] = torch.randint(0, 60, (max(batch - 100, 0),), generator=g)
+        x[95 if batch > 110 else 5] = 700
+        x[-10:] = 0  # trailing empty bags
         lens.append(x)
     lens = torch.cat(lens)
     off = torch.zeros(lens.numel() + 1, dtype=torch.int64)
@@ -80,3 +80,21 @@ def test_out_of_range_lookups_among_single_lookup_bags(vectors):
     rows, dims = table_meta(tables)
     res, sc = backward_reference(rows, dims, batch, kept_ind, kept_off, go, None, False)
     assert_backward_matches(g, res, sc, what="backward")
+
+
+@pytest.mark.parametrize("batch", [100, 1200])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+def test_few_and_many_chunks_integer_tables(batch, weighted, dtype):
+    # A forward with few chunks places them in the gather itself, one with many has a
+    # kernel for it; integer values make every sum exact.
+    import numpy as np
+    from paper_2609_30656_gb300.tbe import TBE
+    tables, ind, off, w, _, _ = _problem(VECTORS, dtype, 77, batch=batch)
+    g = torch.Generator().manual_seed(78)
+    tables = [torch.randint(-8, 9, t.shape, generator=g).to(dtype) for t in tables]
+    w = torch.randint(0, 3, (ind.numel(),), generator=g).float() if weighted else None
+    m = TBE([t.to(DEV) for t in tables], validate=True)
+    y = m.forward(ind.to(DEV), off.to(DEV), None if w is None else w.to(DEV))
+    ref, _ = forward_reference(tables, batch, ind, off, w, False)
+    np.testing.assert_array_equal(y.cpu().double().numpy(), ref)
