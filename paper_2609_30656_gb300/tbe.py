@@ -305,12 +305,17 @@ class TBE:
         off = self._dev(offsets, self.index_dtype)
         w = self._dev(per_sample_weights, torch.float32)
         go = self._dev(grad_out, self.out_dtype)
-        T = len(self.dims)
-        sizes = torch.empty(T + 3, dtype=torch.int64, device=self.device)
-        probe = SparseGrad(sizes, sizes[2:], sizes, None, sizes[:1], sizes[1:2])
+        # The counts and the per-table offsets keep one small buffer through both calls
+        # (each writes them whole, so nothing clears it first).
+        dev = self.device
+        sizes = torch.empty(len(self.dims) + 3, dtype=torch.int64, device=dev)
+        num_unique, num_floats, table_offsets = sizes[:1], sizes[1:2], sizes[2:]
+        probe = SparseGrad(sizes, table_offsets, sizes, None, num_unique, num_floats)
         self.backward_into(probe, ind, off, go, w)
         U, F = sizes[:2].tolist()
-        g = self.alloc_grad(U, F)
+        g = SparseGrad(torch.empty(max(U, 1), dtype=torch.int64, device=dev), table_offsets,
+                       torch.empty(U + 1, dtype=torch.int64, device=dev),
+                       torch.empty(max(F, 4), dtype=torch.float32, device=dev), num_unique, num_floats)
         return self._backward_into(self._lib.cb_tbe_backward_finish, g, ind, off, go, w)
 
     def backward_apply(self, indices, offsets, grad_out, per_sample_weights=None,
