@@ -58,7 +58,10 @@ __device__ __forceinline__ int owner_of(const int64_t* base, int n, int64_t j) {
 
 // The first bag of table t starting at or after x0, and after x1 (lower bounds
 // over the table's offsets, in [t*B, (t+1)*B + 1]), found together by W lanes that
-// probe W points of both ranges at a time.
+// probe W points of both ranges at a time. A range narrows to the points around the
+// first one that is not below x, whatever the later ones say, so that for decreasing
+// offsets too the bag found starts at or after x and the one before it before x:
+// a boundary that moves (see below) never leaves its table.
 template <int W>
 __device__ __forceinline__ void bag_lower_bounds(const Problem& P, int t, int64_t x0, int64_t x1, int lane, int64_t& r0,
                                                  int64_t& r1) {
@@ -75,7 +78,8 @@ __device__ __forceinline__ void bag_lower_bounds(const Problem& P, int t, int64_
             const uint32_t step = max(1u, __umulhi(R, 0xffffffffu / (W + 1)));
             const uint32_t m = a[s] + (R <= W ? sub : (sub + 1) * step);
             const bool below = m < b[s] && load_index(P.offsets, blo + m, P.is32) < x[s];
-            const uint32_t cnt = __popc((__ballot_sync(kFull, below) >> shift) & (kFull >> (32 - W)));
+            const uint32_t all = (__ballot_sync(kFull, below) >> shift) & (kFull >> (32 - W));
+            const uint32_t cnt = __clz(__brev(~all));  // points below x before the first that is not
             if (R <= W) {
                 a[s] += cnt;
                 b[s] = a[s];
