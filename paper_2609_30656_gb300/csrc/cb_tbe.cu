@@ -266,8 +266,11 @@ Plan make_plan(const cb_tbe* h, const Workspace& w, bool bwd, int64_t n) {
     Plan Q;
     Q.chunk_len = static_cast<int32_t>(chunk_len);
     // Chunk boundaries move to the end of the bag they cut unless it is longer
-    // than this, so only heavy bags are split.
-    Q.snap_cap = static_cast<int32_t>(4 * chunk_len);
+    // than this, so only heavy bags are split. Not in the backward: key generation
+    // has no sums to split, and its chunks must hold every position of a table
+    // exactly once whatever the offsets (moved boundaries can pass each other where
+    // offsets decrease), because it counts the sort's digits as it goes.
+    Q.snap_cap = bwd ? 0 : static_cast<int32_t>(4 * chunk_len);
     Q.num_classes = static_cast<int32_t>(bwd ? h->bwd_classes.size() : h->fwd_classes.size());
     Q.class_tables = bwd ? h->d_bwd_class_tables : h->d_fwd_class_tables;
     Q.class_table_start = bwd ? h->d_bwd_class_start : h->d_fwd_class_start;
