@@ -30,8 +30,9 @@
  *   - A handle is not thread-safe. Calls on one handle must be ordered on one
  *     stream, or the caller synchronises between streams.
  *   - Host-side argument errors return at once, before any GPU work.
- *     Device-side checks (index range; offsets under CB_VALIDATE) never trap:
- *     they set a sticky error word. Under CB_VALIDATE the call synchronises
+ *     Device-side checks (index range; a table whose offsets begin before an
+ *     earlier table's; every offset under CB_VALIDATE) never trap: they set a
+ *     sticky error word, and the call goes on inside its buffers. Under CB_VALIDATE the call synchronises
  *     `stream` and returns that error; otherwise cb_tbe_get_error() returns
  *     it later. An out-of-range index (negative, or >= rows_t) contributes
  *     nothing: not to the pooled output, not to any gradient row (its row is not

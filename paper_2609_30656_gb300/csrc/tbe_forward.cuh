@@ -439,10 +439,7 @@ __global__ void __launch_bounds__(kWarpThreads, kPlannedBlocks)
     plan_tables(P, Q, 0, pos, ord, nullptr, sh);
     const int lane = threadIdx.x & 31;
     const int64_t total = min64(ord[P.T], Q.max_chunks);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        Q.class_chunk_base[Q.num_classes] = total;  // for the fix-up
-        if (ord[P.T] > Q.max_chunks) set_error(P.error, CB_ERR_BAD_OFFSETS);
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) Q.class_chunk_base[Q.num_classes] = total;  // for the fix-up
     for (int64_t j = warp_id_global(); j < total; j += warps_in_grid()) {
         const Chunk ch = plan_chunk<32>(P, Q, pos, ord, j, lane);
         if (lane == 0) Q.chunks[j] = ch;

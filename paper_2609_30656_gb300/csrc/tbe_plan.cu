@@ -72,10 +72,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
             Q.class_chunk_base[c] = min64(ord[Q.class_table_start[c]], Q.max_chunks);
             Q.chunk_next[c] = 0;
         }
-        if (tid == 0) {
-            if (ord[P.T] > Q.max_chunks) set_error(P.error, CB_ERR_BAD_OFFSETS);
-            if (S.tile_len > 0) *S.num_tiles = min64(tile_ord[P.T], S.max_tiles);
-        }
+        if (tid == 0 && S.tile_len > 0) *S.num_tiles = min64(tile_ord[P.T], S.max_tiles);
     }
     const int64_t first = static_cast<int64_t>(blockIdx.x) * blockDim.x + tid;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;

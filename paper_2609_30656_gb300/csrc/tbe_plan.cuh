@@ -10,15 +10,30 @@ constexpr int kPlanTables = 1024;  // tables that a block plans in shared memory
 
 // The tables' part of the plan, by one block: item ranges (pos), and the first
 // chunk of every table in class order (ord) and, with tiles, the first sort tile in
-// table order (tile_ord), each with the total at the end.
+// table order (tile_ord), each with the total at the end. Positions never decrease:
+// a table whose first offset lies before an earlier table's (malformed, reported
+// here) begins where that one does. So the tables' ranges do not overlap, and all
+// of them together have no more chunks and tiles than n lookups can (room for the
+// workspace, and in the backward a key in a table's range is one of its rows).
 __device__ __forceinline__ void plan_tables(const Problem& P, const Plan& Q, int64_t tile_len, int64_t* pos, int64_t* ord,
                                             int64_t* tile_ord, int64_t* sh) {
     const int tid = threadIdx.x;
+    auto start = [&](int t) {
+        return min64(max64(load_index(P.offsets, static_cast<int64_t>(t) * P.B, P.is32), 0), P.n);
+    };
+    bool falls = false;
     for (int t = tid; t <= P.T; t += blockDim.x) {
-        const int64_t x = load_index(P.offsets, static_cast<int64_t>(t) * P.B, P.is32);
-        pos[t] = min64(max64(x, 0), P.n);
+        const int64_t x = start(t);
+        pos[t] = x;
+        if (t < P.T) falls = falls || start(t + 1) < x;
     }
-    __syncthreads();
+    if (__syncthreads_or(falls)) {
+        if (tid == 0) {
+            set_error(P.error, CB_ERR_BAD_OFFSETS);
+            for (int t = 1; t <= P.T; ++t) pos[t] = max64(pos[t], pos[t - 1]);
+        }
+        __syncthreads();
+    }
     int64_t chunks = 0, tiles = 0;
     for (int i0 = 0; i0 < P.T; i0 += blockDim.x) {
         const int i = i0 + tid;

@@ -106,3 +106,64 @@ def test_backward_sorts_every_lookup_once(dims, B, max_len, seed):
     assert torch.equal(g.grads[:f0], want.grads[:f0]) and torch.equal(g.grads[f1:F], want.grads[f1:F])
     m.backward_apply(ind, bad, go, w, optimizer="adagrad", state=[s for _, s in state])
     assert _marks_stand(bufs) and _marks_stand(state)
+
+
+# First offsets of the tables as parts of n, and the ranges that the call gives them
+# (no range begins before an earlier one's); inner offsets between each pair.
+BOUNDARIES = [
+    ((0.0, 1.0, 0.0, 1.0), (0.0, 1.0, 1.0, 1.0)),
+    ((0.0, 0.1, 0.05, 0.2), (0.0, 0.1, 0.1, 0.2)),
+    ((0.0, 0.5, -3.0, 0.6), (0.0, 0.5, 0.5, 0.6)),
+    ((0.0, 2.0, 0.2, 0.0), (0.0, 1.0, 1.0, 1.0)),
+]
+
+
+# n around the edges of the chunk lengths (32, 64, .., 512) and of the few-tile sort
+@pytest.mark.parametrize("n,copies", [(50, 1), (5000, 1), (640_000, 1), (2_200_000, 1), (10_500_000, 1),
+                                      (50, 400), (5000, 400), (640_000, 400)])
+@pytest.mark.parametrize("parts,used", BOUNDARIES)
+def test_tables_that_begin_before_an_earlier_one(parts, used, copies, n):
+    """Three tables, or three and 1197 that begin as the third does (more than one block plans)."""
+    from paper_2609_30656_gb300.tbe import CB_ERR_BAD_OFFSETS, SparseGrad, TBE
+    rows, D, B = 1000, 4, 16
+    T = 3 * copies
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    _, ind = _padded(torch.randint(0, rows, (n,), generator=gen, device=DEV), -7)
+    starts = [int(p * n) for p in parts]
+    starts = starts[:3] + [starts[2]] * (T - 3) + starts[3:]
+    off = torch.cat([torch.linspace(a, b, B + 1, dtype=torch.float64, device=DEV)[:B].long()
+                     for a, b in zip(starts, starts[1:])] + [torch.tensor(starts[-1:], device=DEV)])
+    held = [int(p * n) for p in used]
+    held = held[:3] + [held[2]] * (T - 3) + held[3:]
+    w = torch.rand(n, generator=gen, device=DEV)
+    go = torch.randn(B, T * D, generator=gen, device=DEV)
+    bufs = _padded_tables([torch.randn(rows, D) for _ in range(T)])
+    tables = [t for _, t in bufs]
+    m = TBE(tables)
+    ids = torch.cat([ind[a:b].unique() + t * rows for t, (a, b) in enumerate(zip(held, held[1:]))])
+    U = ids.numel()
+    (bi, unique_ids), (bo, grad_offsets), (bg, grads) = (_padded(torch.zeros(k, dtype=d), -7) for k, d in (
+        (U, torch.int64), (U + 1, torch.int64), (U * D, torch.float32)))
+    sizes = torch.zeros(2, dtype=torch.int64, device=DEV)
+    g = SparseGrad(unique_ids, torch.zeros(T + 1, dtype=torch.int64, device=DEV), grad_offsets, grads, sizes[:1], sizes[1:])
+    m.backward_into(g, ind, off, go, w)
+    assert m.get_error() == CB_ERR_BAD_OFFSETS
+    assert torch.equal(m.sorted_payloads(n)[:held[-1]].sort().values, torch.arange(held[-1], device=DEV))
+    assert (g.num_unique, g.num_floats) == (U, U * D)
+    assert torch.equal(unique_ids, ids) and torch.equal(grad_offsets, torch.arange(U + 1, device=DEV) * D)
+    for b in (bi, bo, bg):
+        assert bool((b[:PAD] == -7).all()) and bool((b[-PAD:] == -7).all())
+    m.backward_apply(ind, off, go, w, optimizer="sgd", lr=0.5)
+    assert m.get_error() == CB_ERR_BAD_OFFSETS and _marks_stand(bufs)
+    buf, gw = _padded(torch.empty(n), MARK)
+    m.weight_grad(ind, off, go, out=gw)
+    assert m.get_error() == CB_ERR_BAD_OFFSETS
+    assert bool((buf[:PAD] == MARK).all()) and bool((buf[-PAD:] == MARK).all())
+    m.forward(ind, off, w)
+    assert m.get_error() == CB_ERR_BAD_OFFSETS
+    # the handle is as good as new
+    good = (torch.arange(T * B + 1, device=DEV) * n) // (T * B)
+    other = TBE(tables)
+    assert torch.equal(m.forward(ind, good, w), other.forward(ind, good, w))
+    x, y = m.backward(ind, good, go, w), other.backward(ind, good, go, w)
+    assert torch.equal(x.unique_ids, y.unique_ids) and torch.equal(x.grads, y.grads) and m.get_error() == 0
