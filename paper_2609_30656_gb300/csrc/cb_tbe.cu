@@ -81,6 +81,7 @@ struct Workspace {
     uint32_t* digit_base = nullptr;
     uint32_t* status = nullptr;
     uint32_t* tile_counters = nullptr;
+    uint32_t* timed_out = nullptr;
     uint32_t* tile_digits = nullptr;
     uint32_t* table_digits = nullptr;
     int64_t digit_words = 0;  // zeroed before the sort, from zero_digits on
@@ -185,12 +186,14 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
         const size_t hist_words = static_cast<size_t>(T) * h->passes * 256;
         ws.digit_base = static_cast<uint32_t*>(take(sizeof(uint32_t) * hist_words));
         ws.status_bytes = sizeof(uint32_t) * static_cast<size_t>(h->passes) * ws.sort_tiles * 256;
-        // histograms, status words and tile counters are adjacent: one memset clears them
+        // histograms, status words, tile counters (4) and the timeout word are adjacent:
+        // one memset clears them
         ws.hist = static_cast<uint32_t*>(take(sizeof(uint32_t) * hist_words + ws.status_bytes +
-                                              sizeof(uint32_t) * 4));
+                                              sizeof(uint32_t) * 5));
         ws.status = base ? ws.hist + hist_words : nullptr;
         ws.tile_counters = base ? ws.status + static_cast<size_t>(h->passes) * ws.sort_tiles * 256 : nullptr;
-        ws.status_bytes += sizeof(uint32_t) * hist_words + sizeof(uint32_t) * 4;  // cleared from `hist` on
+        ws.timed_out = base ? ws.tile_counters + 4 : nullptr;
+        ws.status_bytes += sizeof(uint32_t) * hist_words + sizeof(uint32_t) * 5;  // cleared from `hist` on
     } else {
         // Few tiles: every pass's counts, zeroed at the start. Many: one pass's
         // counts, and every pass's counts per table, zeroed at the start. Calls of
@@ -377,6 +380,7 @@ cb_status sort_lookups(cb_tbe* h, const Problem& P, const Workspace& w, const Pl
             S.never_set = h->d_never_set;
             S.force_timeout = (h->flags & CB_DEBUG_FORCE_LOOKBACK_TIMEOUT) && p == 0;
             S.error = h->d_error;
+            S.timed_out = w.timed_out;
             S.timeout_ns = kLookbackTimeoutNs;
             launch_onesweep(S, w.sp_max_tiles, stream);
             h->launches += 1;
@@ -463,6 +467,7 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     O.float_base = w.float_base;
     O.tables_done = h->d_tables_done;
     O.cap_fail = w.cap_fail;
+    O.timed_out = w.timed_out;
     if (a) {
         // No caller buffers: the sizes land in the workspace's own words.
         O.unique_ids = nullptr;

@@ -173,8 +173,13 @@ __device__ __forceinline__ void output_ranges(const Problem& P, const BwdOut& O,
         *O.num_unique = rows;
         *O.num_floats = floats;
         int fail = 0;
-        // After a timed-out sort pass the sorted order is not trustworthy.
-        if (*reinterpret_cast<volatile int*>(P.error) == CB_ERR_TIMEOUT) fail = 1;
+        // After a timed-out sort pass the sorted order is not trustworthy. (The error
+        // word does not tell: it keeps an earlier error of the call, and the host may
+        // have read and cleared it between a size query and its finish.)
+        if (O.timed_out && *O.timed_out) {
+            set_error(P.error, CB_ERR_TIMEOUT);
+            fail = 1;
+        }
         if (O.grads && (rows > O.cap_rows || floats > O.cap_floats)) {
             set_error(P.error, CB_ERR_CAPACITY);
             fail = 1;

@@ -36,6 +36,7 @@ struct SortPass {
     const uint32_t* never_set;   // a zero word no kernel writes (timeout test hook)
     int force_timeout;
     int* error;
+    uint32_t* timed_out;         // set when a wait ran out (zeroed before the first pass)
     uint64_t timeout_ns;
 };
 
@@ -118,6 +119,7 @@ struct BwdOut {
     int64_t* float_base;         // [T + 1]
     uint32_t* tables_done;       // zero between calls
     int* cap_fail;
+    const uint32_t* timed_out;   // a sort pass gave up on its wait (null: no pass waits)
     // caller's buffers
     int64_t* unique_ids;
     int64_t* table_offsets;

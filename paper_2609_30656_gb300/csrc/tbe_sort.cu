@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) onesweep_kernel(SortPass S) {
                 }
                 if (timed_out) {
                     set_error(S.error, CB_ERR_TIMEOUT);
+                    *S.timed_out = 1;
                     atomicExch(&sh_abort, 1);
                     break;
                 }

@@ -66,3 +66,32 @@ def test_finish_needs_the_query_before_it():
     _finish(m, small, ind, off, go, None)
     assert m.get_error() == CB_ERR_CAPACITY
     assert small.num_unique == probe.num_unique
+
+
+@pytest.mark.parametrize("step", ["backward", "finish", "apply"])
+@pytest.mark.parametrize("earlier", [False, True])
+def test_nothing_is_summed_in_an_order_that_timed_out(step, earlier):
+    """Neither an earlier error of the call (an index out of range) nor one that the host
+    read between a query and its finish hides that the sort gave up."""
+    from paper_2609_30656_gb300.tbe import CB_DEBUG_FORCE_LOOKBACK_TIMEOUT, CB_ERR_INDEX_OOB, CB_ERR_TIMEOUT, TBE
+    tables, ind, off, _ = random_problem(36, rows=(1000, 1000, 1000), batch=400, max_len=60)
+    if earlier:
+        ind[0] = -1
+    ind, off = ind.to(DEV), off.to(DEV)
+    go = torch.randn(400, sum(t.shape[1] for t in tables), device=DEV)
+    m = TBE([t.to(DEV) for t in tables], extra_flags=CB_DEBUG_FORCE_LOOKBACK_TIMEOUT)
+    before = [t.clone() for t in m.tables]
+    g = m.alloc_grad(ind.numel(), ind.numel() * 24)
+    for x in (g.unique_ids, g.grads):
+        x.fill_(-7)
+    if step == "apply":
+        m.backward_apply(ind, off, go, optimizer="sgd", lr=1.0)
+        assert all(torch.equal(a, b) for a, b in zip(before, m.tables))
+    elif step == "backward":
+        m.backward_into(g, ind, off, go)
+    else:
+        m.backward_into(m.alloc_grad(0, 0, size_only=True), ind, off, go)
+        assert m.get_error() == (CB_ERR_INDEX_OOB if earlier else CB_ERR_TIMEOUT)
+        _finish(m, g, ind, off, go, None)
+    assert m.get_error() == (CB_ERR_INDEX_OOB if earlier and step != "finish" else CB_ERR_TIMEOUT)
+    assert bool((g.unique_ids == -7).all()) and bool((g.grads == -7).all())
