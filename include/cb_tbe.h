@@ -184,13 +184,13 @@ cb_status cb_tbe_backward(cb_tbe* h, int32_t batch, const void* indices, int64_t
 
 /* Finishes a size query: cb_tbe_backward with g->grads NULL counts U and F and
  * leaves the batch's sorted runs in the handle's workspace; this call, with the
- * same batch (all arguments but g as in that query) and buffers of the sizes it
- * returned, writes the gradient from them, without sorting again. It must follow
- * the query on the handle with no call between them that uses the workspace
- * (forward, backward, weight gradient, reserve). Results, errors and capacity
- * checks as in cb_tbe_backward; CB_ERR_INVALID_ARG when the handle holds no
- * query of this batch size, number of lookups and kind of payload, or
- * g->grads is NULL. */
+ * same batch (all arguments but g and grad_out as in that query, and the buffers
+ * they name unchanged) and buffers of the sizes it returned, writes the gradient
+ * from them, without sorting again. It must follow the query on the handle with
+ * no call between them that uses the workspace (forward, backward, weight
+ * gradient, reserve). Results, errors and capacity checks as in cb_tbe_backward;
+ * CB_ERR_INVALID_ARG when the handle holds no query with these indices, offsets,
+ * weights, sizes and stream that returned CB_OK, or g->grads is NULL. */
 cb_status cb_tbe_backward_finish(cb_tbe* h, int32_t batch, const void* indices, int64_t num_indices,
                                  const void* offsets, const float* per_sample_weights,
                                  const void* grad_out, cb_sparse_grad* g, cudaStream_t stream);

@@ -97,6 +97,19 @@ struct Workspace {
     size_t status_bytes = 0;
 };
 
+// What a call that finishes a size query has to repeat. The addresses are compared
+// and never followed: other buffers are another batch.
+struct Query {
+    int64_t n = 0;
+    int32_t batch = 0;
+    const void *indices = nullptr, *offsets = nullptr, *weights = nullptr;
+    cudaStream_t stream = nullptr;
+    bool operator==(const Query& o) const {
+        return n == o.n && batch == o.batch && indices == o.indices && offsets == o.offsets && weights == o.weights &&
+               stream == o.stream;
+    }
+};
+
 }  // namespace
 
 struct cb_tbe {
@@ -130,11 +143,10 @@ struct cb_tbe {
     void* ws = nullptr;
     size_t ws_bytes = 0;
     cudaStream_t last_stream = nullptr;
-    // A size query whose sorted runs the workspace still holds (n < 0: none):
-    // any call that writes the workspace ends it.
-    int64_t query_n = -1;
-    int32_t query_batch = 0;
-    bool query_packed = false;
+    // A size query whose sorted runs the workspace still holds: any call that writes
+    // the workspace ends it.
+    bool query_held = false;
+    Query query;
     // Sorted payloads of the last backward that reached the sort (workspace).
     const uint32_t* last_sorted = nullptr;
     int64_t last_sorted_n = 0;
@@ -220,7 +232,7 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
 }
 
 cb_status ensure_workspace(cb_tbe* h, int64_t B, int64_t n) {
-    h->query_n = -1;
+    h->query_held = false;
     const size_t need = layout(h, B, n, nullptr, nullptr);
     if (need <= h->ws_bytes) return CB_OK;
     if (h->ws) {
@@ -417,9 +429,8 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
         return CB_ERR_INVALID_ARG;
     if (!current_device_ok(h)) return CB_ERR_INVALID_ARG;
     const bool packed = per_sample_weights != nullptr || h->mode == CB_POOL_MEAN;
-    if (finish && n > 0 && batch > 0 &&
-        (h->query_n != n || h->query_batch != batch || h->query_packed != packed))
-        return CB_ERR_INVALID_ARG;
+    const Query query{n, batch, indices, offsets, per_sample_weights, stream};
+    if (finish && n > 0 && batch > 0 && !(h->query_held && h->query == query)) return CB_ERR_INVALID_ARG;
     h->last_stream = stream;
     h->bwd_timed = false;
     if (!finish) h->last_sorted = nullptr;
@@ -444,7 +455,7 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
         st = ensure_workspace(h, batch, n);
         if (st != CB_OK) return st;
     }
-    h->query_n = -1;
+    h->query_held = false;
     Workspace w;
     layout(h, batch, n, static_cast<char*>(h->ws), &w);
     Plan Q = make_plan(h, w, true, n);
@@ -517,12 +528,10 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
     }
     record(h, h->ev_bwd[4], stream);
     h->bwd_timed = (h->flags & CB_TIMING) != 0;
-    if (!reduce) {
-        h->query_n = n;
-        h->query_batch = batch;
-        h->query_packed = packed;
-    }
-    return finish_call(h, stream);
+    st = finish_call(h, stream);
+    h->query_held = !reduce && st == CB_OK;
+    h->query = query;
+    return st;
 }
 
 bool sparse_grad_ok(const cb_sparse_grad* g) {

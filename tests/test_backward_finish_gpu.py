@@ -95,3 +95,43 @@ def test_nothing_is_summed_in_an_order_that_timed_out(step, earlier):
         _finish(m, g, ind, off, go, None)
     assert m.get_error() == (CB_ERR_INDEX_OOB if earlier and step != "finish" else CB_ERR_TIMEOUT)
     assert bool((g.unique_ids == -7).all()) and bool((g.grads == -7).all())
+
+
+@pytest.mark.parametrize("other", ["indices", "offsets", "weights", "stream"])
+def test_finish_refuses_another_batch_of_the_same_size(other):
+    from paper_2609_30656_gb300.tbe import TBE, CbTbeError
+    tables, ind, off, w = random_problem(7, batch=30, weighted=True)
+    args = {"indices": ind.to(DEV), "offsets": off.to(DEV), "weights": w.to(DEV)}
+    go = torch.randn(30, sum(t.shape[1] for t in tables), device=DEV)
+    m = TBE([t.to(DEV) for t in tables])
+    want = m.backward(args["indices"], args["offsets"], go, args["weights"])
+    g = m.alloc_grad(ind.numel(), ind.numel() * 24)
+    g.grads.fill_(-7)
+    m.backward_into(m.alloc_grad(0, 0, size_only=True), args["indices"], args["offsets"], go, args["weights"])
+    torch.cuda.synchronize()
+    mine = dict(args)
+    stream = torch.cuda.Stream() if other == "stream" else torch.cuda.current_stream()
+    if other != "stream":
+        mine[other] = mine[other].clone()
+    with pytest.raises(CbTbeError), torch.cuda.stream(stream):
+        _finish(m, g, mine["indices"], mine["offsets"], go, mine["weights"])
+    torch.cuda.synchronize()
+    assert bool((g.grads == -7).all())
+    _finish(m, g, args["indices"], args["offsets"], go, args["weights"])  # the query still stands
+    assert torch.equal(g.grads[:want.num_floats], want.grads[:want.num_floats])
+
+
+def test_a_query_that_failed_is_not_finished():
+    from paper_2609_30656_gb300.tbe import CB_ERR_INDEX_OOB, CB_ERR_INVALID_ARG, TBE, CbTbeError
+    tables, ind, off, _ = random_problem(8, batch=30)
+    ind[3] = 1 << 40
+    ind, off = ind.to(DEV), off.to(DEV)
+    go = torch.randn(30, sum(t.shape[1] for t in tables), device=DEV)
+    m = TBE([t.to(DEV) for t in tables], validate=True)
+    g = m.alloc_grad(ind.numel(), ind.numel() * 24)
+    with pytest.raises(CbTbeError) as e:
+        m.backward_into(m.alloc_grad(0, 0, size_only=True), ind, off, go)
+    assert e.value.status == CB_ERR_INDEX_OOB
+    with pytest.raises(CbTbeError) as e:
+        _finish(m, g, ind, off, go, None)
+    assert e.value.status == CB_ERR_INVALID_ARG
