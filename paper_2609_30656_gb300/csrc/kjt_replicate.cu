@@ -51,9 +51,10 @@ template <typename I>
 __global__ void __launch_bounds__(kThreads) replicate_kernel(const Replicate<I> p) {
     __shared__ I starts[kTables + 1];
     begin_kernel();
-    // this block's copies [r0, r1)
-    const int per_part = (p.F + p.parts - 1) / p.parts;
-    const int r0 = blockIdx.y * per_part, r1 = min(r0 + per_part, p.F);
+    // this block's copies [r0, r1), in 64 bits: F may be as large as a 32-bit number gets
+    const int64_t per_part = (static_cast<int64_t>(p.F) + p.parts - 1) / p.parts;
+    const int r0 = static_cast<int>(min64(blockIdx.y * per_part, p.F));
+    const int r1 = static_cast<int>(min64(r0 + per_part, p.F));
     if (static_cast<int>(blockIdx.x) < p.bag_blocks) {
         const int64_t bags = static_cast<int64_t>(p.T) * p.B;
         const int64_t k = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x;

@@ -40,3 +40,16 @@ def test_replicate(T, B, factor, dtype):
     got = tbe.replicate_batch(ind.to(DEV), off.to(DEV), w.to(DEV), T, factor)
     for a, b in zip(got, oracle.replicate_kjt(ind, off, w, T, factor)):
         np.testing.assert_array_equal(a.cpu().numpy(), b)
+
+
+def test_replicate_as_often_as_32_bits_count():
+    from paper_2609_30656_gb300 import tbe
+    F = 2 ** 31 - 1  # one bag of one lookup: the most copies that the entry point takes
+    ind, off = torch.tensor([5], dtype=torch.int32, device=DEV), torch.tensor([0, 1], dtype=torch.int32, device=DEV)
+    got_ind, got_off, _ = tbe.replicate_batch(ind, off, None, 1, F)
+    assert int(got_off[0]) == 0 and int(got_off[-1]) == F
+    step = 1 << 28
+    for a in range(0, F, step):
+        b = min(a + step, F)
+        assert torch.equal(got_off[a:b], torch.arange(a, b, dtype=torch.int32, device=DEV))
+        assert bool((got_ind[a:b] == 5).all())
