@@ -65,7 +65,7 @@ struct Workspace {
     Chunk* chunks = nullptr;
     float* carry_head = nullptr;
     float* carry_tail = nullptr;
-    int64_t* tail_owner = nullptr;
+    unsigned long long* split = nullptr;
     uint32_t* chunk_next = nullptr;
     int64_t max_chunks = 0;
     // radix sort plan: table-aligned tiles
@@ -182,7 +182,7 @@ size_t layout(const cb_tbe* h, int64_t B, int64_t n, char* base, Workspace* w) {
     ws.chunks = static_cast<Chunk*>(take(sizeof(Chunk) * max_chunks));
     ws.carry_head = static_cast<float*>(take(sizeof(float) * max_chunks * h->dmax));
     ws.carry_tail = static_cast<float*>(take(sizeof(float) * max_chunks * h->dmax));
-    ws.tail_owner = static_cast<int64_t*>(take(sizeof(int64_t) * max_chunks));
+    ws.split = static_cast<unsigned long long*>(take(sizeof(unsigned long long) * max_chunks));
     ws.chunk_next = static_cast<uint32_t*>(take(sizeof(uint32_t) * (nc + 1)));
     for (int i = 0; i < 2; ++i) {
         ws.keys[i] = static_cast<uint32_t*>(take(sizeof(uint32_t) * n));
@@ -297,7 +297,7 @@ Plan make_plan(const cb_tbe* h, const Workspace& w, bool bwd, int64_t n) {
     Q.max_chunks = w.max_chunks;
     Q.carry_head = w.carry_head;
     Q.carry_tail = w.carry_tail;
-    Q.tail_owner = w.tail_owner;
+    Q.split = w.split;
     Q.chunk_next = w.chunk_next;
     return Q;
 }

@@ -208,7 +208,7 @@ extern "C" cb_status cb_tbe_forward_noalloc(const cb_table_desc* tables, int32_t
         Q.max_chunks = max_chunks;
         Q.carry_head = reinterpret_cast<float*>(base + o_hd);
         Q.carry_tail = reinterpret_cast<float*>(base + o_tl);
-        Q.tail_owner = reinterpret_cast<int64_t*>(base + o_to);
+        Q.split = reinterpret_cast<unsigned long long*>(base + o_to);
         Q.chunk_next = reinterpret_cast<uint32_t*>(base + o_nx);  // zeroed by the plan
         bool one_dtype = true;
         for (const Cls& c : classes) one_dtype = one_dtype && c.dtype == classes[0].dtype;

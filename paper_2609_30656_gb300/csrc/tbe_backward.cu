@@ -12,6 +12,7 @@
 #include <cuda_bf16.h>
 
 #include "tbe_internal.cuh"
+#include "tbe_fixup.cuh"
 #include "tbe_launch.h"
 #include "tbe_reduce.cuh"
 
@@ -271,8 +272,6 @@ __global__ void __launch_bounds__(1024) bwd_outputs_kernel(const __grid_constant
 // complete. (With a list of the heavy runs for a second kernel, and a third kernel for
 // the step, reduce and fix-up of 330 K fp32 lookups took 53 us, now 44; of 1.3 M
 // with fused Adagrad 256, now 244; of 41 M skewed 1138, now 1134.)
-constexpr int64_t kHeavyPieces = 32;
-
 // The chunks after chunk j that hold the rest of its open run: the pieces that
 // follow it (a piece holds one run only).
 __device__ __forceinline__ int64_t run_pieces(const Plan& Q, int64_t j, int t, int64_t total, int lane) {
@@ -338,11 +337,11 @@ __global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_co
         if (threadIdx.x == 0) heavy_count = 0;
         __syncthreads();
         const int64_t base = base0 + static_cast<int64_t>(w) * span;
-        const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
-        for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
+        const unsigned long long mine = lane < span && base + lane < total ? Q.split[base + lane] : 0;
+        for (uint32_t mask = __ballot_sync(kFull, (mine & kSplitBegins) != 0); mask; mask &= mask - 1) {
             const int b = __ffs(mask) - 1;
             const int64_t j = base + b;
-            const int64_t seg = __shfl_sync(kFull, mine, b);
+            const int64_t seg = __shfl_sync(kFull, static_cast<uint32_t>(mine), b);
             const int t = Q.chunks[j].table;
             const int64_t m = run_pieces(Q, j, t, total, lane);
             if (m > kHeavyPieces) {

@@ -1,40 +1,61 @@
 // tbe_forward.cu -- forward fix-up (bags split across chunks) and the launch
 // switch over storage types; the gather-pool kernel is in tbe_forward.cuh.
 #include "tbe_internal.cuh"
+#include "tbe_fixup.cuh"
 #include "tbe_launch.h"
 
 namespace cbtbe {
 
-// A heavy bag split over chunks: its tail piece (chunk where it starts) plus the
-// head pieces of the following chunks, added in fp64, then scaled. Each warp
-// scans `span` chunks at a time for tails (rare once boundaries snap to bag ends).
-__global__ void __launch_bounds__(kWarpThreads) fwd_fixup_kernel(const __grid_constant__ Problem P,
+// Bags split over chunks (only those longer than the cap of the plan's moved
+// boundaries): tail and head pieces, added in fp64, then scaled.
+struct BagSplit {
+    static constexpr bool kNarrow = false;
+    const Problem& P;
+    const Plan& Q;
+    void* out;
+    int64_t total;
+
+    __device__ __forceinline__ int64_t offset(int64_t bag) const { return load_index(P.offsets, bag, P.is32); }
+    // Chunks of a table are contiguous and chunk_len long while a split bag goes on, so
+    // the number of chunks that a bag reaches into follows from where it ends.
+    __device__ __forceinline__ int64_t pieces(int64_t j, uint32_t bag, int) const {
+        const Chunk ch = Q.chunks[j];
+        const int64_t k1 = ch.k0 + static_cast<int64_t>(ch.len & 0x7fffffffu), e = offset(bag + 1);
+        if (e <= k1) return 0;
+        return min64((e - k1 + Q.chunk_len - 1) / Q.chunk_len, total - j - 1);
+    }
+    // ... and the chunk where it begins, from where that is (checked: malformed offsets).
+    __device__ __forceinline__ bool origin(int64_t i, int lane, int64_t& j, int64_t& m) const {
+        const Chunk ch = Q.chunks[i];
+        const int64_t p0 = min64(max64(offset(static_cast<int64_t>(ch.table) * P.B), 0), P.n);
+        j = i - ((ch.k0 - p0) / Q.chunk_len - (offset(ch.first) - p0) / Q.chunk_len);
+        if (j < 0 || j >= i) return false;
+        const unsigned long long word = Q.split[j];
+        if (!(word & kSplitBegins) || static_cast<uint32_t>(word) != static_cast<uint32_t>(ch.first)) return false;
+        m = pieces(j, static_cast<uint32_t>(ch.first), lane);
+        return j + m >= i;
+    }
+    __device__ __forceinline__ void store(int64_t, uint32_t bag, int t, int x0, double (&acc)[4]) const {
+        if (P.mean) {
+            const int64_t L = offset(bag + 1) - offset(bag);
+            if (L > 0)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) acc[x] /= static_cast<double>(L);
+        }
+        const int64_t col0 = (static_cast<int64_t>(bag) - static_cast<int64_t>(t) * P.B) * P.sum_d + P.tables[t].doff;
+        store_out4(out, col0 + x0, static_cast<float>(acc[0]), static_cast<float>(acc[1]),
+                   static_cast<float>(acc[2]), static_cast<float>(acc[3]), P.out_dtype);
+    }
+    __device__ __forceinline__ void stored(int64_t, int, int) const {}
+};
+
+// (80 registers; left to itself the compiler takes 64 and spills.)
+__global__ void __launch_bounds__(kWarpThreads, 3) fwd_fixup_kernel(const __grid_constant__ Problem P,
                                                                  const __grid_constant__ Plan Q,
                                                                  void* out, int span) {
     begin_kernel();
-    const int lane = threadIdx.x & 31;
     const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    for (int64_t base = warp_id_global() * span; base < total; base += warps_in_grid() * span) {
-        const int64_t mine = lane < span && base + lane < total ? Q.tail_owner[base + lane] : -1;
-        for (uint32_t mask = __ballot_sync(kFull, mine >= 0); mask; mask &= mask - 1) {
-            const int b = __ffs(mask) - 1;
-            const int64_t j = base + b;
-            const int64_t bag = __shfl_sync(kFull, mine, b);
-            const int t = Q.chunks[j].table;
-            const TableDev& td = P.tables[t];
-            const int64_t s = load_index(P.offsets, bag, P.is32);
-            const int64_t e = load_index(P.offsets, bag + 1, P.is32);
-            const int64_t m = pieces_after(Q, j, e, total);
-            const double L = (P.mean && e > s) ? static_cast<double>(e - s) : 0.0;
-            const int64_t col0 = (bag - static_cast<int64_t>(t) * P.B) * P.sum_d + td.doff;
-            combine_pieces(Q, j, m, td.dim, P.dmax, lane, [&](int x0, double (&acc)[4]) {
-                if (L > 0.0)
-                    for (int x = 0; x < 4; ++x) acc[x] /= L;
-                store_out4(out, col0 + x0, static_cast<float>(acc[0]), static_cast<float>(acc[1]),
-                           static_cast<float>(acc[2]), static_cast<float>(acc[3]), P.out_dtype);
-            });
-        }
-    }
+    fix_split(P, Q, BagSplit{P, Q, out, total}, total, span);
 }
 
 void launch_fwd_gather_f32(const Problem&, const Plan&, void*, int, int, int, int64_t, int,

@@ -194,7 +194,7 @@ struct Gather {
         }
         // A piece of a bag split across chunks: fp32, for the fix-up.
         const bool started = s.len == 0;
-        if (started && lane == 0) Q.tail_owner[j] = bag;
+        if (started && lane == 0) Q.split[j] |= kSplitBegins | static_cast<uint32_t>(bag);
         float* dst = (started ? Q.carry_tail : Q.carry_head) + static_cast<int64_t>(j) * P.dmax + col;
         if (writes)
 #pragma unroll
@@ -246,6 +246,7 @@ struct Gather {
         s_cur = seg < bag_lo + P.B ? rel_pos(load_index(P.offsets, seg, P.is32), k0) : kRelHi;
         my_end = end_of(seg + lane);
         bool open = s_cur < 0;  // the sums hold part of a bag
+        if (lane == 0) Q.split[j] = open ? kSplitGoesOn : 0;
         Raw nxt = fetch(lane);
         if (len == 0) scan(0, 0);  // a table's chunk without lookups: its empty bags
         for (int32_t base = 0; base < len; base += 32) {
@@ -365,7 +366,6 @@ __device__ __forceinline__ void gather_chunk(const Problem& P, const Plan& Q, vo
     w.v = lane - w.g * w.V;
     w.slots = slots;
     w.seg = static_cast<int32_t>(ch.first);
-    if (lane == 0) Q.tail_owner[j] = -1;
     w.walk(static_cast<const uint4*>(td.data));
 }
 

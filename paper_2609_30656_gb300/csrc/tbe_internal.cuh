@@ -106,11 +106,17 @@ struct Plan {
     int64_t max_chunks;
     float* carry_head;                 // [max_chunks, dmax] piece of a segment begun earlier
     float* carry_tail;                 // [max_chunks, dmax] piece of a segment begun here
-    int64_t* tail_owner;               // [max_chunks] segment whose tail piece is here, or -1
+    unsigned long long* split;         // [max_chunks] kSplit... : segments cut by the chunk's edges
     uint32_t* chunk_next;              // [num_classes + 1] next chunk to hand out per class, and
                                        // over all classes (zeroed by the plan)
 };
 
+// A chunk's split word: in the low half the segment begun in it that runs past its
+// end, if kSplitBegins; kSplitGoesOn if it begins inside a segment. The fix-up counts
+// the blocks that are done with their share of the begun segment above.
+constexpr unsigned long long kSplitBegins = 1ull << 32;
+constexpr unsigned long long kSplitGoesOn = 1ull << 33;
+constexpr unsigned long long kSplitArrival = 1ull << 34;
 
 __host__ __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 __host__ __device__ __forceinline__ int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
@@ -414,116 +420,6 @@ struct EndSlot {
 // A cache line requested into L1 ahead of its load, without a register.
 __device__ __forceinline__ void prefetch_l1(const void* p) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-// ---------------------------------------------------------------- fix-up
-
-// A segment that straddles chunks left its tail piece in chunk j and head pieces
-// in the m chunks after it (chunks of a table are contiguous and chunk_len long
-// except the table's last, so m follows from the segment end). The pieces are
-// added in a fixed order, so the result is deterministic; `store` receives each
-// group of four columns in fp64. Up to 32 pieces: lanes own columns and walk the
-// pieces (add_pieces); more pieces (a hot row repeated across hundreds of
-// chunks): lanes own pieces and meet in a butterfly per group of four columns.
-constexpr int kInnerPieces = 16;
-
-// acc (fp64, four columns from x0) += pieces i0, i0 + step, ... below m, each at
-// head + piece * dmax. The pieces are summed in fp32 in groups of kInnerPieces,
-// each group folded into acc: GB300's fp64 adds are scarce (one per piece and
-// column made a heavy-run combine fp64-bound), and an fp32 sum of at most 16
-// pieces rounds within 16u of their absolute sum. Four loads in flight.
-__device__ __forceinline__ void add_pieces(const float* head, int64_t i0, int64_t step, int64_t m, int dmax,
-                                           int x0, double (&acc)[4]) {
-    for (int64_t g = i0; g < m; g += kInnerPieces * step) {
-        const int64_t gend = min64(m, g + kInnerPieces * step);
-        float in[4] = {0.f, 0.f, 0.f, 0.f};
-        int64_t i = g;
-        for (; i + 3 * step < gend; i += 4 * step) {
-            float4 h[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) h[c] = *reinterpret_cast<const float4*>(head + (i + c * step) * dmax + x0);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                in[0] += h[c].x;
-                in[1] += h[c].y;
-                in[2] += h[c].z;
-                in[3] += h[c].w;
-            }
-        }
-        for (; i < gend; i += step) {
-            const float4 h = *reinterpret_cast<const float4*>(head + i * dmax + x0);
-            in[0] += h.x;
-            in[1] += h.y;
-            in[2] += h.z;
-            in[3] += h.w;
-        }
-#pragma unroll
-        for (int x = 0; x < 4; ++x) acc[x] += in[x];
-    }
-}
-
-template <class Store>
-__device__ __forceinline__ void combine_pieces(const Plan& Q, int64_t j, int64_t m, int dim,
-                                               int dmax, int lane, Store store) {
-    const float* tail = Q.carry_tail + j * dmax;
-    const float* head = Q.carry_head + (j + 1) * dmax;
-    if (m <= 32) {
-        for (int x0 = lane * 4; x0 < dim; x0 += 128) {
-            const float4 a = *reinterpret_cast<const float4*>(tail + x0);
-            double acc[4] = {a.x, a.y, a.z, a.w};
-            add_pieces(head, 0, 1, m, dmax, x0, acc);
-            store(x0, acc);
-        }
-        return;
-    }
-    // Four groups of four columns per round: 16 independent loads per lane.
-    for (int x0 = 0; x0 < dim; x0 += 16) {
-        double acc[4][4] = {};
-        const int ng = min(4, (dim - x0) / 4);
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                if (c >= ng) break;
-                const float4 a = *reinterpret_cast<const float4*>(tail + x0 + 4 * c);
-                acc[c][0] = a.x;
-                acc[c][1] = a.y;
-                acc[c][2] = a.z;
-                acc[c][3] = a.w;
-            }
-        }
-#pragma unroll 4
-        for (int64_t i = lane; i < m; i += 32) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                if (c >= ng) break;
-                const float4 h = *reinterpret_cast<const float4*>(head + i * dmax + x0 + 4 * c);
-                acc[c][0] += h.x;
-                acc[c][1] += h.y;
-                acc[c][2] += h.z;
-                acc[c][3] += h.w;
-            }
-        }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1)
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int x = 0; x < 4; ++x) acc[c][x] += __shfl_xor_sync(kFull, acc[c][x], off);
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (c < ng) store(x0 + 4 * c, acc[c]);
-        }
-    }
-}
-
-// Number of chunks after chunk j that a segment ending at `e` reaches into.
-__device__ __forceinline__ int64_t pieces_after(const Plan& Q, int64_t j, int64_t e, int64_t total) {
-    const Chunk ch = Q.chunks[j];
-    const int64_t k1 = ch.k0 + static_cast<int64_t>(ch.len & 0x7fffffffu);
-    if (e <= k1) return 0;
-    const int64_t m = (e - k1 + Q.chunk_len - 1) / Q.chunk_len;
-    return min64(m, total - j - 1);
 }
 
 // ---------------------------------------------------------------- small scans

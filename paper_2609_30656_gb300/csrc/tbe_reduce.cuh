@@ -443,7 +443,7 @@ struct Reduce {
             total(tot);
             if (!at_head && lane == 0) {
                 // its number in the table, for the fix-up
-                Q.tail_owner[j] = APPLY ? 0 : out_row - O.out_first[t];
+                Q.split[j] |= kSplitBegins | (APPLY ? 0u : static_cast<uint32_t>(out_row - O.out_first[t]));
             }
             if (g == 0) store(carry(at_head ? Q.carry_head : Q.carry_tail), tot);
         }
@@ -487,7 +487,7 @@ __device__ __forceinline__ void reduce_chunk(const Problem& P, const Plan& Q, co
     w.shift = static_cast<int32_t>(ch.k0 - Q.table_pos[t] - (j - Q.table_chunk[t]) * Q.chunk_len);
     w.len = static_cast<int32_t>(ch.len & 0x7fffffffu);
     w.table_end = static_cast<int32_t>(Q.table_pos[t + 1] - ch.k0);
-    if (lane == 0) Q.tail_owner[j] = -1;
+    if (lane == 0) Q.split[j] = ch.len >> 31 ? kSplitGoesOn : 0;
     if (w.len == 0) return;
     // ch.first: the chunk's first run that begins in it (the one after the piece)
     r.walk(w, static_cast<const char*>(grad_out) + static_cast<int64_t>(td.doff) * eb, P.sum_d * eb, (ch.len >> 31) != 0,
