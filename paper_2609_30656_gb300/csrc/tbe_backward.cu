@@ -265,136 +265,128 @@ __global__ void __launch_bounds__(1024) bwd_outputs_kernel(const __grid_constant
 
 // ---------------------------------------------------------------- (6) fix-up
 
-// Runs split over chunks (hot rows that cover whole cells): each warp scans
-// `span` chunks at a time for tail pieces and combines each such run in fp64; runs
-// spread over more than kHeavyPieces chunks are left to the whole block, after its
-// warps' own. With the optimizer step fused, the row is stepped as soon as its sum is
-// complete. (With a list of the heavy runs for a second kernel, and a third kernel for
-// the step, reduce and fix-up of 330 K fp32 lookups took 53 us, now 44; of 1.3 M
-// with fused Adagrad 256, now 244; of 41 M skewed 1138, now 1134.)
-// The chunks after chunk j that hold the rest of its open run: the pieces that
-// follow it (a piece holds one run only).
-__device__ __forceinline__ int64_t run_pieces(const Plan& Q, int64_t j, int t, int64_t total, int lane) {
-    int64_t m = 0;
-    for (;;) {
-        const int64_t i = j + 1 + m + lane;
-        bool more = false;
-        if (i < total) {
-            const Chunk& ch = Q.chunks[i];
-            more = (ch.len >> 31) != 0 && ch.table == t;
+// Runs split over chunks (hot rows that cover whole cells). With the optimizer step
+// fused, the row is stepped as soon as its sum is complete. (With a list of the heavy
+// runs for a second kernel, and a third kernel for the step, reduce and fix-up of 330 K
+// fp32 lookups took 53 us, in one kernel 44; of 1.3 M with fused Adagrad 256 and 244.)
+struct RunSplit {
+    static constexpr bool kNarrow = true;
+    const Problem& P;
+    const Plan& Q;
+    const BwdOut& O;
+    int total;
+
+    // A run's pieces are consecutive chunks that begin inside a run, and hold nothing but
+    // it. How many of the chunks i0, i0 + dir, ... do: kNear are looked at, all at once (a
+    // serial look, 32 at a time, was the longest chain of a mid-size call's fix-up).
+    static constexpr int kWindows = 4, kNear = 32 * kWindows;
+    struct Near {
+        uint32_t in[kWindows];
+        __device__ __forceinline__ int count() const {
+            int n = 0;
+#pragma unroll
+            for (int u = 0; u < kWindows; ++u)
+                if (n == 32 * u) n += __clz(__brev(~in[u]));
+            return n;
         }
-        const uint32_t b = __ballot_sync(kFull, more);
-        if (b != kFull) return m + __ffs(~b) - 1;
-        m += 32;
+    };
+    __device__ __forceinline__ Near near(int i0, int dir, int lane) const {
+        unsigned long long word[kWindows];
+#pragma unroll
+        for (int u = 0; u < kWindows; ++u) {
+            const int i = i0 + dir * (32 * u + lane);
+            word[u] = i >= 0 && i < total ? Q.split[i] : 0;
+        }
+        Near x;
+#pragma unroll
+        for (int u = 0; u < kWindows; ++u) x.in[u] = __ballot_sync(kFull, (word[u] & kSplitGoesOn) != 0);
+        return x;
     }
-}
+    // Beyond them, a search by 33 parts a round: the pieces of one run are those of its
+    // table with as many runs before them. The last piece of `like`'s run after chunk lo,
+    // and the first before chunk hi, which are pieces of it.
+    __device__ __forceinline__ bool is_piece(int i, const Chunk& like) const {
+        const Chunk& ch = Q.chunks[i];
+        return (ch.len >> 31) != 0 && ch.table == like.table && ch.first == like.first;
+    }
+    __device__ __forceinline__ int last_piece(int lo, int lane) const {
+        const Chunk like = Q.chunks[lo];
+        int hi = total;  // none
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int step = (hi - lo + 32) / 33, p = lo + (lane + 1) * step;
+            const int c = __clz(__brev(~__ballot_sync(kFull, p < hi && is_piece(p, like))));
+            hi = min(hi, lo + (c + 1) * step);
+            lo += c * step;
+        }
+        return lo;
+    }
+    __device__ __forceinline__ int first_piece(int hi, int lane) const {
+        const Chunk like = Q.chunks[hi];
+        int lo = -1;  // none
+#pragma unroll 1
+        while (hi - lo > 1) {
+            const int step = (hi - lo + 32) / 33, p = hi - (lane + 1) * step;
+            const int c = __clz(__brev(~__ballot_sync(kFull, p > lo && is_piece(p, like))));
+            lo = max(lo, hi - (c + 1) * step);
+            hi -= c * step;
+        }
+        return hi;
+    }
 
-// Where the fix-up leaves a split run's sum: its gradient row, or, for a fused step,
-// the tail slot of the chunk where it begins.
-__device__ __forceinline__ float* split_row(const Plan& Q, const BwdOut& O, int64_t dmax, int64_t j, int64_t seg, int t,
-                                            int dim) {
-    return O.apply ? Q.carry_tail + j * dmax : O.grads + O.float_base[t] + seg * dim;
-}
+    __device__ __forceinline__ int pieces(int j, uint32_t, int lane) const {
+        const int n = near(j + 1, 1, lane).count();
+        return n < kNear ? n : last_piece(j + n, lane) - j;
+    }
+    __device__ __forceinline__ bool origin(int i, int lane, int& j, int& m) const {
+        const Near next = near(i + 1, 1, lane), prev = near(i - 1, -1, lane);
+        const int after = next.count(), before = prev.count();
+        const int last = after < kNear ? i + after : last_piece(i + after, lane);
+        j = (before < kNear ? i - before : first_piece(i - before, lane)) - 1;
+        m = last - j;
+        // (a run of out-of-range lookups is not summed: no chunk has it as begun)
+        return j >= 0 && (Q.split[j] & kSplitBegins) != 0;
+    }
+    // Where the sum goes: the gradient row, or, for a fused step, the tail slot of the
+    // chunk where the run begins.
+    __device__ __forceinline__ float* row(int j, uint32_t seg, int t) const {
+        return O.apply ? Q.carry_tail + static_cast<int64_t>(j) * P.dmax
+                       : O.grads + O.float_base[t] + static_cast<int64_t>(seg) * P.tables[t].dim;
+    }
+    __device__ __forceinline__ void store(int j, uint32_t seg, int t, int x0, double (&acc)[4]) const {
+        *reinterpret_cast<float4*>(row(j, seg, t) + x0) =
+            make_float4(static_cast<float>(acc[0]), static_cast<float>(acc[1]),
+                        static_cast<float>(acc[2]), static_cast<float>(acc[3]));
+    }
+    // The fused step of the row: lane l steps columns [4l + 128k, + 4).
+    __device__ __forceinline__ void stored(int j, int t, int lane) const {
+        if (!O.apply) return;
+        const float* g = row(j, 0, t);
+        const TableDev& td = P.tables[t];
+        const Chunk ch = Q.chunks[j];
+        // the chunk's last position belongs to the run
+        const int64_t r = static_cast<int64_t>(O.keys_sorted[ch.k0 + (ch.len & 0x7fffffffu) - 1]) - td.key_base;
+        float sq = 0.f;
+#pragma unroll 1
+        for (int x0 = lane * 4; x0 < td.dim; x0 += 128) sq += sq4(*reinterpret_cast<const float4*>(g + x0));
+        const float scale = step_scale(O, t, r, td.dim, sq);
+#pragma unroll 1
+        for (int x0 = lane * 4; x0 < td.dim; x0 += 128)
+            step_cols(td, r, x0, *reinterpret_cast<const float4*>(g + x0), scale);
+    }
+};
 
-// Lane l stores columns [4l + 128k, + 4), and steps them itself.
-__device__ __forceinline__ void store_grad4(float* dst, int x0, const double (&acc)[4]) {
-    *reinterpret_cast<float4*>(dst + x0) =
-        make_float4(static_cast<float>(acc[0]), static_cast<float>(acc[1]),
-                    static_cast<float>(acc[2]), static_cast<float>(acc[3]));
-}
-
-// The fused step of the run that is open at the end of chunk j, whose complete
-// gradient row `g` each lane of the warp has stored its columns of.
-__device__ __forceinline__ void step_split_run(const Problem& P, const Plan& Q, const BwdOut& O, int64_t j, int t,
-                                               const float* g, int lane) {
-    const TableDev& td = P.tables[t];
-    const Chunk ch = Q.chunks[j];
-    // the chunk's last position belongs to the run
-    const int64_t row = static_cast<int64_t>(O.keys_sorted[ch.k0 + (ch.len & 0x7fffffffu) - 1]) - td.key_base;
-    float sq = 0.f;
-    for (int x0 = lane * 4; x0 < td.dim; x0 += 128) sq += sq4(*reinterpret_cast<const float4*>(g + x0));
-    const float scale = step_scale(O, t, row, td.dim, sq);
-    for (int x0 = lane * 4; x0 < td.dim; x0 += 128)
-        step_cols(td, row, x0, *reinterpret_cast<const float4*>(g + x0), scale);
-}
-
-__global__ void __launch_bounds__(kWarpThreads) bwd_fixup_kernel(const __grid_constant__ Problem P,
-                                                                 const __grid_constant__ Plan Q,
-                                                                 const __grid_constant__ BwdOut O, int span) {
-    constexpr int kWarps = kWarpThreads / 32;
-    // Heavy runs of a round: they begin more than kHeavyPieces chunks apart, in the
-    // at most kWarps * 32 chunks that the block scans.
-    constexpr int kMaxHeavy = kWarps * 32 / static_cast<int>(kHeavyPieces) + 2;
-    __shared__ double sh[kWarps][512];
-    __shared__ int4 heavy[kMaxHeavy];
-    __shared__ int heavy_count;
+// 5 blocks per SM, so that a mid-size call's blocks are resident at once; 48 registers, the
+// heavy part spills. (Backward of 106 K one-hot lookups into kept buffers 70.7 us, at 64
+// registers 75, at 80 and 118 78; fused Adagrad step of 1.3 M 341, 341, 340 and 343.)
+__global__ void __launch_bounds__(kWarpThreads, 5) bwd_fixup_kernel(const __grid_constant__ Problem P,
+                                                                    const __grid_constant__ Plan Q,
+                                                                    const __grid_constant__ BwdOut O, int span,
+                                                                    int scan_blocks) {
     begin_kernel();
     if (*O.cap_fail) return;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t total = min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks);
-    const int64_t round = static_cast<int64_t>(gridDim.x) * kWarps * span;
-    for (int64_t base0 = static_cast<int64_t>(blockIdx.x) * kWarps * span; base0 < total; base0 += round) {
-        if (threadIdx.x == 0) heavy_count = 0;
-        __syncthreads();
-        const int64_t base = base0 + static_cast<int64_t>(w) * span;
-        const unsigned long long mine = lane < span && base + lane < total ? Q.split[base + lane] : 0;
-        for (uint32_t mask = __ballot_sync(kFull, (mine & kSplitBegins) != 0); mask; mask &= mask - 1) {
-            const int b = __ffs(mask) - 1;
-            const int64_t j = base + b;
-            const int64_t seg = __shfl_sync(kFull, static_cast<uint32_t>(mine), b);
-            const int t = Q.chunks[j].table;
-            const int64_t m = run_pieces(Q, j, t, total, lane);
-            if (m > kHeavyPieces) {
-                if (lane == 0) {
-                    const int slot = atomicAdd(&heavy_count, 1);
-                    if (slot < kMaxHeavy)
-                        heavy[slot] = make_int4(static_cast<int>(j), static_cast<int>(seg), static_cast<int>(m), t);
-                }
-                continue;
-            }
-            const int dim = P.tables[t].dim;
-            float* dst = split_row(Q, O, P.dmax, j, seg, t, dim);
-            const float* tail = Q.carry_tail + j * P.dmax;
-            const float* head = Q.carry_head + (j + 1) * P.dmax;
-            for (int x0 = lane * 4; x0 < dim; x0 += 128) {
-                const float4 a = *reinterpret_cast<const float4*>(tail + x0);
-                double acc[4] = {a.x, a.y, a.z, a.w};
-                add_pieces(head, 0, 1, m, P.dmax, x0, acc);
-                store_grad4(dst, x0, acc);
-            }
-            if (O.apply) step_split_run(P, Q, O, j, t, dst, lane);
-        }
-        __syncthreads();
-        // A heavy run: warp w adds pieces w, w + 8, ... (lanes own columns; fp32 groups
-        // folded into fp64), then the warps' partial sums meet in warp order, after
-        // the tail piece. The order is fixed, so the result is deterministic.
-        const int count = min(heavy_count, kMaxHeavy);
-        for (int h = 0; h < count; ++h) {
-            const int64_t j = heavy[h].x, seg = heavy[h].y, m = heavy[h].z;
-            const int t = heavy[h].w;
-            const int dim = P.tables[t].dim;
-            const float* head = Q.carry_head + (j + 1) * P.dmax;
-            for (int x0 = lane * 4; x0 < dim; x0 += 128) {
-                double acc[4] = {0.0, 0.0, 0.0, 0.0};
-                add_pieces(head, w, kWarps, m, P.dmax, x0, acc);
-                for (int x = 0; x < 4; ++x) sh[w][x0 + x] = acc[x];
-            }
-            __syncthreads();
-            if (w == 0) {
-                float* dst = split_row(Q, O, P.dmax, j, seg, t, dim);
-                const float* tail = Q.carry_tail + j * P.dmax;
-                for (int x0 = lane * 4; x0 < dim; x0 += 128) {
-                    const float4 a = *reinterpret_cast<const float4*>(tail + x0);
-                    double acc[4] = {a.x, a.y, a.z, a.w};
-                    for (int ww = 0; ww < kWarps; ++ww)
-                        for (int x = 0; x < 4; ++x) acc[x] += sh[ww][x0 + x];
-                    store_grad4(dst, x0, acc);
-                }
-                if (O.apply) step_split_run(P, Q, O, j, t, dst, lane);
-            }
-            __syncthreads();
-        }
-    }
+    const int total = static_cast<int>(min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks));
+    fix_split(P, Q, RunSplit{P, Q, O, total}, total, span, scan_blocks);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -440,8 +432,8 @@ void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const v
 
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
-    const int span = fixup_span(chunk_bound, num_sms);
-    launch(bwd_fixup_kernel, fixup_grid(chunk_bound, span, num_sms), kWarpThreads, 0, s, P, Q, O, span);
+    const FixupGrid g(chunk_bound, num_sms);
+    launch(bwd_fixup_kernel, g.blocks, kWarpThreads, 0, s, P, Q, O, g.span, g.scan_blocks);
 }
 
 }  // namespace cbtbe

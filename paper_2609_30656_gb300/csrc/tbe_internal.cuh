@@ -11,8 +11,8 @@
 // Work is cut into chunks of item positions of one size per call, so every warp
 // does the same amount of gathering whatever the bag-length distribution (heavy tails,
 // empty bags, one-hot bags). A segment that straddles chunk boundaries is summed
-// piecewise; its pieces are combined afterwards in chunk order, in fp64, by a
-// fix-up pass, so results are deterministic.
+// piecewise; its pieces are combined afterwards in one fixed order, in fp64, by a
+// fix-up pass (tbe_fixup.cuh), so results are deterministic.
 #pragma once
 
 #include <cstdint>

@@ -1,6 +1,7 @@
-"""Bags that span many chunks, at the edges of the fix-up's ways to add their pieces: one
-warp up to 32 pieces, a block above, and groups of 128 chunks whose sums are added by the
-last block to finish. Whole numbers make every sum exact in fp32, so results are equal."""
+"""Bags, and runs of one row's lookups, that span many chunks, at the edges of the fix-up's
+ways to add their pieces: one warp up to 32 pieces, a block up to 256, and above that groups
+of 128 chunks whose sums are added by the last block to finish. Whole numbers make every sum exact in
+fp32, so results are equal."""
 
 import pytest
 import torch
@@ -65,7 +66,7 @@ def test_bags_of_many_pieces(lengths, dim, dtype, out):
 
 def test_one_bag_takes_no_longer_than_many():
     """A million lookups in one bag against the same in bags of a thousand: the pieces are
-    added by the whole GPU (about 1.2 times as long; 25 times with one warp per bag)."""
+    added by the whole GPU (a little longer; 25 times as long with one warp per bag)."""
     from paper_2609_30656_gb300.tbe import TBE
     n, rows = 1_000_000, 100_000
     ind = torch.randint(0, rows, (n,), device=DEV)
@@ -76,3 +77,62 @@ def test_one_bag_takes_no_longer_than_many():
         out = torch.empty(B, 64, device=DEV)
         took.append(_times(lambda: m.forward(ind, off, out=out)))
     assert took[0] < 4 * took[1], took
+
+
+@pytest.mark.parametrize("lengths", LENGTHS)
+@pytest.mark.parametrize("invalid", [False, True])
+@pytest.mark.parametrize("dim,out", [(4, torch.float32), (64, torch.float32), (200, torch.float32),
+                                     (384, torch.bfloat16), (512, torch.float16)])
+def test_runs_of_many_pieces(lengths, invalid, dim, out):
+    """Row r of every table is looked up lengths[r] times, the last row (or, invalid: no
+    row, a run that is dropped) as often as a few chunks hold."""
+    from paper_2609_30656_gb300.tbe import CB_ERR_INDEX_OOB, TBE
+    g = torch.Generator(device=DEV).manual_seed(dim)
+    T, B, rows = 3, 40, len(lengths) + 1
+    counts = [lengths + [0], [7] * (rows - 1) + [150 * C], lengths + [131 * C + 2]]
+    if invalid:  # index `rows` is out of range
+        counts = [c[:-1] + [0, c[-1]] for c in counts]
+    ind = torch.cat([torch.repeat_interleave(torch.arange(len(c), device=DEV), torch.tensor(c, device=DEV))[
+        torch.randperm(sum(c), generator=g, device=DEV)] for c in counts])
+    starts = [0]
+    for c in counts:
+        starts.append(starts[-1] + sum(c))
+    off = torch.cat([(a + (torch.arange(B, device=DEV) * (b - a)) // B) for a, b in zip(starts, starts[1:])]
+                    + [torch.tensor(starts[-1:], device=DEV)])
+    go = torch.randint(-8, 9, (B, T * dim), generator=g, device=DEV).to(out)
+    tables = [torch.randint(-8, 9, (rows, dim), generator=g, device=DEV).float() for _ in range(T)]
+    bag = torch.repeat_interleave(torch.arange(T * B, device=DEV), off[1:] - off[:-1])
+    ids, want = [], []
+    for t in range(T):
+        a, b = starts[t], starts[t + 1]
+        G = torch.zeros(rows + 1, dim, dtype=torch.float64, device=DEV)
+        G.index_add_(0, ind[a:b], go[bag[a:b] - t * B, t * dim:(t + 1) * dim].double())
+        seen = ind[a:b].unique()
+        seen = seen[seen < rows]
+        ids.append(seen + t * rows)
+        want.append(G[:rows])
+    m = TBE(tables, out_dtype=out)
+    got = m.backward(ind, off, go)
+    assert (m.get_error() == CB_ERR_INDEX_OOB) == invalid
+    assert torch.equal(got.unique_ids, torch.cat(ids))
+    expect = torch.cat([w[i - t * rows] for t, (w, i) in enumerate(zip(want, ids))])
+    assert torch.equal(got.grads.view(-1, dim).double(), expect)
+    assert torch.equal(m.backward(ind, off, go).grads, got.grads)
+    before = [t.clone() for t in m.tables]
+    m.backward_apply(ind, off, go, optimizer="sgd", lr=0.25)
+    for t, w, x in zip(m.tables, want, before):
+        assert torch.equal(t.double(), x.double() - 0.25 * w)
+
+
+def test_one_hot_row_takes_no_longer_than_many():
+    """A million lookups of one row against the same over the table."""
+    from paper_2609_30656_gb300.tbe import TBE
+    n, rows, B = 1_000_000, 100_000, 1000
+    m = TBE([torch.randn(rows, 64, device=DEV)])
+    off = torch.arange(B + 1, device=DEV) * (n // B)
+    go = torch.randn(B, 64, device=DEV)
+    g = m.alloc_grad(rows, rows * 64)
+    took = []
+    for ind in (torch.full((n,), 7, device=DEV), torch.randint(0, rows, (n,), device=DEV)):
+        took.append(_times(lambda: m.backward_into(g, ind, off, go)))
+    assert took[0] < 2 * took[1], took
