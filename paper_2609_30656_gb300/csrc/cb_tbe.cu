@@ -510,7 +510,7 @@ cb_status backward_impl(cb_tbe* h, int32_t batch, const void* indices, int64_t n
         launch_bwd_outputs(P, O, stream);
         h->launches += 1;
     } else {
-        launch_bwd_runs(P, Q, O, bound, stream);
+        launch_bwd_runs(P, Q, O, bound, h->num_sms, stream);
         h->launches += 2;
         record(h, h->ev_bwd[3], stream);
         nv.phase("bwd.reduce");

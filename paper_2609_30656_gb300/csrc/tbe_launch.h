@@ -193,7 +193,8 @@ void launch_keygen(const Problem& P, const Plan& Q, const KeyGen& K, bool packed
                    int num_sms, cudaStream_t s);
 // Runs of equal sorted keys: counts per chunk cell, the reduce's chunks (cut at
 // run ends), and the sizes and first output rows of every table.
-void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound, cudaStream_t s);
+void launch_bwd_runs(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound, int num_sms,
+                     cudaStream_t s);
 // The output ranges again, into other caller buffers (after launch_bwd_runs).
 void launch_bwd_outputs(const Problem& P, const BwdOut& O, cudaStream_t s);
 // The segmented reduce (apply: with the optimizer step fused), dispatched on
