@@ -123,7 +123,6 @@ struct cb_tbe {
     int32_t sum_d = 0;
     int32_t dmax = 0;
     int64_t sum_rows = 0;
-    int key_bits = 1;
     int passes = 1;
     std::vector<TableDev> tables;
     std::vector<KernelClass> fwd_classes, bwd_classes;
@@ -623,7 +622,6 @@ cb_status cb_tbe_create(const cb_table_desc* tables, int32_t num_tables, cb_pool
     for (const TableDev& td : h->tables) max_rows = std::max(max_rows, td.rows);
     int bits = 1;
     while (bits < 32 && (int64_t(1) << bits) <= max_rows) ++bits;
-    h->key_bits = bits;
     h->passes = (bits + 7) / 8;
 
     // Kernel classes: tables whose rows (forward: storage type) or grad_out rows

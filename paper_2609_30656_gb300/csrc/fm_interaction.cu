@@ -280,13 +280,14 @@ constexpr int64_t kL2Bytes = int64_t(128) << 20;
 
 // Whether a warp takes a sample, or a block. The block has the samples of a few vectors,
 // several at a time, and those of many steps; also of many in a batch too small to give
-// every SM's warps one, and of many vectors in one larger than L2. Block and warp, us, y of 20 to 64 MB (read from L2; fields x dim).
-// Forward: 10 x 4 (10 vectors) 24.9, 32.4; 2 x 32 (16) 23.2, 25.5; 10 x 8 (20) 36.8, 30.2;
-// 16 x 64 (8 steps) 33.6, 10.2; 40 x 64 (20) 17.6, 9.5; 40 x 96 (40) 12.5, 11.1; 100 x
-// 128 (100) 11.0, 13.1; from HBM (256 MB), 26 x 96 (624 vectors) 56.1, 45.9; 26 x 128 (832) 44.7, 45.3; 40 x 256 (2560) 44.1, 52.4. Gradient from L2:
-// 16 x 4 (16 vectors) 22.2, 26.1; 10 x 8 (20) 24.1, 24.8; 3 x 32 (24) 23.8, 23.1; 16 x 64
-// 43.5, 20.1. (A warp per sample that read in a loop took 14.8 for the forward of 100 x 8,
-// the block 43.4, now 12.6.)
+// every SM's warps one, and of many vectors in one larger than L2. Block and warp, us, y
+// of 20 to 64 MB (read from L2), fields x dim. Forward: 10 x 4 (10 vectors) 24.9, 32.4;
+// 2 x 32 (16) 23.2, 25.5; 10 x 8 (20) 36.8, 30.2; 16 x 64 (8 steps) 33.6, 10.2; 40 x 64
+// (20) 17.6, 9.5; 40 x 96 (40) 12.5, 11.1; 100 x 128 (100) 11.0, 13.1. From HBM (256 MB):
+// 26 x 96 (624 vectors) 56.1, 45.9; 26 x 128 (832) 44.7, 45.3; 40 x 256 (2560) 44.1, 52.4.
+// Gradient from L2: 16 x 4 (16 vectors) 22.2, 26.1; 10 x 8 (20) 24.1, 24.8; 3 x 32 (24)
+// 23.8, 23.1; 16 x 64 43.5, 20.1. (A warp per sample that read in a loop took 14.8 for the
+// forward of 100 x 8, the block 43.4; now 12.6.)
 bool fm_by_warp(int64_t vectors, int64_t steps, int batch, bool backward) {
     if (vectors < (backward ? 21 : 16)) return false;
     if (steps <= 16) return true;

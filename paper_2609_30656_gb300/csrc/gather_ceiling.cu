@@ -128,7 +128,7 @@ cb_status launch(const void* rows, int64_t num_rows, int32_t row_bytes, const ui
     const uint4* r = static_cast<const uint4*>(rows);
     const int64_t full = n / 32;
     if (full > 0) {
-        const int cap = occupancy_grid(gather_ceiling_kernel<G, DT>, kWarpThreads, sms);
+        const int cap = resident_blocks(gather_ceiling_kernel<G, DT>, kWarpThreads) * sms;
         const int64_t need = (full + (kWarpThreads / 32) - 1) / (kWarpThreads / 32);
         const int grid = static_cast<int>(need < cap ? need : cap);
         gather_ceiling_kernel<G, DT><<<grid, kWarpThreads, 0, s>>>(r, num_rows, idx, full, out);

@@ -441,10 +441,6 @@ void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t 
     launch(bwd_fixup_kernel, g.blocks, kWarpThreads, 0, s, P, Q, O, g.span, g.scan_blocks);
 }
 
-}  // namespace cbtbe
-
-namespace cbtbe {
-
 // ---------------------------------------------------------------- (7) sparse step
 
 // The optimizer step from a row-sparse gradient already in memory (written by
@@ -589,7 +585,7 @@ __global__ void __launch_bounds__(kWarpThreads, M == 1 ? CB_APPLY_MIN_BLOCKS : 2
 
 template <int M, int R>
 void launch_apply_sparse_m(const Problem& P, const BwdOut& O, int num_sms, cudaStream_t s) {
-    static int cap = occupancy_grid(apply_sparse_kernel<M, R>, kWarpThreads, num_sms);
+    static const int cap = resident_blocks(apply_sparse_kernel<M, R>, kWarpThreads) * num_sms;
     launch(apply_sparse_kernel<M, R>, cap, kWarpThreads, 0, s, P, O);
 }
 

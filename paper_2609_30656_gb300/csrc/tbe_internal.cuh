@@ -65,7 +65,9 @@ struct TableDev {
     int32_t grad_vecs;  // 16-byte vectors per grad_out row, in the output's type
 };
 
-// A run of at most chunk_len item positions of one table.
+// Consecutive item positions of one table. A boundary that is not moved has chunk_len
+// positions on each side; the forward moves it by up to snap_cap, so its chunks hold up
+// to chunk_len + snap_cap, and the reduce's, cut at run ends, less than 2 * chunk_len.
 struct Chunk {
     int64_t k0;     // first item position
     int64_t first;  // forward: first bag touching k0; backward: first run of the table
@@ -135,8 +137,9 @@ __device__ __forceinline__ int64_t warps_in_grid() {
     return (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
 }
 
-// Every kernel of the library is launched with programmatic stream serialization
-// and begins with begin_kernel(): its launch overlaps the end of the kernel before
+// Every kernel of the lookups, the cross term and the replication (not the gather rate
+// probes) is launched with programmatic stream serialization and begins with
+// begin_kernel(): its launch overlaps the end of the kernel before
 // it, whose results it then waits for (the wait covers everything earlier on the
 // stream too, since that kernel began with the same wait). A call is a chain of 3 to
 // 20 short kernels: a serving request's forward 22 -> 15 us, fp32 step of 330 K
@@ -398,7 +401,6 @@ __device__ __forceinline__ void accumulate(float (&a)[Storage<DT>::kElems], cons
 
 // Forward positions are relative to the chunk start and clamped to
 // [kRelLo, kRelHi], which keeps every comparison with [0, len] exact in 32 bits.
-constexpr uint32_t kInvalid = 0xffffffffu;
 constexpr int32_t kRelLo = -1;
 constexpr int32_t kRelHi = 1 << 30;
 

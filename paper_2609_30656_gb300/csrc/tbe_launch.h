@@ -93,8 +93,8 @@ inline int rows_per_step(int vecs) {
     return 32 / lanes;
 }
 
-// Payload bag of a lookup whose index is out of range: outside every table's
-// bags, so the reduce reads the zero row for it.
+// Payload bag of a lookup whose index is out of range: outside every table's bags (the
+// reduce reads the table's last bag for it, and drops the sum).
 constexpr uint32_t kDeadBag = 0xffffffffu;
 
 struct KeyGen {
@@ -157,6 +157,7 @@ void launch_plan(const Problem& P, const Plan& Q, const TilePlan* S, int64_t chu
                  cudaStream_t s);
 int plan_launches(const Problem& P);  // kernels launch_plan enqueues
 
+constexpr int kPlanTables = 1024;  // tables that a block plans in shared memory
 constexpr int kAllClasses = -1, kPlanned = -2;  // `cls` of launch_fwd_gather
 // Whether a forward of one storage type runs without a plan kernel.
 #ifndef CB_PLANNED_BLOCKS
@@ -164,7 +165,7 @@ constexpr int kAllClasses = -1, kPlanned = -2;  // `cls` of launch_fwd_gather
 #endif
 constexpr int kPlannedBlocks = CB_PLANNED_BLOCKS;  // resident blocks per SM of the kernel that does
 inline bool fwd_plans_itself(int64_t chunk_bound, int64_t T, int num_sms) {
-    return T <= 1024 && chunk_bound <= static_cast<int64_t>(num_sms) * 8 * kPlannedBlocks;
+    return T <= kPlanTables && chunk_bound <= static_cast<int64_t>(num_sms) * 8 * kPlannedBlocks;
 }
 void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int dtype, int vpl,
                        int gc, int64_t chunk_bound, int num_sms, cudaStream_t s);

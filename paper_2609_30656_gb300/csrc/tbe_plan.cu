@@ -2,8 +2,9 @@
 // gather-pool and the backward key generation / segmented reduce.
 //
 // A table's items (lookup positions, key-major so each table's lookups are
-// contiguous) are cut into chunks of at most chunk_len positions; a table with
-// no lookups still gets one (empty) chunk so that its empty bags are written.
+// contiguous) are cut every chunk_len positions, and the forward's cuts moved to bag
+// ends; a table with no lookups still gets one (empty) chunk so that its empty bags
+// are written.
 // Chunks are numbered class by class (tables grouped by kernel instantiation),
 // table by table within a class. The backward's sort tiles are placed with them.
 #include "tbe_internal.cuh"

@@ -3,10 +3,9 @@
 #pragma once
 
 #include "tbe_internal.cuh"
+#include "tbe_launch.h"
 
 namespace cbtbe {
-
-constexpr int kPlanTables = 1024;  // tables that a block plans in shared memory
 
 // The tables' part of the plan, by one block: item ranges (pos), and the first
 // chunk of every table in class order (ord) and, with tiles, the first sort tile in

@@ -13,11 +13,6 @@
 
 namespace cbtbe {
 
-template <class KernelT>
-inline int occupancy_grid(KernelT kernel, int threads, int num_sms) {
-    return resident_blocks(kernel, threads) * num_sms;
-}
-
 // ---------------------------------------------------------------- optimizer step
 
 // Start of a stored row.

@@ -44,7 +44,7 @@ __device__ __forceinline__ void weight_grad_chunk(const Problem& P, const Chunk&
                                                   const void* grad_out, float* grad_w, int lane) {
     constexpr int E = Storage<DT>::kElems;
     constexpr int V = 32 / G;
-        constexpr int U = V < 8 / VPL ? V : 8 / VPL;  // lookups per group whose rows are loaded together
+    constexpr int U = V < 8 / VPL ? V : 8 / VPL;  // lookups per group whose rows are loaded together
     static_assert(VPL == 1 || G == 1, "several vectors per lane: one row per step");
     const int g = lane / V, v = lane - g * V;
     const int row_vecs = td.row_vecs;
