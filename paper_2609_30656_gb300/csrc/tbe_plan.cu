@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
     const int tid = threadIdx.x;
     const int64_t total = min64(ord[P.T], Q.max_chunks);
     if (blockIdx.x == 0) {
+#pragma unroll 1
         for (int i = tid; i <= P.T; i += blockDim.x) {
             if (own) {
                 Q.table_pos[i] = pos[i];
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
             }
             if (i < P.T) Q.table_chunk[Q.class_tables[i]] = ord[i];
         }
+#pragma unroll 1
         for (int c = tid; c <= Q.num_classes; c += blockDim.x) {
             Q.class_chunk_base[c] = min64(ord[Q.class_table_start[c]], Q.max_chunks);
             Q.chunk_next[c] = 0;
@@ -78,6 +80,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
     const int64_t first = static_cast<int64_t>(blockIdx.x) * blockDim.x + tid;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int lane = tid & 31;
+#pragma unroll 1
     for (int64_t w = first; (w - lane) / W < total; w += stride) {  // warp-uniform
         const int64_t j = min64(w / W, total - 1);
         const Chunk ch = plan_chunk<W>(P, Q, pos, ord, j, lane);
@@ -86,6 +89,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
     }
     if (S.tile_len <= 0) return;
     const int64_t tiles = min64(tile_ord[P.T], S.max_tiles);
+#pragma unroll 1
     for (int64_t j = first; j < tiles; j += stride) {
         const int t = owner_of(tile_ord, P.T, j);
         const int64_t p0 = pos[t], p1 = max64(p0, pos[t + 1]);
@@ -96,6 +100,7 @@ __global__ void __launch_bounds__(256, 6) plan_kernel(const __grid_constant__ Pr
         ch.len = static_cast<uint32_t>(min64(S.tile_len, p1 - ch.k0));
         S.tiles[j] = ch;
     }
+#pragma unroll 1
     for (int64_t k = first; k < S.zero_words; k += stride) S.zero[k] = 0;
 }
 

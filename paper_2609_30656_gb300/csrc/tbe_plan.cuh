@@ -21,6 +21,7 @@ __device__ __forceinline__ void plan_tables(const Problem& P, const Plan& Q, int
         return min64(max64(load_index(P.offsets, static_cast<int64_t>(t) * P.B, P.is32), 0), P.n);
     };
     bool falls = false;
+#pragma unroll 1
     for (int t = tid; t <= P.T; t += blockDim.x) {
         const int64_t x = start(t);
         pos[t] = x;
@@ -29,11 +30,13 @@ __device__ __forceinline__ void plan_tables(const Problem& P, const Plan& Q, int
     if (__syncthreads_or(falls)) {
         if (tid == 0) {
             set_error(P.error, CB_ERR_BAD_OFFSETS);
+#pragma unroll 1
             for (int t = 1; t <= P.T; ++t) pos[t] = max64(pos[t], pos[t - 1]);
         }
         __syncthreads();
     }
     int64_t chunks = 0, tiles = 0;
+#pragma unroll 1
     for (int i0 = 0; i0 < P.T; i0 += blockDim.x) {
         const int i = i0 + tid;
         int64_t cnt = 0, tcnt = 0;
