@@ -349,19 +349,19 @@ struct RunSplit {
     }
     // Where the sum goes: the gradient row, or, for a fused step, the tail slot of the
     // chunk where the run begins.
-    __device__ __forceinline__ float* row(int j, uint32_t seg, int t) const {
+    using Dest = float*;
+    __device__ __forceinline__ Dest dest(int j, uint32_t seg, int t) const {
         return O.apply ? Q.carry_tail + static_cast<int64_t>(j) * P.dmax
                        : O.grads + O.float_base[t] + static_cast<int64_t>(seg) * P.tables[t].dim;
     }
-    __device__ __forceinline__ void store(int j, uint32_t seg, int t, int x0, double (&acc)[4]) const {
-        *reinterpret_cast<float4*>(row(j, seg, t) + x0) =
-            make_float4(static_cast<float>(acc[0]), static_cast<float>(acc[1]),
-                        static_cast<float>(acc[2]), static_cast<float>(acc[3]));
+    __device__ __forceinline__ void store(Dest d, int x0, double (&acc)[4]) const {
+        *reinterpret_cast<float4*>(d + x0) = make_float4(static_cast<float>(acc[0]), static_cast<float>(acc[1]),
+                                                         static_cast<float>(acc[2]), static_cast<float>(acc[3]));
     }
     // The fused step of the row: lane l steps columns [4l + 128k, + 4).
     __device__ __forceinline__ void stored(int j, int t, int lane) const {
         if (!O.apply) return;
-        const float* g = row(j, 0, t);
+        const float* g = dest(j, 0, t);
         const TableDev& td = P.tables[t];
         const Chunk ch = Q.chunks[j];
         // the chunk's last position belongs to the run
@@ -376,17 +376,20 @@ struct RunSplit {
     }
 };
 
-// 5 blocks per SM, so that a mid-size call's blocks are resident at once; 48 registers, the
-// heavy part spills. (Backward of 106 K one-hot lookups into kept buffers 70.7 us, at 64
-// registers 75, at 80 and 118 78; fused Adagrad step of 1.3 M 341, 341, 340 and 343.)
-__global__ void __launch_bounds__(kWarpThreads, 5) bwd_fixup_kernel(const __grid_constant__ Problem P,
-                                                                    const __grid_constant__ Plan Q,
-                                                                    const __grid_constant__ BwdOut O, int span,
-                                                                    int scan_blocks) {
+// BLOCKS per SM: 3 (80 registers), or 5 (48, and spills) for a grid of 2 to 4 blocks per SM,
+// which then is resident beside the end of the reduce. Whole backward, us, at 3 and 5: 52 K
+// lookups with the fused step (216 blocks) 75.5, 79.8; 106 K one-hot (446 blocks) 78.4,
+// 71.6; 158 K (657 blocks) 88.1, 89.9; 330 K (736 blocks) 104.4, 106.0; the fix-up alone of
+// 123 M skewed ones 62, 78.
+template <int BLOCKS>
+__global__ void __launch_bounds__(kWarpThreads, BLOCKS) bwd_fixup_kernel(const __grid_constant__ Problem P,
+                                                                         const __grid_constant__ Plan Q,
+                                                                         const __grid_constant__ BwdOut O, int span,
+                                                                         int group_blocks) {
     begin_kernel();
     if (*O.cap_fail) return;
     const int total = static_cast<int>(min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks));
-    fix_split(P, Q, RunSplit{P, Q, O, total}, total, span, scan_blocks);
+    fix_split(P, Q, RunSplit{P, Q, O, total}, total, span, group_blocks);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -438,7 +441,8 @@ void launch_bwd_reduce(const Problem& P, const Plan& Q, const BwdOut& O, const v
 void launch_bwd_fixup(const Problem& P, const Plan& Q, const BwdOut& O, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
     const FixupGrid g(chunk_bound, num_sms);
-    launch(bwd_fixup_kernel, g.blocks, kWarpThreads, 0, s, P, Q, O, g.span, g.scan_blocks);
+    auto* kernel = g.blocks > 2 * num_sms && g.blocks <= 4 * num_sms ? bwd_fixup_kernel<5> : bwd_fixup_kernel<3>;
+    launch(kernel, g.blocks, kWarpThreads, 0, s, P, Q, O, g.span, g.group_blocks);
 }
 
 // ---------------------------------------------------------------- (7) sparse step

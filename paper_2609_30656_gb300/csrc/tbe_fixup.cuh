@@ -48,11 +48,10 @@ struct RowLanes {
         c = lane & (V - 1);
     }
     // acc += this lane's share of rows 0 .. n - 1 of fp32, `stride` floats apart, at
-    // columns 4v .. 4v + 3. NARROW: eight rows in fp32 first, by halves (3u of their
+    // columns 4v .. 4v + 3. Narrow: eight rows in fp32 first, by halves (3u of their
     // absolute sum; GB300's fp64 adds are scarce: a backward of 330 K lookups 106 us so, 119
     // with every row into fp64), else each row into fp64.
-    template <bool NARROW>
-    __device__ __forceinline__ void add(const float* rows, int n, int64_t stride, int v, double (&acc)[4]) const {
+    __device__ __forceinline__ void add(bool narrow, const float* rows, int n, int64_t stride, int v, double (&acc)[4]) const {
         rows += g * stride + 4 * v;
         stride *= G;
 #pragma unroll 1
@@ -62,7 +61,7 @@ struct RowLanes {
             for (int u = 0; u < kRowsInFlight; ++u)
                 h[u] = k + u * G < n ? __ldcg(reinterpret_cast<const float4*>(rows + u * stride))
                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (NARROW) {
+            if (narrow) {
 #pragma unroll
                 for (int w = 1; w < kRowsInFlight; w *= 2)
 #pragma unroll
@@ -72,14 +71,19 @@ struct RowLanes {
                         h[u].z += h[u + w].z;
                         h[u].w += h[u + w].w;
                     }
-            }
+            } else {
 #pragma unroll
-            for (int u = 0; u < (NARROW ? 1 : kRowsInFlight); ++u) {
-                acc[0] += h[u].x;
-                acc[1] += h[u].y;
-                acc[2] += h[u].z;
-                acc[3] += h[u].w;
+                for (int u = 1; u < kRowsInFlight; ++u) {
+                    acc[0] += h[u].x;
+                    acc[1] += h[u].y;
+                    acc[2] += h[u].z;
+                    acc[3] += h[u].w;
+                }
             }
+            acc[0] += h[0].x;
+            acc[1] += h[0].y;
+            acc[2] += h[0].z;
+            acc[3] += h[0].w;
         }
     }
     // The same for n fp64 rows, each the low words in one row of floats and the high
@@ -123,58 +127,51 @@ struct RowLanes {
     }
 };
 
-// Split states what is split: Split::kNarrow; pieces(j, seg, lane), the chunks after
+// Split states what is split: Split::kNarrow, whether heavy segments are added narrow too
+// (the others are); pieces(j, seg, lane), the chunks after
 // chunk j that hold the rest of the segment begun there; origin(i, lane, j, m), the
 // chunk where the segment that chunk i begins inside was begun, and its pieces
-// (false: it has none to add); store(j, seg, t, x0, acc), four columns of a
-// segment's sum; stored(j, t, lane), after all of them. All but store are called by
-// whole warps.
+// (false: it has none to add); dest(j, seg, t), where its sum goes, loaded ahead of the
+// pieces; store(dest, x0, acc), four columns of it; stored(j, t, lane), after all of them.
+// All but store are called by whole warps.
 //
-// The warps of the first scan_blocks blocks look for segments begun in their chunks,
-// span chunks at a time, and leave the heavy ones to their block; the other blocks look
-// for groups of chunks that begin inside a segment (the first chunk of all does not).
+// The warps of the first group_blocks blocks look for groups of chunks that begin inside
+// a heavy segment, a group each, and leave them to their block (the first chunk of all
+// begins inside none); those of the others for segments begun in their chunks, span
+// chunks at a time, and leave the heavy ones to their block.
 template <class Split>
 __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const Split& split, int total, int span,
-                                          int scan_blocks) {
+                                          int group_blocks) {
     constexpr int kWarps = kWarpThreads / 32;
     // Heavy segments of a round: they begin more than kHeavyPieces chunks apart, in the
     // at most kWarps * 32 chunks that the block scans.
     constexpr int kMaxHeavy = kWarps * 32 / kHeavyPieces + 2;
     __shared__ double shares[4][kWarps][32];
-    __shared__ int2 heavy[kMaxHeavy];  // first chunk, pieces
+    __shared__ int4 heavy[kMaxHeavy];  // first chunk, pieces, table, the group's chunk or the segment
     __shared__ int heavy_count;
     __shared__ bool sh_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool scans = static_cast<int>(blockIdx.x) < scan_blocks;
+    const bool scans = static_cast<int>(blockIdx.x) >= group_blocks;
     const int64_t dmax = P.dmax;
-    const int64_t width = scans ? kWarps * span : kPieceGroup;  // chunks of the block's look
-    const int64_t step = width * (scans ? scan_blocks : gridDim.x - scan_blocks);
+    // Scanning, a block takes the chunks of its warps side by side; groups that follow each
+    // other, most likely of one segment, go to different blocks.
+    const int blocks = scans ? gridDim.x - group_blocks : group_blocks, me = scans ? blockIdx.x - group_blocks : blockIdx.x;
+    const int64_t block_step = scans ? kWarps * span : kPieceGroup, warp_step = scans ? span : blocks * kPieceGroup;
+    const int64_t step = scans ? blocks * block_step : kWarps * warp_step;
 #pragma unroll 1
-    for (int64_t at = scans ? width * blockIdx.x : width * (1 + blockIdx.x - scan_blocks); at < total; at += step) {
-        const int base = static_cast<int>(at) + (scans ? warp * span : 0);
-        const unsigned long long mine = (scans ? lane < span && base + lane < total : lane == 0) ? Q.split[base + lane] : 0;
+    for (int64_t at = (scans ? me : me + 1) * block_step; at < total; at += step) {
+        const int64_t base = at + warp * warp_step;
+        const unsigned long long mine = lane < (scans ? span : 1) && base + lane < total ? Q.split[base + lane] : 0;
         // Each warp its own light segments, then the block the heavy ones one by one.
         uint32_t found = __ballot_sync(kFull, (mine & (scans ? kSplitBegins : kSplitGoesOn)) != 0);
-        if (!scans) {
-            if (found == 0) continue;  // block-uniform
-            int j, m;
-            if (warp == 0) {
-                if (!split.origin(base, lane, j, m)) m = 0;
-                if (lane == 0) {
-                    heavy[0] = make_int2(j, m);
-                    heavy_count = m > kGroupedPieces ? 1 : 0;
-                }
-            }
-            found = 0;
-        } else if (threadIdx.x == 0) {
-            heavy_count = 0;
-        }
-        __syncthreads();
+        if (threadIdx.x == 0) heavy_count = 0;
+        if (!__syncthreads_or(found != 0)) continue;
         bool block = false;
         int next = 0;
 #pragma unroll 1
         for (;;) {
-            int j, m;
+            int j, m, t, group = 0;
+            uint32_t seg = 0;
             if (!block) {
                 if (found == 0) {
                     __syncthreads();
@@ -183,28 +180,33 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
                 }
                 const int b = __ffs(found) - 1;
                 found &= found - 1;
-                j = base + b;
-                m = split.pieces(j, __shfl_sync(kFull, static_cast<uint32_t>(mine), b), lane);
+                j = static_cast<int>(base) + b;
+                t = Q.chunks[j].table;
+                seg = __shfl_sync(kFull, static_cast<uint32_t>(mine), b);
+                if (scans) m = split.pieces(j, seg, lane);
+                else if (!split.origin(j, lane, j, m) || m <= kGroupedPieces) continue;
                 if (m > kHeavyPieces) {
                     if (lane == 0) {
                         const int slot = atomicAdd(&heavy_count, 1);
-                        if (slot < kMaxHeavy) heavy[slot] = make_int2(j, m);
+                        if (slot < kMaxHeavy)
+                            heavy[slot] = make_int4(j, m, t, scans ? static_cast<int>(seg) : static_cast<int>(base));
                     }
                     continue;
                 }
             } else {
                 if (next >= min(heavy_count, kMaxHeavy)) break;
-                j = heavy[next].x;
-                m = heavy[next].y;
-                ++next;
+                const int4 h = heavy[next++];
+                j = h.x;
+                m = h.y;
+                t = h.z;
+                group = h.w;
+                seg = static_cast<uint32_t>(h.w);
             }
-            const int t = Q.chunks[j].table;
             const RowLanes w(P.tables[t].dim, block);
             const bool grouped = m > kGroupedPieces;
             const int first = (j / kPieceGroup + 1) * kPieceGroup;               // of the groups after j's
             const int groups = grouped ? (j + m - first) / kPieceGroup + 1 : 0;
             const int single = grouped && (j + m) % kPieceGroup == 0 ? 1 : 0;    // a last group of one piece
-            uint32_t seg = 0;
             // A group's share of its segment's pieces first: left in fp64 in place of the
             // first two (a single piece is its own sum). Then the arrival at the segment, and
             // for the last to arrive (or the only one) the sum: the tail, the pieces up to the
@@ -212,21 +214,21 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
             bool share = !scans;
 #pragma unroll 1
             for (;;) {
-                const int row = share ? base : j + 1;
-                const int n = share ? min(kPieceGroup, j + m + 1 - base) : (grouped ? first - row : m);
-                if (!share) {
-                    if (grouped) {
+                const int row = share ? group : j + 1;
+                const int n = share ? min(kPieceGroup, j + m + 1 - group) : (grouped ? first - row : m);
+                if (!share && grouped) {
+                    __threadfence();
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        sh_last = static_cast<int>(atomicAdd(Q.split + j, kSplitArrival) / kSplitArrival) == groups;
                         __threadfence();
-                        __syncthreads();
-                        if (threadIdx.x == 0) {
-                            sh_last = static_cast<int>(atomicAdd(Q.split + j, kSplitArrival) / kSplitArrival) == groups;
-                            __threadfence();
-                        }
-                        __syncthreads();
-                        if (!sh_last) break;
                     }
+                    __syncthreads();
+                    if (!sh_last) break;
                     seg = static_cast<uint32_t>(Q.split[j]);
                 }
+                typename Split::Dest dest;
+                if (!share) dest = split.dest(j, seg, t);
                 float* rows = Q.carry_head + row * dmax;
 #pragma unroll 1
                 for (int v = w.c; v < w.nv + w.c && !(share && n == 1); v += 32) {  // as often in every lane
@@ -239,7 +241,7 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
                             acc[2] = a.z;
                             acc[3] = a.w;
                         }
-                        w.add<Split::kNarrow>(rows, n, dmax, v, acc);
+                        w.add(Split::kNarrow || !block, rows, n, dmax, v, acc);
                         if (!share && grouped) {
                             w.add64(Q.carry_head + first * dmax, groups - single, kPieceGroup * dmax, dmax, v, acc);
                             if (single && w.g == 0) {
@@ -264,7 +266,7 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
                     }
                     if (w.g == 0 && v < w.nv) {
                         if (share) RowLanes::put64(rows, dmax, v, acc);
-                        else split.store(j, seg, t, 4 * v, acc);
+                        else split.store(dest, 4 * v, acc);
                     }
                 }
                 if (!share) {
@@ -279,14 +281,14 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
     }
 }
 
-// The grid: the scanning blocks, and one for every group but the first, up to what the
-// GPU holds.
+// The grid: a block for every group but the first, up to two per SM (then a warp for every
+// group), and the scanning blocks.
 struct FixupGrid {
-    int span, scan_blocks, blocks;
+    int span, group_blocks, blocks;
     FixupGrid(int64_t chunk_bound, int num_sms) {
         span = fixup_span(chunk_bound, num_sms);
-        scan_blocks = fixup_grid(chunk_bound, span, num_sms);
-        blocks = scan_blocks + static_cast<int>(min64((chunk_bound - 1) / kPieceGroup, static_cast<int64_t>(num_sms) * 2));
+        group_blocks = static_cast<int>(min64((chunk_bound - 1) / kPieceGroup, static_cast<int64_t>(num_sms) * 2));
+        blocks = group_blocks + fixup_grid(chunk_bound, span, num_sms);
     }
 };
 

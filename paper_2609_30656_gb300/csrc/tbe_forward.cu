@@ -20,7 +20,7 @@ struct BagSplit {
     // the number of chunks that a bag reaches into follows from where it ends.
     __device__ __forceinline__ int pieces(int j, uint32_t bag, int) const {
         const Chunk ch = Q.chunks[j];
-        const int64_t k1 = ch.k0 + static_cast<int64_t>(ch.len & 0x7fffffffu), e = offset(bag + 1);
+        const int64_t k1 = ch.k0 + static_cast<int64_t>(ch.len & 0x7fffffffu), e = offset(static_cast<int64_t>(bag) + 1);
         if (e <= k1) return 0;
         return static_cast<int>(min64((e - k1 + Q.chunk_len - 1) / Q.chunk_len, total - j - 1));
     }
@@ -39,27 +39,35 @@ struct BagSplit {
         m = pieces(j, static_cast<uint32_t>(ch.first), lane);
         return j + m >= i;
     }
-    __device__ __forceinline__ void store(int, uint32_t bag, int t, int x0, double (&acc)[4]) const {
-        if (P.mean) {
-            const int64_t L = offset(bag + 1) - offset(bag);
-            if (L > 0)
+    struct Dest {
+        int64_t col;
+        double length;  // mean pooling, else 0
+    };
+    __device__ __forceinline__ Dest dest(int, uint32_t bag, int t) const {
+        const int64_t L = P.mean ? offset(static_cast<int64_t>(bag) + 1) - offset(bag) : 0;
+        return Dest{(static_cast<int64_t>(bag) - static_cast<int64_t>(t) * P.B) * P.sum_d + P.tables[t].doff,
+                    static_cast<double>(L)};
+    }
+    __device__ __forceinline__ void store(const Dest& d, int x0, double (&acc)[4]) const {
+        if (d.length > 0.0)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) acc[x] /= static_cast<double>(L);
-        }
-        const int64_t col0 = (static_cast<int64_t>(bag) - static_cast<int64_t>(t) * P.B) * P.sum_d + P.tables[t].doff;
-        store_out4(out, col0 + x0, static_cast<float>(acc[0]), static_cast<float>(acc[1]),
+            for (int x = 0; x < 4; ++x) acc[x] /= d.length;
+        store_out4(out, d.col + x0, static_cast<float>(acc[0]), static_cast<float>(acc[1]),
                    static_cast<float>(acc[2]), static_cast<float>(acc[3]), P.out_dtype);
     }
     __device__ __forceinline__ void stored(int, int, int) const {}
 };
 
-// (98 registers: a forward of 106 K one-hot lookups 31.6 us, at 64 registers 34, at 80 39.)
-__global__ void __launch_bounds__(kWarpThreads) fwd_fixup_kernel(const __grid_constant__ Problem P,
-                                                                 const __grid_constant__ Plan Q,
-                                                                 void* out, int span, int scan_blocks) {
+// BLOCKS per SM: 2 for small grids, else 4 (64 registers, the heavy part spills). Forward of
+// 106 K one-hot lookups, 424 blocks: 31.6 us at 2, 34.1 at 4; of 330 K, 655 blocks: 33.6 and
+// 32.8; of 1.6 M on odd dims, 1100 blocks: 80.5 and 79.6.
+template <int BLOCKS>
+__global__ void __launch_bounds__(kWarpThreads, BLOCKS) fwd_fixup_kernel(const __grid_constant__ Problem P,
+                                                                         const __grid_constant__ Plan Q, void* out,
+                                                                         int span, int group_blocks) {
     begin_kernel();
     const int total = static_cast<int>(min64(Q.class_chunk_base[Q.num_classes], Q.max_chunks));
-    fix_split(P, Q, BagSplit{P, Q, out, total}, total, span, scan_blocks);
+    fix_split(P, Q, BagSplit{P, Q, out, total}, total, span, group_blocks);
 }
 
 void launch_fwd_gather_f32(const Problem&, const Plan&, void*, int, int, int, int64_t, int,
@@ -79,7 +87,8 @@ void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int 
 void launch_fwd_fixup(const Problem& P, const Plan& Q, void* out, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
     const FixupGrid g(chunk_bound, num_sms);
-    launch(fwd_fixup_kernel, g.blocks, kWarpThreads, 0, s, P, Q, out, g.span, g.scan_blocks);
+    auto* kernel = g.blocks <= 3 * num_sms ? fwd_fixup_kernel<2> : fwd_fixup_kernel<4>;
+    launch(kernel, g.blocks, kWarpThreads, 0, s, P, Q, out, g.span, g.group_blocks);
 }
 
 }  // namespace cbtbe

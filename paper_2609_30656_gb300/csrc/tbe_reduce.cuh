@@ -438,7 +438,8 @@ struct Reduce {
             total(tot);
             if (!at_head && lane == 0) {
                 // its number in the table, for the fix-up
-                Q.split[j] |= kSplitBegins | (APPLY ? 0u : static_cast<uint32_t>(out_row - O.out_first[t]));
+                // (a chunk with a run begun in it begins inside none)
+                Q.split[j] = kSplitBegins | (APPLY ? 0u : static_cast<uint32_t>(out_row - O.out_first[t]));
             }
             if (g == 0) store(carry(at_head ? Q.carry_head : Q.carry_tail), tot);
         }
