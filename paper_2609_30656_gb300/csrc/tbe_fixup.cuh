@@ -17,9 +17,9 @@
 //
 // Against one warp per bag (forward), and a block per run that looked for its pieces 32
 // at a time (backward), us. One table, 80 % of the lookups in one bag, fp32 rows of 64:
-// 20 K lookups 151 -> 38, 300 K 1427 -> 58, 1 M 2362 -> 70, 40 M 12900 -> 579; fp16 rows
-// of 128, 1 M: 4630 -> 85. Every lookup of one row, backward, fp32 columns of 64: 300 K
-// 290 -> 117, 1 M 482 -> 182, 40 M 3043 -> 1436; of 128, 1 M: 503 -> 197.
+// 20 K lookups 151 -> 38, 300 K 1427 -> 56, 1 M 2362 -> 75, 40 M 12900 -> 582; fp16 rows
+// of 128, 1 M: 4630 -> 89. Every lookup of one row, backward, fp32 columns of 64: 300 K
+// 290 -> 115, 1 M 482 -> 177, 40 M 3043 -> 1421; of 128, 1 M: 503 -> 195.
 #pragma once
 
 #include "tbe_internal.cuh"
