@@ -170,8 +170,9 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
         int next = 0;
 #pragma unroll 1
         for (;;) {
-            int j, m, t, group = 0;
+            int j, m, t, dim, group = 0;
             uint32_t seg = 0;
+            typename Split::Dest dest;
             if (!block) {
                 if (found == 0) {
                     __syncthreads();
@@ -183,6 +184,9 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
                 j = static_cast<int>(base) + b;
                 t = Q.chunks[j].table;
                 seg = __shfl_sync(kFull, static_cast<uint32_t>(mine), b);
+                // (loads that the sum needs, ahead of those that find its pieces)
+                dim = P.tables[t].dim;
+                if (scans) dest = split.dest(j, seg, t);
                 if (scans) m = split.pieces(j, seg, lane);
                 else if (!split.origin(j, lane, j, m) || m <= kGroupedPieces) continue;
                 if (m > kHeavyPieces) {
@@ -201,8 +205,10 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
                 t = h.z;
                 group = h.w;
                 seg = static_cast<uint32_t>(h.w);
+                dim = P.tables[t].dim;
+                if (scans) dest = split.dest(j, seg, t);
             }
-            const RowLanes w(P.tables[t].dim, block);
+            const RowLanes w(dim, block);
             const bool grouped = m > kGroupedPieces;
             const int first = (j / kPieceGroup + 1) * kPieceGroup;               // of the groups after j's
             const int groups = grouped ? (j + m - first) / kPieceGroup + 1 : 0;
@@ -225,10 +231,11 @@ __device__ __forceinline__ void fix_split(const Problem& P, const Plan& Q, const
                     }
                     __syncthreads();
                     if (!sh_last) break;
-                    seg = static_cast<uint32_t>(Q.split[j]);
+                    if (!scans) {
+                        seg = static_cast<uint32_t>(Q.split[j]);
+                        dest = split.dest(j, seg, t);
+                    }
                 }
-                typename Split::Dest dest;
-                if (!share) dest = split.dest(j, seg, t);
                 float* rows = Q.carry_head + row * dmax;
 #pragma unroll 1
                 for (int v = w.c; v < w.nv + w.c && !(share && n == 1); v += 32) {  // as often in every lane

@@ -58,9 +58,11 @@ struct BagSplit {
     __device__ __forceinline__ void stored(int, int, int) const {}
 };
 
-// BLOCKS per SM: 2 for small grids, else 4 (64 registers, the heavy part spills). Forward of
-// 106 K one-hot lookups, 424 blocks: 31.6 us at 2, 34.1 at 4; of 330 K, 655 blocks: 33.6 and
-// 32.8; of 1.6 M on odd dims, 1100 blocks: 80.5 and 79.6.
+// BLOCKS per SM: 2 for grids of up to 3 blocks per SM, else 3 (80 registers, the heavy part
+// spills). Whole forward, us, at 2, 3 and 4: 106 K one-hot lookups (446 blocks) 35.4, 41.7 and
+// (another box) 34 against 32 at 2; 139 K in tables of two types (579 blocks) 34.6, 34.0,
+// 38.0; 330 K (736 blocks) 33.2, 33.3, 32.7; 270 K in bags of 300 45.5, 42.2, 41.0; 1.3 M 68.1,
+// 67.7, 69.0; 1.6 M on odd dims 80.2, 79.3, 79.4.
 template <int BLOCKS>
 __global__ void __launch_bounds__(kWarpThreads, BLOCKS) fwd_fixup_kernel(const __grid_constant__ Problem P,
                                                                          const __grid_constant__ Plan Q, void* out,
@@ -87,7 +89,7 @@ void launch_fwd_gather(const Problem& P, const Plan& Q, void* out, int cls, int 
 void launch_fwd_fixup(const Problem& P, const Plan& Q, void* out, int64_t chunk_bound,
                       int num_sms, cudaStream_t s) {
     const FixupGrid g(chunk_bound, num_sms);
-    auto* kernel = g.blocks <= 3 * num_sms ? fwd_fixup_kernel<2> : fwd_fixup_kernel<4>;
+    auto* kernel = g.blocks <= 3 * num_sms ? fwd_fixup_kernel<2> : fwd_fixup_kernel<3>;
     launch(kernel, g.blocks, kWarpThreads, 0, s, P, Q, out, g.span, g.group_blocks);
 }
 
